@@ -2,8 +2,10 @@
 // SlimSell, Section III-C SlimWork, Section III-D SlimChunk, Section II-C DP).
 //
 // Vertex state lives in the relabelled row space of the layout:
-//   lvl[r]      level of row r (SS_INF while unvisited); this is the distance
-//               vector d and, for the tropical semiring, the vector f itself.
+//   claim[r]    level and parent of row r in one 64-bit word (claim_word; 0 while
+//               unvisited): the distance vector d with, for the tropical semiring,
+//               the vector f itself, and the parents (sel-max p_k, or the DP parent).
+//   vis         1-bit image of the visited rows, which SlimWork tests per chunk.
 //   fb[k&1]     1-bit image of the frontier f_k (the rows that entered at level k),
 //               double-buffered by level parity.  Every semiring's f_{k-1} is zero
 //               outside this set, so x_k = A (x) f_{k-1} only needs the semiring
@@ -15,7 +17,6 @@
 //                 real      fr[u], the path count u carried into the frontier
 //                 sel-max   id(u) + 1
 //   fr[r]       real-semiring value of row r when it entered the frontier.
-//   par[r]      parent original id + 1 (0 = none): sel-max p_k, or the DP parent.
 //
 // Neighbours are stored in descending original id, so the first frontier hit
 // of a row (in column order) is its largest-id frontier neighbour: that is the
@@ -173,85 +174,57 @@ struct RowAcc {
 };
 
 // Post-process one chunk (the frontier update of Section III-A): new rows are
-// the unvisited rows whose x_k is non-zero; they get level k, a parent and a
-// frontier bit; the chunk's SlimWork state is refreshed.  All lanes call.
+// the unvisited rows (live: bit r for this lane's row r) whose x_k is non-zero;
+// they get a claim word (level k and the parent), a frontier bit and a visited
+// bit (vis: the chunk's visited bits before).  All lanes call.
 //
 // GROUPED: the warp holds 32 / Q chunks at once, lanes g*Q .. g*Q+Q-1 owning all
 // rows of chunk g (own = this lane's group has a chunk); otherwise lanes 0..Q-1
 // own the rows of the warp's one chunk.
 template <int SR, int C, bool GROUPED = false>
-__device__ __forceinline__ void post_chunk(const Dev& d, int k, int chunk, int lane, int4 lv,
-                                           const RowAcc& a, Counters& cnt, bool own = true) {
+__device__ __forceinline__ void post_chunk(const Dev& d, int k, int chunk, int lane, unsigned live,
+                                           unsigned long long vis, const RowAcc& a, Counters& cnt,
+                                           bool own = true) {
   constexpr int Q = C / 4;
   const int lq = GROUPED ? lane % Q : lane;
   const bool owner = GROUPED ? own : lane < Q;
   const int R0 = chunk * C + 4 * lq;
-  unsigned nib = 0, left = 0;
+  unsigned nib = 0;
   if (owner) {
-    int L[4] = {lv.x, lv.y, lv.z, lv.w};
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const bool unvisited = (L[r] == SS_INF);
+    for (int r = 0; r < 4; ++r)
       // x_k is non-zero exactly where a row has a frontier neighbour (the real
       // semiring's values are positive path counts), so every semiring tests the hit
-      const bool found = a.best[r] >= 0;
-      if (unvisited && found) nib |= 1u << r;
-      else if (unvisited) left = 1;
-    }
+      if ((live >> r & 1u) && a.best[r] >= 0) nib |= 1u << r;
     if (nib) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-        if (nib >> r & 1u) {
-          L[r] = k;
-          d.par[R0 + r] = a.best[r] + 1;  // p_k = p_{k-1} + not(p_{k-1}) (.) x_k / DP parent
-          if (SR == SS_REAL) d.fr[R0 + r] = a.sum[r];
-        }
-      *reinterpret_cast<int4*>(d.lvl + R0) = make_int4(L[0], L[1], L[2], L[3]);
-      // the push variants tell visited vertices apart by their pbest slot
-      *reinterpret_cast<int4*>(d.pbest + R0) =
-          make_int4(L[0] == SS_INF ? -1 : SS_PBEST_VISITED, L[1] == SS_INF ? -1 : SS_PBEST_VISITED,
-                    L[2] == SS_INF ? -1 : SS_PBEST_VISITED, L[3] == SS_INF ? -1 : SS_PBEST_VISITED);
       const int4 dg = *reinterpret_cast<const int4*>(d.rdeg + R0);
       const int D[4] = {dg.x, dg.y, dg.z, dg.w};
 #pragma unroll
       for (int r = 0; r < 4; ++r)
         if (nib >> r & 1u) {
+          d.claim[R0 + r] = claim_word(k, a.best[r]);  // p_k = p_{k-1} + not(p_{k-1}) (.) x_k / DP parent
+          if (SR == SS_REAL) d.fr[R0 + r] = a.sum[r];
           cnt.deg += (unsigned long long)D[r];
           cnt.maxdeg = max(cnt.maxdeg, (unsigned)D[r]);
         }
       cnt.nw += __popc(nib);
     }
   }
-  unsigned lo, hi, any_left;
+  unsigned lo, hi;
   if (GROUPED) {  // OR within each group of Q lanes
     lo = (C <= 32 || lq < 8) ? nib << (4 * (lq & 7)) : 0u;
     hi = (C > 32 && lq >= 8) ? nib << (4 * (lq - 8)) : 0u;
-    any_left = left;
 #pragma unroll
     for (int o = 1; o < Q; o <<= 1) {
       lo |= __shfl_xor_sync(SS_FULL_MASK, lo, o);
       if (C > 32) hi |= __shfl_xor_sync(SS_FULL_MASK, hi, o);
-      any_left |= __shfl_xor_sync(SS_FULL_MASK, any_left, o);
     }
   } else {
     gather_bits<C>(nib, lane, &lo, &hi);
-    any_left = __any_sync(SS_FULL_MASK, left);
   }
   if (owner && lq == 0) {
     store_bits<C>(d.fb[k & 1], chunk, lo, hi);
-    d.act[chunk] = any_left ? 1 : 3;
-  }
-}
-
-// A skipped chunk (SlimWork) has only final rows, so f_k is zero there; its bits
-// in the parity buffer are cleared for the two iterations after its last
-// discovery (states 3 and 2), then left alone (state 0).
-template <int C>
-__device__ __forceinline__ void carry_chunk(const Dev& d, int k, int chunk, int lane, int a) {
-  if (a < 2) return;
-  if (lane == 0) {
-    store_bits<C>(d.fb[k & 1], chunk, 0u, 0u);
-    d.act[chunk] = (a == 3) ? 2 : 0;
+    if (lo | hi) store_bits<C>(d.vis, chunk, (unsigned)vis | lo, (unsigned)(vis >> 32) | hi);
   }
 }
 
@@ -357,6 +330,7 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
   const int wid = blockIdx.x * (PULL_THREADS / 32) + (threadIdx.x >> 5);
   const int nw = gridDim.x * (PULL_THREADS / 32);
   const unsigned* gbm = d.fb[km1 & 1];
+  constexpr unsigned long long ALL_ROWS = C == 64 ? ~0ull : (1ull << C) - 1ull;
   // stage the bitmap prefix of f_{k-1} with asynchronous 16-byte copies
   const int pv = d.ctl->prev_variant;
   const bool light = (pv == VAR_FULL || pv == VAR_SLIMWORK || pv == VAR_FILTERED) &&
@@ -393,25 +367,22 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
     const long long my_it = b0 + (long long)lane * nw;
     int4 my_item = make_int4(0, 0, 0, -1);
     long long my_start = 0;
-    int a = 0;
+    unsigned long long my_vis = ALL_ROWS;  // the chunk's visited rows
+    bool active = false;
     if (my_it < d.n_items) {
       my_item = d.items[my_it];
-      a = (MODE == MODE_FULL) ? 1 : d.act[my_item.x];
+      my_vis = chunk_bits<C>(d.vis, my_item.x);
       my_start = d.cs[my_item.x] + (long long)my_item.y * C;
+      const unsigned long long old = chunk_bits<C>(d.fb[k & 1], my_item.x);  // in flight with vis
+      active = MODE == MODE_FULL || my_vis != ALL_ROWS;
+      // a finished chunk (SlimWork) adds no row: f_k is zero there, so what
+      // f_{k-2} left in the parity buffer is cleared
+      if (!active && my_item.y == 0 && old != 0ull) store_bits<C>(d.fb[k & 1], my_item.x, 0u, 0u);
     }
-    unsigned todo = __ballot_sync(SS_FULL_MASK, a == 1);
-    if (MODE != MODE_FULL) {
-      unsigned carry = __ballot_sync(SS_FULL_MASK, a >= 2 && my_item.y == 0);
-      while (carry) {
-        const int src = __ffs(carry) - 1;
-        carry &= carry - 1;
-        carry_chunk<C>(d, k, __shfl_sync(SS_FULL_MASK, my_item.x, src), lane,
-                       __shfl_sync(SS_FULL_MASK, a, src));
-      }
-    }
+    unsigned todo = __ballot_sync(SS_FULL_MASK, active);
     // short whole chunks (at most SHORT_COLS columns, about half of all chunks of a
     // skewed graph) go 32 / Q at a time, one group of Q lanes each
-    unsigned shortm = __ballot_sync(SS_FULL_MASK, a == 1 && my_item.w < 0 &&
+    unsigned shortm = __ballot_sync(SS_FULL_MASK, active && my_item.w < 0 &&
                                                       my_item.z - my_item.y <= SHORT_COLS);
     todo &= ~shortm;
     while (shortm) {
@@ -432,11 +403,8 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
       const int lq = lane % Q;
       const int ncols = own ? item.z - item.y : 0;
       const int chunk = item.x;
-      const int4 lv = own ? *reinterpret_cast<const int4*>(d.lvl + chunk * C + 4 * lq)
-                          : make_int4(SS_PAD_LEVEL, SS_PAD_LEVEL, SS_PAD_LEVEL, SS_PAD_LEVEL);
-      const int L[4] = {lv.x, lv.y, lv.z, lv.w};
-      const unsigned live = (L[0] == SS_INF ? 1u : 0u) | (L[1] == SS_INF ? 2u : 0u) |
-                            (L[2] == SS_INF ? 4u : 0u) | (L[3] == SS_INF ? 8u : 0u);
+      const unsigned long long vis = __shfl_sync(SS_FULL_MASK, my_vis, sl);
+      const unsigned live = own ? ~(unsigned)(vis >> (4 * lq)) & 0xFu : 0u;
       int first[4] = {-1, -1, -1, -1};
       float sum[4] = {0.f, 0.f, 0.f, 0.f};
       const int4* base = reinterpret_cast<const int4*>(colp + start) + lq;
@@ -472,10 +440,10 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
       RowAcc acc;
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        acc.best[r] = (first[r] >= 0 && L[r] == SS_INF) ? __ldg(d.perm + first[r]) : -1;
+        acc.best[r] = (first[r] >= 0 && (live >> r & 1u)) ? __ldg(d.perm + first[r]) : -1;
         acc.sum[r] = sum[r];
       }
-      post_chunk<SR, C, true>(d, k, chunk, lane, lv, acc, cnt, own);
+      post_chunk<SR, C, true>(d, k, chunk, lane, live, vis, acc, cnt, own);
     }
     while (todo) {
       const int src = __ffs(todo) - 1;
@@ -496,18 +464,14 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
           prefetch_l2(colp + my_start, min(bytes, (unsigned)PREFETCH_BYTES));
         }
       }
-      // levels of this lane's 4 rows (prefetched; only this chunk's post writes them)
-      const int4 lv = *reinterpret_cast<const int4*>(d.lvl + chunk * C + 4 * (lane % Q));
-      const int L[4] = {lv.x, lv.y, lv.z, lv.w};
-      const unsigned live = (L[0] == SS_INF ? 1u : 0u) | (L[1] == SS_INF ? 2u : 0u) |
-                            (L[2] == SS_INF ? 4u : 0u) | (L[3] == SS_INF ? 8u : 0u);
+      // this lane's unvisited rows (only this chunk's post changes them)
+      const unsigned long long vis = __shfl_sync(SS_FULL_MASK, my_vis, src);
+      const unsigned live = ~(unsigned)(vis >> (4 * (lane % Q))) & 0xFu;
       int first[4] = {-1, -1, -1, -1};
       float sum[4] = {0.f, 0.f, 0.f, 0.f};
       bool need = true;
       if (MODE == MODE_FILTERED) {  // only unvisited rows are computed
-        need = false;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) need |= (L[r] == SS_INF);
+        need = live != 0u;
       }
       const int nq = (item.z - item.y) * Q;
       const int4* base = reinterpret_cast<const int4*>(colp + start);
@@ -558,7 +522,7 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
           need = false;
 #pragma unroll
           for (int r = 0; r < 4; ++r)
-            need |= (L[r] == SS_INF) && (SR == SS_REAL || first[r] < 0);
+            need |= (live >> r & 1u) && (SR == SS_REAL || first[r] < 0);
         }
       }
       if (MODE != MODE_FILTERED && lane == 0) cnt.slots += (unsigned long long)(item.z - item.y) * C;
@@ -566,7 +530,7 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
       RowAcc acc;
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        acc.best[r] = (first[r] >= 0 && L[r] == SS_INF) ? __ldg(d.perm + first[r]) : -1;
+        acc.best[r] = (first[r] >= 0 && (live >> r & 1u)) ? __ldg(d.perm + first[r]) : -1;
         acc.sum[r] = sum[r];
       }
       // (a non-zero real sum implies a hit on a live row of the same lane)
@@ -616,7 +580,7 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
         if (lane == 0) d.arrive[item.w] = 0u;
       }
       if (lane == 0) cnt.act += 1;
-      post_chunk<SR, C>(d, k, chunk, lane, lv, acc, cnt);
+      post_chunk<SR, C>(d, k, chunk, lane, live, vis, acc, cnt);
     }
   }
   if (MODE == MODE_FILTERED) cnt.slots = lane_slots;
@@ -624,26 +588,34 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
                                        IterLaunch{variant, cond, use_cond});
 }
 
+// Start of a run: nothing visited, empty frontiers.  The claim words of the rows
+// without neighbours (past n_live) are left alone: no pass reads them.
 __global__ void k_init(Dev d) {
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  for (long long r = t0; r < d.n_pad; r += stride) d.lvl[r] = r < d.n ? SS_INF : SS_PAD_LEVEL;
+  ulonglong2* claim2 = reinterpret_cast<ulonglong2*>(d.claim);  // (n_pad is a multiple of 8)
+  for (long long i = t0; i < (d.n_live + 1) / 2; i += stride) claim2[i] = make_ulonglong2(0ull, 0ull);
   for (long long w = t0; w < d.fb_words; w += stride) {
     d.fb[0][w] = 0u;
     d.fb[1][w] = 0u;
+    const long long real = d.n - 32 * w;  // rows of this word that are no padding
+    d.vis[w] = real >= 32 ? 0u : real <= 0 ? ~0u : ~0u << real;
   }
-  for (long long i = t0; i < d.n_c; i += stride) d.act[i] = 1;
   for (long long s = t0; s < (long long)d.n_split * d.C; s += stride) {
     d.xacc[s] = 0.0f;
     d.xpar[s] = -1;
   }
-  for (long long r = t0; r < d.n_pad; r += stride) d.pbest[r] = -1;  // nothing visited
   if (d.ctl->error) {  // a previous run stopped early: restore the push scratch invariant
     for (long long r = t0; r < d.n_pad; r += stride) d.psum[r] = 0.0f;
   }
 }
 
 __global__ void k_init_root(Dev d, int root) { init_root_state(d, root); }
+
+// Lower half of a claim word: parent + 1.
+__device__ __forceinline__ int* parent_half(const Dev& d, long long r) {
+  return reinterpret_cast<int*>(d.claim) + 2 * r;
+}
 
 // DP transformation as a separate pass (Section II-C): the parent of a row at
 // level L >= 1 is its largest-id neighbour at level L-1.  Neighbours are stored
@@ -673,13 +645,15 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_dp(Dev d) {
       const long long start = __shfl_sync(SS_FULL_MASK, my_start, src);
       const int chunk = item.x;
       const int R0 = chunk * C + 4 * (lane % Q);
-      const int4 lv = *reinterpret_cast<const int4*>(d.lvl + R0);
-      int tgt[4] = {lv.x, lv.y, lv.z, lv.w};
+      // upper halves of the claim words: 0x7fffffff - level, 0 while unvisited;
+      // a row's parents are the neighbours whose half is one larger than its own
+      int tgt[4];
       int hit[4];
       bool need = false;
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        tgt[r] = (tgt[r] >= 1 && tgt[r] != SS_INF) ? tgt[r] - 1 : -2;
+        const int up = (int)(d.claim[R0 + r] >> 32);
+        tgt[r] = (up > 0 && up < 0x7fffffff && R0 + r < d.n_live) ? up + 1 : -2;
         hit[r] = -1;
         need |= tgt[r] >= 0;
       }
@@ -697,10 +671,10 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_dp(Dev d) {
         int Lv[PULL_STEP][4];
 #pragma unroll
         for (int u = 0; u < PULL_STEP; ++u) {
-          Lv[u][0] = d.lvl[max(c[u].x, 0)];
-          Lv[u][1] = d.lvl[max(c[u].y, 0)];
-          Lv[u][2] = d.lvl[max(c[u].z, 0)];
-          Lv[u][3] = d.lvl[max(c[u].w, 0)];
+          Lv[u][0] = (int)(d.claim[max(c[u].x, 0)] >> 32);
+          Lv[u][1] = (int)(d.claim[max(c[u].y, 0)] >> 32);
+          Lv[u][2] = (int)(d.claim[max(c[u].z, 0)] >> 32);
+          Lv[u][3] = (int)(d.claim[max(c[u].w, 0)] >> 32);
         }
         need = false;
 #pragma unroll
@@ -724,11 +698,11 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_dp(Dev d) {
         if (item.w < 0) {
 #pragma unroll
           for (int r = 0; r < 4; ++r)
-            if (tgt[r] >= 0) d.par[R0 + r] = best[r] + 1;
+            if (tgt[r] >= 0) parent_half(d, R0 + r)[0] = best[r] + 1;
         } else {
 #pragma unroll
           for (int r = 0; r < 4; ++r)
-            if (best[r] >= 0) atomicMax(d.par + R0 + r, best[r] + 1);
+            if (best[r] >= 0) atomicMax(parent_half(d, R0 + r), best[r] + 1);
         }
       }
     }
@@ -752,7 +726,8 @@ __global__ void k_dp_clear(Dev d) {
     const int4 item = d.items[it];
     if (item.w >= 0 && item.y == 0)
       for (int l = 0; l < d.C; ++l)
-        if (d.lvl[item.x * d.C + l] >= 1) d.par[item.x * d.C + l] = 0;
+        if (item.x * d.C + l < d.n_live && (d.claim[item.x * d.C + l] >> 32) - 1u < 0x7ffffffeu)
+          *parent_half(d, item.x * d.C + l) = 0;
   }
 }
 
@@ -764,7 +739,7 @@ __global__ void k_values(Dev d, float* out) {
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < d.n;
        v += (long long)gridDim.x * blockDim.x) {
     const int r = d.invperm[v];
-    out[v] = (d.lvl[r] == SS_INF) ? 0.0f : d.fr[r];
+    out[v] = final_claim(d, r, d.ctl->root_row) ? d.fr[r] : 0.0f;
   }
 }
 

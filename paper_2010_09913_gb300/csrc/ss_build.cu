@@ -247,9 +247,10 @@ __global__ void k_identity(int* vals, int n) {
     vals[v] = (int)v;
 }
 
-// perm (padded), invperm, per-row degree
+// perm (padded), invperm, per-row degree; *n_live = 1 + the last row with a neighbour
 __global__ void k_perm_tables(const int* sorted_vals, const int* deg, int n, int n_pad, int* perm,
-                              int* invperm, int* rdeg) {
+                              int* invperm, int* rdeg, int* n_live) {
+  int live = 0;
   for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n_pad;
        r += (long long)gridDim.x * blockDim.x) {
     if (r < n) {
@@ -257,11 +258,14 @@ __global__ void k_perm_tables(const int* sorted_vals, const int* deg, int n, int
       perm[r] = v;
       invperm[v] = (int)r;
       rdeg[r] = deg[v];
+      if (deg[v] > 0) live = (int)r + 1;
     } else {
       perm[r] = -1;
       rdeg[r] = 0;
     }
   }
+  live = __reduce_max_sync(SS_FULL_MASK, live);
+  if ((threadIdx.x & 31) == 0 && live) atomicMax(n_live, live);
 }
 
 // cl[i] = longest row of chunk i; cs[i] = C * cl[i] (scanned afterwards); cs[n_c] = 0
@@ -448,7 +452,7 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
   const int nblk = (n + RS_TILE - 1) / RS_TILE;
   const long long scan_len = std::max<long long>((long long)256 * nblk, (long long)n_c + 1);
   SS_TRY(dmalloc(nullptr, (void**)&deg, sizeof(int) * (size_t)n));
-  SS_TRY(dmalloc(nullptr, (void**)&maxdeg, sizeof(int)));
+  SS_TRY(dmalloc(nullptr, (void**)&maxdeg, 2 * sizeof(int)));  // largest degree, live rows
   SS_TRY(dmalloc(nullptr, (void**)&vals_a, sizeof(int) * (size_t)n));
   SS_TRY(dmalloc(nullptr, (void**)&vals_b, sizeof(int) * (size_t)n));
   SS_TRY(dmalloc(nullptr, (void**)&keys_a, sizeof(unsigned long long) * (size_t)n));
@@ -466,7 +470,7 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
   SS_TRY(dmalloc(h, (void**)&h->cs, sizeof(long long) * (size_t)(n_c + 1)));
 
   // 1. degrees and sort keys
-  SS_TRYC(cudaMemsetAsync(maxdeg, 0, sizeof(int), st));
+  SS_TRYC(cudaMemsetAsync(maxdeg, 0, 2 * sizeof(int), st));
   k_degrees<<<grid, 256, 0, st>>>(row_ptr, n, deg, maxdeg);
   int h_maxdeg = 0;
   SS_TRYC(cudaMemcpyAsync(&h_maxdeg, maxdeg, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -498,12 +502,13 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
   SS_TRYC(cudaGetLastError());
 
   // 3. perm / invperm / row degrees, chunk lengths and starts
-  k_perm_tables<<<grid, 256, 0, st>>>(sorted, deg, n, n_pad, h->perm, h->invperm, h->rdeg);
+  k_perm_tables<<<grid, 256, 0, st>>>(sorted, deg, n, n_pad, h->perm, h->invperm, h->rdeg, maxdeg + 1);
   k_chunk_len<<<grid, 256, 0, st>>>(h->rdeg, n_c, C, h->cl, h->cs);
   SS_TRYC(cudaGetLastError());
   SS_TRY(excl_scan(h->cs, n_c + 1, tmp_scan, st));
   long long slots = 0;
   SS_TRYC(cudaMemcpyAsync(&slots, h->cs + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
+  SS_TRYC(cudaMemcpyAsync(&h->n_live, maxdeg + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
   SS_TRYC(cudaStreamSynchronize(st));
   h->slots = slots;
 
@@ -531,12 +536,12 @@ static ss_status alloc_state(slimsell_graph* h) {
   const size_t np = (size_t)h->n_pad;
   // bitmap words rounded up to whole int4 groups, plus one spare group
   h->fb_words = (long long)((((np + 31) / 32) + 3) / 4 * 4 + 4);
-  if ((s = dmalloc(h, (void**)&h->lvl, sizeof(int) * np)) != SS_OK) return s;
+  if ((s = dmalloc(h, (void**)&h->claim, sizeof(unsigned long long) * np)) != SS_OK) return s;
+  if ((s = dmalloc(h, (void**)&h->vis, sizeof(unsigned) * (size_t)h->fb_words)) != SS_OK) return s;
   if ((s = dmalloc(h, (void**)&h->act, (size_t)h->n_c)) != SS_OK) return s;
   for (int b = 0; b < 2; ++b)
     if ((s = dmalloc(h, (void**)&h->fb[b], sizeof(unsigned) * (size_t)h->fb_words)) != SS_OK) return s;
   if ((s = dmalloc(h, (void**)&h->fr, sizeof(float) * np)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->par, sizeof(int) * np)) != SS_OK) return s;
   const size_t ns = (size_t)(h->n_split > 0 ? h->n_split : 1);
   if ((s = dmalloc(h, (void**)&h->xacc, sizeof(float) * ns * h->C)) != SS_OK) return s;
   if ((s = dmalloc(h, (void**)&h->xpar, sizeof(int) * ns * h->C)) != SS_OK) return s;
@@ -546,7 +551,6 @@ static ss_status alloc_state(slimsell_graph* h) {
   // block units cover PUSH_BLOCK_SLOTS / C columns each: at most one partial unit per chunk
   h->bunits_cap = (long long)h->n_c + h->slots / PUSH_BLOCK_SLOTS + 1024;
   if ((s = dmalloc(h, (void**)&h->bunits, sizeof(int2) * (size_t)h->bunits_cap)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->pbest, sizeof(int) * np)) != SS_OK) return s;
   if ((s = dmalloc(h, (void**)&h->psum, sizeof(float) * np)) != SS_OK) return s;
   if ((s = dmalloc(h, (void**)&h->touched, sizeof(unsigned) * (size_t)h->fb_words)) != SS_OK) return s;
   for (int b = 0; b < 2; ++b) {
@@ -563,7 +567,6 @@ static ss_status alloc_state(slimsell_graph* h) {
     set_error("slimsell_build: no thread-block cluster of the push kernel fits on this device");
     return SS_ERR_CUDA;
   }
-  SS_CUDA(cudaMemset(h->pbest, 0xff, sizeof(int) * np));
   SS_CUDA(cudaMemset(h->psum, 0, sizeof(float) * np));
   SS_CUDA(cudaMemset(h->touched, 0, sizeof(unsigned) * (size_t)h->fb_words));
   if ((s = dmalloc(h, (void**)&h->ctl, sizeof(Ctl))) != SS_OK) return s;
@@ -594,8 +597,8 @@ void free_handle(slimsell_graph* h) {
   ab_release(h);
   bc_release(h);
   void* ptrs[] = {h->perm, h->invperm, h->rdeg, h->cl, h->cs, h->col, h->items, h->split_n,
-                  h->lvl, h->act, h->fb[0], h->fb[1], h->fr, h->par, h->xacc, h->xpar,
-                  h->arrive, h->ctl, h->iters, h->units, h->bunits, h->pbest,
+                  h->claim, h->vis, h->act, h->fb[0], h->fb[1], h->fr, h->xacc, h->xpar,
+                  h->arrive, h->ctl, h->iters, h->units, h->bunits,
                   h->psum, h->touched, h->qlist[0], h->qlist[1], h->qdeg[0], h->qdeg[1], h->qbase[0],
                   h->qbase[1], h->qorig[0], h->qorig[1], h->qovf, h->qovf_n, h->lstat, h->mlp, h->feats, h->mF[0],
                   h->mF[1], h->mV, h->mxacc, h->mroots};
@@ -623,17 +626,18 @@ ss::Dev slimsell_graph::dev() const {
   ss::Dev d;
   d.n = n; d.C = C; d.n_c = n_c; d.n_pad = n_pad; d.n_items = n_items; d.n_split = n_split;
   d.perm = perm; d.invperm = invperm; d.rdeg = rdeg; d.cl = cl; d.cs = cs; d.col = col;
-  d.items = items; d.split_n = split_n; d.lvl = lvl; d.act = act;
+  d.items = items; d.split_n = split_n; d.claim = claim; d.vis = vis; d.act = act;
+  d.n_live = n_live;
   d.fb[0] = fb[0]; d.fb[1] = fb[1]; d.fb_words = fb_words;
   // staged prefix: whole int4 groups, never past the allocated bitmap
   long long need = ((((long long)n_pad + 31) / 32) + 3) / 4 * 4;
   long long cap = (long long)(smem_bytes / 16) * 4;
   d.smem_words = (int)(need < cap ? need : cap);
-  d.fr = fr; d.par = par; d.xacc = xacc; d.xpar = xpar; d.arrive = arrive;
+  d.fr = fr; d.xacc = xacc; d.xpar = xpar; d.arrive = arrive;
   d.units = units; d.units_cap = units_cap;
   d.bunits = bunits; d.bunits_cap = bunits_cap; d.push_blocks = push_blocks;
   d.format = SS_FORMAT_SLIMSELL; d.scol = nullptr; d.sval = nullptr;  // set per call by slimsell_bfs
-  d.pbest = pbest; d.psum = psum; d.touched = touched; d.mlp = mlp; d.feats = feats;
+  d.psum = psum; d.touched = touched; d.mlp = mlp; d.feats = feats;
   d.sel_margin = sel_margin;
   for (int b = 0; b < 2; ++b) {
     d.qlist[b] = qlist[b]; d.qdeg[b] = qdeg[b]; d.qbase[b] = qbase[b]; d.qorig[b] = qorig[b];

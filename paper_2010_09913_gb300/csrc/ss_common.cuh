@@ -12,10 +12,7 @@
 
 #include "slimsell.h"
 
-#define SS_INF 0x7fffffff          // tropical infinity / "unvisited" level
-#define SS_PAD_LEVEL (-1)          // level of padding rows (never unvisited, never in a frontier)
 #define SS_FULL_MASK 0xffffffffu
-#define SS_PBEST_VISITED 0x7fffffff  // pbest of a visited vertex (above every original id)
 #define SS_SMEM_MAX_BYTES 212992   // frontier-bitmap prefix staged per block (1,703,936 vertices)
 #define SS_SMEM_LIMIT_BYTES 214016 // dynamic shared memory requested at most (prefix + guard)
 // threads of a pull-iteration block (one block per SM); the item order assumes it
@@ -56,6 +53,8 @@ struct Ctl {
   unsigned long long dp_slots;    // slots read by the DP pass
   unsigned int blocks_done;       // blocks of the current iteration kernel that finished
   int prev_variant;               // variant of the previous iteration (-1 before the first)
+  int root_row;                   // row of the run's root
+  int pad0;
   unsigned long long prev_slots;  // slots read by the previous iteration
   unsigned long long prev_new;    // |f_{k-1}|: vertices discovered by the previous iteration
   unsigned long long prev_deg;    // their degree sum (frontier edges)
@@ -79,6 +78,7 @@ struct Ctl {
 // Flat view of the handle's device buffers handed to kernels by value.
 struct Dev {
   int n, C, n_c, n_pad, n_items, n_split;
+  int n_live;           // rows from n_live on have no neighbours: a run reaches none but its root
   const int* perm;      // [n_pad] vertex at row position (-1 for padding rows)
   const int* invperm;   // [n] row position of vertex
   const int* rdeg;      // [n_pad] degree of the vertex at each row (0 for padding)
@@ -90,13 +90,14 @@ struct Dev {
   const float* sval;    // [slots] Sell-C-sigma values of the run's semiring (1 edge, its zero padding)
   const int4* items;    // [n_items] (chunk, j0, j1, split index or -1)
   const int* split_n;   // [n_split] items per split chunk
-  int* lvl;             // [n_pad] level (SS_INF = unvisited); the tropical f vector
-  unsigned char* act;   // [n_c] SlimWork state: 1 active, 3/2 inactive with zero writes pending, 0 inactive
+  unsigned long long* claim;  // [n_pad] claim word of a row: level and parent (claim_word), 0 = unvisited
+  unsigned* vis;        // [fb_words] visited bits of the rows (padding rows count as visited)
+  unsigned char* act;   // [n_c] multi-source SlimWork state: 1 active, 3/2 inactive with zero writes
+                        // pending, 0 inactive
   unsigned* fb[2];      // frontier bitmaps (n_pad bits each), indexed by level parity
   long long fb_words;   // allocated words per bitmap
   int smem_words;       // bitmap words staged in shared memory per block (multiple of 4)
   float* fr;            // [n_pad] real-semiring value of a row when it entered the frontier
-  int* par;             // [n_pad] parent original id + 1 (0 = none)
   float* xacc;          // [n_split * C] SlimChunk partial sums (real semiring)
   int* xpar;            // [n_split * C] SlimChunk partial parents (original id, -1 = none)
   unsigned* arrive;     // [n_split] SlimChunk arrival counters
@@ -106,8 +107,6 @@ struct Dev {
                         // block-sparse frontier: chunks whose frontier block is dense
   long long bunits_cap;
   int push_blocks;      // 0: vertex units only, 1: block units for dense blocks, 2: for every block
-  int* pbest;           // [n_pad] push: largest frontier-neighbour original id (-1 = none yet,
-                        // SS_PBEST_VISITED once the vertex has a level)
   float* psum;          // [n_pad] push: real-semiring sum of frontier-neighbour values
   unsigned* touched;    // [fb_words] push: rows reached by the current push
   int* qlist[2];        // [n_pad] vertex lists of a level (cluster push), by parity
@@ -147,6 +146,7 @@ struct slimsell_graph {
   int n = 0, C = 0, sigma = 0, split_w = 0, n_c = 0, n_pad = 0;
   long long nnz = 0, slots = 0;
   int n_items = 0, n_split = 0, max_degree = 0;
+  int n_live = 0;
   int num_sms = 0;
   // layout
   int* perm = nullptr;
@@ -158,12 +158,12 @@ struct slimsell_graph {
   int4* items = nullptr;
   int* split_n = nullptr;
   // BFS state
-  int* lvl = nullptr;
+  unsigned long long* claim = nullptr;
+  unsigned* vis = nullptr;
   unsigned char* act = nullptr;
   unsigned* fb[2] = {nullptr, nullptr};
   long long fb_words = 0;
   float* fr = nullptr;
-  int* par = nullptr;
   float* xacc = nullptr;
   int* xpar = nullptr;
   unsigned* arrive = nullptr;
@@ -172,7 +172,6 @@ struct slimsell_graph {
   int2* bunits = nullptr;
   long long bunits_cap = 0;
   int push_blocks = 1;                 // see SS_OPT_PUSH_BLOCKS
-  int* pbest = nullptr;
   float* psum = nullptr;
   unsigned* touched = nullptr;
   int* qlist[2] = {nullptr, nullptr};

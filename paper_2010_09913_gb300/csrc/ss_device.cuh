@@ -10,6 +10,29 @@ namespace ss {
 enum { VAR_FULL = SS_V_FULL, VAR_SLIMWORK = SS_V_SLIMWORK, VAR_PUSH = SS_V_PUSH,
        VAR_FILTERED = SS_V_PULL_FILTERED, VAR_PUSH_LOCAL = 4, N_VARIANTS = 5 };
 
+// Claim word of a row that enters level `level` with parent `id` (an original
+// id): 64-bit max keeps the earliest level and, within a level, the largest id,
+// so one atomicMax visits a row, keeps its canonical parent and leaves rows of
+// earlier levels alone.  0 is an unvisited row.  Level and parent share a word
+// because every reader wants both: the output gathers one 8-byte word per vertex.
+__host__ __device__ __forceinline__ unsigned long long claim_word(int level, int id) {
+  return ((unsigned long long)(unsigned)(0x7fffffff - level) << 32) | (unsigned)(id + 1);
+}
+__device__ __forceinline__ int claim_level(unsigned long long w) {  // (w != 0)
+  return 0x7fffffff - (int)(w >> 32);
+}
+__device__ __forceinline__ int claim_parent(unsigned long long w) { return (int)(unsigned)w - 1; }
+
+// The bits of one chunk's rows (bit l = row l of the chunk) in a row bitmap.
+template <int C>
+__device__ __forceinline__ unsigned long long chunk_bits(const unsigned* bm, long long chunk) {
+  if (C == 8) return reinterpret_cast<const unsigned char*>(bm)[chunk];
+  if (C == 16) return reinterpret_cast<const unsigned short*>(bm)[chunk];
+  if (C == 32) return bm[chunk];
+  const uint2 v = reinterpret_cast<const uint2*>(bm)[chunk];
+  return ((unsigned long long)v.y << 32) | v.x;
+}
+
 // Frontiers the cluster push takes: at most d.local_max_nf vertices and
 // d.local_max_e edges (SS_LOCAL_SLICE and SS_LOCAL_EDGES_PER_CTA per CTA).
 __device__ __forceinline__ bool local_fits(const Dev& d, unsigned long long nf, unsigned long long mf) {
@@ -220,12 +243,12 @@ __device__ __forceinline__ void store_features(const Dev& d, int k, const float*
 // Root state and control block of a new single-source run (one thread).
 __device__ __forceinline__ void init_root_state(const Dev& d, int root) {
   const int r = d.invperm[root];
-  d.lvl[r] = 0;
-  d.pbest[r] = SS_PBEST_VISITED;
+  d.claim[r] = claim_word(0, root);
+  d.vis[r >> 5] |= 1u << (r & 31);
   d.fb[0][r >> 5] |= 1u << (r & 31);
   d.fr[r] = 1.0f;
-  d.par[r] = root + 1;
   Ctl* c = d.ctl;
+  c->root_row = r;
   c->k = 1; c->done = 0; c->error = 0; c->variant = -1;
   c->new_count = 0; c->new_deg = 0; c->slots = 0; c->active = 0;
   c->reached = 1; c->reached_deg = (unsigned long long)d.rdeg[r];
@@ -243,14 +266,54 @@ __device__ __forceinline__ void init_root_state(const Dev& d, int root) {
   d.iters[0] = s;
 }
 
-// Distances and parents in original vertex ids (grid-stride over vertices).
+// Claim word of a row at the end of a run.  Rows past n_live have no neighbours,
+// are not initialised and hold the word of whatever run had them as its root.
+__device__ __forceinline__ unsigned long long final_claim(const Dev& d, int r, int root_row) {
+  return (r < d.n_live || r == root_row) ? d.claim[r] : 0ull;
+}
+
+// Distances and parents in original vertex ids (grid-stride over groups of four
+// vertices).  Bound by the random 8-byte gathers of the claim words (a 32-byte
+// sector each), so four are in flight per thread and the rows without
+// neighbours (half of a Kronecker graph's) gather nothing.  With one gather each for
+// level and parent over all vertices it took 22 us on Kronecker 22.
 __device__ __forceinline__ void write_outputs(const Dev& d, int* dist, int* parent) {
-  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < d.n;
-       v += (long long)gridDim.x * blockDim.x) {
-    const int r = d.invperm[v];
-    const int L = d.lvl[r];
-    if (dist) dist[v] = (L == SS_INF) ? -1 : L;
-    if (parent) parent[v] = (L == SS_INF) ? -1 : d.par[r] - 1;
+  const int root_row = d.ctl->root_row;
+  // 16-byte stores where the caller's arrays allow them
+  const bool vd = (reinterpret_cast<size_t>(dist) & 15) == 0, vp = (reinterpret_cast<size_t>(parent) & 15) == 0;
+  for (long long v = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); v < d.n;
+       v += 4LL * gridDim.x * blockDim.x) {
+    const int cnt = (int)min((long long)d.n - v, 4LL);
+    int r[4], L[4], P[4];
+    if (cnt == 4) {
+      const int4 q = *reinterpret_cast<const int4*>(d.invperm + v);
+      r[0] = q.x; r[1] = q.y; r[2] = q.z; r[3] = q.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) r[i] = d.invperm[i < cnt ? v + i : v];
+    }
+    unsigned long long w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = final_claim(d, r[i], root_row);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      L[i] = w[i] ? claim_level(w[i]) : -1;
+      P[i] = w[i] ? claim_parent(w[i]) : -1;
+    }
+    if (dist) {
+      if (vd && cnt == 4) *reinterpret_cast<int4*>(dist + v) = make_int4(L[0], L[1], L[2], L[3]);
+      else
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < cnt) dist[v + i] = L[i];
+    }
+    if (parent) {
+      if (vp && cnt == 4) *reinterpret_cast<int4*>(parent + v) = make_int4(P[0], P[1], P[2], P[3]);
+      else
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < cnt) parent[v + i] = P[i];
+    }
   }
 }
 

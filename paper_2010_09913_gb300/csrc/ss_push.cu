@@ -10,12 +10,13 @@
 //                   PUSH_UNIT neighbours;
 //   k_push_scatter  one warp per unit reads the vertex's row (column-major, so
 //                   with stride C) and, for every unvisited neighbour, folds in
-//                   the parent by atomicMax, the real value by atomicAdd and a
-//                   touched bit by atomicOr (reductions: no result is read);
+//                   level and parent by one atomicMax on its claim word, the real
+//                   value by atomicAdd and a touched bit by atomicOr (reductions:
+//                   no result is read);
 //   k_push_post     walks the touched words: a touched word becomes the
 //                   frontier word of level k (fb[k&1] held level k-2, which is
-//                   overwritten), and each touched row gets level k, parent and
-//                   value; the scratch is reset and the iteration tail runs.
+//                   overwritten) and joins the visited bits, and each touched row
+//                   gets its value; the scratch is reset and the iteration tail runs.
 #include <algorithm>
 #include <climits>
 
@@ -28,16 +29,6 @@ namespace ss {
 namespace cg = cooperative_groups;
 
 constexpr int PUSH_THREADS = 256;
-
-// The frontier bits of one chunk (bit l = row l of the chunk) in a 64-bit word.
-template <int C>
-__device__ __forceinline__ unsigned long long chunk_bits(const unsigned* fb, long long chunk) {
-  if (C == 8) return reinterpret_cast<const unsigned char*>(fb)[chunk];
-  if (C == 16) return reinterpret_cast<const unsigned short*>(fb)[chunk];
-  if (C == 32) return fb[chunk];
-  const uint2 v = reinterpret_cast<const uint2*>(fb)[chunk];
-  return ((unsigned long long)v.y << 32) | v.x;
-}
 
 // Emit the block units (chunk, first column) of chunk i, warp-aggregated; all
 // lanes call, lanes with i < 0 emit nothing.
@@ -101,14 +92,15 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_expand(Dev d) {
   }
 }
 
-// Fold the frontier row (original id origu, real value val) into neighbour v
-// when v is unvisited.
+// Fold the frontier row (claim word key, real value val) into neighbour v
+// unless v was visited at an earlier level.
 template <int SR>
-__device__ __forceinline__ void push_fold(const Dev& d, int v, int origu, float val) {
-  if (d.lvl[v] == SS_INF) {
-    // parents and touched bits only grow, so a stale read can only cause a
-    // redundant atomic, never a missed one
-    if (*(volatile const int*)(d.pbest + v) < origu) atomicMax(d.pbest + v, origu);
+__device__ __forceinline__ void push_fold(const Dev& d, int v, unsigned long long key, float val) {
+  // claim words and touched bits only grow, so a stale read can only cause a
+  // redundant atomic, never a missed one
+  const unsigned long long w = *(volatile const unsigned long long*)(d.claim + v);
+  if ((unsigned)(w >> 32) <= (unsigned)(key >> 32)) {
+    if (w < key) atomicMax(d.claim + v, key);
     if (SR == SS_REAL) atomicAdd(d.psum + v, val);
     const unsigned bit = 1u << (v & 31);
     if (!(*(volatile const unsigned*)(d.touched + (v >> 5)) & bit)) atomicOr(d.touched + (v >> 5), bit);
@@ -130,13 +122,13 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_scatter(Dev d) {
     const int deg = d.rdeg[u];
     const int chunk = u / C, l = u % C;
     const int* rowp = d.col + d.cs[chunk] + l;
-    const int origu = __ldg(d.perm + u);
+    const unsigned long long key = claim_word(c->k, __ldg(d.perm + u));
     const float val = (SR == SS_REAL) ? d.fr[u] : 0.0f;
     const int jend = min(un.y + PUSH_UNIT, deg);
     for (int j = un.y + lane; j < jend; j += 32) {
       const int v = __ldg(rowp + (long long)j * C);
       ++my_slots;
-      push_fold<SR>(d, v, origu, val);
+      push_fold<SR>(d, v, key, val);
     }
   }
   // block units: columns [j0, j0 + COLS) of a chunk whose frontier block is
@@ -169,7 +161,7 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_scatter(Dev d) {
         const int cc[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-          if ((mb >> r & 1u) && cc[r] >= 0) push_fold<SR>(d, cc[r], origs[r], vals[r]);
+          if ((mb >> r & 1u) && cc[r] >= 0) push_fold<SR>(d, cc[r], claim_word(c->k, origs[r]), vals[r]);
       }
     }
   }
@@ -198,13 +190,11 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_post(Dev d, IterLaunch il
        w += (long long)gridDim.x * blockDim.x) {
     unsigned bits = d.touched[w];
     fbk[w] = bits;  // f_k: exactly the rows first reached now
+    if (bits) d.vis[w] |= bits;
     while (bits) {
       const int b = __ffs(bits) - 1;
       bits &= bits - 1;
       const int v = (int)(w * 32 + b);
-      d.lvl[v] = k;
-      d.par[v] = d.pbest[v] + 1;  // largest-id frontier neighbour + 1
-      d.pbest[v] = SS_PBEST_VISITED;
       if (SR == SS_REAL) {
         d.fr[v] = d.psum[v];
         d.psum[v] = 0.0f;
@@ -230,12 +220,12 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_post(Dev d, IterLaunch il
 // rows longer than LOCAL_UNIT edges being cut into units spread round-robin
 // over the cluster.  Per level a CTA scatters over its share's edges (each
 // thread a contiguous run: one binary search, then a forward walk) and claims
-// each candidate with one atomicMax on its parent slot: the old value -1 makes
-// this CTA the vertex's owner, visited vertices hold SS_PBEST_VISITED (no id
-// is larger, so their slot never changes), and the slot ends with the largest
-// id among the frontier neighbours, the parent.  Two hardware cluster barriers
-// per level order the scatter before the post step (which reads the final
-// parents) and the post step before the next level; per-CTA counts and
+// each candidate with one atomicMax on its claim word: the old value 0 makes
+// this CTA the vertex's owner, words of earlier levels are larger and never
+// change, and the word ends with this level and the largest id among the
+// frontier neighbours, the parent.  Two hardware cluster barriers per level
+// order the scatter before the post step (which reads the final counts) and
+// the post step before the next level; per-CTA counts and
 // statistics reach every CTA through distributed shared memory.  Spreading the
 // random accesses over many SMs is what makes a level cheap: one SM's L1
 // serves about one uncoalesced line per clock.  Every CTA keeps a copy of the
@@ -249,7 +239,7 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_post(Dev d, IterLaunch il
 //   qlist/qdeg/qbase/qorig[(k-1)&1] = level k-1, qlist[k&1] = level k-2 (lengths in qlen).
 // ---------------------------------------------------------------------------
 constexpr int LOCAL_THREADS = 1024;
-constexpr int LOCAL_BATCH = 16;     // candidate edges per thread in flight
+constexpr int LOCAL_BATCH = 8;      // candidate edges per thread in flight (a full slice: 8 per thread)
 constexpr int LOCAL_NEWCAP = 8192;  // new vertices per CTA kept in shared memory
 constexpr int LOCAL_POST = 2;       // new vertices per thread in flight in the post step
 constexpr int LOCAL_UNIT = 1024;    // edges of one slice entry; longer rows become several units
@@ -400,13 +390,13 @@ __device__ __forceinline__ void local_features(const Dev& d, LocalSmem& S, cg::c
 
 // One scatter pass of the cluster push: thread tid takes edges [ea, ea + per) of
 // the slice (per <= B), finds their rows by one binary search and a forward walk,
-// loads the neighbours, and claims each with one atomicMax (all B in flight
-// before any result is used); one atomicMax both claims a vertex (old value -1),
-// keeps the largest-id parent and tells visited vertices apart (their slot holds
-// SS_PBEST_VISITED, which no id exceeds).
+// loads the neighbours, and claims each with one atomicMax on its claim word (all
+// B in flight before any result is used): the old value 0 makes this thread the
+// vertex's first discoverer, the word keeps level and largest-id parent, and words
+// of earlier levels are larger, so visited vertices keep theirs.
 template <int SR, int C, int B>
 __device__ __forceinline__ void local_scatter(const Dev& d, LocalSmem& S, int p0, int p1, int ns, int e0,
-                                              int per, int Es, int tid) {
+                                              int per, int Es, int tid, int k) {
   const int* sid = S.sid[p1];
   const int ea = e0 + tid * per;
   const int eb = min(ea + per, Es);
@@ -435,20 +425,21 @@ __device__ __forceinline__ void local_scatter(const Dev& d, LocalSmem& S, int p0
       if (SR == SS_REAL) fu[q] = __ldcg(d.fr + sid[i]);  // written during this launch: past L1
     }
   }
-  int old[B];
+  unsigned long long old[B];
 #pragma unroll
   for (int q = 0; q < B; ++q) {
-    old[q] = SS_PBEST_VISITED;
-    if (v[q] >= 0) old[q] = atomicMax(d.pbest + v[q], S.orig[src[q]]);
+    old[q] = ~0ull;
+    if (v[q] >= 0) old[q] = atomicMax(d.claim + v[q], claim_word(k, S.orig[src[q]]));
   }
-  if (SR == SS_REAL) {
+  if (SR == SS_REAL) {  // a neighbour not visited at an earlier level
+    const unsigned lev = 0x7fffffffu - (unsigned)k;
 #pragma unroll
     for (int q = 0; q < B; ++q)
-      if (old[q] != SS_PBEST_VISITED) atomicAdd(d.psum + v[q], fu[q]);
+      if ((unsigned)(old[q] >> 32) <= lev) atomicAdd(d.psum + v[q], fu[q]);
   }
 #pragma unroll
   for (int q = 0; q < B; ++q) {
-    if (old[q] < 0) {  // first discoverer: this CTA owns the vertex
+    if (old[q] == 0ull) {  // first discoverer: this CTA owns the vertex
       const int idx = atomicAdd(&S.nnew, 1);
       if (idx < LOCAL_NEWCAP) {
         S.nid[idx] = v[q];
@@ -471,7 +462,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 template <int SR, int C>
 __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaunch il, int max_levels,
                                                                  int time_levels) {
-  constexpr int BATCH = (SR == SS_REAL) ? LOCAL_BATCH / 2 : LOCAL_BATCH;  // registers
+  constexpr int BATCH = LOCAL_BATCH;
   LocalSmem& S = *reinterpret_cast<LocalSmem*>(ss_local_smem);
   // per-level timing (profiling): the first level also carries the launch's entry
   unsigned long long t_prev = time_levels ? global_ns() : 0ull;
@@ -626,9 +617,9 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
     for (int e0 = 0; e0 < Es; e0 += LOCAL_THREADS * BATCH) {
       const int per = min(BATCH, (Es - e0 + LOCAL_THREADS - 1) / LOCAL_THREADS);
       if (per <= 4)
-        local_scatter<SR, C, 4>(d, S, p0, p1, ns, e0, per, Es, tid);
+        local_scatter<SR, C, 4>(d, S, p0, p1, ns, e0, per, Es, tid, k);
       else
-        local_scatter<SR, C, BATCH>(d, S, p0, p1, ns, e0, per, Es, tid);
+        local_scatter<SR, C, BATCH>(d, S, p0, p1, ns, e0, per, Es, tid, k);
     }
     __syncthreads();
     if (tid < G) {  // tell every CTA how many vertices this one found
@@ -669,7 +660,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
     unsigned long long nd = 0;
     unsigned md = 0;
     for (int i0 = 0; i0 < cnt; i0 += LOCAL_POST * LOCAL_THREADS) {
-      int vv[LOCAL_POST], pb[LOCAL_POST], dv[LOCAL_POST], og[LOCAL_POST];
+      int vv[LOCAL_POST], dv[LOCAL_POST], og[LOCAL_POST];
       long long csv[LOCAL_POST];
       float fv[LOCAL_POST];
 #pragma unroll
@@ -681,7 +672,6 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
 #pragma unroll
       for (int q = 0; q < LOCAL_POST; ++q) {  // every load of the batch before any store
         if (vv[q] >= 0) {
-          pb[q] = __ldcg(d.pbest + vv[q]);
           dv[q] = __ldg(d.rdeg + vv[q]);
           csv[q] = __ldg(d.cs + vv[q] / C);
           og[q] = __ldg(d.perm + vv[q]);
@@ -692,14 +682,12 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
       for (int q = 0; q < LOCAL_POST; ++q) {
         if (vv[q] < 0) continue;
         const int x = vv[q];
-        d.lvl[x] = k;
-        d.par[x] = pb[q] + 1;  // largest-id frontier neighbour + 1
-        d.pbest[x] = SS_PBEST_VISITED;
         if (SR == SS_REAL) {
           d.fr[x] = fv[q];
           d.psum[x] = 0.0f;
         }
         atomicOr(fbk + (x >> 5), 1u << (x & 31));
+        atomicOr(d.vis + (x >> 5), 1u << (x & 31));
         const long long at = off + i0 + q * LOCAL_THREADS + tid;
         const long long bx = csv[q] + (x % C);
         d.qlist[p0][at] = x;
