@@ -57,10 +57,31 @@ namespace ss {
 #endif
 
 constexpr int PULL_THREADS = SS_PULL_THREADS;  // one block per SM
+#ifndef SS_FILTERED_THREADS
+#define SS_FILTERED_THREADS 640
+#endif
+constexpr int FILTERED_THREADS = SS_FILTERED_THREADS;
 #ifndef SS_PULL_SHORT_COLS
 #define SS_PULL_SHORT_COLS 4
 #endif
 constexpr int SHORT_COLS = SS_PULL_SHORT_COLS;  // chunks this short go several per warp
+// The filtered pull's chunks in groups of C/4 lanes: every unsplit chunk starts in a
+// group and goes on in a whole warp once it is still open after GROUP_TRY columns
+// with more than GROUP_LEFT left (8 / 32: 314 us for ER 4 M's largest level; leaving
+// with more than 8 left 344, trying 4 columns 322).  The real semiring needs whole
+// sums, so there only chunks of at most GROUP_COLS columns go in groups.
+#ifndef SS_PULL_GROUP_COLS
+#define SS_PULL_GROUP_COLS 8
+#endif
+#ifndef SS_PULL_GROUP_TRY
+#define SS_PULL_GROUP_TRY 8
+#endif
+#ifndef SS_PULL_GROUP_LEFT
+#define SS_PULL_GROUP_LEFT 32
+#endif
+constexpr int GROUP_COLS = SS_PULL_GROUP_COLS;
+constexpr int GROUP_TRY = SS_PULL_GROUP_TRY;
+constexpr int GROUP_LEFT = SS_PULL_GROUP_LEFT;
 
 // int4 col loads in flight per lane (4 slots each)
 template <int SR, int FMT>
@@ -176,7 +197,8 @@ struct RowAcc {
 // Post-process one chunk (the frontier update of Section III-A): new rows are
 // the unvisited rows (live: bit r for this lane's row r) whose x_k is non-zero;
 // they get a claim word (level k and the parent), a frontier bit and a visited
-// bit (vis: the chunk's visited bits before).  All lanes call.
+// bit (vis: the chunk's visited bits before; prev: rows of this chunk that entered
+// the frontier earlier in this pass; *added: the new rows' bits).  All lanes call.
 //
 // GROUPED: the warp holds 32 / Q chunks at once, lanes g*Q .. g*Q+Q-1 owning all
 // rows of chunk g (own = this lane's group has a chunk); otherwise lanes 0..Q-1
@@ -184,7 +206,8 @@ struct RowAcc {
 template <int SR, int C, bool GROUPED = false>
 __device__ __forceinline__ void post_chunk(const Dev& d, int k, int chunk, int lane, unsigned live,
                                            unsigned long long vis, const RowAcc& a, Counters& cnt,
-                                           bool own = true) {
+                                           bool own = true, unsigned long long prev = 0ull,
+                                           unsigned long long* added = nullptr) {
   constexpr int Q = C / 4;
   const int lq = GROUPED ? lane % Q : lane;
   const bool owner = GROUPED ? own : lane < Q;
@@ -223,9 +246,10 @@ __device__ __forceinline__ void post_chunk(const Dev& d, int k, int chunk, int l
     gather_bits<C>(nib, lane, &lo, &hi);
   }
   if (owner && lq == 0) {
-    store_bits<C>(d.fb[k & 1], chunk, lo, hi);
+    store_bits<C>(d.fb[k & 1], chunk, lo | (unsigned)prev, hi | (unsigned)(prev >> 32));
     if (lo | hi) store_bits<C>(d.vis, chunk, (unsigned)vis | lo, (unsigned)(vis >> 32) | hi);
   }
+  if (added) *added = ((unsigned long long)hi << 32) | lo;
 }
 
 // Scan the slots of one quad: record the first frontier hit per row and, for
@@ -312,6 +336,53 @@ __device__ __forceinline__ void gather_step(const Dev& d, const int4* c, const u
 
 extern __shared__ __align__(16) unsigned ss_smem_bits[];
 
+// The frontier bitmap as a block reads it: words of the staged prefix (sbits bits)
+// from shared memory, the rest from global memory; real semiring on hub levels:
+// the values of the rows below sf from shared memory too.
+struct Staged {
+  const unsigned* sm;
+  const float* smf;
+  int sbits, sf;
+};
+
+// Stage the prefix of f_{k-1}'s bitmap gbm with asynchronous 16-byte copies (all
+// threads of the block call; the copies run until stage_wait).
+template <int SR>
+__device__ __forceinline__ Staged stage_frontier(const Dev& d, const unsigned* gbm) {
+  const int pv = d.ctl->prev_variant;
+  const bool light = (pv == VAR_FULL || pv == VAR_SLIMWORK || pv == VAR_FILTERED) &&
+                     d.ctl->prev_slots < STAGE_MIN_SLOTS;
+  const int sw_all = light ? 0 : d.smem_words;
+  // real semiring on a level whose frontier carries a large share of the edges
+  // (the hub level of a skewed graph): the last sf words of the staging area
+  // hold the values fr of the sf highest-degree rows instead of bitmap words
+  const bool hub = SR == SS_REAL && (unsigned long long)d.ctl->prev_deg * HUB_EDGE_SHARE >
+                                        (unsigned long long)d.nnz;
+  const int sf = hub ? min(HUB_VALUE_ROWS, (sw_all >> 1) & ~3) : 0;
+  const int sw = sw_all - sf;  // bitmap words staged (a multiple of 4)
+  if (threadIdx.x < SMEM_GUARD) ss_smem_bits[threadIdx.x] = 0u;
+  const unsigned sbase = (unsigned)__cvta_generic_to_shared(ss_smem_bits + SMEM_GUARD);
+  for (int i = threadIdx.x; i < (sw >> 2); i += blockDim.x)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sbase + 16u * (unsigned)i),
+                 "l"(reinterpret_cast<const int4*>(gbm) + i)
+                 : "memory");
+  const unsigned fbase = sbase + 4u * (unsigned)sw;
+  for (int i = threadIdx.x; i < (sf >> 2); i += blockDim.x)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(fbase + 16u * (unsigned)i),
+                 "l"(reinterpret_cast<const int4*>(d.fr) + i)
+                 : "memory");
+  Staged s;
+  s.sm = ss_smem_bits + SMEM_GUARD;
+  s.smf = reinterpret_cast<const float*>(s.sm + sw);
+  s.sbits = sw * 32;
+  s.sf = sf;
+  return s;
+}
+__device__ __forceinline__ void stage_wait() {
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
+}
+
 // One frontier expansion x_k = A (x)_S f_{k-1} with fused post-processing.
 // Warp w of the grid owns items w, w + W, w + 2W, ... (W = warps in the grid,
 // the item list is ordered for that assignment); it reads the descriptors and
@@ -331,38 +402,12 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
   const int nw = gridDim.x * (PULL_THREADS / 32);
   const unsigned* gbm = d.fb[km1 & 1];
   constexpr unsigned long long ALL_ROWS = C == 64 ? ~0ull : (1ull << C) - 1ull;
-  // stage the bitmap prefix of f_{k-1} with asynchronous 16-byte copies
-  const int pv = d.ctl->prev_variant;
-  const bool light = (pv == VAR_FULL || pv == VAR_SLIMWORK || pv == VAR_FILTERED) &&
-                     d.ctl->prev_slots < STAGE_MIN_SLOTS;
-  const int sw_all = light ? 0 : d.smem_words;
-  // real semiring on a level whose frontier carries a large share of the edges
-  // (the hub level of a skewed graph): the last sf words of the staging area
-  // hold the values fr of the sf highest-degree rows instead of bitmap words
-  const bool hub = SR == SS_REAL && (unsigned long long)d.ctl->prev_deg * HUB_EDGE_SHARE >
-                                        (unsigned long long)d.nnz;
-  const int sf = hub ? min(HUB_VALUE_ROWS, (sw_all >> 1) & ~3) : 0;
-  const int sw = sw_all - sf;  // bitmap words staged (a multiple of 4)
-  {
-    if (threadIdx.x < SMEM_GUARD) ss_smem_bits[threadIdx.x] = 0u;
-    const unsigned sbase = (unsigned)__cvta_generic_to_shared(ss_smem_bits + SMEM_GUARD);
-    for (int i = threadIdx.x; i < (sw >> 2); i += PULL_THREADS)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sbase + 16u * (unsigned)i),
-                   "l"(reinterpret_cast<const int4*>(gbm) + i)
-                   : "memory");
-    const unsigned fbase = sbase + 4u * (unsigned)sw;
-    for (int i = threadIdx.x; i < (sf >> 2); i += PULL_THREADS)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(fbase + 16u * (unsigned)i),
-                   "l"(reinterpret_cast<const int4*>(d.fr) + i)
-                   : "memory");
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-  }
-  __syncthreads();
-  const unsigned* sm = ss_smem_bits + SMEM_GUARD;
-  const float* smf = reinterpret_cast<const float*>(sm + sw);
-  const int sbits = sw * 32;
+  const Staged sg = stage_frontier<SR>(d, gbm);
+  stage_wait();
+  const unsigned* sm = sg.sm;
+  const float* smf = sg.smf;
+  const int sbits = sg.sbits, sf = sg.sf;
   Counters cnt;
-  unsigned long long lane_slots = 0;
   for (long long b0 = wid; b0 < d.n_items; b0 += 32LL * nw) {
     const long long my_it = b0 + (long long)lane * nw;
     int4 my_item = make_int4(0, 0, 0, -1);
@@ -434,9 +479,8 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
       }
       if (own && lq == 0) {
         cnt.act += 1;
-        if (MODE != MODE_FILTERED) cnt.slots += (unsigned long long)ncols * C;
+        cnt.slots += (unsigned long long)ncols * C;
       }
-      if (MODE == MODE_FILTERED) lane_slots += 4ull * ncols;
       RowAcc acc;
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
@@ -469,18 +513,10 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
       const unsigned live = ~(unsigned)(vis >> (4 * (lane % Q))) & 0xFu;
       int first[4] = {-1, -1, -1, -1};
       float sum[4] = {0.f, 0.f, 0.f, 0.f};
-      bool need = true;
-      if (MODE == MODE_FILTERED) {  // only unvisited rows are computed
-        need = live != 0u;
-      }
       const int nq = (item.z - item.y) * Q;
       const int4* base = reinterpret_cast<const int4*>(colp + start);
       const int4* vbase = reinterpret_cast<const int4*>(d.sval + start);  // (Sell only)
       for (int q0 = 0; q0 < nq; q0 += 32 * PULL_STEP) {
-        if (MODE == MODE_FILTERED) {
-          if (!__any_sync(SS_FULL_MASK, need)) break;
-          if (!need) continue;
-        }
         // keep the prefetch PREFETCH_BYTES ahead inside long items (one lane issues it)
         if (lane == 0) {
           const long long ahead = (long long)(q0 + 32 * PULL_STEP) * 16 + PREFETCH_BYTES;
@@ -505,7 +541,6 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
           } else {
             v[u] = make_int4(0, 0, 0, 0);
           }
-          if (MODE == MODE_FILTERED && q < nq) lane_slots += 4;
         }
         if constexpr (SR == SS_REAL && FMT == SS_FORMAT_SLIMSELL) {
           unsigned mm[PULL_STEP];
@@ -518,14 +553,8 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
           for (int u = 0; u < PULL_STEP; ++u)  // (q0 + 32 u < nq is warp-uniform)
             if (q0 + 32 * u < nq) scan_quad<SR, FMT>(d, sm, sbits, gbm, c[u], v[u], first, sum, live, smf, sf);
         }
-        if (MODE == MODE_FILTERED) {  // a row is done once visited or (not real) hit
-          need = false;
-#pragma unroll
-          for (int r = 0; r < 4; ++r)
-            need |= (live >> r & 1u) && (SR == SS_REAL || first[r] < 0);
-        }
       }
-      if (MODE != MODE_FILTERED && lane == 0) cnt.slots += (unsigned long long)(item.z - item.y) * C;
+      if (lane == 0) cnt.slots += (unsigned long long)(item.z - item.y) * C;
       // the largest original id among this lane's first hits of unvisited rows
       RowAcc acc;
 #pragma unroll
@@ -583,8 +612,330 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
       post_chunk<SR, C>(d, k, chunk, lane, live, vis, acc, cnt);
     }
   }
-  if (MODE == MODE_FILTERED) cnt.slots = lane_slots;
   finish_iteration_block<PULL_THREADS>(d, cnt.nw, cnt.deg, cnt.slots, cnt.act, cnt.maxdeg,
+                                       IterLaunch{variant, cond, use_cond});
+}
+
+// The visited-filtered pull: as k_pull, but only unvisited rows are computed and
+// (but for the real semiring) a row stops at its first frontier neighbour.
+//
+// Hub levels find most rows within their first columns, so what a pass costs is
+// not the stream but the latency chain of each chunk (descriptor, columns, bits,
+// parent, row data).  Hence chunks start in groups of C/4 lanes (32 / (C/4) at a
+// time, GSTEP columns a step, each group taking its next chunk on its own), and
+// the next loads are issued before the finished chunks are post-processed; only
+// long rests and split items take a whole warp.  Reading 16 columns at once with
+// // one chunk per warp took 58 us on Kronecker 22's level after the hubs and 395 us on
+// ER 4 M's largest; this takes 45 and 230 (GSTEP 4: 248; without leaving out the
+// lookups of rows already hit 314).  640 threads, for the registers (768: 246 at
+// GSTEP 4; 1024 spills).
+template <int SR, int C>
+__global__ void __launch_bounds__(FILTERED_THREADS, 1) k_pull_filtered(Dev d, int variant,
+                                                                       cudaGraphConditionalHandle cond,
+                                                                       int use_cond) {
+  constexpr int FMT = SS_FORMAT_SLIMSELL;
+  constexpr int PULL_STEP = pull_step<SR, FMT>();
+  const int* colp = d.col;
+  constexpr int Q = C / 4;
+  if (d.ctl->done) return;
+  const int k = d.ctl->k;
+  const int km1 = k - 1;
+  const int lane = threadIdx.x & 31;
+  const int wid = blockIdx.x * (FILTERED_THREADS / 32) + (threadIdx.x >> 5);
+  const int nw = gridDim.x * (FILTERED_THREADS / 32);
+  const unsigned* gbm = d.fb[km1 & 1];
+  constexpr unsigned long long ALL_ROWS = C == 64 ? ~0ull : (1ull << C) - 1ull;
+  const Staged sg = stage_frontier<SR>(d, gbm);
+  stage_wait();
+  const unsigned* sm = sg.sm;
+  const float* smf = sg.smf;
+  const int sbits = sg.sbits, sf = sg.sf;
+  Counters cnt;
+  unsigned long long lane_slots = 0;
+  for (long long b0 = wid; b0 < d.n_items; b0 += 32LL * nw) {
+    const long long my_it = b0 + (long long)lane * nw;
+    int4 my_item = make_int4(0, 0, 0, -1);
+    long long my_start = 0;
+    unsigned long long my_vis = ALL_ROWS;  // the chunk's visited rows
+    bool active = false;
+    if (my_it < d.n_items) {
+      my_item = d.items[my_it];
+      my_vis = chunk_bits<C>(d.vis, my_item.x);
+      my_start = d.cs[my_item.x] + (long long)my_item.y * C;
+      const unsigned long long old = chunk_bits<C>(d.fb[k & 1], my_item.x);  // in flight with vis
+      active = my_vis != ALL_ROWS;
+      // a finished chunk (SlimWork) adds no row: f_k is zero there, so what
+      // f_{k-2} left in the parity buffer is cleared
+      if (!active && my_item.y == 0 && old != 0ull) store_bits<C>(d.fb[k & 1], my_item.x, 0u, 0u);
+    }
+    unsigned todo = __ballot_sync(SS_FULL_MASK, active);
+    // chunks in groups of Q lanes (see GROUP_COLS).  Each group works through its own
+    // chunk GSTEP columns at a time and takes the next one when it is done; the loads
+    // of the next step are issued before the finished chunks are post-processed.
+    unsigned long long my_new = 0ull;  // rows of this lane's item that the groups have found
+    {
+      constexpr int GROUPS = 32 / Q;
+      constexpr int GSTEP = 2;
+      constexpr bool EARLY = SR != SS_REAL;  // rows stop at their first hit
+      const int lq = lane % Q;
+      unsigned gm = __ballot_sync(SS_FULL_MASK, active && my_item.w < 0 &&
+                                                    (EARLY || my_item.z - my_item.y <= GROUP_COLS));
+      todo &= ~gm;
+      int src = -1, chunk = 0, rem = 0;  // this group's item (its lane), chunk and columns left
+      unsigned live = 0;                 // this lane's unvisited rows of it
+      unsigned long long vis = 0ull;     // its visited rows
+      const int4* cp = nullptr;
+      int first[4];
+      float sum[4];
+      int4 c[GSTEP];
+      // groups that want an item take the next ones; their first step is loaded
+      auto take = [&](bool want) {
+        const unsigned wm = __ballot_sync(SS_FULL_MASK, want);
+        int got = -1;
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g)
+          if (wm >> (g * Q) & 1u) {
+            const int nxt = gm ? __ffs(gm) - 1 : -1;
+            gm &= gm - 1;
+            if (lane / Q == g) got = nxt;
+          }
+        const int sl = got >= 0 ? got : 0;
+        const int nchunk = __shfl_sync(SS_FULL_MASK, my_item.x, sl);
+        const int ncols = __shfl_sync(SS_FULL_MASK, my_item.z, sl) - __shfl_sync(SS_FULL_MASK, my_item.y, sl);
+        const long long start = __shfl_sync(SS_FULL_MASK, my_start, sl);
+        const unsigned long long nvis = __shfl_sync(SS_FULL_MASK, my_vis, sl);
+        if (want) {
+          src = got;
+          rem = got >= 0 ? ncols : 0;
+          chunk = nchunk;
+          vis = nvis;
+          live = got >= 0 ? ~(unsigned)(nvis >> (4 * lq)) & 0xFu : 0u;
+          cp = reinterpret_cast<const int4*>(colp + start) + lq;
+          if (got >= 0 && lq == 0) {
+            cnt.act += 1;
+          }
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            first[r] = -1;
+            sum[r] = 0.f;
+          }
+        }
+      };
+      auto load = [&]() {
+        unsigned open = live;
+        if (EARLY) {
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (first[r] >= 0) open &= ~(1u << r);
+        }
+        const int n = open ? rem : 0;
+        lane_slots += 4ull * (unsigned)max(0, min(n, GSTEP));
+#pragma unroll
+        for (int u = 0; u < GSTEP; ++u) {
+          c[u] = (u < n) ? ld_stream(cp + u * Q) : make_int4(-1, -1, -1, -1);
+        }
+      };
+      if (gm) {
+        take(true);
+        load();
+      }
+      while (__any_sync(SS_FULL_MASK, src >= 0)) {
+        if constexpr (SR == SS_REAL) {
+          unsigned mm[GSTEP];
+#pragma unroll
+          for (int u = 0; u < GSTEP; ++u) mm[u] = quad_hits(sm, sbits, gbm, c[u], first) & live;
+          gather_step<GSTEP>(d, c, mm, sum, smf, sf);
+        } else {
+          // rows hit in an earlier step (or visited) look nothing up: past the staged
+          // prefix a lookup is a memory gather
+          bool shut[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) shut[r] = EARLY && (first[r] >= 0 || !(live >> r & 1u));
+#pragma unroll
+          for (int u = 0; u < GSTEP; ++u) {
+            const int4 q = make_int4(shut[0] ? -1 : c[u].x, shut[1] ? -1 : c[u].y, shut[2] ? -1 : c[u].z,
+                                     shut[3] ? -1 : c[u].w);
+            scan_quad<SR, FMT>(d, sm, sbits, gbm, q, make_int4(0, 0, 0, 0), first, sum, live, smf, sf);
+          }
+        }
+        rem -= GSTEP;
+        cp += GSTEP * Q;
+        bool fin = src >= 0 && rem <= 0, leave = false;
+        if (EARLY) {  // done once every row is visited or hit
+          unsigned open = 0;
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if ((live >> r & 1u) && first[r] < 0) open = 1;
+#pragma unroll
+          for (int o = 1; o < Q; o <<= 1) open |= __shfl_xor_sync(SS_FULL_MASK, open, o);
+          fin = fin || (src >= 0 && !open);
+          // a long rest goes to the whole warp (from this column on)
+          const int used = __shfl_sync(SS_FULL_MASK, my_item.z, max(src, 0)) -
+                           __shfl_sync(SS_FULL_MASK, my_item.y, max(src, 0)) - rem;
+          leave = src >= 0 && !fin && used >= GROUP_TRY && rem > GROUP_LEFT;
+        }
+        const bool out = fin || leave;
+        if (__any_sync(SS_FULL_MASK, out)) {
+          const int ochunk = chunk, osrc = src, orem = rem;
+          const unsigned olive = live;
+          const unsigned long long ovis = vis;
+          RowAcc acc;
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            acc.best[r] = (out && first[r] >= 0 && (live >> r & 1u)) ? first[r] : -1;
+            acc.sum[r] = sum[r];
+          }
+          take(out);
+          load();
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (acc.best[r] >= 0) acc.best[r] = __ldg(d.perm + acc.best[r]);
+          unsigned long long added;
+          post_chunk<SR, C, true>(d, k, ochunk, lane, olive, ovis, acc, cnt, out, 0ull, &added);
+          if (EARLY) {  // hand the left chunks over: lane s holds item s
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) {
+              const int s = __shfl_sync(SS_FULL_MASK, leave ? osrc : -1, g * Q);
+              const int left = __shfl_sync(SS_FULL_MASK, orem, g * Q);
+              const unsigned long long nb = __shfl_sync(SS_FULL_MASK, added, g * Q);
+              if (s >= 0) {
+                todo |= 1u << s;
+                if (lane == s) {
+                  const int y = my_item.z - left;
+                  my_start += (long long)(y - my_item.y) * C;
+                  my_item.y = y;
+                  my_new = nb;
+                  my_vis |= nb;
+                }
+              }
+            }
+          }
+        } else {
+          load();
+        }
+      }
+    }
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int4 item = shfl_int4(my_item, src);
+      const long long start = __shfl_sync(SS_FULL_MASK, my_start, src);
+      const int chunk = item.x;
+      // L2 prefetch: the head of this item beyond the first step, and of the next item
+      if (lane == src) {
+        const unsigned bytes = (unsigned)(item.z - item.y) * C * 4u;
+        if (bytes > 2048u)
+          prefetch_l2(colp + start + 512, min(bytes - 2048u, (unsigned)PREFETCH_BYTES));
+      }
+      if (todo) {
+        const int nxt = __ffs(todo) - 1;
+        if (lane == nxt) {
+          const unsigned bytes = (unsigned)(my_item.z - my_item.y) * C * 4u;
+          prefetch_l2(colp + my_start, min(bytes, (unsigned)PREFETCH_BYTES));
+        }
+      }
+      // this lane's unvisited rows (only this chunk's post changes them)
+      const unsigned long long vis = __shfl_sync(SS_FULL_MASK, my_vis, src);
+      const unsigned live = ~(unsigned)(vis >> (4 * (lane % Q))) & 0xFu;
+      int first[4] = {-1, -1, -1, -1};
+      float sum[4] = {0.f, 0.f, 0.f, 0.f};
+      bool need = live != 0u;  // only unvisited rows are computed
+      const int nq = (item.z - item.y) * Q;
+      const int4* base = reinterpret_cast<const int4*>(colp + start);
+      for (int q0 = 0; q0 < nq; q0 += 32 * PULL_STEP) {
+        if (!__any_sync(SS_FULL_MASK, need)) break;
+        if (!need) continue;
+        // keep the prefetch PREFETCH_BYTES ahead inside long items (one lane issues it)
+        if (lane == 0) {
+          const long long ahead = (long long)(q0 + 32 * PULL_STEP) * 16 + PREFETCH_BYTES;
+          const long long total = (long long)nq * 16;
+          if (ahead < total) {
+            prefetch_l2(reinterpret_cast<const char*>(base) + ahead,
+                        (unsigned)min(total - ahead, (long long)(32 * PULL_STEP * 16)));
+          }
+        }
+        int4 c[PULL_STEP];
+#pragma unroll
+        for (int u = 0; u < PULL_STEP; ++u) {
+          const int q = q0 + lane + 32 * u;
+          c[u] = (q < nq) ? ld_stream(base + q) : make_int4(-1, -1, -1, -1);
+          if (q < nq) lane_slots += 4;
+        }
+        if constexpr (SR == SS_REAL) {
+          unsigned mm[PULL_STEP];
+#pragma unroll
+          for (int u = 0; u < PULL_STEP; ++u)
+            mm[u] = (q0 + 32 * u < nq) ? quad_hits(sm, sbits, gbm, c[u], first) & live : 0u;
+          gather_step<PULL_STEP>(d, c, mm, sum, smf, sf);
+        } else {
+#pragma unroll
+          for (int u = 0; u < PULL_STEP; ++u)  // (q0 + 32 u < nq is warp-uniform)
+            if (q0 + 32 * u < nq) scan_quad<SR, FMT>(d, sm, sbits, gbm, c[u], make_int4(0, 0, 0, 0), first, sum, live, smf, sf);
+        }
+        need = false;  // a row is done once visited or (not real) hit
+#pragma unroll
+        for (int r = 0; r < 4; ++r) need |= (live >> r & 1u) && (SR == SS_REAL || first[r] < 0);
+      }
+      // the largest original id among this lane's first hits of unvisited rows
+      RowAcc acc;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        acc.best[r] = (first[r] >= 0 && (live >> r & 1u)) ? __ldg(d.perm + first[r]) : -1;
+        acc.sum[r] = sum[r];
+      }
+      // (a non-zero real sum implies a hit on a live row of the same lane)
+      const bool any_hit = (acc.best[0] >= 0) | (acc.best[1] >= 0) | (acc.best[2] >= 0) |
+                           (acc.best[3] >= 0);
+      if (__any_sync(SS_FULL_MASK, any_hit)) {  // lanes with equal lane mod Q share rows
+#pragma unroll
+        for (int off = Q; off < 32; off <<= 1)
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            acc.best[r] = max(acc.best[r], __shfl_xor_sync(SS_FULL_MASK, acc.best[r], off));
+            if (SR == SS_REAL) acc.sum[r] += __shfl_xor_sync(SS_FULL_MASK, acc.sum[r], off);
+          }
+      }
+      if (item.w >= 0) {  // SlimChunk: combine partial rows, the last arriving item post-processes
+        const size_t xo = (size_t)item.w * C + 4 * lane;
+        if (lane < Q) {
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            if (acc.best[r] >= 0) atomicMax(d.xpar + xo + r, acc.best[r]);
+            if (SR == SS_REAL && acc.sum[r] != 0.0f) atomicAdd(d.xacc + xo + r, acc.sum[r]);
+          }
+          __threadfence();
+        }
+        __syncwarp();
+        int last = 0;
+        if (lane == 0) {
+          const unsigned old = atomicAdd(d.arrive + item.w, 1u);
+          last = (old == (unsigned)d.split_n[item.w] - 1u);
+        }
+        last = __shfl_sync(SS_FULL_MASK, last, 0);
+        if (!last) continue;
+        __threadfence();
+        if (lane < Q) {
+          // one 16-byte read and reset per array (xo is a multiple of 4 and the
+          // scratch 16-byte aligned); the per-row scalar form of this rarely run
+          // block made the whole real-semiring kernel 20-25 % slower on GB300
+          const int4 b4 = __ldcg(reinterpret_cast<const int4*>(d.xpar + xo));
+          *reinterpret_cast<int4*>(d.xpar + xo) = make_int4(-1, -1, -1, -1);
+          acc.best[0] = b4.x; acc.best[1] = b4.y; acc.best[2] = b4.z; acc.best[3] = b4.w;
+          if (SR == SS_REAL) {
+            const float4 s4 = __ldcg(reinterpret_cast<const float4*>(d.xacc + xo));
+            *reinterpret_cast<float4*>(d.xacc + xo) = make_float4(0.f, 0.f, 0.f, 0.f);
+            acc.sum[0] = s4.x; acc.sum[1] = s4.y; acc.sum[2] = s4.z; acc.sum[3] = s4.w;
+          }
+        }
+        if (lane == 0) d.arrive[item.w] = 0u;
+      }
+      // (a chunk that the groups started is counted already, and has new rows)
+      if (lane == 0 && !(SR != SS_REAL && item.w < 0)) cnt.act += 1;
+      post_chunk<SR, C>(d, k, chunk, lane, live, vis, acc, cnt, true, __shfl_sync(SS_FULL_MASK, my_new, src));
+    }
+  }
+  cnt.slots = lane_slots;
+  finish_iteration_block<FILTERED_THREADS>(d, cnt.nw, cnt.deg, cnt.slots, cnt.act, cnt.maxdeg,
                                        IterLaunch{variant, cond, use_cond});
 }
 
@@ -771,6 +1122,19 @@ static ss_status launch_pull(const slimsell_graph* h, const Dev& d, const IterLa
   return SS_OK;
 }
 
+template <int SR, int C>
+static ss_status launch_filtered(const slimsell_graph* h, const Dev& d, const IterLaunch& il,
+                                 cudaStream_t st) {
+  static std::atomic<unsigned long long> configured{0};
+  if (first_on_device(configured))
+    SS_CUDA(cudaFuncSetAttribute(k_pull_filtered<SR, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 SS_SMEM_LIMIT_BYTES));
+  k_pull_filtered<SR, C><<<pull_grid(h), FILTERED_THREADS, (size_t)(d.smem_words + SMEM_GUARD) * 4, st>>>(
+      d, il.variant, il.cond, il.use_cond);
+  SS_CUDA(cudaGetLastError());
+  return SS_OK;
+}
+
 template <int SR, int MODE, int FMT>
 static ss_status launch_pull_c(const slimsell_graph* h, const Dev& d, const IterLaunch& il,
                                cudaStream_t st) {
@@ -796,7 +1160,12 @@ static ss_status launch_pull_m(const slimsell_graph* h, const Dev& d, int mode, 
       return sell ? launch_pull_c<SR, MODE_SLIMWORK, SS_FORMAT_SELL>(h, d, il, st)
                   : launch_pull_c<SR, MODE_SLIMWORK, SS_FORMAT_SLIMSELL>(h, d, il, st);
     default:
-      return launch_pull_c<SR, MODE_FILTERED, SS_FORMAT_SLIMSELL>(h, d, il, st);
+      switch (h->C) {
+        case 8: return launch_filtered<SR, 8>(h, d, il, st);
+        case 16: return launch_filtered<SR, 16>(h, d, il, st);
+        case 32: return launch_filtered<SR, 32>(h, d, il, st);
+        default: return launch_filtered<SR, 64>(h, d, il, st);
+      }
   }
 }
 

