@@ -264,9 +264,11 @@ ss_status slimsell_bfs_spmv(slimsell_handle h, int32_t root, int32_t semiring, i
  * forward pass per level sums the path counts sigma of the neighbours one
  * level up, per source (the real-semiring BFS step with the counts kept), and a
  * backward pass per level from the deepest sums (1 + delta(w)) / sigma(w) over
- * the neighbours one level down.  fp64 throughout; a row's neighbours are cut
- * into units of 256 that combine with atomicAdd, so the result may differ from
- * a serial sum in the last bits.
+ * the neighbours one level down.  Path counts are 64-bit integers and the
+ * dependency sums 128-bit fixed point (exact sums, at least 60 significant bits
+ * a term) while the counts stay in their range, fp64 past it; a row's
+ * neighbours are cut into units of 256 that combine with atomics, so the result
+ * may differ from a serial fp64 sum in the last bits.
  *   d_sources int32[k] device, k >= 1, each in [0, n) (copied to the host)
  *   d_bc      double[n] device, overwritten
  *   kernel_ms host double* or NULL: summed device time of the level kernels

@@ -73,6 +73,7 @@ struct Ctl {
   unsigned long long new_rowdeg;  // multi-source: degree sum of the rows that gained a source
                                   // in the current iteration (each row counted once)
   unsigned long long prev_rowdeg; // ... in the previous iteration
+  unsigned long long count_bits;  // centrality: every bit set in some path count of the batch
 };
 
 // Flat view of the handle's device buffers handed to kernels by value.
