@@ -35,6 +35,8 @@
 // atomics; the last item of a chunk to arrive runs the post-processing.
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
 #include "ss_device.cuh"
 
 namespace ss {
@@ -310,7 +312,7 @@ __device__ __forceinline__ unsigned quad_hits(const unsigned* sm, int sbits, con
 // issued before the first add, so a warp waits once per step, not once per quad
 // (Kronecker 22 hub level: 322 -> 278 us; the gathers are latency-bound, and
 // staging more hub rows as 8- or 16-bit counts measured no faster).
-template <int U>
+template <int U, bool SHARED = false>
 __device__ __forceinline__ void gather_step(const Dev& d, const int4* c, const unsigned* mm, float sum[4],
                                             const float* smf, int sf) {
   unsigned any = 0;
@@ -324,7 +326,8 @@ __device__ __forceinline__ void gather_step(const Dev& d, const int4* c, const u
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       float v = 0.f;
-      if (mm[u] >> r & 1u) v = (cc[r] < sf) ? smf[cc[r]] : __ldg(d.fr + cc[r]);
+      if (mm[u] >> r & 1u)
+        v = (cc[r] < sf) ? smf[cc[r]] : SHARED ? __ldcg(d.fr + cc[r]) : __ldg(d.fr + cc[r]);
       x[u][r] = v;
     }
   }
@@ -345,6 +348,17 @@ struct Staged {
   int sbits, sf;
 };
 
+// Start copying the first `words` bitmap words (a multiple of 4) behind the guard;
+// returns the shared address of the first one.
+__device__ __forceinline__ unsigned stage_words(const unsigned* gbm, int words) {
+  const unsigned sbase = (unsigned)__cvta_generic_to_shared(ss_smem_bits + SMEM_GUARD);
+  for (int i = threadIdx.x; i < (words >> 2); i += blockDim.x)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sbase + 16u * (unsigned)i),
+                 "l"(reinterpret_cast<const int4*>(gbm) + i)
+                 : "memory");
+  return sbase;
+}
+
 // Stage the prefix of f_{k-1}'s bitmap gbm with asynchronous 16-byte copies (all
 // threads of the block call; the copies run until stage_wait).
 template <int SR>
@@ -361,11 +375,7 @@ __device__ __forceinline__ Staged stage_frontier(const Dev& d, const unsigned* g
   const int sf = hub ? min(HUB_VALUE_ROWS, (sw_all >> 1) & ~3) : 0;
   const int sw = sw_all - sf;  // bitmap words staged (a multiple of 4)
   if (threadIdx.x < SMEM_GUARD) ss_smem_bits[threadIdx.x] = 0u;
-  const unsigned sbase = (unsigned)__cvta_generic_to_shared(ss_smem_bits + SMEM_GUARD);
-  for (int i = threadIdx.x; i < (sw >> 2); i += blockDim.x)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sbase + 16u * (unsigned)i),
-                 "l"(reinterpret_cast<const int4*>(gbm) + i)
-                 : "memory");
+  const unsigned sbase = stage_words(gbm, sw);
   const unsigned fbase = sbase + 4u * (unsigned)sw;
   for (int i = threadIdx.x; i < (sf >> 2); i += blockDim.x)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(fbase + 16u * (unsigned)i),
@@ -383,31 +393,30 @@ __device__ __forceinline__ void stage_wait() {
   __syncthreads();
 }
 
-// One frontier expansion x_k = A (x)_S f_{k-1} with fused post-processing.
-// Warp w of the grid owns items w, w + W, w + 2W, ... (W = warps in the grid,
-// the item list is ordered for that assignment); it reads the descriptors and
-// SlimWork states of 32 of them at once (one per lane) and walks the active ones.
-template <int SR, int C, int MODE, int FMT>
-__global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
-                                                          cudaGraphConditionalHandle cond,
-                                                          int use_cond) {
+struct __align__(8) ItemCache {
+  int chunk, y, z, w;
+  long long start;
+};
+
+// Warp wid of nw walks its items wid, wid + nw, ... of level k (the item list is
+// ordered for such an assignment): it reads the descriptors and visited bits of 32
+// of them at once (one per lane) and processes the active ones.  full: every chunk
+// is active.  SHARED: other SMs have written the bitmaps and values since this
+// kernel began, so those are read past L1 (and the whole bitmap is staged); cache:
+// the threads' item descriptors in shared memory (at most one batch), filled by the
+// first level.
+template <int SR, int C, int FMT, bool SHARED>
+__device__ __forceinline__ void pull_items(const Dev& d, int k, bool full, const unsigned* gbm, const Staged& sg,
+                                           int wid, int nw, Counters& cnt, ItemCache* cache = nullptr,
+                                           bool fill = false) {
   constexpr int PULL_STEP = pull_step<SR, FMT>();
-  const int* colp = (FMT == SS_FORMAT_SELL) ? d.scol : d.col;
   constexpr int Q = C / 4;
-  if (d.ctl->done) return;
-  const int k = d.ctl->k;
-  const int km1 = k - 1;
-  const int lane = threadIdx.x & 31;
-  const int wid = blockIdx.x * (PULL_THREADS / 32) + (threadIdx.x >> 5);
-  const int nw = gridDim.x * (PULL_THREADS / 32);
-  const unsigned* gbm = d.fb[km1 & 1];
   constexpr unsigned long long ALL_ROWS = C == 64 ? ~0ull : (1ull << C) - 1ull;
-  const Staged sg = stage_frontier<SR>(d, gbm);
-  stage_wait();
+  const int* colp = (FMT == SS_FORMAT_SELL) ? d.scol : d.col;
+  const int lane = threadIdx.x & 31;
   const unsigned* sm = sg.sm;
   const float* smf = sg.smf;
   const int sbits = sg.sbits, sf = sg.sf;
-  Counters cnt;
   for (long long b0 = wid; b0 < d.n_items; b0 += 32LL * nw) {
     const long long my_it = b0 + (long long)lane * nw;
     int4 my_item = make_int4(0, 0, 0, -1);
@@ -415,11 +424,19 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
     unsigned long long my_vis = ALL_ROWS;  // the chunk's visited rows
     bool active = false;
     if (my_it < d.n_items) {
-      my_item = d.items[my_it];
-      my_vis = chunk_bits<C>(d.vis, my_item.x);
-      my_start = d.cs[my_item.x] + (long long)my_item.y * C;
-      const unsigned long long old = chunk_bits<C>(d.fb[k & 1], my_item.x);  // in flight with vis
-      active = MODE == MODE_FULL || my_vis != ALL_ROWS;
+      if (SHARED && cache && !fill) {
+        const ItemCache ic = cache[threadIdx.x];
+        my_item = make_int4(ic.chunk, ic.y, ic.z, ic.w);
+        my_start = ic.start;
+      } else {
+        my_item = d.items[my_it];
+        my_start = d.cs[my_item.x] + (long long)my_item.y * C;
+        if (SHARED && cache)
+          cache[threadIdx.x] = ItemCache{my_item.x, my_item.y, my_item.z, my_item.w, my_start};
+      }
+      my_vis = chunk_bits<C, SHARED>(d.vis, my_item.x);
+      const unsigned long long old = chunk_bits<C, SHARED>(d.fb[k & 1], my_item.x);  // in flight with vis
+      active = full || my_vis != ALL_ROWS;
       // a finished chunk (SlimWork) adds no row: f_k is zero there, so what
       // f_{k-2} left in the parity buffer is cleared
       if (!active && my_item.y == 0 && old != 0ull) store_bits<C>(d.fb[k & 1], my_item.x, 0u, 0u);
@@ -471,7 +488,7 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
 #pragma unroll
         for (int u = 0; u < SHORT_COLS; ++u)
           mm[u] = (u < ncols) ? quad_hits(sm, sbits, gbm, c[u], first) & live : 0u;
-        gather_step<SHORT_COLS>(d, c, mm, sum, smf, sf);
+        gather_step<SHORT_COLS, SHARED>(d, c, mm, sum, smf, sf);
       } else {
 #pragma unroll
         for (int u = 0; u < SHORT_COLS; ++u)
@@ -547,7 +564,7 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
 #pragma unroll
           for (int u = 0; u < PULL_STEP; ++u)
             mm[u] = (q0 + 32 * u < nq) ? quad_hits(sm, sbits, gbm, c[u], first) & live : 0u;
-          gather_step<PULL_STEP>(d, c, mm, sum, smf, sf);
+          gather_step<PULL_STEP, SHARED>(d, c, mm, sum, smf, sf);
         } else {
 #pragma unroll
           for (int u = 0; u < PULL_STEP; ++u)  // (q0 + 32 u < nq is warp-uniform)
@@ -612,6 +629,22 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
       post_chunk<SR, C>(d, k, chunk, lane, live, vis, acc, cnt);
     }
   }
+}
+
+// One frontier expansion x_k = A (x)_S f_{k-1} with fused post-processing.
+template <int SR, int C, int MODE, int FMT>
+__global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
+                                                          cudaGraphConditionalHandle cond,
+                                                          int use_cond) {
+  if (d.ctl->done) return;
+  const int k = d.ctl->k;
+  const unsigned* gbm = d.fb[(k - 1) & 1];
+  const Staged sg = stage_frontier<SR>(d, gbm);
+  stage_wait();
+  Counters cnt;
+  pull_items<SR, C, FMT, false>(d, k, MODE == MODE_FULL, gbm, sg,
+                                (int)(blockIdx.x * (PULL_THREADS / 32) + (threadIdx.x >> 5)),
+                                (int)(gridDim.x * (PULL_THREADS / 32)), cnt);
   finish_iteration_block<PULL_THREADS>(d, cnt.nw, cnt.deg, cnt.slots, cnt.act, cnt.maxdeg,
                                        IterLaunch{variant, cond, use_cond});
 }
@@ -939,18 +972,22 @@ __global__ void __launch_bounds__(FILTERED_THREADS, 1) k_pull_filtered(Dev d, in
                                        IterLaunch{variant, cond, use_cond});
 }
 
-// Start of a run: nothing visited, empty frontiers.  The claim words of the rows
-// without neighbours (past n_live) are left alone: no pass reads them.
-__global__ void k_init(Dev d) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// Start of a run, thread t0 of `stride`: nothing visited but the root row (none if
+// negative), empty frontiers.  The claim words of the rows without neighbours (past
+// n_live) are left alone: no pass reads them.
+__device__ __forceinline__ void init_rows(const Dev& d, long long t0, long long stride, int root_row,
+                                          unsigned long long root_word) {
   ulonglong2* claim2 = reinterpret_cast<ulonglong2*>(d.claim);  // (n_pad is a multiple of 8)
-  for (long long i = t0; i < (d.n_live + 1) / 2; i += stride) claim2[i] = make_ulonglong2(0ull, 0ull);
+  const long long pairs = (d.n_live + 1) / 2;
+  for (long long i = t0; i < pairs; i += stride)
+    claim2[i] = make_ulonglong2(2 * i == root_row ? root_word : 0ull, 2 * i + 1 == root_row ? root_word : 0ull);
+  if (t0 == 0 && root_row >= 2 * pairs) d.claim[root_row] = root_word;
   for (long long w = t0; w < d.fb_words; w += stride) {
-    d.fb[0][w] = 0u;
+    const unsigned rb = root_row >= 0 && (root_row >> 5) == w ? 1u << (root_row & 31) : 0u;
+    d.fb[0][w] = rb;
     d.fb[1][w] = 0u;
     const long long real = d.n - 32 * w;  // rows of this word that are no padding
-    d.vis[w] = real >= 32 ? 0u : real <= 0 ? ~0u : ~0u << real;
+    d.vis[w] = (real >= 32 ? 0u : real <= 0 ? ~0u : ~0u << real) | rb;
   }
   for (long long s = t0; s < (long long)d.n_split * d.C; s += stride) {
     d.xacc[s] = 0.0f;
@@ -959,6 +996,96 @@ __global__ void k_init(Dev d) {
   if (d.ctl->error) {  // a previous run stopped early: restore the push scratch invariant
     for (long long r = t0; r < d.n_pad; r += stride) d.psum[r] = 0.0f;
   }
+}
+
+// A whole run (init, every level, outputs) on a small graph in one launch, by one
+// thread-block cluster.  A small graph's pass is a few microseconds of work behind
+// a launch, a control-block read, a grid-wide tail and the next launch, 10 us a level
+// (Kronecker 10: 80 us for five levels); here a level costs the pass, a block
+// reduction and one hardware cluster barrier.  The barrier orders the level's
+// bitmap, visited and value writes before the next level reads them (past L1), and
+// the counters travel through distributed shared memory, double-buffered by level
+// parity, so every thread takes the same exit.  Rank 0 keeps the control block in
+// shared memory and writes it back at the end.  Kronecker 10: 42 us; 64 graphs of scale
+// 10 .. 17 in one batch 0.35 ms, 1.65 with a conditional loop of launches each.
+template <int SR, int C>
+__global__ void __launch_bounds__(PULL_THREADS, 1) k_small(Dev d, SmallIo io, int policy) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int G = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // (a small graph's counters fit 32 bits)
+  __shared__ unsigned part[2][SS_LOCAL_CLUSTER_MAX][5];  // every CTA's counters, by level parity
+  __shared__ unsigned wpart[PULL_THREADS / 32][5];
+  __shared__ Ctl ctl;  // (rank 0)
+  const int nw = G * (PULL_THREADS / 32);
+  ItemCache* cache = d.n_items <= 32 * nw
+                         ? reinterpret_cast<ItemCache*>(ss_smem_bits + SMEM_GUARD + d.smem_words) : nullptr;
+  const int root = io.roots ? io.roots[io.i] : io.root;
+  const int root_row = d.invperm[root];
+  {
+    const long long t0 = (long long)rank * PULL_THREADS + tid, stride = (long long)G * PULL_THREADS;
+    init_rows(d, t0, stride, root_row, claim_word(0, root));
+    if (rank == 0 && tid == PULL_THREADS - 1) {
+      d.fr[root_row] = 1.0f;
+      init_ctl(d, &ctl, root_row);
+    }
+  }
+  cl.sync();
+  unsigned long long reached = 1;
+  for (int k = 1;; ++k) {
+    const unsigned* gbm = d.fb[(k - 1) & 1];
+    Staged sg;
+    sg.sm = ss_smem_bits + SMEM_GUARD;
+    sg.smf = nullptr;
+    sg.sf = 0;
+    sg.sbits = d.smem_words * 32;  // the whole bitmap
+    if (tid < SMEM_GUARD) ss_smem_bits[tid] = 0u;
+    stage_words(gbm, d.smem_words);
+    stage_wait();
+    Counters cnt;
+    pull_items<SR, C, SS_FORMAT_SLIMSELL, true>(d, k, policy == SS_V_FULL, gbm, sg,
+                                                rank * (PULL_THREADS / 32) + warp, nw, cnt, cache, k == 1);
+    const unsigned v[5] = {(unsigned)cnt.nw, (unsigned)cnt.deg, (unsigned)cnt.slots, (unsigned)cnt.act, cnt.maxdeg};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      const unsigned w = i < 4 ? __reduce_add_sync(SS_FULL_MASK, v[i]) : __reduce_max_sync(SS_FULL_MASK, v[i]);
+      if (lane == 0) wpart[warp][i] = w;
+    }
+    __syncthreads();
+    if (warp < 5) {  // counter `warp` over the block's warps, told to every CTA
+      const unsigned x = lane < PULL_THREADS / 32 ? wpart[lane][warp] : 0u;
+      const unsigned w = warp < 4 ? __reduce_add_sync(SS_FULL_MASK, x) : __reduce_max_sync(SS_FULL_MASK, x);
+      if (lane < G) cl.map_shared_rank(&part[0][0][0], lane)[((k & 1) * SS_LOCAL_CLUSTER_MAX + rank) * 5 + warp] = w;
+    }
+    // level k is complete (one CTA alone needs no cluster-wide release of its writes)
+    if (G > 1) cl.sync();
+    else __syncthreads();
+    unsigned tot[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      const unsigned x = lane < G ? part[k & 1][lane][i] : 0u;
+      tot[i] = i < 4 ? __reduce_add_sync(SS_FULL_MASK, x) : __reduce_max_sync(SS_FULL_MASK, x);
+    }
+    reached += tot[0];
+    if (rank == 0 && tid == PULL_THREADS - 1) advance_level(d, &ctl, k, tot[0], tot[1], tot[2], tot[3], tot[4], policy);
+    // the same decision advance_level takes
+    if (tot[0] == 0 || k >= d.n + 1 || reached > d.reach_cap) break;
+  }
+  if (rank == 0) {
+    __syncthreads();
+    const unsigned* src = reinterpret_cast<const unsigned*>(&ctl);
+    unsigned* dst = reinterpret_cast<unsigned*>(d.ctl);
+    for (int i = tid; i < (int)(sizeof(Ctl) / sizeof(unsigned)); i += PULL_THREADS) dst[i] = src[i];
+  }
+  int* dist = io.dists ? io.dists[io.i] : io.dist;
+  int* parent = io.parents ? io.parents[io.i] : io.parent;
+  if (dist || parent)
+    write_outputs(d, dist, parent, root_row, (long long)rank * PULL_THREADS + tid, (long long)G * PULL_THREADS);
+}
+
+__global__ void k_init(Dev d) {
+  init_rows(d, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x, -1, 0ull);
 }
 
 __global__ void k_init_root(Dev d, int root) { init_root_state(d, root); }
@@ -1082,7 +1209,10 @@ __global__ void k_dp_clear(Dev d) {
   }
 }
 
-__global__ void k_output(Dev d, int* dist, int* parent) { write_outputs(d, dist, parent); }
+__global__ void k_output(Dev d, int* dist, int* parent) {
+  write_outputs(d, dist, parent, d.ctl->root_row, (long long)blockIdx.x * blockDim.x + threadIdx.x,
+                (long long)gridDim.x * blockDim.x);
+}
 
 // Real-semiring values f of the last run in original vertex order; rows the run
 // did not reach hold stale values and read as 0.
@@ -1132,6 +1262,121 @@ static ss_status launch_filtered(const slimsell_graph* h, const Dev& d, const It
   k_pull_filtered<SR, C><<<pull_grid(h), FILTERED_THREADS, (size_t)(d.smem_words + SMEM_GUARD) * 4, st>>>(
       d, il.variant, il.cond, il.use_cond);
   SS_CUDA(cudaGetLastError());
+  return SS_OK;
+}
+
+// Graphs whose whole run goes into one launch (k_small): the fixed full and SlimWork
+// policies over SlimSell with the whole bitmap staged, up to SMALL_SLOTS slots where a
+// run has the GPU to itself (a cluster of up to 16 of the 152 SMs: TODO_RULE), up to
+// SMALL_BATCH_SLOTS side by side in a batch, where a cluster's SMs are a graph's share
+// of the GPU and its size follows from its share of the slots (at least
+// SMALL_BATCH_MIN slots a CTA: 32 graphs of scale 10 .. 13 take 171 us, 217 with 16 K).
+#ifndef SS_SMALL_SLOTS
+#define SS_SMALL_SLOTS (32 << 10)
+#endif
+#ifndef SS_SMALL_SLOTS_PER_CTA
+#define SS_SMALL_SLOTS_PER_CTA (16 << 10)
+#endif
+#ifndef SS_SMALL_BATCH_SLOTS
+#define SS_SMALL_BATCH_SLOTS (4 << 20)
+#endif
+#ifndef SS_SMALL_BATCH_MIN
+#define SS_SMALL_BATCH_MIN (64 << 10)
+#endif
+constexpr long long SMALL_SLOTS = SS_SMALL_SLOTS;                  // one run alone on the GPU
+constexpr long long SMALL_SLOTS_PER_CTA = SS_SMALL_SLOTS_PER_CTA;
+constexpr long long SMALL_BATCH_SLOTS = SS_SMALL_BATCH_SLOTS;      // many side by side
+constexpr long long SMALL_BATCH_MIN = SS_SMALL_BATCH_MIN;
+
+static bool whole_run(const slimsell_graph* h, const Dev& d, int policy, long long max_slots) {
+  return (policy == SS_V_FULL || policy == SS_V_SLIMWORK) && d.format == SS_FORMAT_SLIMSELL &&
+         h->slots <= max_slots && (long long)d.smem_words * 32 >= h->n_pad &&
+         (long long)d.smem_words * 4 <= SS_SMEM_LIMIT_BYTES - 16 - (long long)sizeof(ItemCache) * PULL_THREADS;
+}
+bool batch_small(const slimsell_graph* h, const Dev& d, int policy) {
+  return whole_run(h, d, policy, SMALL_BATCH_SLOTS);
+}
+static size_t small_smem(const Dev& d) {
+  return (size_t)(d.smem_words + SMEM_GUARD) * 4 + sizeof(ItemCache) * PULL_THREADS;
+}
+
+// CTAs of the run's cluster: a power of two, at most what the device places.
+static int small_cluster(const slimsell_graph* h, long long slots_per_cta) {
+  int G = 1;
+  while (G < h->local_cluster && G * slots_per_cta < h->slots) G *= 2;
+  return G;
+}
+
+using SmallKernel = void (*)(Dev, SmallIo, int);
+
+template <int SR>
+static SmallKernel small_kernel_c(int C) {
+  switch (C) {
+    case 8: return k_small<SR, 8>;
+    case 16: return k_small<SR, 16>;
+    case 32: return k_small<SR, 32>;
+    default: return k_small<SR, 64>;
+  }
+}
+
+// The kernel of a semiring and chunk height, with its launch limits raised.
+static ss_status small_kernel(const slimsell_graph* h, int sr, SmallKernel* out) {
+  static std::atomic<unsigned long long> configured[4][4];
+  const int c = h->C == 8 ? 0 : h->C == 16 ? 1 : h->C == 32 ? 2 : 3;
+  *out = sr == SS_TROPICAL ? small_kernel_c<SS_TROPICAL>(h->C)
+       : sr == SS_REAL     ? small_kernel_c<SS_REAL>(h->C)
+       : sr == SS_BOOLEAN  ? small_kernel_c<SS_BOOLEAN>(h->C)
+                           : small_kernel_c<SS_SELMAX>(h->C);
+  if (first_on_device(configured[sr][c])) {
+    SS_CUDA(cudaFuncSetAttribute(*out, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM_LIMIT_BYTES));
+    SS_CUDA(cudaFuncSetAttribute(*out, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  }
+  return SS_OK;
+}
+
+static ss_status launch_small(const slimsell_graph* h, const Dev& d, int sr, int policy, const SmallIo& io, int G,
+                              cudaStream_t st) {
+  SmallKernel kern = nullptr;
+  ss_status s = small_kernel(h, sr, &kern);
+  if (s != SS_OK) return s;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(G);
+  cfg.blockDim = dim3(PULL_THREADS);
+  cfg.dynamicSmemBytes = small_smem(d);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = G;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  SS_CUDA(cudaLaunchKernelEx(&cfg, kern, d, io, policy));
+  return SS_OK;
+}
+
+ss_status add_small_node(const slimsell_graph* h, const Dev& d, int sr, int policy, const SmallIo& io,
+                         long long batch_slots, cudaGraph_t g, cudaGraphNode_t* out) {
+  SmallKernel kern = nullptr;
+  ss_status s = small_kernel(h, sr, &kern);
+  if (s != SS_OK) return s;
+  const int G = std::min(8, small_cluster(h, std::max(SMALL_BATCH_MIN, batch_slots / h->num_sms)));
+  Dev dd = d;
+  SmallIo ii = io;
+  int pol = policy;
+  void* args[] = {&dd, &ii, &pol};
+  cudaKernelNodeParams kp = {};
+  kp.func = (void*)kern;
+  kp.gridDim = dim3(G);
+  kp.blockDim = dim3(PULL_THREADS);
+  kp.sharedMemBytes = (unsigned)small_smem(d);
+  kp.kernelParams = args;
+  SS_CUDA(cudaGraphAddKernelNode(out, g, nullptr, 0, &kp));
+  cudaKernelNodeAttrValue v = {};
+  v.clusterDim.x = G;
+  v.clusterDim.y = 1;
+  v.clusterDim.z = 1;
+  SS_CUDA(cudaGraphKernelNodeSetAttribute(*out, cudaLaunchAttributeClusterDimension, &v));
   return SS_OK;
 }
 
@@ -1401,11 +1646,22 @@ ss_status slimsell_bfs(slimsell_handle h, int32_t root, int32_t semiring, int32_
   double iter_ms = 0.0;
   if (prof) SS_CUDA(cudaEventRecord(h->ev_c, st));
 
-  k_init<<<grid, 256, 0, st>>>(d);
-  k_init_root<<<1, 1, 0, st>>>(d, root);
-  SS_CUDA(cudaGetLastError());
+  const bool dp = d_parent && semiring != SS_SELMAX && h->dp_pass;
+  const bool whole = device_loop && whole_run(h, d, policy, SMALL_SLOTS);
+  if (!whole) {
+    k_init<<<grid, 256, 0, st>>>(d);
+    k_init_root<<<1, 1, 0, st>>>(d, root);
+    SS_CUDA(cudaGetLastError());
+  }
 
-  if (device_loop) {
+  if (whole) {
+    SmallIo io{};
+    io.root = root;
+    io.dist = dp ? nullptr : d_dist;  // (with the DP pass, the outputs follow it)
+    io.parent = dp ? nullptr : d_parent;
+    ss_status s = launch_small(h, d, semiring, policy, io, small_cluster(h, SMALL_SLOTS_PER_CTA), st);
+    if (s != SS_OK) return s;
+  } else if (device_loop) {
     cudaGraphExec_t exec = nullptr;
     ss_status s = loop_graph(h, d, semiring, policy, &exec);
     if (s != SS_OK) return s;
@@ -1487,11 +1743,11 @@ ss_status slimsell_bfs(slimsell_handle h, int32_t root, int32_t semiring, int32_
     }
   }
 
-  if (d_parent && semiring != SS_SELMAX && h->dp_pass) {
+  if (dp) {
     ss_status s = launch_dp(h, d, st);
     if (s != SS_OK) return s;
   }
-  if (d_dist || d_parent) {
+  if ((!whole || dp) && (d_dist || d_parent)) {
     k_output<<<grid, 256, 0, st>>>(d, d_dist, d_parent);
     SS_CUDA(cudaGetLastError());
   }

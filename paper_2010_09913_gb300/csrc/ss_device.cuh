@@ -24,12 +24,18 @@ __device__ __forceinline__ int claim_level(unsigned long long w) {  // (w != 0)
 __device__ __forceinline__ int claim_parent(unsigned long long w) { return (int)(unsigned)w - 1; }
 
 // The bits of one chunk's rows (bit l = row l of the chunk) in a row bitmap.
-template <int C>
+// SHARED: read past L1 (another SM may have written it since this kernel began).
+template <class T, bool SHARED>
+__device__ __forceinline__ T ld_word(const T* p) {
+  if constexpr (SHARED) return __ldcg(p);
+  else return *p;
+}
+template <int C, bool SHARED = false>
 __device__ __forceinline__ unsigned long long chunk_bits(const unsigned* bm, long long chunk) {
-  if (C == 8) return reinterpret_cast<const unsigned char*>(bm)[chunk];
-  if (C == 16) return reinterpret_cast<const unsigned short*>(bm)[chunk];
-  if (C == 32) return bm[chunk];
-  const uint2 v = reinterpret_cast<const uint2*>(bm)[chunk];
+  if (C == 8) return ld_word<unsigned char, SHARED>(reinterpret_cast<const unsigned char*>(bm) + chunk);
+  if (C == 16) return ld_word<unsigned short, SHARED>(reinterpret_cast<const unsigned short*>(bm) + chunk);
+  if (C == 32) return ld_word<unsigned, SHARED>(bm + chunk);
+  const uint2 v = ld_word<uint2, SHARED>(reinterpret_cast<const uint2*>(bm) + chunk);
   return ((unsigned long long)v.y << 32) | v.x;
 }
 
@@ -240,14 +246,8 @@ __device__ __forceinline__ void store_features(const Dev& d, int k, const float*
   for (int i = 0; i < SS_SELECTOR_FEATURES; ++i) d.feats[(size_t)k * SS_SELECTOR_FEATURES + i] = f[i];
 }
 
-// Root state and control block of a new single-source run (one thread).
-__device__ __forceinline__ void init_root_state(const Dev& d, int root) {
-  const int r = d.invperm[root];
-  d.claim[r] = claim_word(0, root);
-  d.vis[r >> 5] |= 1u << (r & 31);
-  d.fb[0][r >> 5] |= 1u << (r & 31);
-  d.fr[r] = 1.0f;
-  Ctl* c = d.ctl;
+// Control block of a new single-source run from root row r (one thread).
+__device__ __forceinline__ void init_ctl(const Dev& d, Ctl* c, int r) {
   c->root_row = r;
   c->k = 1; c->done = 0; c->error = 0; c->variant = -1;
   c->new_count = 0; c->new_deg = 0; c->slots = 0; c->active = 0;
@@ -266,23 +266,32 @@ __device__ __forceinline__ void init_root_state(const Dev& d, int root) {
   d.iters[0] = s;
 }
 
+// Root state and control block of a new single-source run (one thread).
+__device__ __forceinline__ void init_root_state(const Dev& d, int root) {
+  const int r = d.invperm[root];
+  d.claim[r] = claim_word(0, root);
+  d.vis[r >> 5] |= 1u << (r & 31);
+  d.fb[0][r >> 5] |= 1u << (r & 31);
+  d.fr[r] = 1.0f;
+  init_ctl(d, d.ctl, r);
+}
+
 // Claim word of a row at the end of a run.  Rows past n_live have no neighbours,
 // are not initialised and hold the word of whatever run had them as its root.
 __device__ __forceinline__ unsigned long long final_claim(const Dev& d, int r, int root_row) {
-  return (r < d.n_live || r == root_row) ? d.claim[r] : 0ull;
+  return (r < d.n_live || r == root_row) ? __ldcg(d.claim + r) : 0ull;
 }
 
-// Distances and parents in original vertex ids (grid-stride over groups of four
-// vertices).  Bound by the random 8-byte gathers of the claim words (a 32-byte
+// Distances and parents in original vertex ids: thread t of `threads` takes every
+// threads-th group of four vertices.  Bound by the random 8-byte gathers of the claim words (a 32-byte
 // sector each), so four are in flight per thread and the rows without
 // neighbours (half of a Kronecker graph's) gather nothing: 10 us on Kronecker 22; with
 // one gather each for level and parent, over all vertices, 22 us.
-__device__ __forceinline__ void write_outputs(const Dev& d, int* dist, int* parent) {
-  const int root_row = d.ctl->root_row;
+__device__ __forceinline__ void write_outputs(const Dev& d, int* dist, int* parent, int root_row, long long t,
+                                              long long threads) {
   // 16-byte stores where the caller's arrays allow them
   const bool vd = (reinterpret_cast<size_t>(dist) & 15) == 0, vp = (reinterpret_cast<size_t>(parent) & 15) == 0;
-  for (long long v = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); v < d.n;
-       v += 4LL * gridDim.x * blockDim.x) {
+  for (long long v = 4 * t; v < d.n; v += 4 * threads) {
     const int cnt = (int)min((long long)d.n - v, 4LL);
     int r[4], L[4], P[4];
     if (cnt == 4) {
@@ -339,6 +348,20 @@ ss_status multi_level(slimsell_graph* h, const MultiDev& m, int W, cudaStream_t 
 ss_status sell_arrays(slimsell_graph* h, cudaStream_t st);
 
 __global__ void k_init(Dev d);
+
+// Whole runs of the fixed full and SlimWork policies on small graphs in one launch (ss_bfs.cu).
+struct SmallIo {
+  int root;               // the root, or (roots given) roots[i]
+  const int* roots;
+  int* dist;              // outputs (NULL: none), or (tables given) dists[i], parents[i]
+  int* parent;
+  int* const* dists;
+  int* const* parents;
+  int i;
+};
+bool batch_small(const slimsell_graph* h, const Dev& d, int policy);  // a batch runs this graph that way
+ss_status add_small_node(const slimsell_graph* h, const Dev& d, int sr, int policy, const SmallIo& io,
+                         long long batch_slots, cudaGraph_t g, cudaGraphNode_t* out);
 
 // Grid sizes that follow the graph size (ss_bfs.cu).
 int pull_grid(const slimsell_graph* h);
