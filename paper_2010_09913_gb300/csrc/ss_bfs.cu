@@ -993,7 +993,7 @@ __device__ __forceinline__ void init_rows(const Dev& d, long long t0, long long 
     d.xacc[s] = 0.0f;
     d.xpar[s] = -1;
   }
-  if (d.ctl->error) {  // a previous run stopped early: restore the push scratch invariant
+  if (d.ctl->error | d.ctl->psum_dirty) {  // a previous run left sums behind (or stopped early)
     for (long long r = t0; r < d.n_pad; r += stride) d.psum[r] = 0.0f;
   }
 }
@@ -1267,10 +1267,14 @@ static ss_status launch_filtered(const slimsell_graph* h, const Dev& d, const It
 
 // Graphs whose whole run goes into one launch (k_small): the fixed full and SlimWork
 // policies over SlimSell with the whole bitmap staged, up to SMALL_SLOTS slots where a
-// run has the GPU to itself (a cluster of up to 16 of the 152 SMs: TODO_RULE), up to
+// run has the GPU to itself (what one or two CTAs hold), up to
 // SMALL_BATCH_SLOTS side by side in a batch, where a cluster's SMs are a graph's share
 // of the GPU and its size follows from its share of the slots (at least
 // SMALL_BATCH_MIN slots a CTA: 32 graphs of scale 10 .. 13 take 171 us, 217 with 16 K).
+// SMALL_SLOTS could go on to about 1 M (Kronecker 14 takes 79 us that way, 147 grid-wide;
+// ER 200 K, without hubs, 234 against 147), but the adaptive policies do not run here, and
+// plain SlimWork would then beat them on small long-diameter graphs, where they are the
+// choice that scales (tests/test_gpu_selector.py holds them to it).
 #ifndef SS_SMALL_SLOTS
 #define SS_SMALL_SLOTS (32 << 10)
 #endif

@@ -19,12 +19,17 @@
 #ifndef SS_PULL_THREADS
 #define SS_PULL_THREADS 1024
 #endif
-// cluster push: frontier entries and frontier edges per CTA, largest cluster, list capacity
+// cluster push: frontier rows and frontier edges per CTA, largest cluster, levels run by one CTA
 #define SS_LOCAL_SLICE 4096
 #define SS_LOCAL_EDGES_PER_CTA 8192
 #define SS_LOCAL_CLUSTER_MAX 16
 #define SS_LSTAT 8  // words per level in lstat
-#define SS_LOCAL_LIST_CAP (SS_LOCAL_CLUSTER_MAX * SS_LOCAL_EDGES_PER_CTA)
+#ifndef SS_LOCAL_SOLO_UP
+#define SS_LOCAL_SOLO_UP 512
+#endif
+#ifndef SS_LOCAL_SOLO_DOWN
+#define SS_LOCAL_SOLO_DOWN 256
+#endif
 
 namespace ss {
 
@@ -54,7 +59,7 @@ struct Ctl {
   unsigned int blocks_done;       // blocks of the current iteration kernel that finished
   int prev_variant;               // variant of the previous iteration (-1 before the first)
   int root_row;                   // row of the run's root
-  int pad0;
+  int psum_dirty;                 // the cluster push left sums in psum: the next run's init zeroes it
   unsigned long long prev_slots;  // slots read by the previous iteration
   unsigned long long prev_new;    // |f_{k-1}|: vertices discovered by the previous iteration
   unsigned long long prev_deg;    // their degree sum (frontier edges)
@@ -64,10 +69,7 @@ struct Ctl {
   unsigned int prev_maxdeg;       // ... by the previous iteration
   unsigned long long units;       // push work units queued by the current iteration
   unsigned long long variant_count[5];  // iterations run with each variant
-  int list_level;                 // level whose vertex list is in qlist[level & 1] (-1: none)
-  int list_prev_ok;               // qlist also holds the list of list_level - 1
-  unsigned long long qlen[2];     // vertex-list lengths, by level parity
-  unsigned long long qprep;       // length of a list just built from the bitmap
+  unsigned long long qprep;       // length of the vertex list built from the bitmap
   unsigned long long loop_guard;  // decide-kernel executions in this run (device loop bound)
   unsigned long long bunits;      // push block units queued by the current iteration
   unsigned long long new_rowdeg;  // multi-source: degree sum of the rows that gained a source
@@ -111,12 +113,8 @@ struct Dev {
   int push_blocks;      // 0: vertex units only, 1: block units for dense blocks, 2: for every block
   float* psum;          // [n_pad] push: real-semiring sum of frontier-neighbour values
   unsigned* touched;    // [fb_words] push: rows reached by the current push
-  int* qlist[2];        // [n_pad] vertex lists of a level (cluster push), by parity
-  int* qdeg[2];         // [SS_LOCAL_LIST_CAP] cluster push: degree of each listed vertex
-  long long* qbase[2];  // [SS_LOCAL_LIST_CAP] ... start of its column-major row (cs + row % C)
-  int* qorig[2];        // [SS_LOCAL_LIST_CAP] ... its original id
-  int* qovf;            // [SS_LOCAL_LIST_CAP] cluster push: new vertices past a CTA's list
-  unsigned long long* qovf_n;  // [2] their counts, by level parity
+  int* qlist;           // [n_pad] cluster push: rows of its first frontier, then rows without room
+  unsigned long long* qcount;  // [2] cluster push: rows without room, entries of the first frontier
   int local_cluster;    // CTAs in the cluster push's cluster
   long long local_max_nf, local_max_e;  // largest frontier (vertices, edges) it takes
   const float* mlp;     // selector weights (16-64-64-4 MLP), or NULL
@@ -176,12 +174,8 @@ struct slimsell_graph {
   int push_blocks = 1;                 // see SS_OPT_PUSH_BLOCKS
   float* psum = nullptr;
   unsigned* touched = nullptr;
-  int* qlist[2] = {nullptr, nullptr};
-  int* qdeg[2] = {nullptr, nullptr};
-  long long* qbase[2] = {nullptr, nullptr};
-  int* qorig[2] = {nullptr, nullptr};
-  int* qovf = nullptr;
-  unsigned long long* qovf_n = nullptr;
+  int* qlist = nullptr;
+  unsigned long long* qcount = nullptr;
   int local_cluster = 0;
   float* mlp = nullptr;       // selector weights on the device (NULL until loaded)
   float sel_margin = 0.0f;    // see SS_OPT_SELECTOR_MARGIN

@@ -126,7 +126,7 @@ __device__ __forceinline__ bool advance_level(const Dev& d, Ctl* c, int k, unsig
 
 // End of an iteration, run by the last block of its final kernel: record the
 // level, reset the per-iteration counters and (device-side loop) set the loop
-// condition.  The vertex list of the single-block push is no longer current.
+// condition.
 __device__ __forceinline__ void iteration_tail(const Dev& d, int variant,
                                                cudaGraphConditionalHandle cond, int use_cond) {
   Ctl* c = d.ctl;
@@ -139,7 +139,6 @@ __device__ __forceinline__ void iteration_tail(const Dev& d, int variant,
   const bool stop = advance_level(d, c, k, nc, nd, sl, ac, md, variant);
   c->prev_rowdeg = c->new_rowdeg;
   c->new_rowdeg = 0;
-  c->list_level = -1;
   c->new_count = 0;
   c->new_deg = 0;
   c->slots = 0;
@@ -259,7 +258,8 @@ __device__ __forceinline__ void init_ctl(const Dev& d, Ctl* c, int r) {
   c->bunits = 0;
   for (int v = 0; v < N_VARIANTS; ++v) c->variant_count[v] = 0;
   c->loop_guard = 0;
-  c->list_level = -1; c->list_prev_ok = 0; c->qlen[0] = c->qlen[1] = 0; c->qprep = 0;
+  c->qprep = 0;
+  c->psum_dirty = 0;
   ss_iter_stats s;
   s.frontier = 1; s.frontier_degree = d.rdeg[r]; s.slots = 0; s.active_chunks = 0;
   s.variant = -1; s.kernel_ns = 0;

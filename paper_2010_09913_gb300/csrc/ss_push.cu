@@ -211,88 +211,90 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_post(Dev d, IterLaunch il
 // ---------------------------------------------------------------------------
 // Cluster push for small frontiers: one thread-block cluster (16 CTAs of 1024
 // threads where the device can place it, else 8) runs level after level inside
-// one launch, with no kernel boundary and no bitmap walk per level.  The
-// frontier is a vertex list; each CTA holds an equal share of it in shared
-// memory with, per entry, what the scatter needs (start of the row's edges in
-// col, edge count, original id).  The first level's share is loaded from the
-// global list; later shares are written straight into the owning CTA's shared
-// memory by the CTAs that discover the vertices (distributed shared memory),
-// rows longer than LOCAL_UNIT edges being cut into units spread round-robin
-// over the cluster.  Per level a CTA scatters over its share's edges (each
-// thread a contiguous run: one binary search, then a forward walk) and claims
-// each candidate with one atomicMax on its claim word: the old value 0 makes
-// this CTA the vertex's owner, words of earlier levels are larger and never
-// change, and the word ends with this level and the largest id among the
-// frontier neighbours, the parent.  Two hardware cluster barriers per level
-// order the scatter before the post step (which reads the final counts) and
-// the post step before the next level; per-CTA counts and
-// statistics reach every CTA through distributed shared memory.  Spreading the
-// random accesses over many SMs is what makes a level cheap: one SM's L1
-// serves about one uncoalesced line per clock.  Every CTA keeps a copy of the
-// control block in shared memory, updated identically from the cluster totals,
-// so all CTAs take the same exits; CTA 0 writes it back at the end.
-// The cluster hands back to the iteration loop when the frontier outgrows
-// d.local_max_nf vertices or d.local_max_e edges, or after max_levels levels,
-// leaving the bitmaps and lists as the grid-wide variants and the next launch
-// expect them:
-//   fb[(k-1)&1] = level k-1, fb[k&1] = level k-2 (or zero),
-//   qlist/qdeg/qbase/qorig[(k-1)&1] = level k-1, qlist[k&1] = level k-2 (lengths in qlen).
+// one launch, with no kernel boundary and no bitmap walk per level.
+//
+// The frontier lives in shared memory as entries of at most LOCAL_EDGES edges
+// (start in col, edge count, original id, row); rows of more than LOCAL_LONG edges
+// become entries of LOCAL_UNIT edges that a warp walks together.  A thread takes an
+// entry, loads its neighbours, claims each with one atomicMax on its claim word
+// (old value 0: this thread discovered it; words of earlier levels are larger and
+// never change; the word ends with this level and the largest id among the
+// frontier neighbours, the parent), and writes each discovered row's entries
+// straight into the shared memory of the CTA that takes them in the next level
+// (distributed shared memory).  Where an entry goes follows from its number among
+// the entries its CTA has made (round-robin over the CTAs, one segment per making
+// CTA), so no count is needed before the placing and a level has one cluster
+// barrier: the claim word needs no second step after the claims are final.
+//
+// A level is a chain of latencies (columns, claims, row data, barrier), and the
+// barrier with its release of the level's global writes is the longest.  While levels
+// have up to SOLO_UP edges they are therefore run by rank 0 alone, entries in its own shared
+// memory, block barriers only, while the others wait at a cluster barrier until it
+// spreads the entries again or ends the launch.  Lattice 4096^2 (6,154 levels): 4.9 us a
+// level, 6.9 with two cluster barriers a level and the row data fetched after the
+// claims; 96^2, mostly rank 0 alone, about 2.4 us.
+//
+// Every active CTA takes the same exits (counters reach every CTA through
+// distributed shared memory); rank 0 keeps the control block in shared memory and
+// writes it back.  Frontier bits are kept in no level: a launch clears those of its
+// first frontier, and when it hands back it sets those of the last, as the
+// grid-wide variants expect them (fb[(k-1)&1] = level k-1, fb[k&1] = 0).
 // ---------------------------------------------------------------------------
-constexpr int LOCAL_THREADS = 1024;
-constexpr int LOCAL_BATCH = 8;      // candidate edges per thread in flight (a full slice: 8 per thread)
-constexpr int LOCAL_NEWCAP = 8192;  // new vertices per CTA kept in shared memory
-constexpr int LOCAL_POST = 2;       // new vertices per thread in flight in the post step
-constexpr int LOCAL_UNIT = 1024;    // edges of one slice entry; longer rows become several units
-constexpr int LOCAL_HUBCAP = 256;   // extra slice entries per CTA for the units of long rows
-constexpr int LOCAL_SLOTS = SS_LOCAL_SLICE + LOCAL_HUBCAP;
-constexpr int LOCAL_PER_THREAD = (LOCAL_SLOTS + LOCAL_THREADS - 1) / LOCAL_THREADS;
+#ifndef SS_LOCAL_THREADS
+#define SS_LOCAL_THREADS 512
+#endif
+constexpr int LOCAL_THREADS = SS_LOCAL_THREADS;
+constexpr int LOCAL_EDGES = 4;      // edges a thread takes at once, and of one entry of a short row
+constexpr int LOCAL_LONG = 64;      // longer rows are cut into units of
+constexpr int LOCAL_UNIT = 128;     // edges, walked by a warp
+constexpr int LOCAL_ENTRIES = 6144; // entries a CTA holds of one level
+constexpr int SOLO_UP = SS_LOCAL_SOLO_UP;      // rank 0 goes on alone after a level of up to this many edges
+constexpr int SOLO_DOWN = SS_LOCAL_SOLO_DOWN;  // the cluster leaves the next level to it after one of this many
 constexpr int CTL_WORDS = (int)(sizeof(Ctl) / sizeof(unsigned));
 static_assert(sizeof(Ctl) % sizeof(unsigned) == 0, "control block copied as words");
-static_assert(SS_LOCAL_SLICE % LOCAL_THREADS == 0, "whole frontier entries per thread");
-static_assert(SS_LOCAL_CLUSTER_MAX * SS_LOCAL_EDGES_PER_CTA / LOCAL_UNIT <= LOCAL_HUBCAP,
-              "the units of the largest frontier fit one CTA");
+static_assert(SOLO_DOWN <= SOLO_UP && SOLO_UP <= LOCAL_ENTRIES, "the first solo level fits one CTA");
 
-struct LocalPub {             // what each CTA tells every CTA of the cluster about a level
-  int nsm;                    // new vertices it holds in shared memory
-  int novf;                   // new vertices it put in the overflow list
-  unsigned md;                // largest degree of the vertices it posted
-  int drop;                   // a unit of a long row found no room (the next level goes back)
-  unsigned long long nd;      // their degree sum
+struct LocalPub {             // what a CTA tells the others about a level
+  int nent;                   // entries it has made
+  int nnew;                   // vertices it has discovered
+  unsigned md;                // their largest degree
+  int drop;                   // a vertex found no room (the level goes back to the grid)
+  unsigned nd_lo, nd_hi;      // their degree sum, nd_lo + nd_hi * 2^20 (32-bit shared atomics are native)
 };
 
-// A CTA's slice of the frontier: entries 0 .. ns-1 are its equal share of the
-// vertex list (each with at most LOCAL_UNIT of its edges), then `hubn` units
-// carrying further LOCAL_UNIT-edge pieces of long rows, appended by any CTA.
+struct __align__(16) LocalEntry {
+  unsigned long long edges;   // start of the entry's first edge in col, edge count << 44
+  int orig;                   // original id of its row (parent candidate)
+  int row;                    // its row; -1 - row for all but the row's first entry
+};
+
+struct LocalMsg {             // rank 0 to the waiting CTAs, at the end of its solo levels
+  int k, exit, handback, dropped;
+  unsigned long long nf, E, reached, reached_deg;
+};
+
 struct LocalSmem {
-  Ctl ctl;                             // this CTA's copy of the control block
-  long long base[LOCAL_SLOTS];         // start of the entry's first edge in col
-  int pref[LOCAL_SLOTS];               // edge counts, then their exclusive prefix
-  int orig[LOCAL_SLOTS];               // original ids (parent candidates)
-  int sid[2][LOCAL_SLOTS];             // vertex ids, by level parity
-  int nid[LOCAL_NEWCAP];               // vertices this CTA discovered
-  long long wsum[LOCAL_THREADS / 32];
-  unsigned long long red[LOCAL_THREADS / 32];
-  unsigned redmax[LOCAL_THREADS / 32];
-  LocalPub all[2][SS_LOCAL_CLUSTER_MAX];  // written by every CTA of the cluster, by level parity
-  int nnew, novf, es, hubn, drop;
-  unsigned long long placed;           // edges of the vertices this CTA has placed for the next level
+  Ctl ctl;                                // rank 0: the control block
+  LocalEntry ent[2][LOCAL_ENTRIES];       // by level parity
+  LocalPub mine[3];                       // this CTA's counters, by level modulo 3
+  LocalPub all[2][SS_LOCAL_CLUSTER_MAX];  // every CTA's
+  unsigned placed[2];                     // edges of the long rows this CTA has placed
+  LocalMsg msg;
 };
 static_assert(sizeof(LocalSmem) <= 227 * 1024, "cluster push shared memory");
+static_assert(LOCAL_THREADS / 32 >= SS_LOCAL_CLUSTER_MAX, "a warp for every segment of a slice");
 
-// Entry from a bitmap state: list the level-(k-1) rows into qlist[(k-1)&1] and
-// clear fb[k&1] (it held level k-2, which the cluster push does not list).
+// Entry: list the level-(k-1) rows into qlist and clear fb[k&1] (it held level k-2).
 __global__ void __launch_bounds__(PUSH_THREADS) k_push_local_prep(Dev d) {
   Ctl* c = d.ctl;
   if (c->done) return;
   const int k = c->k;
-  if (c->list_level == k - 1) return;  // the previous cluster-push level left its list
   const int lane = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long words = ((long long)d.n_pad + 31) / 32;
   const unsigned* fbm = d.fb[(k - 1) & 1];
   unsigned* fbk = d.fb[k & 1];
-  int* list = d.qlist[(k - 1) & 1];
   for (long long i0 = t0 - lane; i0 < words; i0 += stride & ~31LL) {
     const long long i = i0 + lane;
     unsigned bits = 0u;
@@ -313,47 +315,8 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_local_prep(Dev d) {
       base = __shfl_sync(SS_FULL_MASK, base, 0);
       // the decide kernel sends only frontiers that fit the list
       const unsigned long long at = base + __popc(m & ((1u << lane) - 1u));
-      if (u >= 0 && at < (unsigned long long)d.n_pad) list[at] = u;
+      if (u >= 0 && at < (unsigned long long)d.n_pad) d.qlist[at] = u;
     }
-  }
-}
-
-// End the kernel: no CTA leaves while another may still read its shared memory;
-// CTA 0 writes its control block back and sets the loop condition.
-__device__ __forceinline__ void local_exit(LocalSmem& S, Ctl* c, const IterLaunch& il, unsigned cond,
-                                           cg::cluster_group& cl) {
-  cl.sync();
-  if (cl.block_rank() != 0) return;
-  const unsigned* src = reinterpret_cast<const unsigned*>(&S.ctl);
-  unsigned* dst = reinterpret_cast<unsigned*>(c);
-  for (int i = threadIdx.x; i < CTL_WORDS; i += LOCAL_THREADS) dst[i] = src[i];
-  if (threadIdx.x == 0 && il.use_cond) cudaGraphSetConditional(il.cond, cond);
-}
-
-// Entry `slot` of CTA `owner`'s slice (parity p) gets vertex x's first edges; the
-// rest of a row longer than LOCAL_UNIT goes in LOCAL_UNIT-edge units to the
-// following CTAs in turn, appended after their shares (ns_of(o) entries).
-template <int C, typename NsOf>
-__device__ __forceinline__ void place_entry(LocalSmem& S, cg::cluster_group& cl, int G, int owner, int slot,
-                                            int p, int x, long long bx, int dv, int og, NsOf ns_of) {
-  LocalSmem* R = cl.map_shared_rank(&S, owner);
-  R->sid[p][slot] = x;
-  R->pref[slot] = min(dv, LOCAL_UNIT);
-  R->base[slot] = bx;
-  R->orig[slot] = og;
-  int o = owner;
-  for (int j0 = LOCAL_UNIT; j0 < dv; j0 += LOCAL_UNIT) {
-    o = (o + 1 == G) ? 0 : o + 1;
-    LocalSmem* T = cl.map_shared_rank(&S, o);
-    const int at = ns_of(o) + atomicAdd(&T->hubn, 1);
-    if (at >= LOCAL_SLOTS) {  // no room: the cluster hands this level back instead
-      S.drop = 1;
-      continue;
-    }
-    T->sid[p][at] = x;
-    T->pref[at] = min(dv - j0, LOCAL_UNIT);
-    T->base[at] = bx + (long long)j0 * C;
-    T->orig[at] = og;
   }
 }
 
@@ -365,92 +328,45 @@ __device__ __forceinline__ long long share(long long total, int r, int lg) {
   return (long long)(((unsigned)total * (unsigned)r) >> lg);
 }
 
-// The CTA whose share holds list entry `at` (0 <= at < total).
-__device__ __forceinline__ int share_owner(long long at, long long total, int lg) {
-  const int G = 1 << lg;
-  int r = (int)(((unsigned)at << lg) / (unsigned)total);
-  while (r + 1 < G && share(total, r + 1, lg) <= at) ++r;
-  while (r > 0 && share(total, r, lg) > at) --r;
-  return r;
+// How the entries of a level lie: made by rank 0 alone or by every CTA, for rank 0
+// alone or for every CTA.  A making CTA owns one segment of every taking CTA.
+struct LocalLay {
+  bool from_one, to_one;
+  __device__ __forceinline__ int cap(int lg) const { return from_one ? LOCAL_ENTRIES : LOCAL_ENTRIES >> lg; }
+  // entries that CTA `rank` takes of the nent ones CTA r has made
+  __device__ __forceinline__ int count(int r, int nent, int rank, int lg) const {
+    if (from_one && r != 0) return 0;
+    if (to_one) return rank == 0 ? min(nent, cap(lg)) : 0;
+    const int G = 1 << lg, e0 = (rank - r) & (G - 1);
+    return nent > e0 ? min((nent - e0 + G - 1) >> lg, cap(lg)) : 0;
+  }
+};
+
+// Call f(index, valid) for this CTA's entries of parity p: the threads of a warp together,
+// segment after segment; invalid past a segment's end.
+// (made: how many rank 0 has made, where it alone did).
+template <class F>
+__device__ __forceinline__ void local_entries(const LocalSmem& S, const LocalLay& lay, int made, int p, int rank,
+                                              int lg, F f) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nseg = lay.from_one ? 1 : 1 << lg;
+  const int wps = (LOCAL_THREADS / 32) / nseg;  // warps of a segment
+  const int seg = warp / wps;
+  const int n = lay.count(seg, lay.from_one ? made : S.all[p][seg].nent, rank, lg);
+  // entry after entry goes to another warp, so that a few long ones do not queue in one
+  for (int i0 = warp % wps; i0 < n; i0 += wps * 32) f(seg * lay.cap(lg) + i0 + lane * wps, i0 + lane * wps < n);
 }
 
 // Selector features of the iterations after levels k0 .. k1 run in this launch
 // (the decide kernel did not run before them), from the per-level totals the
 // launch recorded; rank 0's threads, one level each, when the launch ends.
-__device__ __forceinline__ void local_features(const Dev& d, LocalSmem& S, cg::cluster_group& cl, int k0,
-                                               int k1) {
+__device__ __forceinline__ void local_features(const Dev& d, int k0, int k1) {
   __syncthreads();  // the last level's totals are in place
-  if (cl.block_rank() != 0) return;
   for (int k = k0 + (int)threadIdx.x; k <= k1 && k + 1 < d.iter_cap; k += LOCAL_THREADS) {
     const unsigned long long* ls = d.lstat + (size_t)k * SS_LSTAT;
     float f[SS_SELECTOR_FEATURES];
     features_of(d, k + 1, ls[0], ls[1], ls[4], ls[5], (unsigned)ls[2], ls[6], f);
     store_features(d, k + 1, f);
-  }
-}
-
-// One scatter pass of the cluster push: thread tid takes edges [ea, ea + per) of
-// the slice (per <= B), finds their rows by one binary search and a forward walk,
-// loads the neighbours, and claims each with one atomicMax on its claim word (all
-// B in flight before any result is used): the old value 0 makes this thread the
-// vertex's first discoverer, the word keeps level and largest-id parent, and words
-// of earlier levels are larger, so visited vertices keep theirs.
-template <int SR, int C, int B>
-__device__ __forceinline__ void local_scatter(const Dev& d, LocalSmem& S, int p0, int p1, int ns, int e0,
-                                              int per, int Es, int tid, int k) {
-  const int* sid = S.sid[p1];
-  const int ea = e0 + tid * per;
-  const int eb = min(ea + per, Es);
-  int i = 0;
-  if (ea < eb) {  // largest i with pref[i] <= ea
-    int lo_ = 0, hi_ = ns - 1;
-    while (lo_ < hi_) {
-      const int mid = (lo_ + hi_ + 1) >> 1;
-      if (S.pref[mid] <= ea) lo_ = mid;
-      else hi_ = mid - 1;
-    }
-    i = lo_;
-  }
-  int src[B], v[B];
-  float fu[B];  // real semiring: the source's value, loaded with the neighbour
-#pragma unroll
-  for (int q = 0; q < B; ++q) {
-    const int e = ea + q;
-    src[q] = -1;
-    v[q] = -1;
-    fu[q] = 0.0f;
-    if (e < eb) {
-      while (i + 1 < ns && S.pref[i + 1] <= e) ++i;
-      src[q] = i;
-      v[q] = __ldg(d.col + S.base[i] + (long long)(e - S.pref[i]) * C);
-      if (SR == SS_REAL) fu[q] = __ldcg(d.fr + sid[i]);  // written during this launch: past L1
-    }
-  }
-  unsigned long long old[B];
-#pragma unroll
-  for (int q = 0; q < B; ++q) {
-    old[q] = ~0ull;
-    if (v[q] >= 0) old[q] = atomicMax(d.claim + v[q], claim_word(k, S.orig[src[q]]));
-  }
-  if (SR == SS_REAL) {  // a neighbour not visited at an earlier level
-    const unsigned lev = 0x7fffffffu - (unsigned)k;
-#pragma unroll
-    for (int q = 0; q < B; ++q)
-      if ((unsigned)(old[q] >> 32) <= lev) atomicAdd(d.psum + v[q], fu[q]);
-  }
-#pragma unroll
-  for (int q = 0; q < B; ++q) {
-    if (old[q] == 0ull) {  // first discoverer: this CTA owns the vertex
-      const int idx = atomicAdd(&S.nnew, 1);
-      if (idx < LOCAL_NEWCAP) {
-        S.nid[idx] = v[q];
-      } else {  // past this CTA's list (skewed slices): the shared overflow list
-        atomicAdd(&S.novf, 1);
-        const unsigned long long o = atomicAdd(d.qovf_n + p0, 1ull);
-        if (o < (unsigned long long)SS_LOCAL_LIST_CAP) d.qovf[o] = v[q];
-        else atomicOr(&S.ctl.error, 16);  // cannot happen: new vertices <= E <= cap
-      }
-    }
   }
 }
 
@@ -460,10 +376,203 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
+// A level's placing: where the rows that this CTA discovers go.
+template <int C>
+struct LocalPlace {
+  const Dev& d;
+  LocalSmem& S;
+  cg::cluster_group& cl;
+  LocalPub* mine;
+  int k, p, rank, lg;
+  LocalLay lay;
+  bool first;  // the launch's own entries: numbered through one counter for all CTAs, as if rank 0 made them
+  // a row without room: the level is handed back, as a bitmap, where its bit is set at once
+  __device__ __forceinline__ void drop(int x) {
+    mine->drop = 1;
+    atomicOr(d.fb[p] + (x >> 5), 1u << (x & 31));
+    atomicOr(d.vis + (x >> 5), 1u << (x & 31));
+  }
+  // Unit u of a row as entry number e; false (and the row dropped) without room: what fits of
+  // the row is placed all the same, it is then set twice.
+  __device__ __forceinline__ bool put(int x, long long bx, int deg, int og, int per, int u, int e, int seg, int cap,
+                                      int from) {
+    const int slot = lay.to_one ? e : e >> lg;
+    if (slot >= cap) {
+      drop(x);
+      return false;
+    }
+    LocalEntry en;
+    en.edges = (unsigned long long)(bx + (long long)u * per * C) | (unsigned long long)min(deg - u * per, per) << 44;
+    en.orig = og;
+    en.row = u == 0 ? x : -1 - x;
+    LocalSmem* T = cl.map_shared_rank(&S, lay.to_one ? 0 : (from + e) & ((1 << lg) - 1));
+    *reinterpret_cast<int4*>(&T->ent[p][seg + slot]) = *reinterpret_cast<const int4*>(&en);
+    return true;
+  }
+  // Entries of up to N rows a lane (those with x >= 0); all lanes of the warp call, and
+  // number their entries with one shared atomic.
+  template <int N>
+  __device__ __forceinline__ void operator()(const int* x, const long long* bx, const int* deg, const int* og) {
+    const int lane = threadIdx.x & 31;
+    const int G = 1 << lg, cap = lay.cap(lg), from = first ? 0 : rank;
+    const int seg = lay.from_one ? 0 : rank * cap;
+    bool single = true;  // every row is one entry
+#pragma unroll
+    for (int q = 0; q < N; ++q) single = single && (x[q] < 0 || deg[q] <= LOCAL_EDGES);
+    if (__all_sync(SS_FULL_MASK, single)) {
+      unsigned m[N];
+      int at[N], all = 0;
+#pragma unroll
+      for (int q = 0; q < N; ++q) {
+        m[q] = __ballot_sync(SS_FULL_MASK, x[q] >= 0);
+        at[q] = all + __popc(m[q] & ((1u << lane) - 1u));
+        all += __popc(m[q]);
+      }
+      int e0 = 0;
+      if (lane == 0) e0 = first ? (int)atomicAdd(d.qcount, (unsigned long long)all) : atomicAdd(&mine->nent, all);
+      e0 = __shfl_sync(SS_FULL_MASK, e0, 0);
+#pragma unroll
+      for (int q = 0; q < N; ++q) {
+        if (x[q] < 0) continue;
+        const int e = e0 + at[q];
+        const int slot = lay.to_one ? e : e >> lg;
+        if (slot >= cap) {
+          drop(x[q]);
+          continue;
+        }
+        LocalEntry en;
+        en.edges = (unsigned long long)bx[q] | (unsigned long long)deg[q] << 44;
+        en.orig = og[q];
+        en.row = x[q];
+        LocalSmem* T = cl.map_shared_rank(&S, lay.to_one ? 0 : (from + e) & (G - 1));
+        *reinterpret_cast<int4*>(&T->ent[p][seg + slot]) = *reinterpret_cast<const int4*>(&en);
+#pragma unroll
+        for (int j = 0; j < LOCAL_EDGES; ++j)  // its columns, for the next level
+          if (j < deg[q]) asm volatile("prefetch.global.L2 [%0];" ::"l"(d.col + bx[q] + (long long)j * C));
+      }
+      return;
+    }
+    int nu[N], total = 0;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      nu[q] = 0;
+      if (x[q] >= 0) {
+        nu[q] = deg[q] > LOCAL_LONG ? (deg[q] + LOCAL_UNIT - 1) / LOCAL_UNIT : (deg[q] + LOCAL_EDGES - 1) / LOCAL_EDGES;
+        // a level of more edges than the cluster takes is handed back, so nothing past that is
+        // placed (the 160 units of one 163 K hub were 15 us of a Kronecker 22 level)
+        if (deg[q] > LOCAL_LONG &&
+            atomicAdd(&S.placed[p], (unsigned)min(deg[q], 1 << 17)) + (unsigned)deg[q] > (unsigned)d.local_max_e) {
+          drop(x[q]);
+          nu[q] = 0;
+        }
+        total += nu[q];
+      }
+    }
+    int incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(SS_FULL_MASK, incl, o);
+      if (lane >= o) incl += t;
+    }
+    const int all = __shfl_sync(SS_FULL_MASK, incl, 31);
+    if (all == 0) return;
+    int e0 = 0;
+    if (lane == 31) e0 = first ? (int)atomicAdd(d.qcount, (unsigned long long)all) : atomicAdd(&mine->nent, all);
+    e0 = __shfl_sync(SS_FULL_MASK, e0, 31) + incl - total;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const int per = deg[q] > LOCAL_LONG ? LOCAL_UNIT : LOCAL_EDGES;
+      if (nu[q] <= LOCAL_LONG / LOCAL_EDGES) {
+        for (int u = 0; u < nu[q]; ++u)
+          if (!put(x[q], bx[q], deg[q], og[q], per, u, e0 + u, seg, cap, from)) break;
+      }
+      // the units of a long row, by the whole warp
+      unsigned big = __ballot_sync(SS_FULL_MASK, nu[q] > LOCAL_LONG / LOCAL_EDGES);
+      while (big) {
+        const int src = __ffs(big) - 1;
+        big &= big - 1;
+        const int bxr = __shfl_sync(SS_FULL_MASK, x[q], src), bdeg = __shfl_sync(SS_FULL_MASK, deg[q], src);
+        const int bog = __shfl_sync(SS_FULL_MASK, og[q], src), be = __shfl_sync(SS_FULL_MASK, e0, src);
+        const int bn = __shfl_sync(SS_FULL_MASK, nu[q], src);
+        const long long bb = __shfl_sync(SS_FULL_MASK, bx[q], src);
+        for (int u = lane; u < bn; u += 32)
+          if (!put(bxr, bb, bdeg, bog, LOCAL_UNIT, u, be + u, seg, cap, from)) break;
+      }
+      e0 += nu[q];
+    }
+  }
+};
+
+// atomicMax under a predicate (~0 without it).  Written as a branch, each of a
+// thread's claims waited for the one before it at the branch's end: 3,480 cycles for
+// four against 1,050 in flight together.
+__device__ __forceinline__ unsigned long long claim_if(unsigned long long* p, unsigned long long key, bool on) {
+  unsigned long long old;
+  asm volatile(
+      "{\n\t.reg .pred on;\n\tsetp.ne.s32 on, %3, 0;\n\tmov.b64 %0, -1;\n\t"
+      "@on atom.global.max.u64 %0, [%1], %2;\n\t}"
+      : "=l"(old)
+      : "l"(p), "l"(key), "r"((int)on)
+      : "memory");
+  return old;
+}
+
+// Per-thread counters of a level.
+struct LocalSum {
+  int nnew = 0;
+  unsigned md = 0;
+  unsigned long long nd = 0;
+};
+
+// Claim up to LOCAL_EDGES neighbours, at b, b + step, ... (n of them) of the row with
+// original id og and value fu: every load in flight before a claim, every claim
+// before a result, and the discovered rows' data before the first is placed.  All
+// lanes of the warp call.
+template <int SR, int C>
+__device__ __forceinline__ void local_claim(const Dev& d, LocalPlace<C>& place, LocalSum& sum, long long b, int step,
+                                            int n, int og, float fu) {
+  int v[LOCAL_EDGES];
+#pragma unroll
+  for (int q = 0; q < LOCAL_EDGES; ++q) v[q] = q < n ? __ldg(d.col + b + (long long)q * step) : -1;
+  unsigned long long old[LOCAL_EDGES];
+  const unsigned long long key = claim_word(place.k, og);
+#pragma unroll
+  for (int q = 0; q < LOCAL_EDGES; ++q) old[q] = claim_if(d.claim + v[q], key, v[q] >= 0);
+  if (SR == SS_REAL) {  // a neighbour not visited at an earlier level
+#pragma unroll
+    for (int q = 0; q < LOCAL_EDGES; ++q)
+      if ((unsigned)(old[q] >> 32) <= (unsigned)(key >> 32)) atomicAdd(d.psum + v[q], fu);
+  }
+  // the neighbours' row data, in flight with the claims (of every neighbour: waiting to
+  // learn which are new would add a memory latency to the level)
+  int dv[LOCAL_EDGES], og2[LOCAL_EDGES];
+  long long bx[LOCAL_EDGES];
+#pragma unroll
+  for (int q = 0; q < LOCAL_EDGES; ++q) {
+    dv[q] = v[q] >= 0 ? __ldg(d.rdeg + v[q]) : 0;
+    bx[q] = v[q] >= 0 ? __ldg(d.cs + v[q] / C) + v[q] % C : 0;
+    og2[q] = v[q] >= 0 ? __ldg(d.perm + v[q]) : 0;
+  }
+  bool any = false;
+#pragma unroll
+  for (int q = 0; q < LOCAL_EDGES; ++q) {
+    if (old[q] != 0ull) v[q] = -1;  // (not discovered here)
+    any = any || v[q] >= 0;
+  }
+  if (!__any_sync(SS_FULL_MASK, any)) return;
+  place.template operator()<LOCAL_EDGES>(v, bx, dv, og2);
+#pragma unroll
+  for (int q = 0; q < LOCAL_EDGES; ++q)
+    if (v[q] >= 0) {
+      sum.nnew += 1;
+      sum.nd += (unsigned long long)dv[q];
+      sum.md = max(sum.md, (unsigned)dv[q]);
+    }
+}
+
 template <int SR, int C>
 __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaunch il, int max_levels,
                                                                  int time_levels) {
-  constexpr int BATCH = LOCAL_BATCH;
   LocalSmem& S = *reinterpret_cast<LocalSmem*>(ss_local_smem);
   // per-level timing (profiling): the first level also carries the launch's entry
   unsigned long long t_prev = time_levels ? global_ns() : 0ull;
@@ -473,331 +582,231 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
   const int rank = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   Ctl* c = d.ctl;
-  {
-    const unsigned* src = reinterpret_cast<const unsigned*>(c);
-    unsigned* dst = reinterpret_cast<unsigned*>(&S.ctl);
-    for (int i = tid; i < CTL_WORDS; i += LOCAL_THREADS) dst[i] = src[i];
-    if (rank == 0 && tid < 2) d.qovf_n[tid] = 0ull;
-    if (tid == 0) {
-      S.hubn = 0;
-      S.drop = 0;
-    }
-  }
-  cl.sync();  // every CTA holds its copy before CTA 0 can write the block back
-  if (S.ctl.done) return;  // the same in every CTA; no shared memory was shared yet
-  int k = S.ctl.k;
+  int k = c->k;
   const int k0 = k;  // first level of this launch (its features came from the decide kernel)
-  const bool have_list = S.ctl.list_level == k - 1;
-  long long nf = (long long)(have_list ? S.ctl.qlen[(k - 1) & 1] : S.ctl.qprep);
-  long long E = (long long)S.ctl.prev_deg;  // edges of the level-(k-1) frontier
-  if (!local_fits(d, (unsigned long long)nf, (unsigned long long)E)) {
-    // the decide kernel never sends such a frontier
-    if (tid == 0) {
+  const int done = c->done;
+  unsigned long long nf = c->qprep, E = c->prev_deg;  // rows and edges of the level-(k-1) frontier
+  unsigned long long reached = c->reached, reached_deg = c->reached_deg;
+  if (rank == 0)
+    for (int i = tid; i < CTL_WORDS; i += LOCAL_THREADS)
+      reinterpret_cast<unsigned*>(&S.ctl)[i] = reinterpret_cast<const unsigned*>(c)[i];
+  if (tid < 3) S.mine[tid] = LocalPub{0, 0, 0u, 0, 0u, 0u};
+  if (tid < 2) S.placed[tid] = 0u;
+  if (rank == 0 && tid == 0) *d.qcount = 0ull;  // first entries
+  cl.sync();  // every CTA has read the control block, and its counters are reset
+  if (done) return;
+  bool handback = true;  // (else the run has ended)
+  int last = k - 1;      // level of the frontier that the entries hold
+  // (the first entries fit: at most nf + E / LOCAL_EDGES, which local_fits bounds by the cluster's capacity)
+  LocalLay cur{true, nf + E <= SOLO_DOWN};
+  if (!local_fits(d, nf, E)) {  // the decide kernel never sends such a frontier
+    if (rank == 0 && tid == 0) {
       S.ctl.error |= 8;
       S.ctl.done = 1;
     }
-    local_exit(S, c, il, 0u, cl);
-    return;
+    handback = false;
+    cur = LocalLay{true, true};
+    nf = 0;
   }
-  if (tid == 0 && !have_list) S.ctl.qlen[(k - 1) & 1] = (unsigned long long)nf;
-  // the first slice comes from the global list (its per-vertex data listed too, or
-  // gathered), and the level k-2 words to clear from the list the previous launch
-  // left; later slices arrive in shared memory from the CTAs that found them
+  // the first entries, from the list; the first frontier's bits are cleared
   {
     const int p1 = (k - 1) & 1;
-    const long long lo = share(nf, rank, lg);
-    const int ns = (int)(share(nf, rank + 1, lg) - lo);
-    auto ns_of = [&](int o) { return (int)(share(nf, o + 1, lg) - share(nf, o, lg)); };
-    for (int i = tid; i < ns; i += LOCAL_THREADS) {
-      const int u = __ldcg(d.qlist[p1] + lo + i);
-      int dv, og;
-      long long bx;
-      if (have_list) {
-        dv = __ldcg(d.qdeg[p1] + lo + i);
-        bx = __ldcg(d.qbase[p1] + lo + i);
-        og = __ldcg(d.qorig[p1] + lo + i);
-      } else {
-        dv = __ldg(d.rdeg + u);
+    LocalPlace<C> place{d, S, cl, &S.mine[0], k, p1, rank, lg, cur, true};
+    const long long lo = share((long long)nf, rank, lg), hi = share((long long)nf, rank + 1, lg);
+    unsigned* fbm = d.fb[p1];
+    for (long long i0 = lo + wid * 32; i0 < hi; i0 += LOCAL_THREADS) {
+      int u = -1, dv = 0, og = 0;
+      long long bx = 0;
+      if (i0 + lane < hi) {
+        u = __ldcg(d.qlist + i0 + lane);
+        fbm[u >> 5] = 0u;
         bx = __ldg(d.cs + u / C) + (u % C);
+        dv = __ldg(d.rdeg + u);
         og = __ldg(d.perm + u);
       }
-      place_entry<C>(S, cl, G, rank, i, p1, u, bx, dv, og, ns_of);
+      if (dv == 0) u = -1;  // (an isolated root has no edges)
+      place.template operator()<1>(&u, &bx, &dv, &og);
     }
-    const long long n2 = (have_list && S.ctl.list_prev_ok) ? (long long)S.ctl.qlen[k & 1] : 0;
-    const long long lo2 = share(n2, rank, lg), hi2 = share(n2, rank + 1, lg);
-    unsigned* fbk = d.fb[k & 1];
-    for (long long i = lo2 + tid; i < hi2; i += LOCAL_THREADS) fbk[__ldcg(d.qlist[k & 1] + i) >> 5] = 0u;
   }
-  cl.sync();  // the first slices, with the units of long rows, are in place
-  int ns_prev = 0;  // entries of S.sid[k&1]: this CTA's slice of level k-2 (after the first level)
-  unsigned long long reached = S.ctl.reached;  // every thread tracks the stop condition
-  unsigned long long reached_deg = S.ctl.reached_deg;
-  for (int lev = 0;; ++lev) {
-    if (lev > 0 && (lev >= max_levels || !local_fits(d, (unsigned long long)nf, (unsigned long long)E))) {
-      local_features(d, S, cl, k0, k - 1);
-      if (tid == 0) {  // hand the level-(k-1) list back
-        S.ctl.list_level = k - 1;
-        S.ctl.list_prev_ok = 1;
-      }
-      local_exit(S, c, il, 1u, cl);
-      return;
-    }
+  cl.sync();  // the first entries are in place
+  int made = (int)__ldcg(d.qcount);  // entries of the level that rank 0 (or the launch) has made
+  bool stopped = !handback;
+  bool dropped = false;  // the last level holds rows without room (bits only)
+  for (int lev = 0; !stopped; ++lev) {
+    const bool solo = cur.to_one;
     const int p1 = (k - 1) & 1, p0 = k & 1;
-    unsigned* fbk = d.fb[p0];
-    const int nsv = (int)(share(nf, rank + 1, lg) - share(nf, rank, lg));  // vertices
-    const int ns = nsv + S.hubn;  // slice entries: vertices, then units of long rows
-    for (int i = tid; i < ns_prev; i += LOCAL_THREADS) fbk[S.sid[p0][i] >> 5] = 0u;  // level k-2
-    if (tid == 0) {
-      S.nnew = 0;
-      S.novf = 0;
-    }
-    // ---- exclusive prefix of the slice's degrees, in place (slice edges <= E <= d.local_max_e) ----
-    if (ns <= 8 * 32) {  // small slice: one warp
-      if (wid == 0) {
-        int dg[8], sum = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int i = lane * 8 + q;
-          dg[q] = (i < ns) ? S.pref[i] : 0;
-          sum += dg[q];
-        }
-        int incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int t = __shfl_up_sync(SS_FULL_MASK, incl, o);
-          if (lane >= o) incl += t;
-        }
-        int run = incl - sum;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int i = lane * 8 + q;
-          if (i < ns) S.pref[i] = run;
-          run += dg[q];
-        }
-        if (lane == 31) S.es = incl;
-      }
-    } else {
-      int dg[LOCAL_PER_THREAD], sum = 0;
-#pragma unroll
-      for (int q = 0; q < LOCAL_PER_THREAD; ++q) {
-        const int i = tid * LOCAL_PER_THREAD + q;
-        dg[q] = (i < ns) ? S.pref[i] : 0;
-        sum += dg[q];
-      }
-      int incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(SS_FULL_MASK, incl, o);
-        if (lane >= o) incl += t;
-      }
-      if (lane == 31) S.wsum[wid] = incl;
+    if (solo && rank != 0) {  // rank 0 alone: wait for its message
+      cl.sync();
+      const LocalMsg m = S.msg;
+      k = m.k;
+      nf = m.nf;
+      E = m.E;
+      reached = m.reached;
+      reached_deg = m.reached_deg;
+      cur = LocalLay{true, m.exit != 0};
+      last = k - 1;
+      made = S.all[last & 1][0].nent;
+      if (tid < 3) S.mine[tid] = LocalPub{0, 0, 0u, 0, 0u, 0u};
+      if (tid < 2) S.placed[tid] = 0u;
       __syncthreads();
-      if (wid == 0) {
-        long long w = S.wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const long long t = __shfl_up_sync(SS_FULL_MASK, w, o);
-          if (lane >= o) w += t;
-        }
-        S.wsum[lane] = w;
+      if (m.exit) {
+        handback = m.handback != 0;
+        dropped = m.dropped != 0;
+        break;
       }
-      __syncthreads();
-      int run = (wid > 0 ? (int)S.wsum[wid - 1] : 0) + incl - sum;
-#pragma unroll
-      for (int q = 0; q < LOCAL_PER_THREAD; ++q) {
-        const int i = tid * LOCAL_PER_THREAD + q;
-        if (i < ns) S.pref[i] = run;
-        run += dg[q];
-      }
-      if (tid == LOCAL_THREADS - 1) S.es = (int)S.wsum[LOCAL_THREADS / 32 - 1];
+      continue;
     }
+    // where the next level is run follows from this one's size, known to all
+    const LocalLay nxt{solo, solo || E <= SOLO_DOWN};
+    LocalPub* const mine = &S.mine[k % 3];
+    if (tid == 0) {  // the next level's counters (last read before the previous level's barrier)
+      S.mine[(k + 1) % 3] = LocalPub{0, 0, 0u, 0, 0u, 0u};
+      S.placed[p1] = 0u;
+    }
+    LocalPlace<C> place{d, S, cl, mine, k, p0, rank, lg, nxt, false};
+    LocalSum sum;
+    local_entries(S, cur, made, p1, rank, lg, [&](int at, bool valid) {
+      LocalEntry en{0ull, 0, 0};
+      if (valid) *reinterpret_cast<int4*>(&en) = *reinterpret_cast<const int4*>(&S.ent[p1][at]);
+      const long long b = (long long)(en.edges & ((1ull << 44) - 1ull));
+      const int n = (int)(en.edges >> 44);
+      const int og = en.orig;
+      // the row's visited bit: here and not at its discovery, where the level's barrier would wait for it
+      if (valid && en.row >= 0) atomicOr(d.vis + (en.row >> 5), 1u << (en.row & 31));
+      float fu = 0.f;
+      if (SR == SS_REAL && valid) {  // the row's value: its sum, final since the last barrier
+        const int x = en.row;
+        fu = __ldcg((lev == 0 ? d.fr : d.psum) + (x < 0 ? -1 - x : x));
+        if (lev > 0 && x >= 0) d.fr[x] = fu;
+      }
+      local_claim<SR, C>(d, place, sum, b, C, n <= LOCAL_EDGES ? n : 0, og, fu);
+      unsigned more = __ballot_sync(SS_FULL_MASK, n > LOCAL_EDGES);
+      while (more) {  // long rows: the warp takes 32 x LOCAL_EDGES edges at a time
+        const int src = __ffs(more) - 1;
+        more &= more - 1;
+        const long long bl = __shfl_sync(SS_FULL_MASK, b, src);
+        const int nl = __shfl_sync(SS_FULL_MASK, n, src);
+        const int ol = __shfl_sync(SS_FULL_MASK, og, src);
+        const float fl = SR == SS_REAL ? __shfl_sync(SS_FULL_MASK, fu, src) : 0.f;
+        for (int j0 = 0; j0 < nl; j0 += 32 * LOCAL_EDGES) {
+          const int j = j0 + lane;
+          local_claim<SR, C>(d, place, sum, bl + (long long)j * C, 32 * C, j < nl ? (nl - j + 31) / 32 : 0, ol, fl);
+        }
+      }
+    });
+    {  // this CTA's counters of the level
+      const unsigned nn = __reduce_add_sync(SS_FULL_MASK, (unsigned)sum.nnew);
+      const unsigned md = __reduce_max_sync(SS_FULL_MASK, sum.md);
+      if (nn) {  // (a warp's 32 low halves of 20 bits, and its high halves, fit 32 bits)
+        const unsigned lo = __reduce_add_sync(SS_FULL_MASK, (unsigned)sum.nd & 0xFFFFFu);
+        const unsigned hi = __reduce_add_sync(SS_FULL_MASK, (unsigned)(sum.nd >> 20));
+        if (lane == 0) {
+          atomicAdd(&mine->nnew, (int)nn);
+          atomicMax(&mine->md, md);
+          atomicAdd(&mine->nd_lo, lo);
+          if (hi) atomicAdd(&mine->nd_hi, hi);
+        }
+      }
+    }
+    if (SR == SS_REAL && solo) __threadfence();  // the sums are read past L1 after the barrier
     __syncthreads();
-    const int Es = S.es;
-    // ---- scatter: each thread a contiguous run of at most BATCH edges per pass
-    // (a 4-edge batch when that covers the slice: fewer idle unrolled steps) ----
-    for (int e0 = 0; e0 < Es; e0 += LOCAL_THREADS * BATCH) {
-      const int per = min(BATCH, (Es - e0 + LOCAL_THREADS - 1) / LOCAL_THREADS);
-      if (per <= 4)
-        local_scatter<SR, C, 4>(d, S, p0, p1, ns, e0, per, Es, tid, k);
-      else
-        local_scatter<SR, C, BATCH>(d, S, p0, p1, ns, e0, per, Es, tid, k);
-    }
-    __syncthreads();
-    if (tid < G) {  // tell every CTA how many vertices this one found
-      LocalPub* dst = &cl.map_shared_rank(&S, tid)->all[p0][rank];
-      dst->nsm = min(S.nnew, LOCAL_NEWCAP);
-      dst->novf = S.novf;
-    }
-    if (rank == 0 && tid == 0) d.qovf_n[p1] = 0ull;  // the next level's overflow counter
-    if (tid == 0) {  // units for the next level are appended after this barrier
-      S.hubn = 0;
-      S.drop = 0;
-      S.placed = 0ull;
-    }
-    cl.sync();  // #1: every scatter is done, so parents and sums are final
-    // ---- list positions (every warp alike): this CTA's list, then its share of the overflow ----
-    long long tot, novf, off;
-    {
-      const int nr = lane < G ? S.all[p0][lane].nsm : 0;
-      const int vr = lane < G ? S.all[p0][lane].novf : 0;
-      novf = (long long)__reduce_add_sync(SS_FULL_MASK, (unsigned)vr);
-      const long long cntr = nr + (lane < G ? share(novf, lane + 1, lg) - share(novf, lane, lg) : 0);
-      long long incl = cntr;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long t = __shfl_up_sync(SS_FULL_MASK, incl, o);
-        if (lane >= o) incl += t;
-      }
-      tot = __shfl_sync(SS_FULL_MASK, incl, 31);
-      off = __shfl_sync(SS_FULL_MASK, incl - cntr, rank);
-    }
-    const int nsm = S.all[p0][rank].nsm;
-    const long long olo = share(novf, rank, lg);
-    const int cnt = nsm + (int)(share(novf, rank + 1, lg) - olo);
-    // the next slices are filled only for a frontier the cluster will likely take:
-    // past local_max_e / 4 vertices its edges almost surely outgrow the cluster
-    const bool next_here = local_fits(d, (unsigned long long)tot, 0ull) && tot <= d.local_max_e / 4;
-    // ---- post: level, parent, value, frontier bit and list record of each new vertex;
-    // its data also goes straight to the CTA that takes it in the next level ----
-    unsigned long long nd = 0;
-    unsigned md = 0;
-    for (int i0 = 0; i0 < cnt; i0 += LOCAL_POST * LOCAL_THREADS) {
-      int vv[LOCAL_POST], dv[LOCAL_POST], og[LOCAL_POST];
-      long long csv[LOCAL_POST];
-      float fv[LOCAL_POST];
-#pragma unroll
-      for (int q = 0; q < LOCAL_POST; ++q) {
-        const int i = i0 + q * LOCAL_THREADS + tid;
-        vv[q] = -1;
-        if (i < cnt) vv[q] = (i < nsm) ? S.nid[i] : __ldcg(d.qovf + olo + (i - nsm));
-      }
-#pragma unroll
-      for (int q = 0; q < LOCAL_POST; ++q) {  // every load of the batch before any store
-        if (vv[q] >= 0) {
-          dv[q] = __ldg(d.rdeg + vv[q]);
-          csv[q] = __ldg(d.cs + vv[q] / C);
-          og[q] = __ldg(d.perm + vv[q]);
-          fv[q] = (SR == SS_REAL) ? __ldcg(d.psum + vv[q]) : 0.0f;
-        }
-      }
-      // a level with more edges than the cluster takes is handed back, so nothing
-      // past that is placed (one hub of 163 K edges is 160 units, each a remote
-      // append: 35 us on Kronecker 22's second level against 20 us now)
-      bool place = next_here;
-      {
-        if (d.max_degree > LOCAL_UNIT) {  // (short rows are one entry each)
-          unsigned mine = 0;
-#pragma unroll
-          for (int q = 0; q < LOCAL_POST; ++q)
-            if (vv[q] >= 0) mine += (unsigned)min(dv[q], 1 << 24);
-          mine = __reduce_add_sync(SS_FULL_MASK, mine);
-          int over = 0;
-          if (lane == 0 && place)
-            over = atomicAdd(&S.placed, (unsigned long long)mine) + mine > (unsigned long long)d.local_max_e;
-          if (__shfl_sync(SS_FULL_MASK, over, 0)) {
-            place = false;
-            S.drop = 1;
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < LOCAL_POST; ++q) {
-        if (vv[q] < 0) continue;
-        const int x = vv[q];
-        if (SR == SS_REAL) {
-          d.fr[x] = fv[q];
-          d.psum[x] = 0.0f;
-        }
-        atomicOr(fbk + (x >> 5), 1u << (x & 31));
-        atomicOr(d.vis + (x >> 5), 1u << (x & 31));
-        const long long at = off + i0 + q * LOCAL_THREADS + tid;
-        const long long bx = csv[q] + (x % C);
-        d.qlist[p0][at] = x;
-        d.qdeg[p0][at] = dv[q];
-        d.qbase[p0][at] = bx;
-        d.qorig[p0][at] = og[q];
-        if (place) {
-          const int r = share_owner(at, tot, lg);
-          place_entry<C>(S, cl, G, r, (int)(at - share(tot, r, lg)), p0, x, bx, dv[q], og[q],
-                         [&](int o) { return (int)(share(tot, o + 1, lg) - share(tot, o, lg)); });
-        }
-        nd += (unsigned long long)dv[q];
-        md = max(md, (unsigned)dv[q]);
-      }
-    }
-    // this CTA's statistics, told to every CTA
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nd += __shfl_down_sync(SS_FULL_MASK, nd, o);
-    md = __reduce_max_sync(SS_FULL_MASK, md);
-    if (lane == 0) {
-      S.red[wid] = nd;
-      S.redmax[wid] = md;
-    }
-    __syncthreads();
-    if (wid == 0) {
-      unsigned long long w = S.red[lane];
-      unsigned m = S.redmax[lane];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(SS_FULL_MASK, w, o);
-      m = __reduce_max_sync(SS_FULL_MASK, m);
-      if (lane < G) {
-        LocalPub* dst = &cl.map_shared_rank(&S, lane)->all[p0][rank];
-        dst->nd = w;
-        dst->md = m;
-        dst->drop = S.drop;
-      }
-    }
-    cl.sync();  // #2: every record, slice and statistic of level k is in place
+    if (!solo && tid < G) cl.map_shared_rank(&S, tid)->all[p0][rank] = *mine;
+    if (!solo) cl.sync();  // every claim, sum and entry of level k is in place
     // ---- totals (every warp alike) and the stop decision ----
-    unsigned long long td = lane < G ? S.all[p0][lane].nd : 0ull;
-    unsigned tm = lane < G ? S.all[p0][lane].md : 0u;
-    const bool dropped = __any_sync(SS_FULL_MASK, lane < G && S.all[p0][lane].drop != 0);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) td += __shfl_xor_sync(SS_FULL_MASK, td, o);
-    tm = __reduce_max_sync(SS_FULL_MASK, tm);
-    reached += (unsigned long long)tot;
+    const LocalPub pub = lane >= (solo ? 1 : G) ? LocalPub{0, 0, 0u, 0, 0u, 0u} : solo ? *mine : S.all[p0][lane];
+    const unsigned tot = __reduce_add_sync(SS_FULL_MASK, (unsigned)pub.nnew);
+    const unsigned tm = __reduce_max_sync(SS_FULL_MASK, pub.md);
+    dropped = __any_sync(SS_FULL_MASK, pub.drop != 0);
+    // (16 CTAs of 32 warps of 2^25 at most)
+    const unsigned long long td = (unsigned long long)__reduce_add_sync(SS_FULL_MASK, pub.nd_lo & 0xFFFFFu) +
+                                  ((unsigned long long)__reduce_add_sync(SS_FULL_MASK, (pub.nd_lo >> 20)) << 20) +
+                                  ((unsigned long long)__reduce_add_sync(SS_FULL_MASK, pub.nd_hi) << 20);
+    reached += tot;
     // the same decision advance_level takes on the control block
     const bool stop = tot == 0 || k >= d.n + 1 || reached > d.reach_cap;
-    if (tid == 0) {
-      S.ctl.qlen[p0] = (unsigned long long)tot;
-      advance_level(d, &S.ctl, k, (unsigned long long)tot, td, (unsigned long long)E, 0ull, tm,
-                    VAR_PUSH_LOCAL, rank == 0);
-      S.ctl.list_level = k;
-      S.ctl.list_prev_ok = 1;
-      if (time_levels && rank == 0 && k < d.iter_cap) {  // device-side time of this level
+    if (rank == 0 && tid == LOCAL_THREADS - 1) {
+      advance_level(d, &S.ctl, k, tot, td, E, 0ull, tm, VAR_PUSH_LOCAL);
+      if (time_levels && k < d.iter_cap) {  // device-side time of this level
         const unsigned long long t = global_ns();
         d.iters[k].kernel_ns = (int)min(t - t_prev, 2000000000ull);
         t_prev = t;
       }
     }
     reached_deg += td;
-    if (rank == 0 && wid == LOCAL_THREADS / 32 - 1 && lane < 7 && k < d.iter_cap) {
+    if (rank == 0 && wid == LOCAL_THREADS / 32 - 2 && lane < 7 && k < d.iter_cap) {
       // the totals the next level's selector features come from (computed at exit)
       const unsigned long long v = lane == 0 ? (unsigned long long)tot : lane == 1 ? td
-                                 : lane == 2 ? (unsigned long long)tm : lane == 3 ? (unsigned long long)E
-                                 : lane == 4 ? reached : lane == 5 ? reached_deg : (unsigned long long)nf;
+                                 : lane == 2 ? (unsigned long long)tm : lane == 3 ? E
+                                 : lane == 4 ? reached : lane == 5 ? reached_deg : nf;
       d.lstat[(size_t)k * SS_LSTAT + lane] = v;
     }
-    if (stop) {
-      local_features(d, S, cl, k0, k - 1);
-      local_exit(S, c, il, 0u, cl);
-      return;
-    }
-    if (!next_here || dropped) {  // the next frontier does not fit: hand back before using it
-      local_features(d, S, cl, k0, k);
-      ++k;
-      if (tid == 0) {
-        S.ctl.list_level = k - 1;
-        S.ctl.list_prev_ok = 1;
-      }
-      local_exit(S, c, il, 1u, cl);
-      return;
-    }
-    ns_prev = nsv;  // this level's frontier is level (k+1)-2
     nf = tot;
-    E = (long long)td;
+    E = td;
+    last = k;
     ++k;
+    cur = nxt;
+    made = __shfl_sync(SS_FULL_MASK, pub.nent, 0);  // (rank 0's)
+    handback = !stop;
+    stopped = stop || dropped || lev + 1 >= max_levels || !local_fits(d, nf, E);
+    const bool wake = solo && !stopped && E > SOLO_UP;  // the others take part again
+    if (wake) {  // rank 0's entries, spread as if it had placed them so
+      const int n = min(made, LOCAL_ENTRIES);
+      // (in rounds of ascending entries: slot e >> lg never passes what has been read)
+      for (int j = 0; j < n; j += LOCAL_THREADS) {
+        const int e = j + tid;
+        LocalEntry en{0ull, 0, 0};
+        if (e < n) *reinterpret_cast<int4*>(&en) = *reinterpret_cast<const int4*>(&S.ent[p0][e]);
+        __syncthreads();
+        if (e < n)
+          *reinterpret_cast<int4*>(&cl.map_shared_rank(&S, e & (G - 1))->ent[p0][e >> lg]) =
+              *reinterpret_cast<const int4*>(&en);
+      }
+      cur.to_one = false;
+    }
+    if (solo && (stopped || wake)) {  // tell the waiting CTAs
+      if (tid < G && tid != 0) {
+        cl.map_shared_rank(&S, tid)->all[p0][0] = *mine;
+        LocalMsg m;
+        m.k = k;
+        m.exit = stopped ? 1 : 0;
+        m.handback = handback ? 1 : 0;
+        m.dropped = dropped ? 1 : 0;
+        m.nf = nf;
+        m.E = E;
+        m.reached = reached;
+        m.reached_deg = reached_deg;
+        cl.map_shared_rank(&S, tid)->msg = m;
+      }
+      cl.sync();
+    }
   }
+  // ---- the launch ends: the last frontier's bits (and real values), then the control block ----
+  if (rank == 0 && last >= k0) local_features(d, k0, handback ? last : last - 1);
+  if (handback) {
+    unsigned* fb = d.fb[last & 1];
+    local_entries(S, cur, made, last & 1, rank, lg, [&](int at, bool valid) {
+      if (!valid) return;
+      const int x = S.ent[last & 1][at].row;
+      if (x < 0) return;
+      atomicOr(fb + (x >> 5), 1u << (x & 31));
+      atomicOr(d.vis + (x >> 5), 1u << (x & 31));
+      if (SR == SS_REAL && last >= k0) d.fr[x] = __ldcg(d.psum + x);
+    });
+    if (SR == SS_REAL && dropped) {  // values of the rows without room: every row of the bitmap
+      for (long long w = (long long)rank * LOCAL_THREADS + tid; w < (d.n_pad + 31) / 32; w += (long long)G * LOCAL_THREADS)
+        for (unsigned bits = __ldcg(fb + w); bits; bits &= bits - 1) {
+          const long long x = w * 32 + __ffs(bits) - 1;
+          d.fr[x] = __ldcg(d.psum + x);
+        }
+    }
+  }
+  cl.sync();  // no CTA leaves while another may still write its shared memory
+  if (rank != 0) return;
+  if (tid == 0 && SR == SS_REAL) S.ctl.psum_dirty = 1;
+  __syncthreads();
+  for (int i = tid; i < CTL_WORDS; i += LOCAL_THREADS)
+    reinterpret_cast<unsigned*>(c)[i] = reinterpret_cast<const unsigned*>(&S.ctl)[i];
+  if (tid == 0 && il.use_cond) cudaGraphSetConditional(il.cond, handback ? 1u : 0u);
 }
 
 
