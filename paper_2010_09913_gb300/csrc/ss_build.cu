@@ -553,8 +553,7 @@ static ss_status alloc_state(slimsell_graph* h) {
   if ((s = dmalloc(h, (void**)&h->bunits, sizeof(int2) * (size_t)h->bunits_cap)) != SS_OK) return s;
   if ((s = dmalloc(h, (void**)&h->psum, sizeof(float) * np)) != SS_OK) return s;
   if ((s = dmalloc(h, (void**)&h->touched, sizeof(unsigned) * (size_t)h->fb_words)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->qlist, sizeof(int) * np)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->qcount, 2 * sizeof(unsigned long long))) != SS_OK) return s;
+  if ((s = dmalloc(h, (void**)&h->qcount, sizeof(unsigned long long))) != SS_OK) return s;
   h->local_cluster = push_local_cluster_size();
   if (h->local_cluster <= 0) {
     set_error("slimsell_build: no thread-block cluster of the push kernel fits on this device");
@@ -592,7 +591,7 @@ void free_handle(slimsell_graph* h) {
   void* ptrs[] = {h->perm, h->invperm, h->rdeg, h->cl, h->cs, h->col, h->items, h->split_n,
                   h->claim, h->vis, h->act, h->fb[0], h->fb[1], h->fr, h->xacc, h->xpar,
                   h->arrive, h->ctl, h->iters, h->units, h->bunits,
-                  h->psum, h->touched, h->qlist, h->qcount, h->lstat, h->mlp, h->feats, h->mF[0],
+                  h->psum, h->touched, h->qcount, h->lstat, h->mlp, h->feats, h->mF[0],
                   h->mF[1], h->mV, h->mxacc, h->mroots};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -631,7 +630,7 @@ ss::Dev slimsell_graph::dev() const {
   d.format = SS_FORMAT_SLIMSELL; d.scol = nullptr; d.sval = nullptr;  // set per call by slimsell_bfs
   d.psum = psum; d.touched = touched; d.mlp = mlp; d.feats = feats;
   d.sel_margin = sel_margin;
-  d.qlist = qlist; d.qcount = qcount;
+  d.qcount = qcount;
   d.local_cluster = local_cluster;
   d.local_max_nf = (long long)local_cluster * SS_LOCAL_SLICE;
   d.local_max_e = (long long)local_cluster * SS_LOCAL_EDGES_PER_CTA;

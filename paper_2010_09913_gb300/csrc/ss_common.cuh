@@ -69,7 +69,6 @@ struct Ctl {
   unsigned int prev_maxdeg;       // ... by the previous iteration
   unsigned long long units;       // push work units queued by the current iteration
   unsigned long long variant_count[5];  // iterations run with each variant
-  unsigned long long qprep;       // length of the vertex list built from the bitmap
   unsigned long long loop_guard;  // decide-kernel executions in this run (device loop bound)
   unsigned long long bunits;      // push block units queued by the current iteration
   unsigned long long new_rowdeg;  // multi-source: degree sum of the rows that gained a source
@@ -113,8 +112,7 @@ struct Dev {
   int push_blocks;      // 0: vertex units only, 1: block units for dense blocks, 2: for every block
   float* psum;          // [n_pad] push: real-semiring sum of frontier-neighbour values
   unsigned* touched;    // [fb_words] push: rows reached by the current push
-  int* qlist;           // [n_pad] cluster push: rows of its first frontier, then rows without room
-  unsigned long long* qcount;  // [2] cluster push: rows without room, entries of the first frontier
+  unsigned long long* qcount;  // [1] cluster push: entries of its first frontier
   int local_cluster;    // CTAs in the cluster push's cluster
   long long local_max_nf, local_max_e;  // largest frontier (vertices, edges) it takes
   const float* mlp;     // selector weights (16-64-64-4 MLP), or NULL
@@ -174,7 +172,6 @@ struct slimsell_graph {
   int push_blocks = 1;                 // see SS_OPT_PUSH_BLOCKS
   float* psum = nullptr;
   unsigned* touched = nullptr;
-  int* qlist = nullptr;
   unsigned long long* qcount = nullptr;
   int local_cluster = 0;
   float* mlp = nullptr;       // selector weights on the device (NULL until loaded)

@@ -113,7 +113,6 @@ __device__ __forceinline__ bool advance_level(const Dev& d, Ctl* c, int k, unsig
   if (variant >= 0 && variant < N_VARIANTS) c->variant_count[variant] += 1;
   c->units = 0;
   c->bunits = 0;
-  c->qprep = 0;
   bool stop = (nc == 0);
   if (k >= d.n + 1 || c->reached > d.reach_cap) {
     c->error |= 1;
@@ -258,7 +257,6 @@ __device__ __forceinline__ void init_ctl(const Dev& d, Ctl* c, int r) {
   c->bunits = 0;
   for (int v = 0; v < N_VARIANTS; ++v) c->variant_count[v] = 0;
   c->loop_guard = 0;
-  c->qprep = 0;
   c->psum_dirty = 0;
   ss_iter_stats s;
   s.frontier = 1; s.frontier_degree = d.rdeg[r]; s.slots = 0; s.active_chunks = 0;

@@ -243,7 +243,6 @@ __global__ void k_multi_roots(MultiDev m, int W, int* parent) {
     c->prev2_new = 0; c->prev_active = 0; c->new_maxdeg = 0; c->prev_maxdeg = 0; c->units = 0; c->bunits = 0;
     c->loop_guard = 0;
     for (int v = 0; v < N_VARIANTS; ++v) c->variant_count[v] = 0;
-    c->qprep = 0;
     c->new_rowdeg = 0;
     c->prev_rowdeg = rd;  // the roots' rows (a repeated root counted again: an upper bound)
     ss_iter_stats st;

@@ -284,49 +284,7 @@ struct LocalSmem {
 static_assert(sizeof(LocalSmem) <= 227 * 1024, "cluster push shared memory");
 static_assert(LOCAL_THREADS / 32 >= SS_LOCAL_CLUSTER_MAX, "a warp for every segment of a slice");
 
-// Entry: list the level-(k-1) rows into qlist and clear fb[k&1] (it held level k-2).
-__global__ void __launch_bounds__(PUSH_THREADS) k_push_local_prep(Dev d) {
-  Ctl* c = d.ctl;
-  if (c->done) return;
-  const int k = c->k;
-  const int lane = threadIdx.x & 31;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long words = ((long long)d.n_pad + 31) / 32;
-  const unsigned* fbm = d.fb[(k - 1) & 1];
-  unsigned* fbk = d.fb[k & 1];
-  for (long long i0 = t0 - lane; i0 < words; i0 += stride & ~31LL) {
-    const long long i = i0 + lane;
-    unsigned bits = 0u;
-    if (i < words) {
-      bits = fbm[i];
-      fbk[i] = 0u;
-    }
-    while (__any_sync(SS_FULL_MASK, bits != 0u)) {
-      int u = -1;
-      if (bits) {
-        const int b = __ffs(bits) - 1;
-        bits &= bits - 1;
-        u = (int)(i * 32 + b);
-      }
-      const unsigned m = __ballot_sync(SS_FULL_MASK, u >= 0);
-      unsigned long long base = 0;
-      if (lane == 0) base = atomicAdd(&c->qprep, (unsigned long long)__popc(m));
-      base = __shfl_sync(SS_FULL_MASK, base, 0);
-      // the decide kernel sends only frontiers that fit the list
-      const unsigned long long at = base + __popc(m & ((1u << lane) - 1u));
-      if (u >= 0 && at < (unsigned long long)d.n_pad) d.qlist[at] = u;
-    }
-  }
-}
-
 extern __shared__ __align__(16) unsigned char ss_local_smem[];
-
-// CTA r's first entry of a list of `total` entries split into G = 2^lg equal
-// shares (every list here has fewer than 2^27 entries, so 32 bits hold total * G).
-__device__ __forceinline__ long long share(long long total, int r, int lg) {
-  return (long long)(((unsigned)total * (unsigned)r) >> lg);
-}
 
 // How the entries of a level lie: made by rank 0 alone or by every CTA, for rank 0
 // alone or for every CTA.  A making CTA owns one segment of every taking CTA.
@@ -585,7 +543,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
   int k = c->k;
   const int k0 = k;  // first level of this launch (its features came from the decide kernel)
   const int done = c->done;
-  unsigned long long nf = c->qprep, E = c->prev_deg;  // rows and edges of the level-(k-1) frontier
+  unsigned long long nf = c->prev_new, E = c->prev_deg;  // rows and edges of the level-(k-1) frontier
   unsigned long long reached = c->reached, reached_deg = c->reached_deg;
   if (rank == 0)
     for (int i = tid; i < CTL_WORDS; i += LOCAL_THREADS)
@@ -608,24 +566,47 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
     cur = LocalLay{true, true};
     nf = 0;
   }
-  // the first entries, from the list; the first frontier's bits are cleared
-  {
+  // the first entries, from the frontier bitmap (a kernel of its own, listing the rows first,
+  // cost each launch 3 us more); the first frontier's bits are cleared, and those of level k-2
+  if (handback) {
     const int p1 = (k - 1) & 1;
     LocalPlace<C> place{d, S, cl, &S.mine[0], k, p1, rank, lg, cur, true};
-    const long long lo = share((long long)nf, rank, lg), hi = share((long long)nf, rank + 1, lg);
-    unsigned* fbm = d.fb[p1];
-    for (long long i0 = lo + wid * 32; i0 < hi; i0 += LOCAL_THREADS) {
-      int u = -1, dv = 0, og = 0;
-      long long bx = 0;
-      if (i0 + lane < hi) {
-        u = __ldcg(d.qlist + i0 + lane);
-        fbm[u >> 5] = 0u;
-        bx = __ldg(d.cs + u / C) + (u % C);
-        dv = __ldg(d.rdeg + u);
-        og = __ldg(d.perm + u);
+    const long long words = ((long long)d.n_pad + 31) / 32;
+    unsigned *fbm = d.fb[p1], *fbk = d.fb[k & 1];
+    constexpr int AHEAD = 8;  // words in flight per thread
+    // a thread takes 1 / 2^sp of a word's bits, so that the rows of a small graph's few words
+    // spread over the cluster (the parts of a word lie in one warp)
+    const long long threads = (long long)G * LOCAL_THREADS;
+    int sp = 0;
+    while (sp < 5 && (words << (sp + 1)) <= threads) ++sp;
+    const unsigned part = (sp ? (1u << (32 >> sp)) - 1u : ~0u) << ((tid & ((1 << sp) - 1)) * (32 >> sp));
+    for (long long t0 = (long long)rank * LOCAL_THREADS + tid; t0 - lane < words << sp; t0 += AHEAD * threads) {
+      unsigned bits[AHEAD];
+#pragma unroll
+      for (int j = 0; j < AHEAD; ++j) {
+        const long long w = (t0 + j * threads) >> sp;
+        bits[j] = w < words ? __ldcg(fbm + w) : 0u;
+        if (w < words) fbk[w] = 0u;
       }
-      if (dv == 0) u = -1;  // (an isolated root has no edges)
-      place.template operator()<1>(&u, &bx, &dv, &og);
+#pragma unroll
+      for (int j = 0; j < AHEAD; ++j) {
+        const long long w = (t0 + j * threads) >> sp;
+        if (bits[j]) fbm[w] = 0u;
+        bits[j] &= part;
+        while (__any_sync(SS_FULL_MASK, bits[j] != 0u)) {
+          int u = -1, dv = 0, og = 0;
+          long long bx = 0;
+          if (bits[j]) {
+            u = (int)(w * 32 + __ffs(bits[j]) - 1);
+            bits[j] &= bits[j] - 1;
+            bx = __ldg(d.cs + u / C) + (u % C);
+            dv = __ldg(d.rdeg + u);
+            og = __ldg(d.perm + u);
+          }
+          if (dv == 0) u = -1;  // (an isolated root has no edges)
+          place.template operator()<1>(&u, &bx, &dv, &og);
+        }
+      }
     }
   }
   cl.sync();  // the first entries are in place
@@ -856,8 +837,6 @@ static ss_status launch_push_local_c(const slimsell_graph* h, const Dev& d, cons
     SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocalSmem)));
     SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   }
-  k_push_local_prep<<<vertex_grid(h, 32 * PUSH_THREADS), PUSH_THREADS, 0, st>>>(d);
-  SS_CUDA(cudaGetLastError());
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(d.local_cluster);
   cfg.blockDim = dim3(LOCAL_THREADS);
