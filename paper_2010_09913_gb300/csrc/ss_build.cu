@@ -9,7 +9,7 @@
 #include <cstdarg>
 #include <climits>
 #include <algorithm>
-#include <cstring>
+#include <utility>
 #include <vector>
 
 #include "ss_device.cuh"
@@ -43,6 +43,27 @@ ss_status dmalloc(slimsell_graph* h, void** p, size_t bytes) {
   if (h) h->device_bytes += (long long)bytes;
   return SS_OK;
 }
+
+namespace {
+// Several arrays in one device allocation (a handle made 47 cudaMalloc and 47
+// cudaFree calls, 3 ms of a 7.5 ms build of Kronecker 22): arrays are announced,
+// then placed at 256-byte boundaries of one allocation.
+struct Slab {
+  std::vector<std::pair<void**, size_t>> want;
+  size_t total = 0;
+  template <class T>
+  void add(T** p, size_t count) {
+    want.push_back({(void**)p, total});
+    total += (std::max<size_t>(count, 1) * sizeof(T) + 255) / 256 * 256;
+  }
+  ss_status place(slimsell_graph* h, void** base) {
+    ss_status s = dmalloc(h, base, total);
+    if (s != SS_OK) return s;
+    for (auto& w : want) *w.first = (char*)*base + w.second;
+    return SS_OK;
+  }
+};
+}  // namespace
 
 // ---------------------------------------------------------------------------
 // Exclusive prefix sum over int64 (three passes: tile sums, scan of sums, tile scans)
@@ -316,25 +337,68 @@ __global__ void k_item_fill(const int* cl, int n_c, int W, const long long* off,
   }
 }
 
-// one warp per item: col[cs_i + j*C + l] for slots j0*C .. j1*C of the chunk
-__global__ void k_pack(const int4* items, int n_items, const long long* cs, int C, const int* perm,
-                       const int* invperm, const int* rdeg, const long long* row_ptr,
-                       const int* csr_col, int* col) {
+// col[cs_i + j*C + l] for the columns of every item, one warp per item.  A lane owns a
+// row (C = 64: two in turn; C < 32: 32 / C columns side by side) and walks its
+// neighbours from the last, PACK_STEP at a time: consecutive entries of one row share
+// sectors, and the stores of a column are coalesced.  Bound by the random gathers of
+// invperm (one per edge, from L2); working out row and column of every slot anew, with
+// four dependent loads each, took 2.2 ms on Kronecker 22; this one takes 0.86.
+constexpr int PACK_STEP = 8;
+template <int C>
+__global__ void __launch_bounds__(256) k_pack(const int4* items, int n_items, const long long* cs,
+                                              const int* perm, const int* __restrict__ invperm,
+                                              const int* rdeg, const long long* row_ptr,
+                                              const int* __restrict__ csr_col, int* __restrict__ col) {
+  constexpr int ROWS = C < 32 ? C : 32, SIDE = 32 / ROWS;
   const int lane = threadIdx.x & 31;
   const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long it = wid; it < n_items; it += nw) {
-    int4 item = items[it];
+    const int4 item = items[it];
     const long long c0 = cs[item.x];
-    const long long s_end = (long long)item.z * C;
-    for (long long s = (long long)item.y * C + lane; s < s_end; s += 32) {
-      int j = (int)(s / C), l = (int)(s % C);
-      long long r = (long long)item.x * C + l;
-      int v = perm[r];
-      int out = -1;
-      if (v >= 0 && j < rdeg[r]) out = invperm[csr_col[row_ptr[v + 1] - 1 - j]];
-      col[c0 + s] = out;
+#pragma unroll
+    for (int l = lane % ROWS; l < C; l += 32) {
+      const long long r = (long long)item.x * C + l;
+      const int v = perm[r];
+      const int deg = v >= 0 ? rdeg[r] : 0;
+      const int* src = csr_col + (v >= 0 ? row_ptr[v + 1] - 1 : 0);
+      int* dst = col + c0 + l;
+      for (int j0 = item.y + lane / ROWS; j0 < item.z; j0 += PACK_STEP * SIDE) {
+        int u[PACK_STEP];
+#pragma unroll
+        for (int q = 0; q < PACK_STEP; ++q) {
+          const int j = j0 + q * SIDE;
+          u[q] = (j < deg && j < item.z) ? __ldg(src - j) : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < PACK_STEP; ++q)
+          if (u[q] >= 0) u[q] = __ldg(invperm + u[q]);
+#pragma unroll
+        for (int q = 0; q < PACK_STEP; ++q) {
+          const int j = j0 + q * SIDE;
+          if (j < item.z) dst[(long long)j * C] = u[q];
+        }
+      }
     }
+  }
+}
+
+// Sort keys of the work items: longest first.
+__global__ void k_item_keys(const int4* items, int n, int longest, unsigned long long* keys, int* vals) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    keys[i] = (unsigned long long)(longest - (items[i].z - items[i].y));
+    vals[i] = (int)i;
+  }
+}
+
+// Items by descending length (sorted) in snake order: position p of round p / W
+// comes from the mirrored position in every other round.
+__global__ void k_item_snake(const int4* items, const int* sorted, int n, int W, int4* out) {
+  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
+       p += (long long)gridDim.x * blockDim.x) {
+    const long long r = p / W, w = p % W, len = min((long long)W, n - r * W);
+    out[p] = items[sorted[(r & 1) ? r * W + (len - 1 - w) : p]];
   }
 }
 
@@ -347,135 +411,101 @@ static int bit_width(unsigned long long x) {
   return b;
 }
 
-// build an item table of width W; returns the item count through *n_items_out
-static ss_status make_items(slimsell_graph* h, int W, long long* tmp_cnt, long long* tmp_flag,
-                            long long* tmp_scan, int4** items_out, int* n_items_out, int** split_n_out,
-                            int* n_split_out, bool owned, cudaStream_t st) {
-  const int n_c = h->n_c;
-  const int grid = 4 * h->num_sms;
-  k_item_count<<<grid, 256, 0, st>>>(h->cl, n_c, W, tmp_cnt, split_n_out ? tmp_flag : nullptr);
-  SS_CUDA(cudaGetLastError());
-  ss_status s = excl_scan(tmp_cnt, n_c + 1, tmp_scan, st);
-  if (s != SS_OK) return s;
-  if (split_n_out) {
-    s = excl_scan(tmp_flag, n_c + 1, tmp_scan, st);
+// Stable sort of n (key, value) pairs by the low `bits` bits; the sorted values end in *out.
+static ss_status sort_pairs(unsigned long long* keys_a, unsigned long long* keys_b, int* vals_a, int* vals_b,
+                            int n, int bits, long long* hist, long long* tmp_scan, int** out, cudaStream_t st) {
+  const int nblk = (n + RS_TILE - 1) / RS_TILE;
+  for (int shift = 0; shift < bits; shift += 8) {
+    k_rs_hist<<<nblk, RS_THREADS, 0, st>>>(keys_a, n, shift, hist, nblk);
+    ss_status s = excl_scan(hist, (long long)256 * nblk, tmp_scan, st);
     if (s != SS_OK) return s;
+    k_rs_scatter<<<nblk, RS_THREADS, 0, st>>>(keys_a, vals_a, keys_b, vals_b, n, shift, hist, nblk);
+    std::swap(keys_a, keys_b);
+    std::swap(vals_a, vals_b);
   }
-  long long nitems = 0, nsplit = 0;
-  SS_CUDA(cudaMemcpyAsync(&nitems, tmp_cnt + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
-  if (split_n_out)
-    SS_CUDA(cudaMemcpyAsync(&nsplit, tmp_flag + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
-  SS_CUDA(cudaStreamSynchronize(st));
-  if (nitems > 0x7fffffffLL) {
-    set_error("too many work items (%lld)", nitems);
-    return SS_ERR_UNSUPPORTED;
-  }
-  int4* items = nullptr;
-  s = dmalloc(owned ? h : nullptr, (void**)&items, sizeof(int4) * (size_t)nitems);
-  if (s != SS_OK) return s;
-  int* split_n = nullptr;
-  if (split_n_out) {
-    s = dmalloc(h, (void**)&split_n, sizeof(int) * (size_t)(nsplit > 0 ? nsplit : 1));
-    if (s != SS_OK) {
-      cudaFree(items);
-      return s;
-    }
-  }
-  k_item_fill<<<grid, 256, 0, st>>>(h->cl, n_c, W, tmp_cnt, split_n_out ? tmp_flag : nullptr, items,
-                                    split_n);
   SS_CUDA(cudaGetLastError());
-  *items_out = items;
-  *n_items_out = (int)nitems;
-  if (split_n_out) {
-    *split_n_out = split_n;
-    *n_split_out = (int)nsplit;
-  }
+  *out = vals_a;
   return SS_OK;
 }
 
-// Order the BFS work items for the iteration kernels, whose warp w takes items
-// w, w + W, w + 2W, ... (W = warps in the grid): items are sorted by estimated
-// cost (slots plus a fixed per-item overhead), largest first, and every other
-// group of W items is reversed ("snake" order) so each warp's total is balanced.
-static ss_status order_items(slimsell_graph* h, cudaStream_t st) {
-  const int n = h->n_items;
-  if (n <= 1) return SS_OK;
-  std::vector<int4> items((size_t)n), out((size_t)n);
-  SS_CUDA(cudaMemcpyAsync(items.data(), h->items, sizeof(int4) * (size_t)n, cudaMemcpyDeviceToHost, st));
-  SS_CUDA(cudaStreamSynchronize(st));
-  std::vector<int> idx((size_t)n);
-  for (int i = 0; i < n; ++i) idx[i] = i;
-  const long long C = h->C, overhead = 24LL * h->C;
-  std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) {
-    return (items[a].z - items[a].y) * C + overhead > (items[b].z - items[b].y) * C + overhead;
-  });
-  const long long W = (long long)h->num_sms * (SS_PULL_THREADS / 32);
-  for (long long p = 0; p < n; ++p) {
-    const long long r = p / W, w = p % W;
-    const long long round_len = std::min<long long>(W, n - r * W);
-    const long long src = (r & 1) ? r * W + (round_len - 1 - w) : p;
-    out[(size_t)p] = items[(size_t)idx[(size_t)src]];
-  }
-  SS_CUDA(cudaMemcpyAsync(h->items, out.data(), sizeof(int4) * (size_t)n, cudaMemcpyHostToDevice, st));
-  SS_CUDA(cudaStreamSynchronize(st));
-  return SS_OK;
+template <int C>
+static void launch_pack(const slimsell_graph* h, const int4* items, int n_items, const long long* row_ptr,
+                        const int* csr_col, cudaStream_t st) {
+  k_pack<C><<<8 * h->num_sms, 256, 0, st>>>(items, n_items, h->cs, h->perm, h->invperm, h->rdeg, row_ptr,
+                                            csr_col, h->col);
 }
 
-static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const int* csr_col,
+// Widest BFS items that the packing takes as they are (one warp each); wider ones
+// (hub chunks unsplit) are packed from a table of their own.
+constexpr int PACK_WIDTH = 1024;
+
+static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const int* csr_col, void** temps,
                             cudaStream_t st) {
   const int n = h->n, C = h->C;
   const int n_c = h->n_c, n_pad = h->n_pad;
   const int grid = 8 * h->num_sms;
+  const size_t np = (size_t)n_pad;
   ss_status s;
 
-  // temporaries
-  int *deg = nullptr, *maxdeg = nullptr, *vals_a = nullptr, *vals_b = nullptr;
+  // temporaries (temps: allocations that the caller frees)
+  int *deg = nullptr, *flags = nullptr, *vals_a = nullptr, *vals_b = nullptr;
   unsigned long long *keys_a = nullptr, *keys_b = nullptr;
-  long long *hist = nullptr, *tmp_scan = nullptr, *tmp_cnt = nullptr, *tmp_flag = nullptr;
-  int4* pack_items = nullptr;
-  int n_pack_items = 0;
-  auto cleanup = [&]() {
-    cudaFree(deg); cudaFree(maxdeg); cudaFree(vals_a); cudaFree(vals_b);
-    cudaFree(keys_a); cudaFree(keys_b); cudaFree(hist); cudaFree(tmp_scan);
-    cudaFree(tmp_cnt); cudaFree(tmp_flag); cudaFree(pack_items);
-  };
-#define SS_TRY(x)            \
-  do {                       \
-    s = (x);                 \
-    if (s != SS_OK) {        \
-      cleanup();             \
-      return s;              \
-    }                        \
-  } while (0)
-#define SS_TRYC(x) SS_TRY(((x) == cudaSuccess) ? SS_OK : cuda_fail(cudaGetLastError(), #x))
-
+  long long *hist = nullptr, *tmp_scan = nullptr, *cnt = nullptr, *split = nullptr, *pack_cnt = nullptr;
+  const bool own_pack = h->split_w <= 0 || h->split_w > PACK_WIDTH;
   const int nblk = (n + RS_TILE - 1) / RS_TILE;
   const long long scan_len = std::max<long long>((long long)256 * nblk, (long long)n_c + 1);
-  SS_TRY(dmalloc(nullptr, (void**)&deg, sizeof(int) * (size_t)n));
-  SS_TRY(dmalloc(nullptr, (void**)&maxdeg, 2 * sizeof(int)));  // largest degree, live rows
-  SS_TRY(dmalloc(nullptr, (void**)&vals_a, sizeof(int) * (size_t)n));
-  SS_TRY(dmalloc(nullptr, (void**)&vals_b, sizeof(int) * (size_t)n));
-  SS_TRY(dmalloc(nullptr, (void**)&keys_a, sizeof(unsigned long long) * (size_t)n));
-  SS_TRY(dmalloc(nullptr, (void**)&keys_b, sizeof(unsigned long long) * (size_t)n));
-  SS_TRY(dmalloc(nullptr, (void**)&hist, sizeof(long long) * (size_t)256 * nblk));
-  SS_TRY(dmalloc(nullptr, (void**)&tmp_scan, sizeof(long long) * (size_t)(scan_len / SCAN_TILE + 2)));
-  SS_TRY(dmalloc(nullptr, (void**)&tmp_cnt, sizeof(long long) * (size_t)(n_c + 1)));
-  SS_TRY(dmalloc(nullptr, (void**)&tmp_flag, sizeof(long long) * (size_t)(n_c + 1)));
+  {
+    Slab t;
+    t.add(&deg, (size_t)n);
+    t.add(&flags, 2);  // largest degree, live rows
+    t.add(&vals_a, (size_t)n);
+    t.add(&vals_b, (size_t)n);
+    t.add(&keys_a, (size_t)n);
+    t.add(&keys_b, (size_t)n);
+    t.add(&hist, (size_t)256 * nblk);
+    t.add(&tmp_scan, (size_t)(scan_len / SCAN_TILE + 2));
+    t.add(&cnt, (size_t)n_c + 1);
+    t.add(&split, (size_t)n_c + 1);
+    if (own_pack) t.add(&pack_cnt, (size_t)n_c + 1);
+    if ((s = t.place(nullptr, &temps[0])) != SS_OK) return s;
+  }
 
-  // permanent layout arrays
-  SS_TRY(dmalloc(h, (void**)&h->perm, sizeof(int) * (size_t)n_pad));
-  SS_TRY(dmalloc(h, (void**)&h->invperm, sizeof(int) * (size_t)n));
-  SS_TRY(dmalloc(h, (void**)&h->rdeg, sizeof(int) * (size_t)n_pad));
-  SS_TRY(dmalloc(h, (void**)&h->cl, sizeof(int) * (size_t)n_c));
-  SS_TRY(dmalloc(h, (void**)&h->cs, sizeof(long long) * (size_t)(n_c + 1)));
+  // permanent arrays whose size follows from n and nnz: the layout's tables and the BFS state
+  // bitmap words rounded up to whole int4 groups, plus one spare group
+  h->fb_words = (long long)((((np + 31) / 32) + 3) / 4 * 4 + 4);
+  h->units_cap = (long long)np + h->nnz / 256 + 1024;  // any frontier fits
+  h->iter_cap = 1 << 16;
+  {
+    Slab p;
+    p.add(&h->perm, np);
+    p.add(&h->invperm, (size_t)n);
+    p.add(&h->rdeg, np);
+    p.add(&h->cl, (size_t)n_c);
+    p.add(&h->cs, (size_t)n_c + 1);
+    p.add(&h->claim, np);
+    p.add(&h->vis, (size_t)h->fb_words);
+    p.add(&h->act, (size_t)n_c);
+    for (int b = 0; b < 2; ++b) p.add(&h->fb[b], (size_t)h->fb_words);
+    p.add(&h->fr, np);
+    p.add(&h->units, (size_t)h->units_cap);
+    p.add(&h->psum, np);
+    p.add(&h->touched, (size_t)h->fb_words);
+    p.add(&h->qcount, 1);
+    p.add(&h->ctl, 1);
+    p.add(&h->feats, SS_SELECTOR_FEATURES * (size_t)h->iter_cap);
+    p.add(&h->iters, (size_t)h->iter_cap);
+    p.add(&h->lstat, SS_LSTAT * (size_t)h->iter_cap);
+    if ((s = p.place(h, &h->slab[0])) != SS_OK) return s;
+  }
+  SS_CUDA(cudaMemsetAsync(h->psum, 0, sizeof(float) * np, st));
+  SS_CUDA(cudaMemsetAsync(h->touched, 0, sizeof(unsigned) * (size_t)h->fb_words, st));
+  SS_CUDA(cudaMemsetAsync(h->ctl, 0, sizeof(Ctl), st));
 
   // 1. degrees and sort keys
-  SS_TRYC(cudaMemsetAsync(maxdeg, 0, 2 * sizeof(int), st));
-  k_degrees<<<grid, 256, 0, st>>>(row_ptr, n, deg, maxdeg);
-  int h_maxdeg = 0;
-  SS_TRYC(cudaMemcpyAsync(&h_maxdeg, maxdeg, sizeof(int), cudaMemcpyDeviceToHost, st));
-  SS_TRYC(cudaStreamSynchronize(st));
-  h->max_degree = h_maxdeg;
+  SS_CUDA(cudaMemsetAsync(flags, 0, 2 * sizeof(int), st));
+  k_degrees<<<grid, 256, 0, st>>>(row_ptr, n, deg, flags);
+  SS_CUDA(cudaMemcpyAsync(&h->max_degree, flags, sizeof(int), cudaMemcpyDeviceToHost, st));
+  SS_CUDA(cudaStreamSynchronize(st));
 
   // 2. sigma-window sort by descending degree (stable: ties keep ascending id)
   int* sorted = vals_a;
@@ -483,101 +513,117 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
     k_identity<<<grid, 256, 0, st>>>(vals_a, n);
   } else {
     const int sigma = h->sigma >= n ? n : h->sigma;  // already a multiple of C (or >= n)
-    const int dbits = bit_width((unsigned long long)h_maxdeg);
+    const int dbits = bit_width((unsigned long long)h->max_degree);
     const long long nwin = ((long long)n + sigma - 1) / sigma;
-    const int wbits = bit_width((unsigned long long)(nwin - 1));
-    const int bits = dbits + wbits;
-    k_make_keys<<<grid, 256, 0, st>>>(deg, n, sigma, h_maxdeg, dbits, keys_a, vals_a);
-    unsigned long long *kin = keys_a, *kout = keys_b;
-    int *vin = vals_a, *vout = vals_b;
-    for (int shift = 0; shift < bits; shift += 8) {
-      k_rs_hist<<<nblk, RS_THREADS, 0, st>>>(kin, n, shift, hist, nblk);
-      SS_TRY(excl_scan(hist, (long long)256 * nblk, tmp_scan, st));
-      k_rs_scatter<<<nblk, RS_THREADS, 0, st>>>(kin, vin, kout, vout, n, shift, hist, nblk);
-      std::swap(kin, kout);
-      std::swap(vin, vout);
-    }
-    sorted = vin;
+    const int bits = dbits + bit_width((unsigned long long)(nwin - 1));
+    k_make_keys<<<grid, 256, 0, st>>>(deg, n, sigma, h->max_degree, dbits, keys_a, vals_a);
+    if ((s = sort_pairs(keys_a, keys_b, vals_a, vals_b, n, bits, hist, tmp_scan, &sorted, st)) != SS_OK) return s;
   }
-  SS_TRYC(cudaGetLastError());
+  SS_CUDA(cudaGetLastError());
 
-  // 3. perm / invperm / row degrees, chunk lengths and starts
-  k_perm_tables<<<grid, 256, 0, st>>>(sorted, deg, n, n_pad, h->perm, h->invperm, h->rdeg, maxdeg + 1);
+  // 3. perm / invperm / row degrees, chunk lengths and starts, work items per chunk
+  k_perm_tables<<<grid, 256, 0, st>>>(sorted, deg, n, n_pad, h->perm, h->invperm, h->rdeg, flags + 1);
   k_chunk_len<<<grid, 256, 0, st>>>(h->rdeg, n_c, C, h->cl, h->cs);
-  SS_TRYC(cudaGetLastError());
-  SS_TRY(excl_scan(h->cs, n_c + 1, tmp_scan, st));
-  long long slots = 0;
-  SS_TRYC(cudaMemcpyAsync(&slots, h->cs + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
-  SS_TRYC(cudaMemcpyAsync(&h->n_live, maxdeg + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
-  SS_TRYC(cudaStreamSynchronize(st));
+  k_item_count<<<grid, 256, 0, st>>>(h->cl, n_c, h->split_w, cnt, split);
+  if (own_pack) k_item_count<<<grid, 256, 0, st>>>(h->cl, n_c, 256, pack_cnt, nullptr);
+  SS_CUDA(cudaGetLastError());
+  if ((s = excl_scan(h->cs, n_c + 1, tmp_scan, st)) != SS_OK) return s;
+  if ((s = excl_scan(cnt, n_c + 1, tmp_scan, st)) != SS_OK) return s;
+  if ((s = excl_scan(split, n_c + 1, tmp_scan, st)) != SS_OK) return s;
+  if (own_pack && (s = excl_scan(pack_cnt, n_c + 1, tmp_scan, st)) != SS_OK) return s;
+  long long slots = 0, nitems = 0, nsplit = 0, npack = 0;
+  SS_CUDA(cudaMemcpyAsync(&slots, h->cs + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
+  SS_CUDA(cudaMemcpyAsync(&h->n_live, flags + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
+  SS_CUDA(cudaMemcpyAsync(&nitems, cnt + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
+  SS_CUDA(cudaMemcpyAsync(&nsplit, split + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
+  if (own_pack) SS_CUDA(cudaMemcpyAsync(&npack, pack_cnt + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
+  SS_CUDA(cudaStreamSynchronize(st));
+  if (nitems > 0x7fffffffLL || npack > 0x7fffffffLL) {
+    set_error("too many work items (%lld)", std::max(nitems, npack));
+    return SS_ERR_UNSUPPORTED;
+  }
   h->slots = slots;
+  h->n_items = (int)nitems;
+  h->n_split = (int)nsplit;
 
-  // 4. item tables
-  SS_TRY(make_items(h, 256, tmp_cnt, tmp_flag, tmp_scan, &pack_items, &n_pack_items, nullptr,
-                    nullptr, false, st));
-  SS_TRY(make_items(h, h->split_w, tmp_cnt, tmp_flag, tmp_scan, &h->items, &h->n_items, &h->split_n,
-                    &h->n_split, true, st));
-  SS_TRY(order_items(h, st));
+  // permanent arrays whose size follows from the layout; temporaries of the item order
+  // block units cover PUSH_BLOCK_SLOTS / C columns each: at most one partial unit per chunk
+  h->bunits_cap = (long long)n_c + slots / PUSH_BLOCK_SLOTS + 1024;
+  {
+    Slab p;
+    p.add(&h->col, (size_t)slots);
+    p.add(&h->items, (size_t)nitems);
+    p.add(&h->split_n, (size_t)nsplit);
+    p.add(&h->xacc, (size_t)nsplit * C);
+    p.add(&h->xpar, (size_t)nsplit * C);
+    p.add(&h->arrive, (size_t)nsplit);
+    p.add(&h->bunits, (size_t)h->bunits_cap);
+    if ((s = p.place(h, &h->slab[1])) != SS_OK) return s;
+  }
+  SS_CUDA(cudaMemsetAsync(h->arrive, 0, sizeof(unsigned) * (size_t)std::max(nsplit, 1LL), st));
+  int4 *fresh = nullptr, *pack_items = nullptr;
+  unsigned long long *ik_a = keys_a, *ik_b = keys_b;
+  int *iv_a = vals_a, *iv_b = vals_b;
+  long long *ihist = hist, *iscan = tmp_scan;
+  {
+    const size_t iblk = (size_t)((nitems + RS_TILE - 1) / RS_TILE);
+    Slab t;
+    t.add(&fresh, (size_t)nitems);
+    if (own_pack) t.add(&pack_items, (size_t)npack);
+    if (nitems > n) {  // (narrow splits: more items than vertices)
+      t.add(&ik_a, (size_t)nitems);
+      t.add(&ik_b, (size_t)nitems);
+      t.add(&iv_a, (size_t)nitems);
+      t.add(&iv_b, (size_t)nitems);
+      t.add(&ihist, 256 * iblk);
+      t.add(&iscan, 256 * iblk / SCAN_TILE + 2);
+    }
+    if ((s = t.place(nullptr, &temps[1])) != SS_OK) return s;
+  }
+
+  // 4. the BFS work items, ordered for the iteration kernels, whose warp w takes items
+  // w, w + W, w + 2W, ... (W = warps in the grid): longest first, and every other group of
+  // W items is reversed ("snake" order) so each warp's total is balanced
+  k_item_fill<<<grid, 256, 0, st>>>(h->cl, n_c, h->split_w, cnt, split, fresh, h->split_n);
+  if (nitems > 0) {
+    const int longest = h->split_w > 0 ? std::min(h->split_w, h->max_degree) : h->max_degree;
+    int* order = nullptr;
+    k_item_keys<<<grid, 256, 0, st>>>(fresh, h->n_items, longest, ik_a, iv_a);
+    if ((s = sort_pairs(ik_a, ik_b, iv_a, iv_b, h->n_items, bit_width((unsigned long long)(longest - 1)), ihist,
+                        iscan, &order, st)) != SS_OK)
+      return s;
+    k_item_snake<<<grid, 256, 0, st>>>(fresh, order, h->n_items, h->num_sms * (SS_PULL_THREADS / 32), h->items);
+  }
+  if (own_pack) k_item_fill<<<grid, 256, 0, st>>>(h->cl, n_c, 256, pack_cnt, nullptr, pack_items, nullptr);
+  SS_CUDA(cudaGetLastError());
 
   // 5. pack
-  SS_TRY(dmalloc(h, (void**)&h->col, sizeof(int) * (size_t)(slots > 0 ? slots : 1)));
-  k_pack<<<grid, 256, 0, st>>>(pack_items, n_pack_items, h->cs, C, h->perm, h->invperm, h->rdeg,
-                               row_ptr, csr_col, h->col);
-  SS_TRYC(cudaGetLastError());
-  SS_TRYC(cudaStreamSynchronize(st));
-  cleanup();
-#undef SS_TRY
-#undef SS_TRYC
+  const int4* pitems = own_pack ? pack_items : h->items;
+  const int np_items = own_pack ? (int)npack : h->n_items;
+  switch (C) {
+    case 8: launch_pack<8>(h, pitems, np_items, row_ptr, csr_col, st); break;
+    case 16: launch_pack<16>(h, pitems, np_items, row_ptr, csr_col, st); break;
+    case 32: launch_pack<32>(h, pitems, np_items, row_ptr, csr_col, st); break;
+    default: launch_pack<64>(h, pitems, np_items, row_ptr, csr_col, st); break;
+  }
+  SS_CUDA(cudaGetLastError());
+  SS_CUDA(cudaStreamSynchronize(st));
   return SS_OK;
 }
 
-static ss_status alloc_state(slimsell_graph* h) {
-  ss_status s;
-  const size_t np = (size_t)h->n_pad;
-  // bitmap words rounded up to whole int4 groups, plus one spare group
-  h->fb_words = (long long)((((np + 31) / 32) + 3) / 4 * 4 + 4);
-  if ((s = dmalloc(h, (void**)&h->claim, sizeof(unsigned long long) * np)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->vis, sizeof(unsigned) * (size_t)h->fb_words)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->act, (size_t)h->n_c)) != SS_OK) return s;
-  for (int b = 0; b < 2; ++b)
-    if ((s = dmalloc(h, (void**)&h->fb[b], sizeof(unsigned) * (size_t)h->fb_words)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->fr, sizeof(float) * np)) != SS_OK) return s;
-  const size_t ns = (size_t)(h->n_split > 0 ? h->n_split : 1);
-  if ((s = dmalloc(h, (void**)&h->xacc, sizeof(float) * ns * h->C)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->xpar, sizeof(int) * ns * h->C)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->arrive, sizeof(unsigned) * ns)) != SS_OK) return s;
-  h->units_cap = (long long)np + h->nnz / 256 + 1024;  // any frontier fits
-  if ((s = dmalloc(h, (void**)&h->units, sizeof(int2) * (size_t)h->units_cap)) != SS_OK) return s;
-  // block units cover PUSH_BLOCK_SLOTS / C columns each: at most one partial unit per chunk
-  h->bunits_cap = (long long)h->n_c + h->slots / PUSH_BLOCK_SLOTS + 1024;
-  if ((s = dmalloc(h, (void**)&h->bunits, sizeof(int2) * (size_t)h->bunits_cap)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->psum, sizeof(float) * np)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->touched, sizeof(unsigned) * (size_t)h->fb_words)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->qcount, sizeof(unsigned long long))) != SS_OK) return s;
+// Host-side state of a handle.
+static ss_status host_state(slimsell_graph* h) {
   h->local_cluster = push_local_cluster_size();
   if (h->local_cluster <= 0) {
     set_error("slimsell_build: no thread-block cluster of the push kernel fits on this device");
     return SS_ERR_CUDA;
   }
-  SS_CUDA(cudaMemset(h->psum, 0, sizeof(float) * np));
-  SS_CUDA(cudaMemset(h->touched, 0, sizeof(unsigned) * (size_t)h->fb_words));
-  if ((s = dmalloc(h, (void**)&h->ctl, sizeof(Ctl))) != SS_OK) return s;
-  h->iter_cap = 1 << 16;
-  if ((s = dmalloc(h, (void**)&h->feats, sizeof(float) * SS_SELECTOR_FEATURES * (size_t)h->iter_cap)) != SS_OK)
-    return s;
-  if ((s = dmalloc(h, (void**)&h->iters, sizeof(ss_iter_stats) * (size_t)h->iter_cap)) != SS_OK) return s;
-  if ((s = dmalloc(h, (void**)&h->lstat, sizeof(unsigned long long) * SS_LSTAT * (size_t)h->iter_cap)) != SS_OK)
-    return s;
-  SS_CUDA(cudaMemset(h->arrive, 0, sizeof(unsigned) * ns));
-  SS_CUDA(cudaMemset(h->fb[0], 0, sizeof(unsigned) * (size_t)h->fb_words));
-  SS_CUDA(cudaMemset(h->fb[1], 0, sizeof(unsigned) * (size_t)h->fb_words));
   SS_CUDA(cudaHostAlloc((void**)&h->h_ctl, sizeof(Ctl), cudaHostAllocDefault));
   SS_CUDA(cudaEventCreate(&h->ev_a));
   SS_CUDA(cudaEventCreate(&h->ev_b));
   SS_CUDA(cudaEventCreate(&h->ev_c));
   SS_CUDA(cudaEventCreate(&h->ev_d));
   SS_CUDA(cudaEventCreateWithFlags(&h->ev_done, cudaEventDisableTiming));
-  SS_CUDA(cudaMemset(h->ctl, 0, sizeof(Ctl)));
   return SS_OK;
 }
 
@@ -588,11 +634,7 @@ void free_handle(slimsell_graph* h) {
   if (!h) return;
   ab_release(h);
   bc_release(h);
-  void* ptrs[] = {h->perm, h->invperm, h->rdeg, h->cl, h->cs, h->col, h->items, h->split_n,
-                  h->claim, h->vis, h->act, h->fb[0], h->fb[1], h->fr, h->xacc, h->xpar,
-                  h->arrive, h->ctl, h->iters, h->units, h->bunits,
-                  h->psum, h->touched, h->qcount, h->lstat, h->mlp, h->feats, h->mF[0],
-                  h->mF[1], h->mV, h->mxacc, h->mroots};
+  void* ptrs[] = {h->slab[0], h->slab[1], h->mlp, h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->h_ctl) cudaFreeHost(h->h_ctl);
@@ -679,8 +721,12 @@ ss_status slimsell_build(const int64_t* d_row_ptr, const int32_t* d_col, int32_t
   h->split_w = split_w;
   h->n_c = (int)n_c;
   h->n_pad = (int)(n_c * C);
-  ss_status s = ss::build_impl(h, (const long long*)d_row_ptr, d_col, st);
-  if (s == SS_OK) s = ss::alloc_state(h);
+  void* temps[2] = {nullptr, nullptr};
+  ss_status s = ss::host_state(h);
+  if (s == SS_OK) s = ss::build_impl(h, (const long long*)d_row_ptr, d_col, temps, st);
+  if (s != SS_OK) cudaStreamSynchronize(st);  // queued work may still use the temporaries
+  for (void* t : temps)
+    if (t) cudaFree(t);
   if (s != SS_OK) {
     ss::free_handle(h);
     return s;

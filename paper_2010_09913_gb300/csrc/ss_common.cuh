@@ -146,6 +146,8 @@ struct slimsell_graph {
   int n_items = 0, n_split = 0, max_degree = 0;
   int n_live = 0;
   int num_sms = 0;
+  // device allocations of the layout and the BFS state: the arrays below lie in them
+  void* slab[2] = {nullptr, nullptr};
   // layout
   int* perm = nullptr;
   int* invperm = nullptr;
