@@ -132,7 +132,8 @@ template <>
 struct BcVal<BC_COUNT> {
   using T = unsigned long long;
   T v = 0ull;
-  __device__ __forceinline__ void add(const T* p) { v += *p; }
+  static __device__ __forceinline__ T zero() { return 0ull; }
+  __device__ __forceinline__ void add(T x) { v += x; }
   __device__ __forceinline__ void store(T* p) const { *p = v; }
   __device__ __forceinline__ unsigned long long merge(T* p) const { return v ? atomicAdd(p, v) + v : 0ull; }
   __device__ __forceinline__ unsigned long long bits() const { return v; }
@@ -141,7 +142,10 @@ template <>
 struct BcVal<BC_FP64> {
   using T = double;
   T v = 0.0;
-  __device__ __forceinline__ void add(const T* p) { v += *p; }
+  static __device__ __forceinline__ T zero() { return 0.0; }
+  __device__ __forceinline__ void add(T x) {
+    if (x != 0.0) v += x;  // (a skipped fp64 add frees the pipe)
+  }
   __device__ __forceinline__ void store(T* p) const { *p = v; }
   __device__ __forceinline__ unsigned long long merge(T* p) const {
     if (v != 0.0) atomicAdd(p, v);
@@ -153,8 +157,8 @@ template <>
 struct BcVal<BC_FIXED> {
   using T = ulonglong2;  // x low, y high
   unsigned long long lo = 0ull, hi = 0ull;
-  __device__ __forceinline__ void add(const T* p) {
-    const T q = *p;
+  static __device__ __forceinline__ T zero() { return make_ulonglong2(0ull, 0ull); }
+  __device__ __forceinline__ void add(T q) {
     lo += q.x;
     hi += q.y + (lo < q.x ? 1ull : 0ull);
   }
@@ -174,6 +178,10 @@ struct BcVal<BC_FIXED> {
 // lf_x = LF[L-1], val = out = sigma.  Backward: lf_v = LF[L], lf_x = LF[L+1],
 // val = t, out = the sums.  A row of one unit is stored, others are merged.
 // ctl->count_bits collects the bits of every finished path count.
+#ifndef SS_BC_GATHER
+#define SS_BC_GATHER 4
+#endif
+constexpr int GATHER = SS_BC_GATHER;
 template <int KIND>
 __global__ void __launch_bounds__(256) k_bcm_gather(Dev d, const unsigned long long* __restrict__ lf_v,
                                                     const unsigned long long* __restrict__ lf_x,
@@ -202,14 +210,27 @@ __global__ void __launch_bounds__(256) k_bcm_gather(Dev d, const unsigned long l
         mx = __ldg(lf_x + x) & mv;
       }
       unsigned any = __ballot_sync(SS_FULL_MASK, mx != 0ull);
-      while (any) {  // the neighbours holding a source of this row, in turn
-        const int q = __ffs(any) - 1;
-        any &= any - 1;
-        const unsigned mlo = __shfl_sync(SS_FULL_MASK, (unsigned)mx, q);
-        const unsigned mhi = __shfl_sync(SS_FULL_MASK, (unsigned)(mx >> 32), q);
-        const typename BcVal<KIND>::T* row = val + (long long)__shfl_sync(SS_FULL_MASK, x, q) * BCM_S + lane;
-        if (mlo >> lane & 1u) a0.add(row);
-        if (mhi >> lane & 1u) a1.add(row + 32);
+      // the neighbours holding a source of this row, GATHER at a time: every load of the group
+      // before the first add, which otherwise waits out a memory latency per neighbour
+      // (64 sources on Kronecker 22: 40.6 ms, 36.7 so)
+      while (any) {
+        typename BcVal<KIND>::T x0[GATHER], x1[GATHER];
+#pragma unroll
+        for (int t = 0; t < GATHER; ++t) {
+          const int q = any ? __ffs(any) - 1 : 0;
+          unsigned mlo = __shfl_sync(SS_FULL_MASK, (unsigned)mx, q);
+          unsigned mhi = __shfl_sync(SS_FULL_MASK, (unsigned)(mx >> 32), q);
+          const typename BcVal<KIND>::T* row = val + (long long)__shfl_sync(SS_FULL_MASK, x, q) * BCM_S + lane;
+          if (!any) mlo = mhi = 0u;
+          any &= any - 1;
+          x0[t] = (mlo >> lane & 1u) ? *row : BcVal<KIND>::zero();
+          x1[t] = (mhi >> lane & 1u) ? row[32] : BcVal<KIND>::zero();
+        }
+#pragma unroll
+        for (int t = 0; t < GATHER; ++t) {
+          a0.add(x0[t]);
+          a1.add(x1[t]);
+        }
       }
     }
     typename BcVal<KIND>::T* const o = out + v * BCM_S + lane;
@@ -266,15 +287,18 @@ __device__ __forceinline__ double fixed_to_double(unsigned long long lo, unsigne
 
 // Backward post of level L: delta = sigma * sum for the row's sources at level L
 // (leaf: the deepest level, whose sums are 0), bc += their sum, and the pair's
-// slot becomes t = sum + 1 / sigma.  A warp takes 32 rows' level words at once.
+// slot becomes t = sum + 1 / sigma.  A warp takes up to 32 rows' level words at once
+// (fewer on a small graph, whose rows then spread over the warps: 13 sources on
+// Kronecker 10 took 717 us with 32 rows a warp always, and take 595).
 __global__ void __launch_bounds__(256) k_bcm_post_fixed(Dev d, const unsigned long long* __restrict__ lf,
                                                         const unsigned long long* __restrict__ sigma,
                                                         ulonglong2* dep, int F, int leaf, double* bc) {
   const int lane = threadIdx.x & 31;
   const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long r0 = wid * 32; r0 < d.n_pad; r0 += nw * 32) {
-    const unsigned long long word = r0 + lane < d.n_pad ? lf[r0 + lane] : 0ull;
+  const int per = (int)min(32LL, (d.n_pad + nw - 1) / nw);
+  for (long long r0 = wid * per; r0 < d.n_pad; r0 += nw * per) {
+    const unsigned long long word = lane < per && r0 + lane < d.n_pad ? lf[r0 + lane] : 0ull;
     unsigned rows = __ballot_sync(SS_FULL_MASK, word != 0ull);
     while (rows) {
       const int q = __ffs(rows) - 1;
