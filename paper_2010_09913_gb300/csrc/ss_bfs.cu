@@ -37,7 +37,7 @@
 
 #include <cooperative_groups.h>
 
-#include "ss_device.cuh"
+#include "ss_pull.cuh"
 
 namespace ss {
 
@@ -53,9 +53,6 @@ namespace ss {
 #endif
 #ifndef SS_PULL_PREFETCH
 #define SS_PULL_PREFETCH 0  // bulk L2 prefetch distance beyond the next step (0: next step only)
-#endif
-#ifndef SS_PULL_LOAD
-#define SS_PULL_LOAD 2  // col loads: 0 evict-first, 1 no-L1 with 256-byte L2 fetches, 2 no-L1
 #endif
 
 constexpr int PULL_THREADS = SS_PULL_THREADS;  // one block per SM
@@ -102,9 +99,6 @@ __device__ __forceinline__ int4 sell_edges(int4 c, int4 v) {
   constexpr int Z = sell_zero_bits<SR>();
   return make_int4(v.x == Z ? -1 : c.x, v.y == Z ? -1 : c.y, v.z == Z ? -1 : c.z, v.w == Z ? -1 : c.w);
 }
-// Stage the bitmap prefix only when the previous iteration read at least this
-// many slots; below it, reading frontier bits from global memory is cheaper.
-constexpr unsigned long long STAGE_MIN_SLOTS = 2ull << 20;
 
 enum { MODE_FULL = 0, MODE_SLIMWORK = 1, MODE_FILTERED = 3 };
 
@@ -118,24 +112,6 @@ enum { MODE_FULL = 0, MODE_SLIMWORK = 1, MODE_FILTERED = 3 };
 constexpr int HUB_VALUE_ROWS = SS_HUB_VALUE_ROWS;
 constexpr unsigned long long HUB_EDGE_SHARE = 16;
 
-__device__ __forceinline__ int4 ld_stream(const int4* p) {
-#if SS_PULL_LOAD == 1
-  int4 v;
-  asm("ld.global.nc.L1::no_allocate.L2::256B.v4.s32 {%0, %1, %2, %3}, [%4];"
-      : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-      : "l"(p));
-  return v;
-#elif SS_PULL_LOAD == 2
-  int4 v;
-  asm("ld.global.nc.L1::no_allocate.v4.s32 {%0, %1, %2, %3}, [%4];"
-      : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-      : "l"(p));
-  return v;
-#else
-  return __ldcs(p);
-#endif
-}
-
 // Ask the TMA unit to pull [p, p + bytes) into L2 ahead of the warp's loads
 // (p 16-byte aligned, bytes a positive multiple of 16).
 __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
@@ -148,27 +124,6 @@ constexpr int PREFETCH_BYTES = SS_PULL_PREFETCH;  // col bytes prefetched ahead 
 __device__ __forceinline__ int4 shfl_int4(int4 v, int src) {
   return make_int4(__shfl_sync(SS_FULL_MASK, v.x, src), __shfl_sync(SS_FULL_MASK, v.y, src),
                    __shfl_sync(SS_FULL_MASK, v.z, src), __shfl_sync(SS_FULL_MASK, v.w, src));
-}
-
-// Shared-memory image of the bitmap: SMEM_GUARD zero words, then the staged
-// prefix.  The padding marker c = -1 has c >> 5 = -1 and lands on the last guard
-// word, so it needs no branch; vertices past the prefix read the global bitmap.
-constexpr int SMEM_GUARD = 4;
-
-__device__ __forceinline__ unsigned frontier_bit(const unsigned* smw, int sbits, const unsigned* gbm,
-                                                 int c) {
-  const int wi = c >> 5;
-  const unsigned w = (c < sbits) ? smw[wi] : __ldg(gbm + wi);
-  return (w >> (c & 31)) & 1u;
-}
-
-// Store the C frontier bits of one chunk (bit l = row l) into the bitmap.
-template <int C>
-__device__ __forceinline__ void store_bits(unsigned* fb, int chunk, unsigned lo, unsigned hi) {
-  if (C == 8) reinterpret_cast<unsigned char*>(fb)[chunk] = (unsigned char)lo;
-  else if (C == 16) reinterpret_cast<unsigned short*>(fb)[chunk] = (unsigned short)lo;
-  else if (C == 32) fb[chunk] = lo;
-  else reinterpret_cast<uint2*>(fb)[chunk] = make_uint2(lo, hi);
 }
 
 // Combine the 4-bit masks of lanes 0 .. C/4-1 into the chunk's bit words (all lanes call).
@@ -337,7 +292,6 @@ __device__ __forceinline__ void gather_step(const Dev& d, const int4* c, const u
     for (int r = 0; r < 4; ++r) sum[r] += x[u][r];
 }
 
-extern __shared__ __align__(16) unsigned ss_smem_bits[];
 
 // The frontier bitmap as a block reads it: words of the staged prefix (sbits bits)
 // from shared memory, the rest from global memory; real semiring on hub levels:
@@ -347,17 +301,6 @@ struct Staged {
   const float* smf;
   int sbits, sf;
 };
-
-// Start copying the first `words` bitmap words (a multiple of 4) behind the guard;
-// returns the shared address of the first one.
-__device__ __forceinline__ unsigned stage_words(const unsigned* gbm, int words) {
-  const unsigned sbase = (unsigned)__cvta_generic_to_shared(ss_smem_bits + SMEM_GUARD);
-  for (int i = threadIdx.x; i < (words >> 2); i += blockDim.x)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sbase + 16u * (unsigned)i),
-                 "l"(reinterpret_cast<const int4*>(gbm) + i)
-                 : "memory");
-  return sbase;
-}
 
 // Stage the prefix of f_{k-1}'s bitmap gbm with asynchronous 16-byte copies (all
 // threads of the block call; the copies run until stage_wait).
@@ -388,11 +331,6 @@ __device__ __forceinline__ Staged stage_frontier(const Dev& d, const unsigned* g
   s.sf = sf;
   return s;
 }
-__device__ __forceinline__ void stage_wait() {
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
-  __syncthreads();
-}
-
 struct __align__(8) ItemCache {
   int chunk, y, z, w;
   long long start;

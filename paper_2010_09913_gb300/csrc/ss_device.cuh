@@ -332,6 +332,8 @@ struct MultiDev {
   unsigned long long* V;
   unsigned long long* xacc;  // [n_split][C][W]
   int* dist;                 // [n][k] in original vertex order, or NULL
+  unsigned long long* planes;  // level bit planes (ss_multi.cu), plane_words words each, or NULL
+  long long plane_words;
   int vec_dist;              // k % 4 == 0 and dist 16-byte aligned: 16-byte group writes
   const int* roots;          // [k]
   int k;

@@ -29,7 +29,7 @@
 #include <cstdint>
 #include <vector>
 
-#include "ss_device.cuh"
+#include "ss_pull.cuh"
 
 namespace ss {
 
@@ -40,6 +40,36 @@ constexpr int MULTI_BATCH = SS_MULTI_BATCH;  // columns per thread in flight
 #ifndef SS_MULTI_BLOCKS_PER_SM
 #define SS_MULTI_BLOCKS_PER_SM 0  // resident blocks per SM (0: as many as fit)
 #endif
+
+// Levels are kept as bit planes until the end of an epoch of MULTI_EPOCH levels: the
+// four planes of word (row, w), one 32-byte sector, hold the bits of the level (within
+// the epoch) at which the row entered each of the 64 sources' frontiers.
+// k_multi_levels then writes the distances in vertex order, a sector gathered per 64
+// entries.  Written at each discovery instead, into
+// an array first filled with -1, they were 16-byte read-modify-writes scattered over
+// the n x k output: 0.8 of the 2.5 ms of 64 sources on Kronecker 22 (0.64 in the
+// pulls, 0.16 the fill).
+constexpr int MULTI_PLANES = 4;
+constexpr int MULTI_EPOCH = (1 << MULTI_PLANES) - 1;
+
+// Out of line, so that the gather loops' register allocation does not depend on it.
+__device__ __noinline__ void keep_levels(unsigned long long* planes, unsigned long long nb, int level) {
+  const int code = (level - 1) % MULTI_EPOCH + 1;
+#pragma unroll
+  for (int i = 0; i < MULTI_PLANES; ++i)
+    if (code >> i & 1) planes[i] |= nb;
+}
+
+// The other way, at each discovery into an output first filled with -1, stays for
+// outputs of fewer than MULTI_PLANES_OUT entries, where k_multi_levels' launch and latency
+// are not made up for (32 sources on Kronecker 16: 376 us; by way of planes 408), and
+// for k of at most half the words' sources, whose planes are mostly empty (48 sources in
+// two words on Kronecker 20: 1115 us and 1188; 2 on Kronecker 21, with parents: 1.34 ms
+// and 1.89).  Also where the planes do not fit in the device's memory.
+constexpr long long MULTI_PLANES_OUT = 16LL << 20;
+static bool multi_planes(const slimsell_graph* h, int k, int W) {
+  return k > 32 * W && (long long)h->n * k >= MULTI_PLANES_OUT;
+}
 
 // Distances of the new sources (bits of nb) of one 64-source word, in 16-byte
 // groups of 4: a group with no earlier discovery (bits of vold) still holds -1
@@ -60,16 +90,75 @@ __device__ __noinline__ void write_levels_vec(int* out, unsigned long long nb, u
   }
 }
 
-// The C summary bits of one chunk (bit l = row l) into the bitmap.
-template <int C>
-__device__ __forceinline__ void store_summary(unsigned* fa, int chunk, unsigned lo, unsigned hi) {
-  if (C == 8) reinterpret_cast<unsigned char*>(fa)[chunk] = (unsigned char)lo;
-  else if (C == 16) reinterpret_cast<unsigned short*>(fa)[chunk] = (unsigned short)lo;
-  else if (C == 32) fa[chunk] = lo;
-  else reinterpret_cast<uint2*>(fa)[chunk] = make_uint2(lo, hi);
+// Distances of an epoch (levels base + 1 .. base + MULTI_EPOCH) from its planes; the
+// first epoch writes every entry (-1 where nothing was found), later ones what they
+// found, and the planes are cleared for the next.  Sixteen lanes write the 64
+// entries of a vertex's word as 16-byte groups where the output allows it.  (In row
+// order the writes of 256 bytes went to scattered places: 347 us on Kronecker 22.)
+__global__ void __launch_bounds__(256) k_multi_levels(MultiDev m, int W, int lgW, int base) {
+  const Dev& d = m.d;
+  const long long words = (long long)d.n << lgW;  // word i: word i & (W - 1) of vertex i >> lgW
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long groups = (long long)gridDim.x * blockDim.x >> 4;  // 16 lanes each
+  const int g = (int)(t & 15);
+  constexpr int U = 4;  // words in flight per group
+  for (long long w0 = t >> 4; w0 < words; w0 += U * groups) {
+    unsigned b[U][MULTI_PLANES], found[U];
+    int row[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const long long word = w0 + u * groups;
+      row[u] = word < words ? __ldg(d.invperm + (word >> lgW)) : d.n_live;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      found[u] = 0;
+#pragma unroll
+      for (int p = 0; p < MULTI_PLANES; ++p) b[u][p] = 0;
+      if (row[u] < d.n_live) {  // (rows without neighbours have no levels)
+        const ulonglong2* q = reinterpret_cast<const ulonglong2*>(
+            m.planes + (((long long)row[u] << lgW) + ((w0 + u * groups) & (W - 1))) * MULTI_PLANES);
+        const ulonglong2 x = __ldg(q), y = __ldg(q + 1);
+        b[u][0] = (unsigned)(x.x >> (4 * g)) & 0xFu;
+        b[u][1] = (unsigned)(x.y >> (4 * g)) & 0xFu;
+        b[u][2] = (unsigned)(y.x >> (4 * g)) & 0xFu;
+        b[u][3] = (unsigned)(y.y >> (4 * g)) & 0xFu;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const long long word = w0 + u * groups;
+      const int s0 = 64 * (int)(word & (W - 1)) + 4 * g;
+#pragma unroll
+      for (int p = 0; p < MULTI_PLANES; ++p) found[u] |= b[u][p];
+      if (word >= words || s0 >= m.k || (base > 0 && !found[u])) continue;
+      int v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        int code = 0;
+#pragma unroll
+        for (int p = 0; p < MULTI_PLANES; ++p) code |= (b[u][p] >> j & 1u) << p;
+        v[j] = code ? base + code : -1;
+      }
+      int* out = m.dist + (word >> lgW) * m.k + s0;
+      if (m.vec_dist && (base == 0 || found[u] == 0xFu)) {
+        __stcs(reinterpret_cast<int4*>(out), make_int4(v[0], v[1], v[2], v[3]));
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (s0 + j < m.k && (base == 0 || v[j] >= 0)) out[j] = v[j];
+      }
+    }
+  }
 }
 
-template <int C, int W, bool SLIMWORK>
+// The sources' own distances, after the first epoch has written every entry.
+__global__ void k_multi_root_levels(MultiDev m) {
+  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < m.k; s += gridDim.x * blockDim.x)
+    m.dist[(long long)m.roots[s] * m.k + s] = 0;
+}
+
+template <int C, int W, bool SLIMWORK, bool PLANES>
 __global__ void __launch_bounds__(C * W) k_multi_pull(MultiDev m, IterLaunch il) {
   constexpr int T = C * W;
   const Dev& d = m.d;
@@ -98,7 +187,7 @@ __global__ void __launch_bounds__(C * W) k_multi_pull(MultiDev m, IterLaunch il)
         if (a >= 2 && item.y == 0) {
           Fn[row * W + w] = 0ull;  // f_k is zero on a finished chunk
           if (tid == 0) {
-            store_summary<C>(FAn, chunk, 0u, 0u);
+            store_bits<C>(FAn, chunk, 0u, 0u);
             d.act[chunk] = (a == 3) ? 2 : 0;
           }
         }
@@ -157,7 +246,9 @@ __global__ void __launch_bounds__(C * W) k_multi_pull(MultiDev m, IterLaunch il)
       nw += (unsigned long long)pc;
       deg += (unsigned long long)pc * (unsigned long long)dv;
       maxdeg = max(maxdeg, (unsigned)dv);
-      if (m.dist) {
+      if constexpr (PLANES) {
+        keep_levels(m.planes + (row * W + w) * MULTI_PLANES, nb, level);
+      } else if (m.dist) {
         int* out = m.dist + (long long)d.perm[row] * m.k + 64 * w;
         if (m.vec_dist) {
           write_levels_vec(out, nb, vold, level);
@@ -175,7 +266,7 @@ __global__ void __launch_bounds__(C * W) k_multi_pull(MultiDev m, IterLaunch il)
     const int left = __syncthreads_or((vold | nb) != ~0ull);
     if (w == 0 && ((s_fa[r >> 5] >> (r & 31)) & 1u)) atomicAdd(&s_rowdeg, (unsigned long long)d.rdeg[row]);
     if (tid == 0) {
-      store_summary<C>(FAn, chunk, s_fa[0], s_fa[1]);
+      store_bits<C>(FAn, chunk, s_fa[0], s_fa[1]);
       d.act[chunk] = left ? 1 : 3;
       act += 1;
     }
@@ -188,6 +279,273 @@ __global__ void __launch_bounds__(C * W) k_multi_pull(MultiDev m, IterLaunch il)
     __threadfence();  // before this block counts itself done
   }
   finish_iteration_block<T>(d, nw, deg, slots, act, maxdeg, il);
+}
+
+// The level pull for one word of sources (k <= 64): as k_multi_pull, with the pull
+// kernel's layout.  One persistent block per SM stages the frontier summary's prefix
+// in shared memory; a warp takes an item (chunks of at most MULTI_SHORT columns go
+// 32 / Q at a time), lane l loading 16-byte quads of col and keeping the words of
+// rows 4 (l mod Q) .. + 3.  A thread per row read the summary and the words from
+// global memory, two dependent gathers a slot, 32 one-warp blocks an SM; here the
+// summary bit is a shared-memory lookup, and a word is gathered (8 bytes, mostly from
+// L2) only where some source has the neighbour in its frontier and some source
+// still misses the row.  64 sources on Kronecker 22: the first two levels 283 and 376 us in
+// k_multi_pull, 185 and 272 here.
+#ifndef SS_MULTI_ONE_THREADS
+#define SS_MULTI_ONE_THREADS 640
+#endif
+#ifndef SS_MULTI_ONE_STEP
+#define SS_MULTI_ONE_STEP 4
+#endif
+constexpr int MULTI_ONE_THREADS = SS_MULTI_ONE_THREADS;
+constexpr int MULTI_ONE_STEP = SS_MULTI_ONE_STEP;  // quads in flight per lane
+constexpr int MULTI_SHORT = 4;
+
+struct OneSum {
+  unsigned long long nw = 0, deg = 0, rowdeg = 0;
+  unsigned quads = 0, act = 0, maxdeg = 0;
+};
+
+// OR the frontier words of U quads into the rows' accumulators: every summary lookup
+// of the step first, then every gather.
+template <int U>
+__device__ __forceinline__ void one_step(const unsigned* sm, int sbits, const unsigned* FAp,
+                                         const unsigned long long* Fp, const int4* c, unsigned live,
+                                         unsigned long long acc[4]) {
+  unsigned hit = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int cc[4] = {c[u].x, c[u].y, c[u].z, c[u].w};
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      hit |= frontier_bit(sm, sbits, FAp, (live >> r & 1u) ? cc[r] : -1) << (4 * u + r);
+  }
+  if (!hit) return;
+  unsigned long long f[U][4];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int cc[4] = {c[u].x, c[u].y, c[u].z, c[u].w};
+#pragma unroll
+    for (int r = 0; r < 4; ++r) f[u][r] = (hit >> (4 * u + r) & 1u) ? __ldg(Fp + cc[r]) : 0ull;
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[r] |= f[u][r];
+}
+
+// New words of four rows (from R0): visited and frontier words, level planes,
+// counters; returns the bits of the rows that gained a source, *left = some row
+// still misses one.
+__device__ __forceinline__ unsigned one_post(const MultiDev& m, long long R0, int level,
+                                             const unsigned long long acc[4], const unsigned long long V[4],
+                                             unsigned long long* Fn, OneSum& sum, bool* left) {
+  const Dev& d = m.d;
+  unsigned long long nb[4];
+  unsigned nib = 0;
+  *left = false;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    nb[r] = acc[r] & ~V[r];
+    if (nb[r]) nib |= 1u << r;
+    if ((V[r] | nb[r]) != ~0ull) *left = true;
+  }
+  ulonglong2* fn = reinterpret_cast<ulonglong2*>(Fn + R0);
+  fn[0] = make_ulonglong2(nb[0], nb[1]);
+  fn[1] = make_ulonglong2(nb[2], nb[3]);
+  if (nib) {
+    ulonglong2* vv = reinterpret_cast<ulonglong2*>(m.V + R0);
+    vv[0] = make_ulonglong2(V[0] | nb[0], V[1] | nb[1]);
+    vv[1] = make_ulonglong2(V[2] | nb[2], V[3] | nb[3]);
+    const int4 dg = *reinterpret_cast<const int4*>(d.rdeg + R0);
+    const int D[4] = {dg.x, dg.y, dg.z, dg.w};
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (nib >> r & 1u) {
+        const int pc = __popcll(nb[r]);
+        sum.nw += (unsigned long long)pc;
+        sum.deg += (unsigned long long)pc * (unsigned long long)D[r];
+        sum.rowdeg += (unsigned long long)D[r];
+        sum.maxdeg = max(sum.maxdeg, (unsigned)D[r]);
+        if (m.planes) keep_levels(m.planes + (R0 + r) * MULTI_PLANES, nb[r], level);
+      }
+  }
+  return nib;
+}
+
+template <int C, bool SLIMWORK>
+__global__ void __launch_bounds__(MULTI_ONE_THREADS, 1) k_multi_one(MultiDev m, IterLaunch il) {
+  constexpr int Q = C / 4;
+  const Dev& d = m.d;
+  Ctl* c = d.ctl;
+  if (c->done) return;
+  const int level = c->k;
+  const int lane = threadIdx.x & 31, lq = lane % Q;
+  const int wid = blockIdx.x * (MULTI_ONE_THREADS / 32) + (threadIdx.x >> 5);
+  const int nw = gridDim.x * (MULTI_ONE_THREADS / 32);
+  const unsigned long long* Fp = m.F[(level - 1) & 1];
+  unsigned long long* Fn = m.F[level & 1];
+  const unsigned* FAp = d.fb[(level - 1) & 1];
+  unsigned* FAn = d.fb[level & 1];
+  if (threadIdx.x < SMEM_GUARD) ss_smem_bits[threadIdx.x] = 0u;
+  // below STAGE_MIN_SLOTS slots in the previous level, reading the bits from global memory is cheaper
+  const int words = level > 1 && c->prev_slots < STAGE_MIN_SLOTS ? 0 : d.smem_words;
+  stage_words(FAp, words);
+  stage_wait();
+  const unsigned* sm = ss_smem_bits + SMEM_GUARD;
+  const int sbits = words * 32;
+  OneSum sum;
+  for (long long b0 = wid; b0 < d.n_items; b0 += 32LL * nw) {
+    const long long my_it = b0 + (long long)lane * nw;
+    int4 my_item = make_int4(0, 0, 0, -1);
+    long long my_start = 0;
+    int a = 0;
+    if (my_it < d.n_items) {
+      my_item = d.items[my_it];
+      a = SLIMWORK ? d.act[my_item.x] : 1;
+      my_start = d.cs[my_item.x] + (long long)my_item.y * C;
+    }
+    unsigned todo = __ballot_sync(SS_FULL_MASK, a == 1);
+    if (SLIMWORK) {  // f_k is zero on a finished chunk: clear what f_{k-2} left, twice
+      unsigned carry = __ballot_sync(SS_FULL_MASK, a >= 2 && my_item.y == 0);
+      while (carry) {
+        const int src = __ffs(carry) - 1;
+        carry &= carry - 1;
+        const int chunk = __shfl_sync(SS_FULL_MASK, my_item.x, src);
+        const int state = __shfl_sync(SS_FULL_MASK, a, src);
+        for (int l = lane; l < C; l += 32) Fn[(long long)chunk * C + l] = 0ull;
+        if (lane == 0) {
+          store_bits<C>(FAn, chunk, 0u, 0u);
+          d.act[chunk] = (state == 3) ? 2 : 0;
+        }
+      }
+    }
+    unsigned shortm = __ballot_sync(SS_FULL_MASK, a == 1 && my_item.w < 0 && my_item.z - my_item.y <= MULTI_SHORT);
+    todo &= ~shortm;
+    while (shortm) {  // short whole chunks, one group of Q lanes each
+      int mysrc = -1;
+#pragma unroll
+      for (int g = 0; g < 32 / Q; ++g) {
+        const int sidx = shortm ? __ffs(shortm) - 1 : -1;
+        if (lane / Q == g) mysrc = sidx;
+        shortm &= shortm - 1;
+      }
+      const bool own = mysrc >= 0;
+      const int sl = own ? mysrc : 0;
+      const int chunk = __shfl_sync(SS_FULL_MASK, my_item.x, sl);
+      const int ncols = __shfl_sync(SS_FULL_MASK, my_item.z, sl) - __shfl_sync(SS_FULL_MASK, my_item.y, sl);
+      const long long start = __shfl_sync(SS_FULL_MASK, my_start, sl);
+      const long long R0 = (long long)chunk * C + 4 * lq;
+      unsigned nib = 0;
+      bool left = false;
+      if (own) {
+        const int4* base = reinterpret_cast<const int4*>(d.col + start) + lq;
+        int4 q[MULTI_SHORT];
+#pragma unroll
+        for (int u = 0; u < MULTI_SHORT; ++u)
+          q[u] = u < ncols ? ld_stream(base + u * Q) : make_int4(-1, -1, -1, -1);
+        const ulonglong2 va = *reinterpret_cast<const ulonglong2*>(m.V + R0);
+        const ulonglong2 vb = *reinterpret_cast<const ulonglong2*>(m.V + R0 + 2);
+        const unsigned long long V[4] = {va.x, va.y, vb.x, vb.y};
+        unsigned live = 0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) live |= (V[r] != ~0ull ? 1u : 0u) << r;
+        unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
+        one_step<MULTI_SHORT>(sm, sbits, FAp, Fp, q, live, acc);
+        nib = one_post(m, R0, level, acc, V, Fn, sum, &left);
+        sum.quads += (unsigned)ncols;
+        if (lq == 0) sum.act += 1;
+      }
+      unsigned lo = (C <= 32 || lq < 8) ? nib << (4 * (lq & 7)) : 0u;
+      unsigned hi = (C > 32 && lq >= 8) ? nib << (4 * (lq - 8)) : 0u;
+      unsigned open = left;
+#pragma unroll
+      for (int o = 1; o < Q; o <<= 1) {
+        lo |= __shfl_xor_sync(SS_FULL_MASK, lo, o);
+        if (C > 32) hi |= __shfl_xor_sync(SS_FULL_MASK, hi, o);
+        open |= __shfl_xor_sync(SS_FULL_MASK, open, o);
+      }
+      if (own && lq == 0) {
+        store_bits<C>(FAn, chunk, lo, hi);
+        d.act[chunk] = open ? 1 : 3;
+      }
+    }
+    while (todo) {  // longer items, one at a time
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int chunk = __shfl_sync(SS_FULL_MASK, my_item.x, src);
+      const int sidx = __shfl_sync(SS_FULL_MASK, my_item.w, src);
+      const int nq = (__shfl_sync(SS_FULL_MASK, my_item.z, src) - __shfl_sync(SS_FULL_MASK, my_item.y, src)) * Q;
+      const int4* base = reinterpret_cast<const int4*>(d.col + __shfl_sync(SS_FULL_MASK, my_start, src));
+      const long long R0 = (long long)chunk * C + 4 * lq;
+      const ulonglong2 va = *reinterpret_cast<const ulonglong2*>(m.V + R0);
+      const ulonglong2 vb = *reinterpret_cast<const ulonglong2*>(m.V + R0 + 2);
+      const unsigned long long V[4] = {va.x, va.y, vb.x, vb.y};
+      unsigned live = 0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) live |= (V[r] != ~0ull ? 1u : 0u) << r;
+      unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
+      for (int q0 = 0; q0 < nq; q0 += 32 * MULTI_ONE_STEP) {
+        int4 q[MULTI_ONE_STEP];
+#pragma unroll
+        for (int u = 0; u < MULTI_ONE_STEP; ++u) {
+          const int at = q0 + lane + 32 * u;
+          q[u] = at < nq ? ld_stream(base + at) : make_int4(-1, -1, -1, -1);
+        }
+        one_step<MULTI_ONE_STEP>(sm, sbits, FAp, Fp, q, live, acc);
+      }
+      if (lane == 0) sum.quads += (unsigned)nq;
+      if (__any_sync(SS_FULL_MASK, (acc[0] | acc[1] | acc[2] | acc[3]) != 0ull)) {  // lanes that share rows
+#pragma unroll
+        for (int off = Q; off < 32; off <<= 1)
+#pragma unroll
+          for (int r = 0; r < 4; ++r) acc[r] |= __shfl_xor_sync(SS_FULL_MASK, acc[r], off);
+      }
+      if (sidx >= 0) {  // SlimChunk: OR the partial rows, the last item to arrive post-processes
+        unsigned long long* xa = m.xacc + (size_t)sidx * C + 4 * lane;
+        if (lane < Q) {
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (acc[r]) atomicOr(xa + r, acc[r]);
+          __threadfence();
+        }
+        __syncwarp();
+        int arrived = 0;
+        if (lane == 0) arrived = (atomicAdd(d.arrive + sidx, 1u) == (unsigned)d.split_n[sidx] - 1u);
+        if (!__shfl_sync(SS_FULL_MASK, arrived, 0)) continue;
+        __threadfence();
+        if (lane < Q) {
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            acc[r] = __ldcg(xa + r);
+            xa[r] = 0ull;
+          }
+        }
+        if (lane == 0) d.arrive[sidx] = 0u;
+      }
+      unsigned nib = 0;
+      bool left = false;
+      if (lane < Q) nib = one_post(m, R0, level, acc, V, Fn, sum, &left);
+      const unsigned lo = __reduce_or_sync(SS_FULL_MASK, lane < 8 ? nib << (4 * lane) : 0u);
+      const unsigned hi = C > 32 ? __reduce_or_sync(SS_FULL_MASK, (lane >= 8 && lane < 16) ? nib << (4 * (lane - 8)) : 0u) : 0u;
+      const bool open = __any_sync(SS_FULL_MASK, left);
+      if (lane == 0) {
+        store_bits<C>(FAn, chunk, lo, hi);
+        d.act[chunk] = open ? 1 : 3;
+        sum.act += 1;
+      }
+    }
+  }
+  // degree sum of the rows that gained a source, each row counted once (the
+  // parents pass picks its direction from it)
+  unsigned long long rd = sum.rowdeg;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) rd += __shfl_down_sync(SS_FULL_MASK, rd, o);
+  if (lane == 0 && rd) {
+    atomicAdd(&c->new_rowdeg, rd);
+    __threadfence();  // before this block counts itself done
+  }
+  finish_iteration_block<MULTI_ONE_THREADS>(d, sum.nw, sum.deg, 4ull * sum.quads, sum.act, sum.maxdeg, il);
 }
 
 __global__ void k_multi_init(MultiDev m, int W) {
@@ -228,7 +586,7 @@ __global__ void k_multi_roots(MultiDev m, int W, int* parent) {
     atomicOr(m.V + r * W + s / 64, bit);
     atomicOr(m.F[0] + r * W + s / 64, bit);
     atomicOr(d.fb[0] + (r >> 5), 1u << (r & 31));
-    if (m.dist) m.dist[(long long)v * m.k + s] = 0;
+    if (m.dist && !m.planes) m.dist[(long long)v * m.k + s] = 0;
     if (parent) parent[(long long)v * m.k + s] = v;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -407,6 +765,30 @@ __global__ void __launch_bounds__(256) k_multi_par_scatter(MultiDev m, int W, in
   }
 }
 
+template <int C>
+static ss_status launch_multi_one(const slimsell_graph* h, const MultiDev& m, bool slimwork,
+                                  const IterLaunch& il, cudaStream_t st) {
+  static std::atomic<unsigned long long> configured{0};
+  if (first_on_device(configured)) {
+    SS_CUDA(cudaFuncSetAttribute(k_multi_one<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM_LIMIT_BYTES));
+    SS_CUDA(cudaFuncSetAttribute(k_multi_one<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM_LIMIT_BYTES));
+  }
+  const size_t smem = (size_t)(m.d.smem_words + SMEM_GUARD) * 4;
+  if (slimwork) k_multi_one<C, true><<<pull_grid(h), MULTI_ONE_THREADS, smem, st>>>(m, il);
+  else k_multi_one<C, false><<<pull_grid(h), MULTI_ONE_THREADS, smem, st>>>(m, il);
+  SS_CUDA(cudaGetLastError());
+  return SS_OK;
+}
+
+// Which kernel takes a one-word level.  Not k_multi_one where the last frontier was dense
+// (below); where distances are written at each discovery; or where a warp of it would get
+// fewer than four items, each of them a serial chain of the chunk's columns (63 sources on
+// G(200001, 8n) in chunks of 64: 464 us; a thread per row 399).
+static bool multi_one(const slimsell_graph* h, const MultiDev& m) {
+  return !h->multi_dense && (m.planes || !m.dist) &&
+         (long long)h->n_items >= 4LL * (MULTI_ONE_THREADS / 32) * h->num_sms;
+}
+
 template <int C, int W>
 static ss_status launch_multi_cw(const slimsell_graph* h, const MultiDev& m, bool slimwork,
                                  const IterLaunch& il, cudaStream_t st) {
@@ -414,17 +796,22 @@ static ss_status launch_multi_cw(const slimsell_graph* h, const MultiDev& m, boo
     set_error("slimsell_bfs_multi: C * ceil(k / 64) must be at least 32");
     return SS_ERR_UNSUPPORTED;
   } else {
-    static int grid[64][2];  // per device (zero: not measured yet)
-    int& g = grid[h->device & 63][slimwork ? 1 : 0];
+    if constexpr (W == 1)
+      if (multi_one(h, m))
+        return launch_multi_one<C>(h, m, slimwork, il, st);
+    using Kernel = void (*)(MultiDev, IterLaunch);
+    static const Kernel kernels[4] = {k_multi_pull<C, W, false, false>, k_multi_pull<C, W, true, false>,
+                                      k_multi_pull<C, W, false, true>, k_multi_pull<C, W, true, true>};
+    static int grid[64][4];  // per device (zero: not measured yet)
+    const int which = (slimwork ? 1 : 0) + (m.planes ? 2 : 0);
+    int& g = grid[h->device & 63][which];
     if (!g) {
       int b = 0;
-      if (slimwork) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_multi_pull<C, W, true>, C * W, 0);
-      else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_multi_pull<C, W, false>, C * W, 0);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernels[which], C * W, 0);
       if (SS_MULTI_BLOCKS_PER_SM > 0) b = std::min(b, SS_MULTI_BLOCKS_PER_SM);
       g = (b > 0 ? b : 1) * h->num_sms;
     }
-    if (slimwork) k_multi_pull<C, W, true><<<g, C * W, 0, st>>>(m, il);
-    else k_multi_pull<C, W, false><<<g, C * W, 0, st>>>(m, il);
+    kernels[which]<<<g, C * W, 0, st>>>(m, il);
     SS_CUDA(cudaGetLastError());
     return SS_OK;
   }
@@ -452,14 +839,25 @@ static ss_status launch_multi(const slimsell_graph* h, const MultiDev& m, int W,
   }
 }
 
+// Which kernel takes the next one-word level (from the counters just read): where the
+// frontier's rows hold over 1 / MULTI_DENSE_SHARE of the edges, most lookups hit, and what
+// counts is how many of the gathered words L1 holds; the block kernel leaves it all of L1,
+// k_multi_one uses it for the bits (64 sources on Kronecker 22, the dense level: 615 us,
+// 1155 in k_multi_one).
+constexpr unsigned long long MULTI_DENSE_SHARE = 8;
+static bool multi_dense(const slimsell_graph* h) {
+  return h->h_ctl->prev_rowdeg * MULTI_DENSE_SHARE > (unsigned long long)h->nnz;
+}
+
 // Multi-source scratch, grown on demand and kept with the handle.
 static ss_status ensure_multi_scratch(slimsell_graph* h, int W) {
   if (h->multi_w >= W) return SS_OK;
-  void* ptrs[] = {h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots};
+  void* ptrs[] = {h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots, h->mplanes};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   h->mF[0] = h->mF[1] = h->mV = h->mxacc = nullptr;
   h->mroots = nullptr;
+  h->mplanes = nullptr;
   h->multi_w = 0;
   const size_t words = (size_t)h->n_pad * W;
   ss_status s;
@@ -470,6 +868,29 @@ static ss_status ensure_multi_scratch(slimsell_graph* h, int W) {
   if ((s = dmalloc(h, (void**)&h->mxacc, sizeof(unsigned long long) * ns)) != SS_OK) return s;
   if ((s = dmalloc(h, (void**)&h->mroots, sizeof(int) * 1024)) != SS_OK) return s;
   h->multi_w = W;
+  return SS_OK;
+}
+
+// Level planes, allocated by the first call that wants distances.
+static ss_status ensure_multi_planes(slimsell_graph* h) {
+  if (h->mplanes) return SS_OK;
+  const ss_status s = dmalloc(h, (void**)&h->mplanes,
+                              sizeof(unsigned long long) * MULTI_PLANES * (size_t)h->n_pad * (size_t)h->multi_w);
+  if (s != SS_OK) cudaGetLastError();  // the caller does without; the launches' checks see nothing
+  return s;
+}
+
+// Write the distances of the epoch that ends with `level` (planes cleared for the next
+// epoch when more levels follow).
+static ss_status write_levels(const slimsell_graph* h, const MultiDev& m, int W, int level, bool more,
+                              cudaStream_t st) {
+  int lgW = 0;
+  while ((1 << lgW) < W) ++lgW;
+  const int base = (level - 1) / MULTI_EPOCH * MULTI_EPOCH;
+  k_multi_levels<<<16 * h->num_sms, 256, 0, st>>>(m, W, lgW, base);
+  if (base == 0) k_multi_root_levels<<<(m.k + 255) / 256, 256, 0, st>>>(m);
+  SS_CUDA(cudaGetLastError());
+  if (more) SS_CUDA(cudaMemsetAsync(m.planes, 0, sizeof(unsigned long long) * MULTI_PLANES * (size_t)m.plane_words, st));
   return SS_OK;
 }
 
@@ -486,6 +907,7 @@ ss_status multi_start(slimsell_graph* h, const int32_t* d_roots, int k, cudaStre
   while (h->C * W < 32) W *= 2;
   if (h->pending) SS_CUDA(cudaEventSynchronize(h->ev_done));
   h->pending = 0;
+  h->multi_dense = false;
   ss_status s = ensure_multi_scratch(h, W);
   if (s != SS_OK) return s;
   SS_CUDA(cudaMemcpyAsync(h->mroots, d_roots, sizeof(int) * (size_t)k, cudaMemcpyDeviceToDevice, st));
@@ -497,6 +919,8 @@ ss_status multi_start(slimsell_graph* h, const int32_t* d_roots, int k, cudaStre
   m->xacc = h->mxacc;
   m->dist = nullptr;
   m->vec_dist = 0;
+  m->planes = nullptr;
+  m->plane_words = 0;
   m->roots = h->mroots;
   m->k = k;
   k_multi_init<<<8 * h->num_sms, 256, 0, st>>>(*m, W);
@@ -519,6 +943,7 @@ ss_status multi_level(slimsell_graph* h, const MultiDev& m, int W, cudaStream_t 
     return SS_ERR_CUDA;
   }
   *done = h->h_ctl->done != 0;
+  h->multi_dense = multi_dense(h);
   return SS_OK;
 }
 
@@ -572,6 +997,12 @@ extern "C" ss_status slimsell_bfs_multi_parents(slimsell_handle h, const int32_t
   m.V = h->mV;
   m.xacc = h->mxacc;
   m.dist = d_dist;
+  m.planes = nullptr;
+  m.plane_words = (long long)h->n_pad * W;
+  if (d_dist && multi_planes(h, k, W) && ensure_multi_planes(h) == SS_OK) {
+    m.planes = h->mplanes;
+    SS_CUDA(cudaMemsetAsync(m.planes, 0, sizeof(unsigned long long) * MULTI_PLANES * (size_t)m.plane_words, st));
+  }
   m.vec_dist = (k % 4 == 0) && ((reinterpret_cast<uintptr_t>(d_dist) & 15u) == 0);
   m.roots = h->mroots;
   m.k = k;
@@ -579,7 +1010,7 @@ extern "C" ss_status slimsell_bfs_multi_parents(slimsell_handle h, const int32_t
   h->iter_ns.clear();
   double iter_ms = 0.0;
   if (prof) SS_CUDA(cudaEventRecord(h->ev_c, st));
-  if (d_dist) SS_CUDA(cudaMemsetAsync(d_dist, 0xff, sizeof(int) * (size_t)h->n * (size_t)k, st));
+  if (d_dist && !m.planes) SS_CUDA(cudaMemsetAsync(d_dist, 0xff, sizeof(int) * (size_t)h->n * (size_t)k, st));
   if (d_parent) SS_CUDA(cudaMemsetAsync(d_parent, 0xff, sizeof(int) * (size_t)h->n * (size_t)k, st));
   k_multi_init<<<8 * h->num_sms, 256, 0, st>>>(m, W);
   k_multi_roots<<<(k + 255) / 256, 256, 0, st>>>(m, W, d_parent);
@@ -591,6 +1022,7 @@ extern "C" ss_status slimsell_bfs_multi_parents(slimsell_handle h, const int32_t
     SS_CUDA(cudaStreamSynchronize(st));
   }
   const IterLaunch il{policy, 0, 0};
+  h->multi_dense = false;
   const long long max_iter = (long long)h->n + 2;
   for (long long it = 0;; ++it) {
     if (it > max_iter) {
@@ -626,7 +1058,11 @@ extern "C" ss_status slimsell_bfs_multi_parents(slimsell_handle h, const int32_t
       iter_ms += ms;
       h->iter_ns.push_back((int)(ms * 1.0e6f));
     }
-    if (h->h_ctl->done) break;
+    const bool done = h->h_ctl->done != 0;
+    h->multi_dense = multi_dense(h);
+    if (m.planes && (done || (it + 1) % MULTI_EPOCH == 0))
+      if ((s = write_levels(h, m, W, (int)(it + 1), !done, st)) != SS_OK) return s;
+    if (done) break;
   }
   if (prof) SS_CUDA(cudaEventRecord(h->ev_d, st));
   SS_CUDA(cudaMemcpyAsync(h->h_ctl, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
