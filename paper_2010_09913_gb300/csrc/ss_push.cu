@@ -300,19 +300,47 @@ struct LocalLay {
   }
 };
 
-// Call f(index, valid) for this CTA's entries of parity p: the threads of a warp together,
-// segment after segment; invalid past a segment's end.
+// Call f(index, valid) for this CTA's entries of parity p: the threads of a warp together;
+// invalid past the last entry.
 // (made: how many rank 0 has made, where it alone did).
 template <class F>
 __device__ __forceinline__ void local_entries(const LocalSmem& S, const LocalLay& lay, int made, int p, int rank,
                                               int lg, F f) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int NW = LOCAL_THREADS / 32;
   const int nseg = lay.from_one ? 1 : 1 << lg;
-  const int wps = (LOCAL_THREADS / 32) / nseg;  // warps of a segment
-  const int seg = warp / wps;
-  const int n = lay.count(seg, lay.from_one ? made : S.all[p][seg].nent, rank, lg);
-  // entry after entry goes to another warp, so that a few long ones do not queue in one
-  for (int i0 = warp % wps; i0 < n; i0 += wps * 32) f(seg * lay.cap(lg) + i0 + lane * wps, i0 + lane * wps < n);
+  const int nent = lane < nseg ? lay.count(lane, lay.from_one ? made : S.all[p][lane].nent, rank, lg) : 0;
+  const int total = (int)__reduce_add_sync(SS_FULL_MASK, (unsigned)nent);
+  const int most = (int)__reduce_max_sync(SS_FULL_MASK, (unsigned)nent);
+  // Each segment has warps of its own, and entry after entry goes to another of them, so that a
+  // few long ones do not queue in one.  Uneven segments are one list for all the warps instead:
+  // in a level made by a few CTAs alone (three units of a hub) as few warps had all the work
+  // (282 rows of 92,934 edges on Kronecker 14: 81 us, 22 so).  The search for an entry's
+  // segment made a lattice's small levels 8 % longer where it was always done.
+  const bool list = most >= 8 && most * nseg > 2 * total;
+  int incl = nent;
+  if (list) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(SS_FULL_MASK, incl, o);
+      if (lane >= o) incl += t;
+    }
+  }
+  const int before = incl - nent;
+  const int wps = list ? NW : NW / nseg;  // warps of a segment
+  const int own = warp / wps;
+  const int n = list ? total : __shfl_sync(SS_FULL_MASK, nent, own);
+  for (int i0 = warp % wps; i0 < n; i0 += wps * 32) {
+    const int i = i0 + lane * wps;
+    int seg = own, at = i;
+    if (list) {
+      seg = 0;  // segments that end at or before entry i
+      for (int step = nseg >> 1; step; step >>= 1)
+        if (__shfl_sync(SS_FULL_MASK, incl, seg + step - 1) <= i) seg += step;
+      at -= __shfl_sync(SS_FULL_MASK, before, seg);
+    }
+    f(seg * lay.cap(lg) + at, i < n);
+  }
 }
 
 // Selector features of the iterations after levels k0 .. k1 run in this launch
@@ -343,6 +371,7 @@ struct LocalPlace {
   LocalPub* mine;
   int k, p, rank, lg;
   LocalLay lay;
+  bool late;   // a level of more edges than the cluster's threads take in one round
   bool first;  // the launch's own entries: numbered through one counter for all CTAs, as if rank 0 made them
   // a row without room: the level is handed back, as a bitmap, where its bit is set at once
   __device__ __forceinline__ void drop(int x) {
@@ -502,7 +531,13 @@ __device__ __forceinline__ void local_claim(const Dev& d, LocalPlace<C>& place, 
       if ((unsigned)(old[q] >> 32) <= (unsigned)(key >> 32)) atomicAdd(d.psum + v[q], fu);
   }
   // the neighbours' row data, in flight with the claims (of every neighbour: waiting to
-  // learn which are new would add a memory latency to the level)
+  // learn which are new would add a memory latency to the level); in a level of several
+  // rounds, bound by its gathers and not by their latency, of the new ones alone
+  if (place.late) {
+#pragma unroll
+    for (int q = 0; q < LOCAL_EDGES; ++q)
+      if (old[q] != 0ull) v[q] = -1;
+  }
   int dv[LOCAL_EDGES], og2[LOCAL_EDGES];
   long long bx[LOCAL_EDGES];
 #pragma unroll
@@ -570,7 +605,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
   // cost each launch 3 us more); the first frontier's bits are cleared, and those of level k-2
   if (handback) {
     const int p1 = (k - 1) & 1;
-    LocalPlace<C> place{d, S, cl, &S.mine[0], k, p1, rank, lg, cur, true};
+    LocalPlace<C> place{d, S, cl, &S.mine[0], k, p1, rank, lg, cur, false, true};
     const long long words = ((long long)d.n_pad + 31) / 32;
     unsigned *fbm = d.fb[p1], *fbk = d.fb[k & 1];
     constexpr int AHEAD = 8;  // words in flight per thread
@@ -644,7 +679,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
       S.mine[(k + 1) % 3] = LocalPub{0, 0, 0u, 0, 0u, 0u};
       S.placed[p1] = 0u;
     }
-    LocalPlace<C> place{d, S, cl, mine, k, p0, rank, lg, nxt, false};
+    LocalPlace<C> place{d, S, cl, mine, k, p0, rank, lg, nxt, E > 4ull * LOCAL_THREADS * G, false};
     LocalSum sum;
     local_entries(S, cur, made, p1, rank, lg, [&](int at, bool valid) {
       LocalEntry en{0ull, 0, 0};
