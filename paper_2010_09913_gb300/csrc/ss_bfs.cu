@@ -569,6 +569,77 @@ __device__ __forceinline__ void pull_items(const Dev& d, int k, bool full, const
   }
 }
 
+// The first level, whose frontier is the root alone: x_1 is non-zero exactly in the
+// rows of the slots that hold the root, so the pass streams the whole column array
+// against one row number, eight 16-byte quads in flight per lane, with no item walk, no
+// bitmap and no lookup, and is bound by HBM.  A slot that holds the root (one per
+// neighbour) finds its chunk by bisection; only that row's chunk is SlimWork-skipped
+// (and its slots not counted) when its rows are all visited.  Not for the real semiring,
+// where a repeated edge counts twice.  From ROOT_MIN_SLOTS slots on: below, the level
+// is launch and latency either way.  Level 1 of Kronecker 22: 128 us to 96 (533 MB), of
+// Kronecker 24 520 to 332 (2.2 GB); a whole run of Kronecker 18 178 to 160.
+#ifndef SS_ROOT_MIN_SLOTS
+#define SS_ROOT_MIN_SLOTS (4LL << 20)
+#endif
+constexpr long long ROOT_MIN_SLOTS = SS_ROOT_MIN_SLOTS;
+template <int C>
+__device__ __forceinline__ void pull_root(const Dev& d, bool full, Counters& cnt) {
+  constexpr int U = 8;
+  const int root_row = d.ctl->root_row;
+  const int root = __ldg(d.perm + root_row);
+  const int lane = threadIdx.x & 31;
+  const long long nq = d.total_slots >> 2;
+  const long long warps = (long long)gridDim.x * (PULL_THREADS / 32);
+  const int4* col = reinterpret_cast<const int4*>(d.col);
+  for (long long q0 = ((long long)blockIdx.x * (PULL_THREADS / 32) + (threadIdx.x >> 5)) * (32 * U); q0 < nq;
+       q0 += warps * (32 * U)) {
+    int4 c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const long long q = q0 + lane + 32 * u;
+      c[u] = q < nq ? ld_stream(col + q) : make_int4(-1, -1, -1, -1);
+    }
+    bool any = false;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      any = any || c[u].x == root_row || c[u].y == root_row || c[u].z == root_row || c[u].w == root_row;
+    if (!any) continue;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int cc[4] = {c[u].x, c[u].y, c[u].z, c[u].w};
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (cc[r] != root_row) continue;
+        const long long slot = 4 * (q0 + lane + 32 * u) + r;
+        int lo = 0, hi = d.n_c - 1;  // the last chunk that starts at or before the slot
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (__ldg(d.cs + mid) <= slot) lo = mid;
+          else hi = mid - 1;
+        }
+        const long long row = (long long)lo * C + (slot - __ldg(d.cs + lo)) % C;
+        const unsigned bit = 1u << (row & 31);
+        if (atomicOr(d.vis + (row >> 5), bit) & bit) continue;  // the root, or a repeated edge
+        const int dg = __ldg(d.rdeg + row);
+        d.claim[row] = claim_word(1, root);
+        atomicOr(d.fb[1] + (row >> 5), bit);
+        cnt.nw += 1;
+        cnt.deg += (unsigned long long)dg;
+        cnt.maxdeg = max(cnt.maxdeg, (unsigned)dg);
+      }
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    cnt.slots = (unsigned long long)d.total_slots;
+    cnt.act = (unsigned long long)d.n_busy;
+    const int rc = root_row / C;  // its chunk is finished when the root is its only real row
+    if (!full && d.cl[rc] > 0 && d.n - rc * C == 1) {
+      cnt.slots -= (unsigned long long)d.cl[rc] * C;
+      cnt.act -= 1;
+    }
+  }
+}
+
 // One frontier expansion x_k = A (x)_S f_{k-1} with fused post-processing.
 template <int SR, int C, int MODE, int FMT>
 __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
@@ -576,10 +647,16 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
                                                           int use_cond) {
   if (d.ctl->done) return;
   const int k = d.ctl->k;
+  Counters cnt;
+  if (FMT == SS_FORMAT_SLIMSELL && SR != SS_REAL && k == 1 && d.total_slots >= ROOT_MIN_SLOTS) {
+    pull_root<C>(d, MODE == MODE_FULL, cnt);
+    finish_iteration_block<PULL_THREADS>(d, cnt.nw, cnt.deg, cnt.slots, cnt.act, cnt.maxdeg,
+                                         IterLaunch{variant, cond, use_cond});
+    return;
+  }
   const unsigned* gbm = d.fb[(k - 1) & 1];
   const Staged sg = stage_frontier<SR>(d, gbm);
   stage_wait();
-  Counters cnt;
   pull_items<SR, C, FMT, false>(d, k, MODE == MODE_FULL, gbm, sg,
                                 (int)(blockIdx.x * (PULL_THREADS / 32) + (threadIdx.x >> 5)),
                                 (int)(gridDim.x * (PULL_THREADS / 32)), cnt);

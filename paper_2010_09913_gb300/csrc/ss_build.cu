@@ -290,7 +290,9 @@ __global__ void k_perm_tables(const int* sorted_vals, const int* deg, int n, int
 }
 
 // cl[i] = longest row of chunk i; cs[i] = C * cl[i] (scanned afterwards); cs[n_c] = 0
-__global__ void k_chunk_len(const int* rdeg, int n_c, int C, int* cl, long long* cs) {
+// *busy = chunks with at least one column.
+__global__ void k_chunk_len(const int* rdeg, int n_c, int C, int* cl, long long* cs, int* busy) {
+  int mine = 0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i <= n_c;
        i += (long long)gridDim.x * blockDim.x) {
     if (i == n_c) {
@@ -301,7 +303,10 @@ __global__ void k_chunk_len(const int* rdeg, int n_c, int C, int* cl, long long*
     for (int l = 0; l < C; ++l) m = max(m, rdeg[i * C + l]);
     cl[i] = m;
     cs[i] = (long long)C * m;
+    mine += m > 0;
   }
+  mine = __reduce_add_sync(SS_FULL_MASK, mine);
+  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(busy, mine);
 }
 
 // items per chunk for a given width W (0 = one item per chunk); split flags
@@ -457,7 +462,7 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
   {
     Slab t;
     t.add(&deg, (size_t)n);
-    t.add(&flags, 2);  // largest degree, live rows
+    t.add(&flags, 3);  // largest degree, live rows, busy chunks
     t.add(&vals_a, (size_t)n);
     t.add(&vals_b, (size_t)n);
     t.add(&keys_a, (size_t)n);
@@ -502,7 +507,7 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
   SS_CUDA(cudaMemsetAsync(h->ctl, 0, sizeof(Ctl), st));
 
   // 1. degrees and sort keys
-  SS_CUDA(cudaMemsetAsync(flags, 0, 2 * sizeof(int), st));
+  SS_CUDA(cudaMemsetAsync(flags, 0, 3 * sizeof(int), st));
   k_degrees<<<grid, 256, 0, st>>>(row_ptr, n, deg, flags);
   SS_CUDA(cudaMemcpyAsync(&h->max_degree, flags, sizeof(int), cudaMemcpyDeviceToHost, st));
   SS_CUDA(cudaStreamSynchronize(st));
@@ -523,7 +528,7 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
 
   // 3. perm / invperm / row degrees, chunk lengths and starts, work items per chunk
   k_perm_tables<<<grid, 256, 0, st>>>(sorted, deg, n, n_pad, h->perm, h->invperm, h->rdeg, flags + 1);
-  k_chunk_len<<<grid, 256, 0, st>>>(h->rdeg, n_c, C, h->cl, h->cs);
+  k_chunk_len<<<grid, 256, 0, st>>>(h->rdeg, n_c, C, h->cl, h->cs, flags + 2);
   k_item_count<<<grid, 256, 0, st>>>(h->cl, n_c, h->split_w, cnt, split);
   if (own_pack) k_item_count<<<grid, 256, 0, st>>>(h->cl, n_c, 256, pack_cnt, nullptr);
   SS_CUDA(cudaGetLastError());
@@ -533,7 +538,8 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
   if (own_pack && (s = excl_scan(pack_cnt, n_c + 1, tmp_scan, st)) != SS_OK) return s;
   long long slots = 0, nitems = 0, nsplit = 0, npack = 0;
   SS_CUDA(cudaMemcpyAsync(&slots, h->cs + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
-  SS_CUDA(cudaMemcpyAsync(&h->n_live, flags + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
+  int rows_chunks[2] = {0, 0};
+  SS_CUDA(cudaMemcpyAsync(rows_chunks, flags + 1, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
   SS_CUDA(cudaMemcpyAsync(&nitems, cnt + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
   SS_CUDA(cudaMemcpyAsync(&nsplit, split + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
   if (own_pack) SS_CUDA(cudaMemcpyAsync(&npack, pack_cnt + n_c, sizeof(long long), cudaMemcpyDeviceToHost, st));
@@ -542,6 +548,8 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
     set_error("too many work items (%lld)", std::max(nitems, npack));
     return SS_ERR_UNSUPPORTED;
   }
+  h->n_live = rows_chunks[0];
+  h->n_busy = rows_chunks[1];
   h->slots = slots;
   h->n_items = (int)nitems;
   h->n_split = (int)nsplit;
@@ -660,7 +668,7 @@ ss::Dev slimsell_graph::dev() const {
   d.n = n; d.C = C; d.n_c = n_c; d.n_pad = n_pad; d.n_items = n_items; d.n_split = n_split;
   d.perm = perm; d.invperm = invperm; d.rdeg = rdeg; d.cl = cl; d.cs = cs; d.col = col;
   d.items = items; d.split_n = split_n; d.claim = claim; d.vis = vis; d.act = act;
-  d.n_live = n_live; d.max_degree = max_degree;
+  d.n_live = n_live; d.max_degree = max_degree; d.n_busy = n_busy;
   d.fb[0] = fb[0]; d.fb[1] = fb[1]; d.fb_words = fb_words;
   // staged prefix: whole int4 groups, never past the allocated bitmap
   long long need = ((((long long)n_pad + 31) / 32) + 3) / 4 * 4;

@@ -81,6 +81,7 @@ struct Ctl {
 struct Dev {
   int n, C, n_c, n_pad, n_items, n_split;
   int max_degree;
+  int n_busy;           // chunks with at least one column
   int n_live;           // rows from n_live on have no neighbours: a run reaches none but its root
   const int* perm;      // [n_pad] vertex at row position (-1 for padding rows)
   const int* invperm;   // [n] row position of vertex
@@ -144,7 +145,7 @@ struct slimsell_graph {
   int n = 0, C = 0, sigma = 0, split_w = 0, n_c = 0, n_pad = 0;
   long long nnz = 0, slots = 0;
   int n_items = 0, n_split = 0, max_degree = 0;
-  int n_live = 0;
+  int n_live = 0, n_busy = 0;
   int num_sms = 0;
   // device allocations of the layout and the BFS state: the arrays below lie in them
   void* slab[2] = {nullptr, nullptr};
