@@ -623,6 +623,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
         bits[j] = w < words ? __ldcg(fbm + w) : 0u;
         if (w < words) fbk[w] = 0u;
       }
+      __syncwarp();  // every lane has read the words that it shares with others before one clears them
 #pragma unroll
       for (int j = 0; j < AHEAD; ++j) {
         const long long w = (t0 + j * threads) >> sp;
