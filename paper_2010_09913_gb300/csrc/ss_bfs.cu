@@ -863,6 +863,7 @@ __global__ void __launch_bounds__(FILTERED_THREADS, 1) k_pull_filtered(Dev d, in
         }
       }
     }
+    __syncwarp();  // a left chunk's bits, stored by its group's first lane, are stored again by lane 0
     while (todo) {
       const int src = __ffs(todo) - 1;
       todo &= todo - 1;
