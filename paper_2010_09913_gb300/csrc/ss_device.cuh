@@ -244,8 +244,9 @@ __device__ __forceinline__ void store_features(const Dev& d, int k, const float*
   for (int i = 0; i < SS_SELECTOR_FEATURES; ++i) d.feats[(size_t)k * SS_SELECTOR_FEATURES + i] = f[i];
 }
 
-// Control block of a new single-source run from root row r (one thread).
-__device__ __forceinline__ void init_ctl(const Dev& d, Ctl* c, int r) {
+// Control block of a new single-source run from root row r (one thread): every field,
+// since k_small's block starts as uninitialised shared memory.
+__host__ __device__ __forceinline__ void init_ctl(const Dev& d, Ctl* c, int r) {
   c->root_row = r;
   c->k = 1; c->done = 0; c->error = 0; c->variant = -1;
   c->new_count = 0; c->new_deg = 0; c->slots = 0; c->active = 0;
@@ -258,6 +259,7 @@ __device__ __forceinline__ void init_ctl(const Dev& d, Ctl* c, int r) {
   for (int v = 0; v < N_VARIANTS; ++v) c->variant_count[v] = 0;
   c->loop_guard = 0;
   c->psum_dirty = 0;
+  c->new_rowdeg = 0; c->prev_rowdeg = 0; c->count_bits = 0;
   ss_iter_stats s;
   s.frontier = 1; s.frontier_degree = d.rdeg[r]; s.slots = 0; s.active_chunks = 0;
   s.variant = -1; s.kernel_ns = 0;
