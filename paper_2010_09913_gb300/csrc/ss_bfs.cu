@@ -1106,11 +1106,6 @@ __global__ void k_init(Dev d) {
 
 __global__ void k_init_root(Dev d, int root) { init_root_state(d, root); }
 
-// Lower half of a claim word: parent + 1.
-__device__ __forceinline__ int* parent_half(const Dev& d, long long r) {
-  return reinterpret_cast<int*>(d.claim) + 2 * r;
-}
-
 // DP transformation as a separate pass (Section II-C): the parent of a row at
 // level L >= 1 is its largest-id neighbour at level L-1.  Neighbours are stored
 // in descending original id, so each lane's first hit in its column sequence is

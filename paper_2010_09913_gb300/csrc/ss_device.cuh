@@ -15,13 +15,18 @@ enum { VAR_FULL = SS_V_FULL, VAR_SLIMWORK = SS_V_SLIMWORK, VAR_PUSH = SS_V_PUSH,
 // so one atomicMax visits a row, keeps its canonical parent and leaves rows of
 // earlier levels alone.  0 is an unvisited row.  Level and parent share a word
 // because every reader wants both: the output gathers one 8-byte word per vertex.
+__host__ __device__ __forceinline__ unsigned claim_upper(int level) { return (unsigned)(0x7fffffff - level); }
 __host__ __device__ __forceinline__ unsigned long long claim_word(int level, int id) {
-  return ((unsigned long long)(unsigned)(0x7fffffff - level) << 32) | (unsigned)(id + 1);
+  return ((unsigned long long)claim_upper(level) << 32) | (unsigned)(id + 1);
 }
 __device__ __forceinline__ int claim_level(unsigned long long w) {  // (w != 0)
   return 0x7fffffff - (int)(w >> 32);
 }
 __device__ __forceinline__ int claim_parent(unsigned long long w) { return (int)(unsigned)w - 1; }
+// Lower half of row r's claim word: parent + 1.
+__device__ __forceinline__ int* parent_half(const Dev& d, long long r) {
+  return reinterpret_cast<int*>(d.claim) + 2 * r;
+}
 
 // The bits of one chunk's rows (bit l = row l of the chunk) in a row bitmap.
 // SHARED: read past L1 (another SM may have written it since this kernel began).
