@@ -70,7 +70,7 @@ typedef enum {
 } ss_policy;
 
 /* Executed-variant id (ss_iter_stats.variant, not a policy) of the cluster
- * push: one thread-block cluster (16 CTAs of 1024 threads, else 8) runs
+ * push: one thread-block cluster (16 CTAs of 512 threads, else 8) runs
  * consecutive small levels in one launch with the frontier kept as vertex
  * lists in shared memory; push and the adaptive policies use it for frontiers
  * of at most 4096 vertices and 8192 edges per CTA (high-diameter graphs). */

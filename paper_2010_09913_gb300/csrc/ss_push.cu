@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_post(Dev d, IterLaunch il
 }
 
 // ---------------------------------------------------------------------------
-// Cluster push for small frontiers: one thread-block cluster (16 CTAs of 1024
+// Cluster push for small frontiers: one thread-block cluster (16 CTAs of 512
 // threads where the device can place it, else 8) runs level after level inside
 // one launch, with no kernel boundary and no bitmap walk per level.
 //
@@ -239,9 +239,16 @@ __global__ void __launch_bounds__(PUSH_THREADS) k_push_post(Dev d, IterLaunch il
 // barrier with its release of the level's global writes is the longest.  While levels
 // have up to SOLO_UP edges they are therefore run by rank 0 alone, entries in its own shared
 // memory, block barriers only, while the others wait at a cluster barrier until it
-// spreads the entries again or ends the launch.  Lattice 4096^2 (6,154 levels): 4.9 us a
-// level, 6.9 with two cluster barriers a level and the row data fetched after the
-// claims; 96^2, mostly rank 0 alone, about 2.4 us.
+// spreads the entries again or ends the launch.  Lattice 4096^2 (6,154 levels): 4.5 us a
+// level, 7.2 with two cluster barriers a level; 96^2, mostly rank 0 alone, about 2.4 us.
+//
+// A level of more edges than the cluster has threads is bound not by that chain but by its
+// scattered accesses, on graphs past L2 to DRAM.  Such a level (`late`) therefore reads row data
+// of new rows only, after the claims, and asks for no columns ahead of the next level.  Lattice
+// 8192^2 (14,900 levels), us a level of 8 .. 16 K edges / 16 .. 24 K / 24 .. 32 K, and a run:
+// 7.1 / 13.3 / 19.8, 167 ms, with every neighbour's row data up to 32 K edges;
+// 5.8 / 10.0 / 15.2, 134 ms, with new rows' alone; 5.8 / 9.4 / 13.4, 124 ms, so (7.8 / 10.3 / 12.2,
+// 139 ms, by the two-barrier form).  4096^2: 31.0 ms, 28.2 so; from 4 K edges on 28.1.
 //
 // Every active CTA takes the same exits (counters reach every CTA through
 // distributed shared memory); rank 0 keeps the control block in shared memory and
@@ -324,9 +331,11 @@ __device__ __forceinline__ void local_entries(const LocalSmem& S, const LocalLay
   // Each segment has warps of its own, and entry after entry goes to another of them, so that a
   // few long ones do not queue in one.  Uneven segments are one list for all the warps instead:
   // in a level made by a few CTAs alone (three units of a hub) as few warps had all the work
-  // (282 rows of 92,934 edges on Kronecker 14: 81 us, 22 so).  The search for an entry's
-  // segment made a lattice's small levels 8 % longer where it was always done.
-  const bool list = most >= 8 && most * nseg > 2 * total;
+  // (282 rows of 92,934 edges on Kronecker 14: 81 us, 22 so), and so are segments of more
+  // entries than their warps' lanes, a few of which would be a second round (levels of 24 .. 32 K
+  // edges on lattice 8192^2: 14.0 us, 13.4 so).  The search for an entry's segment made a
+  // lattice's small levels 8 % longer where it was always done.
+  const bool list = most >= 8 && (most * nseg > 2 * total || most > 32 * (NW / nseg));
   int incl = nent;
   if (list) {
 #pragma unroll
@@ -380,7 +389,7 @@ struct LocalPlace {
   LocalPub* mine;
   int k, p, rank, lg;
   LocalLay lay;
-  bool late;   // a level of more edges than the cluster's threads take in one round
+  bool late;   // a level of more edges than the cluster has threads
   bool first;  // the launch's own entries: numbered through one counter for all CTAs, as if rank 0 made them
   // a row without room: the level is handed back, as a bitmap, where its bit is set at once
   __device__ __forceinline__ void drop(int x) {
@@ -444,7 +453,7 @@ struct LocalPlace {
         *reinterpret_cast<int4*>(&T->ent[p][seg + slot]) = *reinterpret_cast<const int4*>(&en);
 #pragma unroll
         for (int j = 0; j < LOCAL_EDGES; ++j)  // its columns, for the next level
-          if (j < deg[q]) asm volatile("prefetch.global.L2 [%0];" ::"l"(d.col + bx[q] + (long long)j * C));
+          if (j < deg[q] && !late) asm volatile("prefetch.global.L2 [%0];" ::"l"(d.col + bx[q] + (long long)j * C));
       }
       return;
     }
@@ -540,8 +549,8 @@ __device__ __forceinline__ void local_claim(const Dev& d, LocalPlace<C>& place, 
       if ((unsigned)(old[q] >> 32) <= (unsigned)(key >> 32)) atomicAdd(d.psum + v[q], fu);
   }
   // the neighbours' row data, in flight with the claims (of every neighbour: waiting to
-  // learn which are new would add a memory latency to the level); in a level of several
-  // rounds, bound by its gathers and not by their latency, of the new ones alone
+  // learn which are new would add a memory latency to the level); in a large level, bound
+  // by its accesses and not by their latency, of the new ones alone
   if (place.late) {
 #pragma unroll
     for (int q = 0; q < LOCAL_EDGES; ++q)
@@ -689,7 +698,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
       S.mine[(k + 1) % 3] = LocalPub{0, 0, 0u, 0, 0u, 0u};
       S.placed[p1] = 0u;
     }
-    LocalPlace<C> place{d, S, cl, mine, k, p0, rank, lg, nxt, E > 4ull * LOCAL_THREADS * G, false};
+    LocalPlace<C> place{d, S, cl, mine, k, p0, rank, lg, nxt, E > (unsigned long long)LOCAL_THREADS * G, false};
     LocalSum sum;
     local_entries(S, cur, made, p1, rank, lg, [&](int at, bool valid) {
       LocalEntry en{0ull, 0, 0};
@@ -743,7 +752,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) k_push_local(Dev d, IterLaun
     const unsigned tot = __reduce_add_sync(SS_FULL_MASK, (unsigned)pub.nnew);
     const unsigned tm = __reduce_max_sync(SS_FULL_MASK, pub.md);
     dropped = __any_sync(SS_FULL_MASK, pub.drop != 0);
-    // (16 CTAs of 32 warps of 2^25 at most)
+    // (16 CTAs of 16 warps of 2^25 at most)
     const unsigned long long td = (unsigned long long)__reduce_add_sync(SS_FULL_MASK, pub.nd_lo & 0xFFFFFu) +
                                   ((unsigned long long)__reduce_add_sync(SS_FULL_MASK, (pub.nd_lo >> 20)) << 20) +
                                   ((unsigned long long)__reduce_add_sync(SS_FULL_MASK, pub.nd_hi) << 20);
