@@ -3,7 +3,7 @@
 // independent chain
 //     k_init -> k_batch_root (root read from a device array) -> device-side
 //     iteration loop (conditional WHILE node) -> k_batch_output
-// or, for the fixed policies on small graphs, the one node k_small; so one
+// or, for the fixed policies on small graphs (batch_small), the one node k_small; so one
 // cudaGraphLaunch runs every BFS, the chains overlapping on the GPU, and the same
 // executable graph is replayed with new roots and output pointers.
 #include <algorithm>
@@ -125,6 +125,8 @@ ss_status slimsell_batch_create(const slimsell_handle* hs, int32_t g, int32_t se
     order[(size_t)i] = i;
     batch_slots += b->hs[(size_t)i]->slots;
   }
+  long long ctas = 0;
+  for (auto* h : b->hs) ctas += batch_ctas(h, h->dev(), policy, batch_slots);
   std::stable_sort(order.begin(), order.end(),
                    [&](int x, int y) { return b->hs[(size_t)x]->slots > b->hs[(size_t)y]->slots; });
   for (int o = 0; o < g && s == SS_OK; ++o) {
@@ -135,7 +137,7 @@ ss_status slimsell_batch_create(const slimsell_handle* hs, int32_t g, int32_t se
     int* roots = b->d_roots;
     int** dist = b->d_dist;
     int** par = b->d_par;
-    if (batch_small(h, d, policy)) {  // the whole chain in one node
+    if (batch_small(h, d, policy, ctas)) {  // the whole chain in one node
       SmallIo io{};
       io.roots = roots;
       io.dists = dist;

@@ -1284,8 +1284,8 @@ static ss_status launch_filtered(const slimsell_graph* h, const Dev& d, const It
 // Graphs whose whole run goes into one launch (k_small): the fixed full and SlimWork
 // policies over SlimSell with the whole bitmap staged, up to SMALL_SLOTS slots where a
 // run has the GPU to itself (what one or two CTAs hold), up to
-// SMALL_BATCH_SLOTS side by side in a batch, where a cluster's SMs are a graph's share
-// of the GPU and its size follows from its share of the slots (at least
+// SMALL_BATCH_SLOTS side by side in a batch (batch_small), where a cluster's SMs are a
+// graph's share of the GPU and its size follows from its share of the slots (at least
 // SMALL_BATCH_MIN slots a CTA: 32 graphs of scale 10 .. 13 take 171 us, 217 with 16 K).
 // SMALL_SLOTS could go on to about 1 M (Kronecker 14 takes 79 us that way, 147 grid-wide;
 // ER 200 K, without hubs, 234 against 147), but the adaptive policies do not run here, and
@@ -1307,14 +1307,13 @@ constexpr long long SMALL_SLOTS = SS_SMALL_SLOTS;                  // one run al
 constexpr long long SMALL_SLOTS_PER_CTA = SS_SMALL_SLOTS_PER_CTA;
 constexpr long long SMALL_BATCH_SLOTS = SS_SMALL_BATCH_SLOTS;      // many side by side
 constexpr long long SMALL_BATCH_MIN = SS_SMALL_BATCH_MIN;
+constexpr long long SMALL_BATCH_ALONE = 512 << 10;  // slots, or live rows, up to which a graph of a
+constexpr int SMALL_BATCH_ROWS = 64 << 10;          // batch is a cluster whatever its company (batch_small)
 
 static bool whole_run(const slimsell_graph* h, const Dev& d, int policy, long long max_slots) {
   return (policy == SS_V_FULL || policy == SS_V_SLIMWORK) && d.format == SS_FORMAT_SLIMSELL &&
          h->slots <= max_slots && (long long)d.smem_words * 32 >= h->n_pad &&
          (long long)d.smem_words * 4 <= SS_SMEM_LIMIT_BYTES - 16 - (long long)sizeof(ItemCache) * PULL_THREADS;
-}
-bool batch_small(const slimsell_graph* h, const Dev& d, int policy) {
-  return whole_run(h, d, policy, SMALL_BATCH_SLOTS);
 }
 static size_t small_smem(const Dev& d) {
   return (size_t)(d.smem_words + SMEM_GUARD) * 4 + sizeof(ItemCache) * PULL_THREADS;
@@ -1325,6 +1324,34 @@ static int small_cluster(const slimsell_graph* h, long long slots_per_cta) {
   int G = 1;
   while (G < h->local_cluster && G * slots_per_cta < h->slots) G *= 2;
   return G;
+}
+
+// CTAs of a graph's cluster in a batch of batch_slots slots, 0 where it cannot run as one.
+static int batch_cluster(const slimsell_graph* h, long long batch_slots) {
+  return std::min(8, small_cluster(h, std::max(SMALL_BATCH_MIN, batch_slots / h->num_sms)));
+}
+int batch_ctas(const slimsell_graph* h, const Dev& d, int policy, long long batch_slots) {
+  if (h->slots < SMALL_BATCH_MIN) return 0;
+  return whole_run(h, d, policy, SMALL_BATCH_SLOTS) ? batch_cluster(h, batch_slots) : 1;
+}
+
+// Whether a graph of a batch runs as one cluster or as a loop of grid-wide launches.  A loop's
+// passes have the whole GPU, eight CTAs a twentieth of it; but a loop pays its launches, which
+// those of other loops queue behind (about 4 us a level and loop), and its grids wait for SMs
+// that clusters hold.  So the larger graphs run as clusters only where the batch's clusters,
+// those of graphs that earn a CTA or more (ctas), fill the GPU, or, for sparse graphs, whose
+// runs are many short levels, two fifths of it.  SlimWork, clusters / loops:
+//   Kronecker 16 (2.1 M slots) alone 202 us / 229, 17 (4.1 M) 261 / 192, 16 of 17 536 / 467, 64 1091 / 1648;
+//   G(60 K, 8n) (1 M) 175 / 181, G(120 K) (1.9 M) 271 / 188, 16 of it 535 / 476, 64 1056 / 1733;
+//   G(200 K) (3.2 M) 434 / 189, 16 of it 868 / 637, 64 1763 / 2363;
+//   lattice 300^2 (0.3 M) 2.3 ms / 3.6, 500^2 (0.9 M) 8.7 / 7.8, 16 of it 17.7 / 32.9,
+//   900^2 (3.1 M) 56 / 20, 4 of it 62 / 46, 16 of it 113 / 177;
+//   64 graphs of Kronecker 10 .. 17 (192 CTAs), all clusters 432 us, those of 17 in loops 503.
+bool batch_small(const slimsell_graph* h, const Dev& d, int policy, long long ctas) {
+  if (!whole_run(h, d, policy, SMALL_BATCH_SLOTS)) return false;
+  if (h->slots <= SMALL_BATCH_ALONE || h->n_live <= SMALL_BATCH_ROWS) return true;
+  const bool sparse = h->nnz < 8LL * h->n_live;
+  return ctas >= (sparse ? 2LL * h->num_sms / 5 : (long long)h->num_sms);
 }
 
 using SmallKernel = void (*)(Dev, SmallIo, int);
@@ -1380,7 +1407,7 @@ ss_status add_small_node(const slimsell_graph* h, const Dev& d, int sr, int poli
   SmallKernel kern = nullptr;
   ss_status s = small_kernel(h, sr, &kern);
   if (s != SS_OK) return s;
-  const int G = std::min(8, small_cluster(h, std::max(SMALL_BATCH_MIN, batch_slots / h->num_sms)));
+  const int G = batch_cluster(h, batch_slots);
   Dev dd = d;
   SmallIo ii = io;
   int pol = policy;

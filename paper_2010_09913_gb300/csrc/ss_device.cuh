@@ -366,7 +366,10 @@ struct SmallIo {
   int* const* parents;
   int i;
 };
-bool batch_small(const slimsell_graph* h, const Dev& d, int policy);  // a batch runs this graph that way
+// A batch runs this graph that way: what it counts for in the rule (CTAs), and the rule, from the
+// sum of those over the batch.
+int batch_ctas(const slimsell_graph* h, const Dev& d, int policy, long long batch_slots);
+bool batch_small(const slimsell_graph* h, const Dev& d, int policy, long long ctas);
 ss_status add_small_node(const slimsell_graph* h, const Dev& d, int sr, int policy, const SmallIo& io,
                          long long batch_slots, cudaGraph_t g, cudaGraphNode_t* out);
 
