@@ -1282,15 +1282,22 @@ static ss_status launch_filtered(const slimsell_graph* h, const Dev& d, const It
 }
 
 // Graphs whose whole run goes into one launch (k_small): the fixed full and SlimWork
-// policies over SlimSell with the whole bitmap staged, up to SMALL_SLOTS slots where a
-// run has the GPU to itself (what one or two CTAs hold), up to
-// SMALL_BATCH_SLOTS side by side in a batch (batch_small), where a cluster's SMs are a
-// graph's share of the GPU and its size follows from its share of the slots (at least
-// SMALL_BATCH_MIN slots a CTA: 32 graphs of scale 10 .. 13 take 171 us, 217 with 16 K).
-// SMALL_SLOTS could go on to about 1 M (Kronecker 14 takes 79 us that way, 147 grid-wide;
-// ER 200 K, without hubs, 234 against 147), but the adaptive policies do not run here, and
-// plain SlimWork would then beat them on small long-diameter graphs, where they are the
-// choice that scales (tests/test_gpu_selector.py holds them to it).
+// policies over SlimSell with the whole bitmap staged.  Where a run has the GPU to itself
+// that is a graph of up to SMALL_ROWS live rows (8 a thread of one CTA) and SMALL_DENSE_SLOTS
+// slots (what 16 CTAs stream in a few microseconds), whatever its layout, but for
+// layouts that are mostly padding, whose few long items leave most warps idle; and any
+// graph of up to SMALL_SLOTS slots.  One launch / grid-wide, SlimWork tropical, us a call that
+// is waited for:
+//   Kronecker 10 in chunks of 32 69 / 118, of 64 93 / 131, of 32 sorted in windows of 256 69 / 118;
+//   Kronecker 13 129 / 195, in chunks of 8 91 / 161; G(8 K, 8n) 82 / 165, G(8 K, 60n) 105 / 250;
+//   lattice 64^2 422 / 1202; Kronecker 11 unsorted in unsplit chunks of 64 (13 slots an edge) 465 / 413.
+// It goes on to gain past SMALL_ROWS (lattice 128^2 823 / 1678, Kronecker 14 154 / 229), but the
+// adaptive policies do not run here, and from there on they, who scale, would lose to
+// plain SlimWork on small long-diameter graphs.
+// In a batch, where graphs run side by side: up to SMALL_BATCH_SLOTS (batch_small); a
+// cluster's SMs are a graph's share of the GPU and its size follows from its share of the
+// slots (at least SMALL_BATCH_MIN slots a CTA: 32 graphs of scale 10 .. 13 take 171 us,
+// 217 with 16 K).
 #ifndef SS_SMALL_SLOTS
 #define SS_SMALL_SLOTS (32 << 10)
 #endif
@@ -1304,6 +1311,8 @@ static ss_status launch_filtered(const slimsell_graph* h, const Dev& d, const It
 #define SS_SMALL_BATCH_MIN (64 << 10)
 #endif
 constexpr long long SMALL_SLOTS = SS_SMALL_SLOTS;                  // one run alone on the GPU
+constexpr int SMALL_ROWS = 8 << 10;
+constexpr long long SMALL_DENSE_SLOTS = 512 << 10;
 constexpr long long SMALL_SLOTS_PER_CTA = SS_SMALL_SLOTS_PER_CTA;
 constexpr long long SMALL_BATCH_SLOTS = SS_SMALL_BATCH_SLOTS;      // many side by side
 constexpr long long SMALL_BATCH_MIN = SS_SMALL_BATCH_MIN;
@@ -1314,6 +1323,10 @@ static bool whole_run(const slimsell_graph* h, const Dev& d, int policy, long lo
   return (policy == SS_V_FULL || policy == SS_V_SLIMWORK) && d.format == SS_FORMAT_SLIMSELL &&
          h->slots <= max_slots && (long long)d.smem_words * 32 >= h->n_pad &&
          (long long)d.smem_words * 4 <= SS_SMEM_LIMIT_BYTES - 16 - (long long)sizeof(ItemCache) * PULL_THREADS;
+}
+static bool run_small(const slimsell_graph* h, const Dev& d, int policy) {
+  const bool rows = h->n_live <= SMALL_ROWS && h->slots <= 4 * h->nnz;
+  return whole_run(h, d, policy, rows ? SMALL_DENSE_SLOTS : SMALL_SLOTS);
 }
 static size_t small_smem(const Dev& d) {
   return (size_t)(d.smem_words + SMEM_GUARD) * 4 + sizeof(ItemCache) * PULL_THREADS;
@@ -1694,7 +1707,7 @@ ss_status slimsell_bfs(slimsell_handle h, int32_t root, int32_t semiring, int32_
   if (prof) SS_CUDA(cudaEventRecord(h->ev_c, st));
 
   const bool dp = d_parent && semiring != SS_SELMAX && h->dp_pass;
-  const bool whole = device_loop && whole_run(h, d, policy, SMALL_SLOTS);
+  const bool whole = device_loop && run_small(h, d, policy);
   if (!whole) {
     k_init<<<grid, 256, 0, st>>>(d);
     k_init_root<<<1, 1, 0, st>>>(d, root);
