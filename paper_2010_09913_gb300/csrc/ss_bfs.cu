@@ -67,24 +67,22 @@ constexpr int SHORT_COLS = SS_PULL_SHORT_COLS;  // chunks this short go several 
 // The filtered pull's chunks in groups of C/4 lanes: every unsplit chunk starts in a
 // group and goes on in a whole warp once it is still open after GROUP_TRY columns
 // with more than GROUP_LEFT left (8 / 32: 314 us for ER 4 M's largest level; leaving
-// with more than 8 left 344, trying 4 columns 322).  The real semiring needs whole
-// sums, so there only chunks of at most GROUP_COLS columns go in groups.
-#ifndef SS_PULL_GROUP_COLS
-#define SS_PULL_GROUP_COLS 8
-#endif
+// with more than 8 left 344, trying 4 columns 322).
 #ifndef SS_PULL_GROUP_TRY
 #define SS_PULL_GROUP_TRY 8
 #endif
 #ifndef SS_PULL_GROUP_LEFT
 #define SS_PULL_GROUP_LEFT 32
 #endif
-constexpr int GROUP_COLS = SS_PULL_GROUP_COLS;
 constexpr int GROUP_TRY = SS_PULL_GROUP_TRY;
 constexpr int GROUP_LEFT = SS_PULL_GROUP_LEFT;
 
-// int4 col loads in flight per lane (4 slots each)
-template <int SR, int FMT>
+// int4 col loads in flight per lane (4 slots each).  STOP: in the filtered pass, whose 20 warps
+// an SM have 96 registers a thread for them (a level with few hits on Kronecker 22: 181 us with
+// the streaming pass's 4, 170 with 8; real 276 with 3, 254 with 6, 269 with 4).
+template <int SR, int FMT, bool STOP = false>
 __host__ __device__ constexpr int pull_step() {
+  if (STOP) return SR == SS_REAL ? 6 : 8;
   return FMT == SS_FORMAT_SELL ? SS_PULL_STEP_SELL : (SR == SS_REAL ? SS_PULL_STEP_REAL : SS_PULL_STEP);
 }
 // Bits of the semiring's zero, the value of a Sell-C-sigma padding slot.
@@ -336,18 +334,167 @@ struct __align__(8) ItemCache {
   long long start;
 };
 
+// The items of a warp's batch that take a whole warp each (todo: their lanes, lane s holding
+// item s).  STOP (the filtered pass): rows that are visited or, but for the real semiring,
+// hit load nothing more; counted: items that are counted as active already; found: rows of
+// this lane's item that entered the frontier earlier in this pass.
+template <int SR, int C, int FMT, bool SHARED, bool STOP>
+__device__ __forceinline__ void pull_whole(const Dev& d, int k, const unsigned* gbm, const Staged& sg, unsigned todo,
+                                           const int4& my_item, long long my_start, unsigned long long my_vis,
+                                           Counters& cnt, unsigned counted = 0u, unsigned long long found = 0ull) {
+  constexpr int PULL_STEP = pull_step<SR, FMT, STOP>();
+  constexpr int Q = C / 4;
+  const int* colp = (FMT == SS_FORMAT_SELL) ? d.scol : d.col;
+  const int lane = threadIdx.x & 31;
+  const unsigned* sm = sg.sm;
+  const float* smf = sg.smf;
+  const int sbits = sg.sbits, sf = sg.sf;
+  while (todo) {
+    const int src = __ffs(todo) - 1;
+    todo &= todo - 1;
+    const int4 item = shfl_int4(my_item, src);
+    const long long start = __shfl_sync(SS_FULL_MASK, my_start, src);
+    const int chunk = item.x;
+    // L2 prefetch: the head of this item beyond the first step, and of the next item
+    if (lane == src) {
+      const unsigned bytes = (unsigned)(item.z - item.y) * C * 4u;
+      if (bytes > 2048u)
+        prefetch_l2(colp + start + 512, min(bytes - 2048u, (unsigned)PREFETCH_BYTES));
+    }
+    if (todo) {
+      const int nxt = __ffs(todo) - 1;
+      if (lane == nxt) {
+        const unsigned bytes = (unsigned)(my_item.z - my_item.y) * C * 4u;
+        prefetch_l2(colp + my_start, min(bytes, (unsigned)PREFETCH_BYTES));
+      }
+    }
+    // this lane's unvisited rows (only this chunk's post changes them)
+    const unsigned long long vis = __shfl_sync(SS_FULL_MASK, my_vis, src);
+    const unsigned live = ~(unsigned)(vis >> (4 * (lane % Q))) & 0xFu;
+    int first[4] = {-1, -1, -1, -1};
+    float sum[4] = {0.f, 0.f, 0.f, 0.f};
+    bool need = live != 0u;  // (STOP)
+    const int nq = (item.z - item.y) * Q;
+    const int4* base = reinterpret_cast<const int4*>(colp + start);
+    const int4* vbase = reinterpret_cast<const int4*>(d.sval + start);  // (Sell only)
+    for (int q0 = 0; q0 < nq; q0 += 32 * PULL_STEP) {
+      if (STOP) {
+        if (!__any_sync(SS_FULL_MASK, need)) break;
+        if (!need) continue;
+      }
+      // keep the prefetch PREFETCH_BYTES ahead inside long items (one lane issues it)
+      if (lane == 0) {
+        const long long ahead = (long long)(q0 + 32 * PULL_STEP) * 16 + PREFETCH_BYTES;
+        const long long total = (long long)nq * 16;
+        if (ahead < total) {
+          prefetch_l2(reinterpret_cast<const char*>(base) + ahead,
+                      (unsigned)min(total - ahead, (long long)(32 * PULL_STEP * 16)));
+          if (FMT == SS_FORMAT_SELL)
+            prefetch_l2(reinterpret_cast<const char*>(vbase) + ahead,
+                        (unsigned)min(total - ahead, (long long)(32 * PULL_STEP * 16)));
+        }
+      }
+      int4 c[PULL_STEP], v[PULL_STEP];
+#pragma unroll
+      for (int u = 0; u < PULL_STEP; ++u) {
+        const int q = q0 + lane + 32 * u;
+        c[u] = (q < nq) ? ld_stream(base + q) : make_int4(-1, -1, -1, -1);
+        if (STOP && q < nq) cnt.slots += 4;
+        if (FMT == SS_FORMAT_SELL) {
+          const int4 vq = (q < nq) ? ld_stream(vbase + q) : make_int4(0, 0, 0, 0);
+          c[u] = sell_edges<SR>(c[u], vq);
+          v[u] = SR == SS_REAL ? vq : make_int4(0, 0, 0, 0);
+        } else {
+          v[u] = make_int4(0, 0, 0, 0);
+        }
+      }
+      if constexpr (SR == SS_REAL && FMT == SS_FORMAT_SLIMSELL) {
+        unsigned mm[PULL_STEP];
+#pragma unroll
+        for (int u = 0; u < PULL_STEP; ++u)
+          mm[u] = (q0 + 32 * u < nq) ? quad_hits(sm, sbits, gbm, c[u], first) & live : 0u;
+        gather_step<PULL_STEP, SHARED>(d, c, mm, sum, smf, sf);
+      } else {
+#pragma unroll
+        for (int u = 0; u < PULL_STEP; ++u)  // (q0 + 32 u < nq is warp-uniform)
+          if (q0 + 32 * u < nq) scan_quad<SR, FMT>(d, sm, sbits, gbm, c[u], v[u], first, sum, live, smf, sf);
+      }
+      if (STOP) {  // a row is done once visited or (not real) hit
+        need = false;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) need |= (live >> r & 1u) && (SR == SS_REAL || first[r] < 0);
+      }
+    }
+    if (!STOP && lane == 0) cnt.slots += (unsigned long long)(item.z - item.y) * C;
+    // the largest original id among this lane's first hits of unvisited rows
+    RowAcc acc;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      acc.best[r] = (first[r] >= 0 && (live >> r & 1u)) ? __ldg(d.perm + first[r]) : -1;
+      acc.sum[r] = sum[r];
+    }
+    // (a non-zero real sum implies a hit on a live row of the same lane)
+    const bool any_hit = (acc.best[0] >= 0) | (acc.best[1] >= 0) | (acc.best[2] >= 0) |
+                         (acc.best[3] >= 0);
+    if (__any_sync(SS_FULL_MASK, any_hit)) {  // lanes with equal lane mod Q share rows
+#pragma unroll
+      for (int off = Q; off < 32; off <<= 1)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          acc.best[r] = max(acc.best[r], __shfl_xor_sync(SS_FULL_MASK, acc.best[r], off));
+          if (SR == SS_REAL) acc.sum[r] += __shfl_xor_sync(SS_FULL_MASK, acc.sum[r], off);
+        }
+    }
+    if (item.w >= 0) {  // SlimChunk: combine partial rows, the last arriving item post-processes
+      const size_t xo = (size_t)item.w * C + 4 * lane;
+      if (lane < Q) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          if (acc.best[r] >= 0) atomicMax(d.xpar + xo + r, acc.best[r]);
+          if (SR == SS_REAL && acc.sum[r] != 0.0f) atomicAdd(d.xacc + xo + r, acc.sum[r]);
+        }
+        __threadfence();
+      }
+      __syncwarp();
+      int last = 0;
+      if (lane == 0) {
+        const unsigned old = atomicAdd(d.arrive + item.w, 1u);
+        last = (old == (unsigned)d.split_n[item.w] - 1u);
+      }
+      last = __shfl_sync(SS_FULL_MASK, last, 0);
+      if (!last) continue;
+      __threadfence();
+      if (lane < Q) {
+        // one 16-byte read and reset per array (xo is a multiple of 4 and the
+        // scratch 16-byte aligned); the per-row scalar form of this rarely run
+        // block made the whole real-semiring kernel 20-25 % slower on GB300
+        const int4 b4 = __ldcg(reinterpret_cast<const int4*>(d.xpar + xo));
+        *reinterpret_cast<int4*>(d.xpar + xo) = make_int4(-1, -1, -1, -1);
+        acc.best[0] = b4.x; acc.best[1] = b4.y; acc.best[2] = b4.z; acc.best[3] = b4.w;
+        if (SR == SS_REAL) {
+          const float4 s4 = __ldcg(reinterpret_cast<const float4*>(d.xacc + xo));
+          *reinterpret_cast<float4*>(d.xacc + xo) = make_float4(0.f, 0.f, 0.f, 0.f);
+          acc.sum[0] = s4.x; acc.sum[1] = s4.y; acc.sum[2] = s4.z; acc.sum[3] = s4.w;
+        }
+      }
+      if (lane == 0) d.arrive[item.w] = 0u;
+    }
+    if (lane == 0 && !(STOP && (counted >> src & 1u))) cnt.act += 1;
+    post_chunk<SR, C>(d, k, chunk, lane, live, vis, acc, cnt, true, STOP ? __shfl_sync(SS_FULL_MASK, found, src) : 0ull);
+  }
+}
+
 // Warp wid of nw walks its items wid, wid + nw, ... of level k (the item list is
 // ordered for such an assignment): it reads the descriptors and visited bits of 32
 // of them at once (one per lane) and processes the active ones.  full: every chunk
 // is active.  SHARED: other SMs have written the bitmaps and values since this
 // kernel began, so those are read past L1 (and the whole bitmap is staged); cache:
 // the threads' item descriptors in shared memory (at most one batch), filled by the
-// first level.
-template <int SR, int C, int FMT, bool SHARED>
+// first level.  STOP: see pull_whole.
+template <int SR, int C, int FMT, bool SHARED, bool STOP = false>
 __device__ __forceinline__ void pull_items(const Dev& d, int k, bool full, const unsigned* gbm, const Staged& sg,
                                            int wid, int nw, Counters& cnt, ItemCache* cache = nullptr,
                                            bool fill = false) {
-  constexpr int PULL_STEP = pull_step<SR, FMT>();
   constexpr int Q = C / 4;
   constexpr unsigned long long ALL_ROWS = C == 64 ? ~0ull : (1ull << C) - 1ull;
   const int* colp = (FMT == SS_FORMAT_SELL) ? d.scol : d.col;
@@ -444,128 +591,7 @@ __device__ __forceinline__ void pull_items(const Dev& d, int k, bool full, const
       }
       post_chunk<SR, C, true>(d, k, chunk, lane, live, vis, acc, cnt, own);
     }
-    while (todo) {
-      const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const int4 item = shfl_int4(my_item, src);
-      const long long start = __shfl_sync(SS_FULL_MASK, my_start, src);
-      const int chunk = item.x;
-      // L2 prefetch: the head of this item beyond the first step, and of the next item
-      if (lane == src) {
-        const unsigned bytes = (unsigned)(item.z - item.y) * C * 4u;
-        if (bytes > 2048u)
-          prefetch_l2(colp + start + 512, min(bytes - 2048u, (unsigned)PREFETCH_BYTES));
-      }
-      if (todo) {
-        const int nxt = __ffs(todo) - 1;
-        if (lane == nxt) {
-          const unsigned bytes = (unsigned)(my_item.z - my_item.y) * C * 4u;
-          prefetch_l2(colp + my_start, min(bytes, (unsigned)PREFETCH_BYTES));
-        }
-      }
-      // this lane's unvisited rows (only this chunk's post changes them)
-      const unsigned long long vis = __shfl_sync(SS_FULL_MASK, my_vis, src);
-      const unsigned live = ~(unsigned)(vis >> (4 * (lane % Q))) & 0xFu;
-      int first[4] = {-1, -1, -1, -1};
-      float sum[4] = {0.f, 0.f, 0.f, 0.f};
-      const int nq = (item.z - item.y) * Q;
-      const int4* base = reinterpret_cast<const int4*>(colp + start);
-      const int4* vbase = reinterpret_cast<const int4*>(d.sval + start);  // (Sell only)
-      for (int q0 = 0; q0 < nq; q0 += 32 * PULL_STEP) {
-        // keep the prefetch PREFETCH_BYTES ahead inside long items (one lane issues it)
-        if (lane == 0) {
-          const long long ahead = (long long)(q0 + 32 * PULL_STEP) * 16 + PREFETCH_BYTES;
-          const long long total = (long long)nq * 16;
-          if (ahead < total) {
-            prefetch_l2(reinterpret_cast<const char*>(base) + ahead,
-                        (unsigned)min(total - ahead, (long long)(32 * PULL_STEP * 16)));
-            if (FMT == SS_FORMAT_SELL)
-              prefetch_l2(reinterpret_cast<const char*>(vbase) + ahead,
-                          (unsigned)min(total - ahead, (long long)(32 * PULL_STEP * 16)));
-          }
-        }
-        int4 c[PULL_STEP], v[PULL_STEP];
-#pragma unroll
-        for (int u = 0; u < PULL_STEP; ++u) {
-          const int q = q0 + lane + 32 * u;
-          c[u] = (q < nq) ? ld_stream(base + q) : make_int4(-1, -1, -1, -1);
-          if (FMT == SS_FORMAT_SELL) {
-            const int4 vq = (q < nq) ? ld_stream(vbase + q) : make_int4(0, 0, 0, 0);
-            c[u] = sell_edges<SR>(c[u], vq);
-            v[u] = SR == SS_REAL ? vq : make_int4(0, 0, 0, 0);
-          } else {
-            v[u] = make_int4(0, 0, 0, 0);
-          }
-        }
-        if constexpr (SR == SS_REAL && FMT == SS_FORMAT_SLIMSELL) {
-          unsigned mm[PULL_STEP];
-#pragma unroll
-          for (int u = 0; u < PULL_STEP; ++u)
-            mm[u] = (q0 + 32 * u < nq) ? quad_hits(sm, sbits, gbm, c[u], first) & live : 0u;
-          gather_step<PULL_STEP, SHARED>(d, c, mm, sum, smf, sf);
-        } else {
-#pragma unroll
-          for (int u = 0; u < PULL_STEP; ++u)  // (q0 + 32 u < nq is warp-uniform)
-            if (q0 + 32 * u < nq) scan_quad<SR, FMT>(d, sm, sbits, gbm, c[u], v[u], first, sum, live, smf, sf);
-        }
-      }
-      if (lane == 0) cnt.slots += (unsigned long long)(item.z - item.y) * C;
-      // the largest original id among this lane's first hits of unvisited rows
-      RowAcc acc;
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        acc.best[r] = (first[r] >= 0 && (live >> r & 1u)) ? __ldg(d.perm + first[r]) : -1;
-        acc.sum[r] = sum[r];
-      }
-      // (a non-zero real sum implies a hit on a live row of the same lane)
-      const bool any_hit = (acc.best[0] >= 0) | (acc.best[1] >= 0) | (acc.best[2] >= 0) |
-                           (acc.best[3] >= 0);
-      if (__any_sync(SS_FULL_MASK, any_hit)) {  // lanes with equal lane mod Q share rows
-#pragma unroll
-        for (int off = Q; off < 32; off <<= 1)
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            acc.best[r] = max(acc.best[r], __shfl_xor_sync(SS_FULL_MASK, acc.best[r], off));
-            if (SR == SS_REAL) acc.sum[r] += __shfl_xor_sync(SS_FULL_MASK, acc.sum[r], off);
-          }
-      }
-      if (item.w >= 0) {  // SlimChunk: combine partial rows, the last arriving item post-processes
-        const size_t xo = (size_t)item.w * C + 4 * lane;
-        if (lane < Q) {
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            if (acc.best[r] >= 0) atomicMax(d.xpar + xo + r, acc.best[r]);
-            if (SR == SS_REAL && acc.sum[r] != 0.0f) atomicAdd(d.xacc + xo + r, acc.sum[r]);
-          }
-          __threadfence();
-        }
-        __syncwarp();
-        int last = 0;
-        if (lane == 0) {
-          const unsigned old = atomicAdd(d.arrive + item.w, 1u);
-          last = (old == (unsigned)d.split_n[item.w] - 1u);
-        }
-        last = __shfl_sync(SS_FULL_MASK, last, 0);
-        if (!last) continue;
-        __threadfence();
-        if (lane < Q) {
-          // one 16-byte read and reset per array (xo is a multiple of 4 and the
-          // scratch 16-byte aligned); the per-row scalar form of this rarely run
-          // block made the whole real-semiring kernel 20-25 % slower on GB300
-          const int4 b4 = __ldcg(reinterpret_cast<const int4*>(d.xpar + xo));
-          *reinterpret_cast<int4*>(d.xpar + xo) = make_int4(-1, -1, -1, -1);
-          acc.best[0] = b4.x; acc.best[1] = b4.y; acc.best[2] = b4.z; acc.best[3] = b4.w;
-          if (SR == SS_REAL) {
-            const float4 s4 = __ldcg(reinterpret_cast<const float4*>(d.xacc + xo));
-            *reinterpret_cast<float4*>(d.xacc + xo) = make_float4(0.f, 0.f, 0.f, 0.f);
-            acc.sum[0] = s4.x; acc.sum[1] = s4.y; acc.sum[2] = s4.z; acc.sum[3] = s4.w;
-          }
-        }
-        if (lane == 0) d.arrive[item.w] = 0u;
-      }
-      if (lane == 0) cnt.act += 1;
-      post_chunk<SR, C>(d, k, chunk, lane, live, vis, acc, cnt);
-    }
+    pull_whole<SR, C, FMT, SHARED, STOP>(d, k, gbm, sg, todo, my_item, my_start, my_vis, cnt);
   }
 }
 
@@ -667,39 +693,27 @@ __global__ void __launch_bounds__(PULL_THREADS, 1) k_pull(Dev d, int variant,
 // The visited-filtered pull: as k_pull, but only unvisited rows are computed and
 // (but for the real semiring) a row stops at its first frontier neighbour.
 //
-// Hub levels find most rows within their first columns, so what a pass costs is
-// not the stream but the latency chain of each chunk (descriptor, columns, bits,
-// parent, row data).  Hence chunks start in groups of C/4 lanes (32 / (C/4) at a
-// time, GSTEP columns a step, each group taking its next chunk on its own), and
-// the next loads are issued before the finished chunks are post-processed; only
-// long rests and split items take a whole warp.  Reading 16 columns at once with
-// // one chunk per warp took 58 us on Kronecker 22's level after the hubs and 395 us on
-// ER 4 M's largest; this takes 45 and 230 (GSTEP 4: 248; without leaving out the
-// lookups of rows already hit 314).  640 threads, for the registers (768: 246 at
-// GSTEP 4; 1024 spills).
+// Where the frontier's rows hold a good share of all edges (frontier_hits_soon), most rows
+// stop within their first columns, so what a pass costs is not the stream but the
+// latency chain of each chunk (descriptor, columns, bits, parent, row data).  There
+// chunks start in groups of C/4 lanes (32 / (C/4) at a time, GSTEP columns a step, each
+// group taking its next chunk on its own), and the next loads are issued before the
+// finished chunks are post-processed; only long rests and split items take a whole warp.
+// Reading 16 columns at once with one chunk per warp took 64 us on Kronecker 22's level
+// after the hubs and 301 us on ER 4 M's largest; this takes 48 and 158 (GSTEP 4: 248 where
+// GSTEP 2 took 230; without leaving out the lookups of rows already hit 314).  Elsewhere,
+// and for the real semiring, which needs whole sums, the columns are streamed as in
+// k_pull: in groups, levels with few hits took 44 us on ER 1 M and 186 on Kronecker 22, and
+// 37 and 170 so.  640 threads, for the registers (768: 246 at GSTEP 4; 1024 spills).
+// The levels with many hits.
 template <int SR, int C>
-__global__ void __launch_bounds__(FILTERED_THREADS, 1) k_pull_filtered(Dev d, int variant,
-                                                                       cudaGraphConditionalHandle cond,
-                                                                       int use_cond) {
+__device__ __forceinline__ void pull_groups(const Dev& d, int k, const unsigned* gbm, const Staged& sg, int wid, int nw,
+                                            Counters& cnt) {
   constexpr int FMT = SS_FORMAT_SLIMSELL;
-  constexpr int PULL_STEP = pull_step<SR, FMT>();
-  const int* colp = d.col;
   constexpr int Q = C / 4;
-  if (d.ctl->done) return;
-  const int k = d.ctl->k;
-  const int km1 = k - 1;
-  const int lane = threadIdx.x & 31;
-  const int wid = blockIdx.x * (FILTERED_THREADS / 32) + (threadIdx.x >> 5);
-  const int nw = gridDim.x * (FILTERED_THREADS / 32);
-  const unsigned* gbm = d.fb[km1 & 1];
   constexpr unsigned long long ALL_ROWS = C == 64 ? ~0ull : (1ull << C) - 1ull;
-  const Staged sg = stage_frontier<SR>(d, gbm);
-  stage_wait();
-  const unsigned* sm = sg.sm;
-  const float* smf = sg.smf;
-  const int sbits = sg.sbits, sf = sg.sf;
-  Counters cnt;
-  unsigned long long lane_slots = 0;
+  const int* colp = d.col;
+  const int lane = threadIdx.x & 31;
   for (long long b0 = wid; b0 < d.n_items; b0 += 32LL * nw) {
     const long long my_it = b0 + (long long)lane * nw;
     int4 my_item = make_int4(0, 0, 0, -1);
@@ -717,24 +731,23 @@ __global__ void __launch_bounds__(FILTERED_THREADS, 1) k_pull_filtered(Dev d, in
       if (!active && my_item.y == 0 && old != 0ull) store_bits<C>(d.fb[k & 1], my_item.x, 0u, 0u);
     }
     unsigned todo = __ballot_sync(SS_FULL_MASK, active);
-    // chunks in groups of Q lanes (see GROUP_COLS).  Each group works through its own
+    // unsplit chunks in groups of Q lanes.  Each group works through its own
     // chunk GSTEP columns at a time and takes the next one when it is done; the loads
     // of the next step are issued before the finished chunks are post-processed.
     unsigned long long my_new = 0ull;  // rows of this lane's item that the groups have found
+    const unsigned grouped = __ballot_sync(SS_FULL_MASK, active && my_item.w < 0);
     {
       constexpr int GROUPS = 32 / Q;
       constexpr int GSTEP = 2;
-      constexpr bool EARLY = SR != SS_REAL;  // rows stop at their first hit
       const int lq = lane % Q;
-      unsigned gm = __ballot_sync(SS_FULL_MASK, active && my_item.w < 0 &&
-                                                    (EARLY || my_item.z - my_item.y <= GROUP_COLS));
+      unsigned gm = grouped;
       todo &= ~gm;
       int src = -1, chunk = 0, rem = 0;  // this group's item (its lane), chunk and columns left
       unsigned live = 0;                 // this lane's unvisited rows of it
       unsigned long long vis = 0ull;     // its visited rows
       const int4* cp = nullptr;
       int first[4];
-      float sum[4];
+      float none[4] = {0.f, 0.f, 0.f, 0.f};  // (no sums but for the real semiring)
       int4 c[GSTEP];
       // groups that want an item take the next ones; their first step is loaded
       auto take = [&](bool want) {
@@ -759,69 +772,50 @@ __global__ void __launch_bounds__(FILTERED_THREADS, 1) k_pull_filtered(Dev d, in
           vis = nvis;
           live = got >= 0 ? ~(unsigned)(nvis >> (4 * lq)) & 0xFu : 0u;
           cp = reinterpret_cast<const int4*>(colp + start) + lq;
-          if (got >= 0 && lq == 0) {
-            cnt.act += 1;
-          }
+          if (got >= 0 && lq == 0) cnt.act += 1;
 #pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            first[r] = -1;
-            sum[r] = 0.f;
-          }
+          for (int r = 0; r < 4; ++r) first[r] = -1;
         }
       };
       auto load = [&]() {
         unsigned open = live;
-        if (EARLY) {
 #pragma unroll
-          for (int r = 0; r < 4; ++r)
-            if (first[r] >= 0) open &= ~(1u << r);
-        }
+        for (int r = 0; r < 4; ++r)
+          if (first[r] >= 0) open &= ~(1u << r);
         const int n = open ? rem : 0;
-        lane_slots += 4ull * (unsigned)max(0, min(n, GSTEP));
+        cnt.slots += 4ull * (unsigned)max(0, min(n, GSTEP));
 #pragma unroll
-        for (int u = 0; u < GSTEP; ++u) {
-          c[u] = (u < n) ? ld_stream(cp + u * Q) : make_int4(-1, -1, -1, -1);
-        }
+        for (int u = 0; u < GSTEP; ++u) c[u] = (u < n) ? ld_stream(cp + u * Q) : make_int4(-1, -1, -1, -1);
       };
       if (gm) {
         take(true);
         load();
       }
       while (__any_sync(SS_FULL_MASK, src >= 0)) {
-        if constexpr (SR == SS_REAL) {
-          unsigned mm[GSTEP];
+        // rows hit in an earlier step (or visited) look nothing up: past the staged
+        // prefix a lookup is a memory gather
+        bool shut[4];
 #pragma unroll
-          for (int u = 0; u < GSTEP; ++u) mm[u] = quad_hits(sm, sbits, gbm, c[u], first) & live;
-          gather_step<GSTEP>(d, c, mm, sum, smf, sf);
-        } else {
-          // rows hit in an earlier step (or visited) look nothing up: past the staged
-          // prefix a lookup is a memory gather
-          bool shut[4];
+        for (int r = 0; r < 4; ++r) shut[r] = first[r] >= 0 || !(live >> r & 1u);
 #pragma unroll
-          for (int r = 0; r < 4; ++r) shut[r] = EARLY && (first[r] >= 0 || !(live >> r & 1u));
-#pragma unroll
-          for (int u = 0; u < GSTEP; ++u) {
-            const int4 q = make_int4(shut[0] ? -1 : c[u].x, shut[1] ? -1 : c[u].y, shut[2] ? -1 : c[u].z,
-                                     shut[3] ? -1 : c[u].w);
-            scan_quad<SR, FMT>(d, sm, sbits, gbm, q, make_int4(0, 0, 0, 0), first, sum, live, smf, sf);
-          }
+        for (int u = 0; u < GSTEP; ++u) {
+          const int4 q = make_int4(shut[0] ? -1 : c[u].x, shut[1] ? -1 : c[u].y, shut[2] ? -1 : c[u].z,
+                                   shut[3] ? -1 : c[u].w);
+          scan_quad<SR, FMT>(d, sg.sm, sg.sbits, gbm, q, make_int4(0, 0, 0, 0), first, none, live, sg.smf, sg.sf);
         }
         rem -= GSTEP;
         cp += GSTEP * Q;
-        bool fin = src >= 0 && rem <= 0, leave = false;
-        if (EARLY) {  // done once every row is visited or hit
-          unsigned open = 0;
+        unsigned open = 0;  // done once every row is visited or hit
 #pragma unroll
-          for (int r = 0; r < 4; ++r)
-            if ((live >> r & 1u) && first[r] < 0) open = 1;
+        for (int r = 0; r < 4; ++r)
+          if ((live >> r & 1u) && first[r] < 0) open = 1;
 #pragma unroll
-          for (int o = 1; o < Q; o <<= 1) open |= __shfl_xor_sync(SS_FULL_MASK, open, o);
-          fin = fin || (src >= 0 && !open);
-          // a long rest goes to the whole warp (from this column on)
-          const int used = __shfl_sync(SS_FULL_MASK, my_item.z, max(src, 0)) -
-                           __shfl_sync(SS_FULL_MASK, my_item.y, max(src, 0)) - rem;
-          leave = src >= 0 && !fin && used >= GROUP_TRY && rem > GROUP_LEFT;
-        }
+        for (int o = 1; o < Q; o <<= 1) open |= __shfl_xor_sync(SS_FULL_MASK, open, o);
+        const bool fin = src >= 0 && (rem <= 0 || !open);
+        // a long rest goes to the whole warp (from this column on)
+        const int used = __shfl_sync(SS_FULL_MASK, my_item.z, max(src, 0)) -
+                         __shfl_sync(SS_FULL_MASK, my_item.y, max(src, 0)) - rem;
+        const bool leave = src >= 0 && !fin && used >= GROUP_TRY && rem > GROUP_LEFT;
         const bool out = fin || leave;
         if (__any_sync(SS_FULL_MASK, out)) {
           const int ochunk = chunk, osrc = src, orem = rem;
@@ -831,7 +825,7 @@ __global__ void __launch_bounds__(FILTERED_THREADS, 1) k_pull_filtered(Dev d, in
 #pragma unroll
           for (int r = 0; r < 4; ++r) {
             acc.best[r] = (out && first[r] >= 0 && (live >> r & 1u)) ? first[r] : -1;
-            acc.sum[r] = sum[r];
+            acc.sum[r] = 0.f;
           }
           take(out);
           load();
@@ -840,21 +834,20 @@ __global__ void __launch_bounds__(FILTERED_THREADS, 1) k_pull_filtered(Dev d, in
             if (acc.best[r] >= 0) acc.best[r] = __ldg(d.perm + acc.best[r]);
           unsigned long long added;
           post_chunk<SR, C, true>(d, k, ochunk, lane, olive, ovis, acc, cnt, out, 0ull, &added);
-          if (EARLY) {  // hand the left chunks over: lane s holds item s
+          // hand the left chunks over: lane s holds item s
 #pragma unroll
-            for (int g = 0; g < GROUPS; ++g) {
-              const int s = __shfl_sync(SS_FULL_MASK, leave ? osrc : -1, g * Q);
-              const int left = __shfl_sync(SS_FULL_MASK, orem, g * Q);
-              const unsigned long long nb = __shfl_sync(SS_FULL_MASK, added, g * Q);
-              if (s >= 0) {
-                todo |= 1u << s;
-                if (lane == s) {
-                  const int y = my_item.z - left;
-                  my_start += (long long)(y - my_item.y) * C;
-                  my_item.y = y;
-                  my_new = nb;
-                  my_vis |= nb;
-                }
+          for (int g = 0; g < GROUPS; ++g) {
+            const int s = __shfl_sync(SS_FULL_MASK, leave ? osrc : -1, g * Q);
+            const int left = __shfl_sync(SS_FULL_MASK, orem, g * Q);
+            const unsigned long long nb = __shfl_sync(SS_FULL_MASK, added, g * Q);
+            if (s >= 0) {
+              todo |= 1u << s;
+              if (lane == s) {
+                const int y = my_item.z - left;
+                my_start += (long long)(y - my_item.y) * C;
+                my_item.y = y;
+                my_new = nb;
+                my_vis |= nb;
               }
             }
           }
@@ -864,128 +857,27 @@ __global__ void __launch_bounds__(FILTERED_THREADS, 1) k_pull_filtered(Dev d, in
       }
     }
     __syncwarp();  // a left chunk's bits, stored by its group's first lane, are stored again by lane 0
-    while (todo) {
-      const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const int4 item = shfl_int4(my_item, src);
-      const long long start = __shfl_sync(SS_FULL_MASK, my_start, src);
-      const int chunk = item.x;
-      // L2 prefetch: the head of this item beyond the first step, and of the next item
-      if (lane == src) {
-        const unsigned bytes = (unsigned)(item.z - item.y) * C * 4u;
-        if (bytes > 2048u)
-          prefetch_l2(colp + start + 512, min(bytes - 2048u, (unsigned)PREFETCH_BYTES));
-      }
-      if (todo) {
-        const int nxt = __ffs(todo) - 1;
-        if (lane == nxt) {
-          const unsigned bytes = (unsigned)(my_item.z - my_item.y) * C * 4u;
-          prefetch_l2(colp + my_start, min(bytes, (unsigned)PREFETCH_BYTES));
-        }
-      }
-      // this lane's unvisited rows (only this chunk's post changes them)
-      const unsigned long long vis = __shfl_sync(SS_FULL_MASK, my_vis, src);
-      const unsigned live = ~(unsigned)(vis >> (4 * (lane % Q))) & 0xFu;
-      int first[4] = {-1, -1, -1, -1};
-      float sum[4] = {0.f, 0.f, 0.f, 0.f};
-      bool need = live != 0u;  // only unvisited rows are computed
-      const int nq = (item.z - item.y) * Q;
-      const int4* base = reinterpret_cast<const int4*>(colp + start);
-      for (int q0 = 0; q0 < nq; q0 += 32 * PULL_STEP) {
-        if (!__any_sync(SS_FULL_MASK, need)) break;
-        if (!need) continue;
-        // keep the prefetch PREFETCH_BYTES ahead inside long items (one lane issues it)
-        if (lane == 0) {
-          const long long ahead = (long long)(q0 + 32 * PULL_STEP) * 16 + PREFETCH_BYTES;
-          const long long total = (long long)nq * 16;
-          if (ahead < total) {
-            prefetch_l2(reinterpret_cast<const char*>(base) + ahead,
-                        (unsigned)min(total - ahead, (long long)(32 * PULL_STEP * 16)));
-          }
-        }
-        int4 c[PULL_STEP];
-#pragma unroll
-        for (int u = 0; u < PULL_STEP; ++u) {
-          const int q = q0 + lane + 32 * u;
-          c[u] = (q < nq) ? ld_stream(base + q) : make_int4(-1, -1, -1, -1);
-          if (q < nq) lane_slots += 4;
-        }
-        if constexpr (SR == SS_REAL) {
-          unsigned mm[PULL_STEP];
-#pragma unroll
-          for (int u = 0; u < PULL_STEP; ++u)
-            mm[u] = (q0 + 32 * u < nq) ? quad_hits(sm, sbits, gbm, c[u], first) & live : 0u;
-          gather_step<PULL_STEP>(d, c, mm, sum, smf, sf);
-        } else {
-#pragma unroll
-          for (int u = 0; u < PULL_STEP; ++u)  // (q0 + 32 u < nq is warp-uniform)
-            if (q0 + 32 * u < nq) scan_quad<SR, FMT>(d, sm, sbits, gbm, c[u], make_int4(0, 0, 0, 0), first, sum, live, smf, sf);
-        }
-        need = false;  // a row is done once visited or (not real) hit
-#pragma unroll
-        for (int r = 0; r < 4; ++r) need |= (live >> r & 1u) && (SR == SS_REAL || first[r] < 0);
-      }
-      // the largest original id among this lane's first hits of unvisited rows
-      RowAcc acc;
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        acc.best[r] = (first[r] >= 0 && (live >> r & 1u)) ? __ldg(d.perm + first[r]) : -1;
-        acc.sum[r] = sum[r];
-      }
-      // (a non-zero real sum implies a hit on a live row of the same lane)
-      const bool any_hit = (acc.best[0] >= 0) | (acc.best[1] >= 0) | (acc.best[2] >= 0) |
-                           (acc.best[3] >= 0);
-      if (__any_sync(SS_FULL_MASK, any_hit)) {  // lanes with equal lane mod Q share rows
-#pragma unroll
-        for (int off = Q; off < 32; off <<= 1)
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            acc.best[r] = max(acc.best[r], __shfl_xor_sync(SS_FULL_MASK, acc.best[r], off));
-            if (SR == SS_REAL) acc.sum[r] += __shfl_xor_sync(SS_FULL_MASK, acc.sum[r], off);
-          }
-      }
-      if (item.w >= 0) {  // SlimChunk: combine partial rows, the last arriving item post-processes
-        const size_t xo = (size_t)item.w * C + 4 * lane;
-        if (lane < Q) {
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            if (acc.best[r] >= 0) atomicMax(d.xpar + xo + r, acc.best[r]);
-            if (SR == SS_REAL && acc.sum[r] != 0.0f) atomicAdd(d.xacc + xo + r, acc.sum[r]);
-          }
-          __threadfence();
-        }
-        __syncwarp();
-        int last = 0;
-        if (lane == 0) {
-          const unsigned old = atomicAdd(d.arrive + item.w, 1u);
-          last = (old == (unsigned)d.split_n[item.w] - 1u);
-        }
-        last = __shfl_sync(SS_FULL_MASK, last, 0);
-        if (!last) continue;
-        __threadfence();
-        if (lane < Q) {
-          // one 16-byte read and reset per array (xo is a multiple of 4 and the
-          // scratch 16-byte aligned); the per-row scalar form of this rarely run
-          // block made the whole real-semiring kernel 20-25 % slower on GB300
-          const int4 b4 = __ldcg(reinterpret_cast<const int4*>(d.xpar + xo));
-          *reinterpret_cast<int4*>(d.xpar + xo) = make_int4(-1, -1, -1, -1);
-          acc.best[0] = b4.x; acc.best[1] = b4.y; acc.best[2] = b4.z; acc.best[3] = b4.w;
-          if (SR == SS_REAL) {
-            const float4 s4 = __ldcg(reinterpret_cast<const float4*>(d.xacc + xo));
-            *reinterpret_cast<float4*>(d.xacc + xo) = make_float4(0.f, 0.f, 0.f, 0.f);
-            acc.sum[0] = s4.x; acc.sum[1] = s4.y; acc.sum[2] = s4.z; acc.sum[3] = s4.w;
-          }
-        }
-        if (lane == 0) d.arrive[item.w] = 0u;
-      }
-      // (a chunk that the groups started is counted already, and has new rows)
-      if (lane == 0 && !(SR != SS_REAL && item.w < 0)) cnt.act += 1;
-      post_chunk<SR, C>(d, k, chunk, lane, live, vis, acc, cnt, true, __shfl_sync(SS_FULL_MASK, my_new, src));
-    }
+    pull_whole<SR, C, FMT, false, true>(d, k, gbm, sg, todo, my_item, my_start, my_vis, cnt, grouped, my_new);
   }
-  cnt.slots = lane_slots;
+}
+
+template <int SR, int C>
+__global__ void __launch_bounds__(FILTERED_THREADS, 1) k_pull_filtered(Dev d, int variant,
+                                                                       cudaGraphConditionalHandle cond,
+                                                                       int use_cond) {
+  if (d.ctl->done) return;
+  const int k = d.ctl->k;
+  const unsigned* gbm = d.fb[(k - 1) & 1];
+  const Staged sg = stage_frontier<SR>(d, gbm);
+  const bool many_hits = frontier_hits_soon(d, d.ctl);
+  stage_wait();
+  const int wid = blockIdx.x * (FILTERED_THREADS / 32) + (threadIdx.x >> 5);
+  const int nw = gridDim.x * (FILTERED_THREADS / 32);
+  Counters cnt;
+  if (SR != SS_REAL && many_hits) pull_groups<SR, C>(d, k, gbm, sg, wid, nw, cnt);
+  else pull_items<SR, C, SS_FORMAT_SLIMSELL, false, true>(d, k, false, gbm, sg, wid, nw, cnt);
   finish_iteration_block<FILTERED_THREADS>(d, cnt.nw, cnt.deg, cnt.slots, cnt.act, cnt.maxdeg,
-                                       IterLaunch{variant, cond, use_cond});
+                                           IterLaunch{variant, cond, use_cond});
 }
 
 // Start of a run, thread t0 of `stride`: nothing visited but the root row (none if

@@ -242,6 +242,12 @@ __device__ __forceinline__ void compute_features(const Dev& d, const Ctl* c, flo
   features_of(d, c->k, c->prev_new, c->prev_deg, c->reached, c->reached_deg, c->prev_maxdeg, c->prev2_new, f);
 }
 
+// The frontier's rows hold a good share (a fifth) of all edges: a row's first frontier
+// neighbour comes within a few columns.
+__device__ __forceinline__ bool frontier_hits_soon(const Dev& d, const Ctl* c) {
+  return 5ull * c->prev_deg >= (unsigned long long)d.nnz;
+}
+
 // Write the features of iteration k into d.feats (one thread).
 __device__ __forceinline__ void store_features(const Dev& d, int k, const float* f) {
   if (k >= d.iter_cap) return;

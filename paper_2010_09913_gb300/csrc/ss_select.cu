@@ -37,7 +37,7 @@ static_assert(N_PARAMS % 4 == 0, "weights are staged as float4");
 // with 50 % 84 / 80; ER 4 M with 26 % 375 / 230, with 2 % 328 / 360; ER 300 K with
 // 14 % 20 / 25, with 76 % 20 / 16.
 __device__ __forceinline__ int pull_variant(const Dev& d, const Ctl* c) {
-  return 5ull * c->prev_deg >= (unsigned long long)d.nnz ? VAR_FILTERED : VAR_SLIMWORK;
+  return frontier_hits_soon(d, c) ? VAR_FILTERED : VAR_SLIMWORK;
 }
 
 // Frontier-size rule (top-down / bottom-up switching with alpha = 14, beta = 24).
