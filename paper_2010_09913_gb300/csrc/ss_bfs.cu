@@ -1450,7 +1450,7 @@ ss_status add_loop_node(slimsell_graph* h, const Dev& d, int sr, int policy, cud
   cudaGraphNodeParams sp = {};
   e = cudaGraphConditionalHandleCreate(&csw, body, 0, 0);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGraphConditionalHandleCreate(switch)");
-  ss_status s = add_decide_node(h, d, policy, csw, cw, body, &dnode);
+  ss_status s = add_decide_node(h, d, sr, policy, csw, cw, body, &dnode);
   if (s != SS_OK) return s;
   sp.type = cudaGraphNodeTypeConditional;
   sp.conditional.handle = csw;
@@ -1638,7 +1638,7 @@ ss_status slimsell_bfs(slimsell_handle h, int32_t root, int32_t semiring, int32_
         return SS_ERR_CUDA;
       }
       for (int j = 0; j < QUEUE_BATCH; ++j) {
-        ss_status s = launch_decide(h, d, policy, 0, 0, st);  // logs the iteration's features
+        ss_status s = launch_decide(h, d, semiring, policy, 0, 0, st);  // logs the iteration's features
         if (s != SS_OK) return s;
         if (prof) SS_CUDA(cudaEventRecord(h->evq[2 * j], st));
         s = launch_variant(h, d, semiring, policy, IterLaunch{policy, 0, 0}, st);
@@ -1666,7 +1666,7 @@ ss_status slimsell_bfs(slimsell_handle h, int32_t root, int32_t semiring, int32_
         return SS_ERR_CUDA;
       }
       // the decide kernel logs the iteration's features; adaptive policies read its choice
-      ss_status s = launch_decide(h, d, policy, 0, 0, st);
+      ss_status s = launch_decide(h, d, semiring, policy, 0, 0, st);
       if (s != SS_OK) return s;
       int variant = policy;
       if (adaptive(policy)) {

@@ -31,25 +31,35 @@ static_assert(N_PARAMS % 4 == 0, "weights are staged as float4");
 
 // The pull of a level: stopping rows at their first hit pays when hits come within
 // a few columns, that is when the frontier's rows hold a good share of all edges;
-// with few hits the filtered pass reads most slots anyway, in shorter steps than the
+// with few hits the filtered pass reads most slots anyway, with fewer warps than the
 // streaming pass.  SlimWork / filtered, us: Kronecker 22 with 8 % of the edges
-// 139 / 184, with 89 % 59 / 45; Kronecker 24 with 7 % 563 / 756; Kronecker 20 (C = 16)
-// with 50 % 84 / 80; ER 4 M with 26 % 375 / 230, with 2 % 328 / 360; ER 300 K with
+// 139 / 179, with 89 % 74 / 48; Kronecker 24 with 7 % 563 / 756; Kronecker 20 (C = 16)
+// with 50 % 84 / 80; ER 4 M with 28 % 305 / 158, with 2 % 256 / 264; ER 300 K with
 // 14 % 20 / 25, with 76 % 20 / 16.
-__device__ __forceinline__ int pull_variant(const Dev& d, const Ctl* c) {
-  return frontier_hits_soon(d, c) ? VAR_FILTERED : VAR_SLIMWORK;
+// The real semiring's rows never stop: what the filtered pass saves there is the columns of
+// chunks whose lanes have no unvisited row, so it pays once few rows are left (ER 4 M with 97 %
+// reached 176 / 119, with 29 % 467 / 471; Kronecker 22 with 34 % 126 / 135, with 1 % 246 / 292,
+// with 71 % 57 / 62; ER 1 M with 63 % 61 / 70, with 79 % 57 / 65), and, for its finer grid, on
+// graphs whose streaming grid, a block per 128 items, leaves SMs idle (Kronecker 18 75 / 56;
+// ER 300 K 29 / 25).
+constexpr int REAL_FULL_GRID_ITEMS = 128 * 152;
+__device__ __forceinline__ int pull_variant(const Dev& d, const Ctl* c, int sr) {
+  const bool filtered = sr == SS_REAL && d.n_items >= REAL_FULL_GRID_ITEMS
+                            ? 8ull * c->reached >= 7ull * (unsigned long long)d.n_live
+                            : frontier_hits_soon(d, c);
+  return filtered ? VAR_FILTERED : VAR_SLIMWORK;
 }
 
 // Frontier-size rule (top-down / bottom-up switching with alpha = 14, beta = 24).
-__device__ int heuristic_variant(const Dev& d, const Ctl* c) {
+__device__ int heuristic_variant(const Dev& d, const Ctl* c, int sr) {
   const unsigned long long nf = c->prev_new, mf = c->prev_deg;
   const unsigned long long mu = (unsigned long long)d.nnz - c->reached_deg;
   if (c->prev_variant < 0) return VAR_PUSH;
   // a frontier the cluster push takes is cheaper there than in any grid-wide pass
   if (local_fits(d, nf, mf)) return VAR_PUSH;
-  if (c->prev_variant == VAR_PUSH || c->prev_variant == VAR_PUSH_LOCAL) return (14ull * mf > mu) ? pull_variant(d, c) : VAR_PUSH;
+  if (c->prev_variant == VAR_PUSH || c->prev_variant == VAR_PUSH_LOCAL) return (14ull * mf > mu) ? pull_variant(d, c, sr) : VAR_PUSH;
   const bool shrinking = c->prev_new < c->prev2_new;
-  return (24ull * nf < (unsigned long long)d.n && shrinking) ? VAR_PUSH : pull_variant(d, c);
+  return (24ull * nf < (unsigned long long)d.n && shrinking) ? VAR_PUSH : pull_variant(d, c, sr);
 }
 
 __device__ __forceinline__ bool push_fits(const Dev& d, const Ctl* c) {
@@ -61,7 +71,7 @@ __device__ __forceinline__ bool push_fits(const Dev& d, const Ctl* c) {
 // device-side loop it also ends the loop (WHILE condition 0) if the run is
 // already done or has looped more than n + 2 times, so termination never
 // depends on a later kernel.
-__global__ void __launch_bounds__(DECIDE_THREADS) k_decide(Dev d, int policy, cudaGraphConditionalHandle sw,
+__global__ void __launch_bounds__(DECIDE_THREADS) k_decide(Dev d, int sr, int policy, cudaGraphConditionalHandle sw,
                                                             int use_sw, cudaGraphConditionalHandle cw,
                                                             int use_cw) {
   __shared__ float x[F_IN], h1[F_H], h2[F_H], y[F_OUT];
@@ -105,7 +115,7 @@ __global__ void __launch_bounds__(DECIDE_THREADS) k_decide(Dev d, int policy, cu
       case SS_V_SLIMWORK: v = VAR_SLIMWORK; break;
       case SS_V_PUSH: v = VAR_PUSH; break;
       case SS_V_PULL_FILTERED: v = VAR_FILTERED; break;
-      default: v = heuristic_variant(d, c); break;
+      default: v = heuristic_variant(d, c, sr); break;
     }
     choice = v;
   }
@@ -156,20 +166,20 @@ __global__ void __launch_bounds__(DECIDE_THREADS) k_decide(Dev d, int policy, cu
   }
 }
 
-ss_status launch_decide(const slimsell_graph* h, const Dev& d, int policy,
+ss_status launch_decide(const slimsell_graph* h, const Dev& d, int sr, int policy,
                         cudaGraphConditionalHandle sw, int use_sw, cudaStream_t st) {
-  k_decide<<<1, DECIDE_THREADS, 0, st>>>(d, policy, sw, use_sw, 0, 0);
+  k_decide<<<1, DECIDE_THREADS, 0, st>>>(d, sr, policy, sw, use_sw, 0, 0);
   SS_CUDA(cudaGetLastError());
   return SS_OK;
 }
 
-ss_status add_decide_node(const slimsell_graph* h, const Dev& d, int policy,
+ss_status add_decide_node(const slimsell_graph* h, const Dev& d, int sr, int policy,
                           cudaGraphConditionalHandle sw, cudaGraphConditionalHandle cw,
                           cudaGraph_t g, cudaGraphNode_t* out) {
   Dev dd = d;
-  int pol = policy, use = 1, usew = 1;
+  int semiring = sr, pol = policy, use = 1, usew = 1;
   cudaGraphConditionalHandle hs = sw, hw = cw;
-  void* args[] = {&dd, &pol, &hs, &use, &hw, &usew};
+  void* args[] = {&dd, &semiring, &pol, &hs, &use, &hw, &usew};
   cudaKernelNodeParams kp = {};
   kp.func = (void*)k_decide;
   kp.gridDim = dim3(1);
