@@ -158,8 +158,20 @@ __global__ void k_multi_root_levels(MultiDev m) {
     m.dist[(long long)m.roots[s] * m.k + s] = 0;
 }
 
+// Resident blocks asked of the compiler (0: its choice) so that MULTI_BATCH columns stay in
+// flight: left alone, it gave the plane form of some shapes fewer registers than the loads
+// take and a spill (64 sources in chunks of 64: 32 registers; Kronecker 20 in items of 1024
+// columns 2407 us, 1247 with 40; 128 sources there 1869 us, 1504 with 64; in chunks of 32
+// on G(1 M, 8n) 1071 us, 1031).  Writing distances at once they were 40 to 48 from the start.
+template <int C, int W, bool PLANES>
+__host__ __device__ constexpr int multi_blocks() {
+  if (!PLANES) return 0;
+  if (C == 64 && W == 2) return 8;
+  return C * W == 64 ? 24 : 0;
+}
+
 template <int C, int W, bool SLIMWORK, bool PLANES>
-__global__ void __launch_bounds__(C * W) k_multi_pull(MultiDev m, IterLaunch il) {
+__global__ void __launch_bounds__(C * W, multi_blocks<C, W, PLANES>()) k_multi_pull(MultiDev m, IterLaunch il) {
   constexpr int T = C * W;
   const Dev& d = m.d;
   Ctl* c = d.ctl;
