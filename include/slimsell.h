@@ -110,7 +110,8 @@ typedef struct {
   int64_t reached_degree;  /* sum of their degrees = 2 * edges in the component       */
   int64_t slots;           /* total col slots read                                    */
   int64_t dp_slots;        /* col slots read by the DP pass (0 for sel-max)           */
-  double iter_kernel_ms;   /* CUDA-event time of the iteration kernels (if profiling) */
+  double iter_kernel_ms;   /* CUDA-event time of the iteration kernels, those that write a
+                              multi-source run's distances included (if profiling)    */
   double total_ms;         /* CUDA-event time of the whole call (if profiling)        */
 } ss_run_stats;
 

@@ -1072,8 +1072,18 @@ extern "C" ss_status slimsell_bfs_multi_parents(slimsell_handle h, const int32_t
     }
     const bool done = h->h_ctl->done != 0;
     h->multi_dense = multi_dense(h);
-    if (m.planes && (done || (it + 1) % MULTI_EPOCH == 0))
+    if (m.planes && (done || (it + 1) % MULTI_EPOCH == 0)) {
+      if (prof) SS_CUDA(cudaEventRecord(h->ev_a, st));
       if ((s = write_levels(h, m, W, (int)(it + 1), !done, st)) != SS_OK) return s;
+      if (prof) {  // the epoch's distance writes are work of its last level
+        SS_CUDA(cudaEventRecord(h->ev_b, st));
+        SS_CUDA(cudaEventSynchronize(h->ev_b));
+        float ms = 0.f;
+        SS_CUDA(cudaEventElapsedTime(&ms, h->ev_a, h->ev_b));
+        iter_ms += ms;
+        h->iter_ns.back() += (int)(ms * 1.0e6f);
+      }
+    }
     if (done) break;
   }
   if (prof) SS_CUDA(cudaEventRecord(h->ev_d, st));
