@@ -642,7 +642,7 @@ void free_handle(slimsell_graph* h) {
   if (!h) return;
   ab_release(h);
   bc_release(h);
-  void* ptrs[] = {h->slab[0], h->slab[1], h->mlp, h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots, h->mplanes};
+  void* ptrs[] = {h->slab[0], h->slab[1], h->mlp, h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots, h->mplanes[0], h->mplanes[1]};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->h_ctl) cudaFreeHost(h->h_ctl);

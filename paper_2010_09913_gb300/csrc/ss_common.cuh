@@ -186,7 +186,7 @@ struct slimsell_graph {
   unsigned long long* mV = nullptr;
   unsigned long long* mxacc = nullptr;
   int* mroots = nullptr;
-  unsigned long long* mplanes = nullptr;  // level planes of the multi-source distances
+  unsigned long long* mplanes[2] = {nullptr, nullptr};  // level planes of the multi-source distances (short, long epochs)
   bool multi_dense = false;               // the next level's frontier holds many edges (ss_multi.cu)
   int smem_bytes = SS_SMEM_MAX_BYTES;  // bitmap prefix staged in shared memory
   int dp_pass = 0;                     // 1: parents by a separate DP pass after the iterations

@@ -345,8 +345,9 @@ struct MultiDev {
   unsigned long long* V;
   unsigned long long* xacc;  // [n_split][C][W]
   int* dist;                 // [n][k] in original vertex order, or NULL
-  unsigned long long* planes;  // level bit planes (ss_multi.cu), plane_words words each, or NULL
+  unsigned long long* planes;  // level bit planes (ss_multi.cu) of plane_words words, or NULL
   long long plane_words;
+  int long_epoch;              // eight planes a word, not four
   int vec_dist;              // k % 4 == 0 and dist 16-byte aligned: 16-byte group writes
   const int* roots;          // [k]
   int k;

@@ -41,22 +41,32 @@ constexpr int MULTI_BATCH = SS_MULTI_BATCH;  // columns per thread in flight
 #define SS_MULTI_BLOCKS_PER_SM 0  // resident blocks per SM (0: as many as fit)
 #endif
 
-// Levels are kept as bit planes until the end of an epoch of MULTI_EPOCH levels: the
-// four planes of word (row, w), one 32-byte sector, hold the bits of the level (within
-// the epoch) at which the row entered each of the 64 sources' frontiers.
-// k_multi_levels then writes the distances in vertex order, a sector gathered per 64
-// entries.  Written at each discovery instead, into
-// an array first filled with -1, they were 16-byte read-modify-writes scattered over
-// the n x k output: 0.8 of the 2.5 ms of 64 sources on Kronecker 22 (0.64 in the
-// pulls, 0.16 the fill).
-constexpr int MULTI_PLANES = 4;
-constexpr int MULTI_EPOCH = (1 << MULTI_PLANES) - 1;
+// Levels are kept as bit planes until the end of an epoch of 2^P - 1 levels: the P
+// planes of word (row, w) hold the bits of the level (within the epoch) at which the row
+// entered each of the 64 sources' frontiers.  k_multi_levels then writes the distances in
+// vertex order.  Written at each discovery instead, into an array first filled with -1, they
+// were 16-byte read-modify-writes scattered over the n x k output: 0.8 of the 2.5 ms of
+// 64 sources on Kronecker 22 (0.64 in the pulls, 0.16 the fill).
+// The first epoch has four planes, a 32-byte sector a word, which most runs end in.  A longer
+// run goes on with eight in an array of their own, 255 levels an epoch: an epoch's end (the
+// writes, and the planes cleared) is 22 us on a 512^2 lattice, 3 to 4 % of a run of a thousand
+// levels that paid it every 15.  Where their memory is not to be had the epochs stay short.
+constexpr int MULTI_SHORT_PLANES = 4, MULTI_LONG_PLANES = 8;
+constexpr int MULTI_EPOCH = (1 << MULTI_SHORT_PLANES) - 1, MULTI_EPOCH_LONG = (1 << MULTI_LONG_PLANES) - 1;
+
+// How a level pass keeps its levels: not (written at once, or not wanted), in the planes of the
+// short first epoch, or in those of a long one.  A parameter of the kernels, each form with
+// its own code, as the gather loops' register allocation follows the slightest change of it.
+enum { KEEP_NOT = 0, KEEP_SHORT = 1, KEEP_LONG = 2 };
+template <int KEEP>
+__host__ __device__ constexpr int planes_of() { return KEEP == KEEP_LONG ? MULTI_LONG_PLANES : MULTI_SHORT_PLANES; }
 
 // Out of line, so that the gather loops' register allocation does not depend on it.
+template <int KEEP>
 __device__ __noinline__ void keep_levels(unsigned long long* planes, unsigned long long nb, int level) {
-  const int code = (level - 1) % MULTI_EPOCH + 1;
+  const int code = KEEP == KEEP_LONG ? (level - 1 - MULTI_EPOCH) % MULTI_EPOCH_LONG + 1 : (level - 1) % MULTI_EPOCH + 1;
 #pragma unroll
-  for (int i = 0; i < MULTI_PLANES; ++i)
+  for (int i = 0; i < planes_of<KEEP>(); ++i)
     if (code >> i & 1) planes[i] |= nb;
 }
 
@@ -90,20 +100,21 @@ __device__ __noinline__ void write_levels_vec(int* out, unsigned long long nb, u
   }
 }
 
-// Distances of an epoch (levels base + 1 .. base + MULTI_EPOCH) from its planes; the
+// Distances of an epoch (levels base + 1 on) from its P planes; the
 // first epoch writes every entry (-1 where nothing was found), later ones what they
 // found, and the planes are cleared for the next.  Sixteen lanes write the 64
 // entries of a vertex's word as 16-byte groups where the output allows it.  (In row
 // order the writes of 256 bytes went to scattered places: 347 us on Kronecker 22.)
+template <int P>
 __global__ void __launch_bounds__(256) k_multi_levels(MultiDev m, int W, int lgW, int base) {
   const Dev& d = m.d;
   const long long words = (long long)d.n << lgW;  // word i: word i & (W - 1) of vertex i >> lgW
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long groups = (long long)gridDim.x * blockDim.x >> 4;  // 16 lanes each
   const int g = (int)(t & 15);
-  constexpr int U = 4;  // words in flight per group
+  constexpr int U = 16 / P;  // words in flight per group
   for (long long w0 = t >> 4; w0 < words; w0 += U * groups) {
-    unsigned b[U][MULTI_PLANES], found[U];
+    unsigned b[U][P], found[U];
     int row[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -114,15 +125,16 @@ __global__ void __launch_bounds__(256) k_multi_levels(MultiDev m, int W, int lgW
     for (int u = 0; u < U; ++u) {
       found[u] = 0;
 #pragma unroll
-      for (int p = 0; p < MULTI_PLANES; ++p) b[u][p] = 0;
+      for (int p = 0; p < P; ++p) b[u][p] = 0;
       if (row[u] < d.n_live) {  // (rows without neighbours have no levels)
         const ulonglong2* q = reinterpret_cast<const ulonglong2*>(
-            m.planes + (((long long)row[u] << lgW) + ((w0 + u * groups) & (W - 1))) * MULTI_PLANES);
-        const ulonglong2 x = __ldg(q), y = __ldg(q + 1);
-        b[u][0] = (unsigned)(x.x >> (4 * g)) & 0xFu;
-        b[u][1] = (unsigned)(x.y >> (4 * g)) & 0xFu;
-        b[u][2] = (unsigned)(y.x >> (4 * g)) & 0xFu;
-        b[u][3] = (unsigned)(y.y >> (4 * g)) & 0xFu;
+            m.planes + (((long long)row[u] << lgW) + ((w0 + u * groups) & (W - 1))) * P);
+#pragma unroll
+        for (int p = 0; p < P; p += 2) {
+          const ulonglong2 x = __ldg(q + p / 2);
+          b[u][p] = (unsigned)(x.x >> (4 * g)) & 0xFu;
+          b[u][p + 1] = (unsigned)(x.y >> (4 * g)) & 0xFu;
+        }
       }
     }
 #pragma unroll
@@ -130,14 +142,14 @@ __global__ void __launch_bounds__(256) k_multi_levels(MultiDev m, int W, int lgW
       const long long word = w0 + u * groups;
       const int s0 = 64 * (int)(word & (W - 1)) + 4 * g;
 #pragma unroll
-      for (int p = 0; p < MULTI_PLANES; ++p) found[u] |= b[u][p];
+      for (int p = 0; p < P; ++p) found[u] |= b[u][p];
       if (word >= words || s0 >= m.k || (base > 0 && !found[u])) continue;
       int v[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         int code = 0;
 #pragma unroll
-        for (int p = 0; p < MULTI_PLANES; ++p) code |= (b[u][p] >> j & 1u) << p;
+        for (int p = 0; p < P; ++p) code |= (b[u][p] >> j & 1u) << p;
         v[j] = code ? base + code : -1;
       }
       int* out = m.dist + (word >> lgW) * m.k + s0;
@@ -163,15 +175,15 @@ __global__ void k_multi_root_levels(MultiDev m) {
 // take and a spill (64 sources in chunks of 64: 32 registers; Kronecker 20 in items of 1024
 // columns 2407 us, 1247 with 40; 128 sources there 1869 us, 1504 with 64; in chunks of 32
 // on G(1 M, 8n) 1071 us, 1031).  Writing distances at once they were 40 to 48 from the start.
-template <int C, int W, bool PLANES>
+template <int C, int W, int KEEP>
 __host__ __device__ constexpr int multi_blocks() {
-  if (!PLANES) return 0;
+  if (KEEP == KEEP_NOT) return 0;
   if (C == 64 && W == 2) return 8;
   return C * W == 64 ? 24 : 0;
 }
 
-template <int C, int W, bool SLIMWORK, bool PLANES>
-__global__ void __launch_bounds__(C * W, multi_blocks<C, W, PLANES>()) k_multi_pull(MultiDev m, IterLaunch il) {
+template <int C, int W, bool SLIMWORK, int KEEP>
+__global__ void __launch_bounds__(C * W, multi_blocks<C, W, KEEP>()) k_multi_pull(MultiDev m, IterLaunch il) {
   constexpr int T = C * W;
   const Dev& d = m.d;
   Ctl* c = d.ctl;
@@ -258,8 +270,8 @@ __global__ void __launch_bounds__(C * W, multi_blocks<C, W, PLANES>()) k_multi_p
       nw += (unsigned long long)pc;
       deg += (unsigned long long)pc * (unsigned long long)dv;
       maxdeg = max(maxdeg, (unsigned)dv);
-      if constexpr (PLANES) {
-        keep_levels(m.planes + (row * W + w) * MULTI_PLANES, nb, level);
+      if constexpr (KEEP != KEEP_NOT) {
+        keep_levels<KEEP>(m.planes + (row * W + w) * planes_of<KEEP>(), nb, level);
       } else if (m.dist) {
         int* out = m.dist + (long long)d.perm[row] * m.k + 64 * w;
         if (m.vec_dist) {
@@ -349,6 +361,7 @@ __device__ __forceinline__ void one_step(const unsigned* sm, int sbits, const un
 // New words of four rows (from R0): visited and frontier words, level planes,
 // counters; returns the bits of the rows that gained a source, *left = some row
 // still misses one.
+template <int KEEP>
 __device__ __forceinline__ unsigned one_post(const MultiDev& m, long long R0, int level,
                                              const unsigned long long acc[4], const unsigned long long V[4],
                                              unsigned long long* Fn, OneSum& sum, bool* left) {
@@ -379,13 +392,13 @@ __device__ __forceinline__ unsigned one_post(const MultiDev& m, long long R0, in
         sum.deg += (unsigned long long)pc * (unsigned long long)D[r];
         sum.rowdeg += (unsigned long long)D[r];
         sum.maxdeg = max(sum.maxdeg, (unsigned)D[r]);
-        if (m.planes) keep_levels(m.planes + (R0 + r) * MULTI_PLANES, nb[r], level);
+        if (m.planes) keep_levels<KEEP>(m.planes + (R0 + r) * planes_of<KEEP>(), nb[r], level);
       }
   }
   return nib;
 }
 
-template <int C, bool SLIMWORK>
+template <int C, bool SLIMWORK, int KEEP>  // (KEEP_SHORT also where no planes are kept)
 __global__ void __launch_bounds__(MULTI_ONE_THREADS, 1) k_multi_one(MultiDev m, IterLaunch il) {
   constexpr int Q = C / 4;
   const Dev& d = m.d;
@@ -464,7 +477,7 @@ __global__ void __launch_bounds__(MULTI_ONE_THREADS, 1) k_multi_one(MultiDev m, 
         for (int r = 0; r < 4; ++r) live |= (V[r] != ~0ull ? 1u : 0u) << r;
         unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
         one_step<MULTI_SHORT>(sm, sbits, FAp, Fp, q, live, acc);
-        nib = one_post(m, R0, level, acc, V, Fn, sum, &left);
+        nib = one_post<KEEP>(m, R0, level, acc, V, Fn, sum, &left);
         sum.quads += (unsigned)ncols;
         if (lq == 0) sum.act += 1;
       }
@@ -537,7 +550,7 @@ __global__ void __launch_bounds__(MULTI_ONE_THREADS, 1) k_multi_one(MultiDev m, 
       }
       unsigned nib = 0;
       bool left = false;
-      if (lane < Q) nib = one_post(m, R0, level, acc, V, Fn, sum, &left);
+      if (lane < Q) nib = one_post<KEEP>(m, R0, level, acc, V, Fn, sum, &left);
       const unsigned lo = __reduce_or_sync(SS_FULL_MASK, lane < 8 ? nib << (4 * lane) : 0u);
       const unsigned hi = C > 32 ? __reduce_or_sync(SS_FULL_MASK, (lane >= 8 && lane < 16) ? nib << (4 * (lane - 8)) : 0u) : 0u;
       const bool open = __any_sync(SS_FULL_MASK, left);
@@ -780,14 +793,15 @@ __global__ void __launch_bounds__(256) k_multi_par_scatter(MultiDev m, int W, in
 template <int C>
 static ss_status launch_multi_one(const slimsell_graph* h, const MultiDev& m, bool slimwork,
                                   const IterLaunch& il, cudaStream_t st) {
+  using Kernel = void (*)(MultiDev, IterLaunch);
+  static const Kernel kernels[4] = {k_multi_one<C, false, KEEP_SHORT>, k_multi_one<C, true, KEEP_SHORT>,
+                                    k_multi_one<C, false, KEEP_LONG>, k_multi_one<C, true, KEEP_LONG>};
   static std::atomic<unsigned long long> configured{0};
-  if (first_on_device(configured)) {
-    SS_CUDA(cudaFuncSetAttribute(k_multi_one<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM_LIMIT_BYTES));
-    SS_CUDA(cudaFuncSetAttribute(k_multi_one<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM_LIMIT_BYTES));
-  }
+  if (first_on_device(configured))
+    for (Kernel kern : kernels)
+      SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM_LIMIT_BYTES));
   const size_t smem = (size_t)(m.d.smem_words + SMEM_GUARD) * 4;
-  if (slimwork) k_multi_one<C, true><<<pull_grid(h), MULTI_ONE_THREADS, smem, st>>>(m, il);
-  else k_multi_one<C, false><<<pull_grid(h), MULTI_ONE_THREADS, smem, st>>>(m, il);
+  kernels[(slimwork ? 1 : 0) + (m.long_epoch ? 2 : 0)]<<<pull_grid(h), MULTI_ONE_THREADS, smem, st>>>(m, il);
   SS_CUDA(cudaGetLastError());
   return SS_OK;
 }
@@ -812,10 +826,11 @@ static ss_status launch_multi_cw(const slimsell_graph* h, const MultiDev& m, boo
       if (multi_one(h, m))
         return launch_multi_one<C>(h, m, slimwork, il, st);
     using Kernel = void (*)(MultiDev, IterLaunch);
-    static const Kernel kernels[4] = {k_multi_pull<C, W, false, false>, k_multi_pull<C, W, true, false>,
-                                      k_multi_pull<C, W, false, true>, k_multi_pull<C, W, true, true>};
-    static int grid[64][4];  // per device (zero: not measured yet)
-    const int which = (slimwork ? 1 : 0) + (m.planes ? 2 : 0);
+    static const Kernel kernels[6] = {k_multi_pull<C, W, false, KEEP_NOT>,   k_multi_pull<C, W, true, KEEP_NOT>,
+                                      k_multi_pull<C, W, false, KEEP_SHORT>, k_multi_pull<C, W, true, KEEP_SHORT>,
+                                      k_multi_pull<C, W, false, KEEP_LONG>,  k_multi_pull<C, W, true, KEEP_LONG>};
+    static int grid[64][6];  // per device (zero: not measured yet)
+    const int which = (slimwork ? 1 : 0) + (m.planes ? (m.long_epoch ? 4 : 2) : 0);
     int& g = grid[h->device & 63][which];
     if (!g) {
       int b = 0;
@@ -864,12 +879,12 @@ static bool multi_dense(const slimsell_graph* h) {
 // Multi-source scratch, grown on demand and kept with the handle.
 static ss_status ensure_multi_scratch(slimsell_graph* h, int W) {
   if (h->multi_w >= W) return SS_OK;
-  void* ptrs[] = {h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots, h->mplanes};
+  void* ptrs[] = {h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots, h->mplanes[0], h->mplanes[1]};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   h->mF[0] = h->mF[1] = h->mV = h->mxacc = nullptr;
   h->mroots = nullptr;
-  h->mplanes = nullptr;
+  h->mplanes[0] = h->mplanes[1] = nullptr;
   h->multi_w = 0;
   const size_t words = (size_t)h->n_pad * W;
   ss_status s;
@@ -883,27 +898,48 @@ static ss_status ensure_multi_scratch(slimsell_graph* h, int W) {
   return SS_OK;
 }
 
-// Level planes, allocated by the first call that wants distances.
-static ss_status ensure_multi_planes(slimsell_graph* h) {
-  if (h->mplanes) return SS_OK;
-  const ss_status s = dmalloc(h, (void**)&h->mplanes,
-                              sizeof(unsigned long long) * MULTI_PLANES * (size_t)h->n_pad * (size_t)h->multi_w);
-  if (s != SS_OK) cudaGetLastError();  // the caller does without; the launches' checks see nothing
-  return s;
+// Planes of the next epoch, cleared; allocated by the first call that wants them.
+// SS_ERR_OOM: the caller does with shorter epochs, or without.
+static ss_status next_planes(slimsell_graph* h, MultiDev* m, bool long_epoch, cudaStream_t st) {
+  const size_t planes = long_epoch ? MULTI_LONG_PLANES : MULTI_SHORT_PLANES;
+  unsigned long long*& p = h->mplanes[long_epoch ? 1 : 0];
+  if (!p) {
+    const ss_status s = dmalloc(h, (void**)&p, sizeof(unsigned long long) * planes * (size_t)h->n_pad * (size_t)h->multi_w);
+    if (s != SS_OK) {  // neither the launches' checks nor the user are to see it
+      cudaGetLastError();
+      set_error("");
+      return s;
+    }
+  }
+  m->planes = p;
+  m->long_epoch = long_epoch ? 1 : 0;
+  SS_CUDA(cudaMemsetAsync(p, 0, sizeof(unsigned long long) * planes * (size_t)m->plane_words, st));
+  return SS_OK;
 }
 
-// Write the distances of the epoch that ends with `level` (planes cleared for the next
-// epoch when more levels follow).
-static ss_status write_levels(const slimsell_graph* h, const MultiDev& m, int W, int level, bool more,
-                              cudaStream_t st) {
+// Whether the epoch under way ends with `level`, and the last level before it.
+static bool epoch_ends(const MultiDev& m, int level) {
+  return m.long_epoch ? (level - MULTI_EPOCH) % MULTI_EPOCH_LONG == 0 : level % MULTI_EPOCH == 0;
+}
+static int epoch_base(const MultiDev& m, int level) {
+  return m.long_epoch ? MULTI_EPOCH + (level - 1 - MULTI_EPOCH) / MULTI_EPOCH_LONG * MULTI_EPOCH_LONG
+                      : (level - 1) / MULTI_EPOCH * MULTI_EPOCH;
+}
+
+// Write the distances of the epoch that ends with `level`, and clear planes for the next one
+// when more levels follow.
+static ss_status write_levels(slimsell_graph* h, MultiDev* m, int W, int level, bool more, cudaStream_t st) {
   int lgW = 0;
   while ((1 << lgW) < W) ++lgW;
-  const int base = (level - 1) / MULTI_EPOCH * MULTI_EPOCH;
-  k_multi_levels<<<16 * h->num_sms, 256, 0, st>>>(m, W, lgW, base);
-  if (base == 0) k_multi_root_levels<<<(m.k + 255) / 256, 256, 0, st>>>(m);
+  const int base = epoch_base(*m, level);
+  if (m->long_epoch) k_multi_levels<MULTI_LONG_PLANES><<<16 * h->num_sms, 256, 0, st>>>(*m, W, lgW, base);
+  else k_multi_levels<MULTI_SHORT_PLANES><<<16 * h->num_sms, 256, 0, st>>>(*m, W, lgW, base);
+  if (base == 0) k_multi_root_levels<<<(m->k + 255) / 256, 256, 0, st>>>(*m);
   SS_CUDA(cudaGetLastError());
-  if (more) SS_CUDA(cudaMemsetAsync(m.planes, 0, sizeof(unsigned long long) * MULTI_PLANES * (size_t)m.plane_words, st));
-  return SS_OK;
+  if (!more) return SS_OK;
+  // (long epochs begin after the first short one or not at all)
+  const ss_status s = next_planes(h, m, m->long_epoch || level == MULTI_EPOCH, st);
+  return s == SS_ERR_OOM ? next_planes(h, m, false, st) : s;
 }
 
 // Level-by-level multi-source BFS for the passes built on it (betweenness
@@ -933,6 +969,7 @@ ss_status multi_start(slimsell_graph* h, const int32_t* d_roots, int k, cudaStre
   m->vec_dist = 0;
   m->planes = nullptr;
   m->plane_words = 0;
+  m->long_epoch = 0;
   m->roots = h->mroots;
   m->k = k;
   k_multi_init<<<8 * h->num_sms, 256, 0, st>>>(*m, W);
@@ -1011,9 +1048,10 @@ extern "C" ss_status slimsell_bfs_multi_parents(slimsell_handle h, const int32_t
   m.dist = d_dist;
   m.planes = nullptr;
   m.plane_words = (long long)h->n_pad * W;
-  if (d_dist && multi_planes(h, k, W) && ensure_multi_planes(h) == SS_OK) {
-    m.planes = h->mplanes;
-    SS_CUDA(cudaMemsetAsync(m.planes, 0, sizeof(unsigned long long) * MULTI_PLANES * (size_t)m.plane_words, st));
+  m.long_epoch = 0;
+  if (d_dist && multi_planes(h, k, W)) {
+    s = next_planes(h, &m, false, st);
+    if (s != SS_OK && s != SS_ERR_OOM) return s;
   }
   m.vec_dist = (k % 4 == 0) && ((reinterpret_cast<uintptr_t>(d_dist) & 15u) == 0);
   m.roots = h->mroots;
@@ -1072,9 +1110,9 @@ extern "C" ss_status slimsell_bfs_multi_parents(slimsell_handle h, const int32_t
     }
     const bool done = h->h_ctl->done != 0;
     h->multi_dense = multi_dense(h);
-    if (m.planes && (done || (it + 1) % MULTI_EPOCH == 0)) {
+    if (m.planes && (done || epoch_ends(m, (int)(it + 1)))) {
       if (prof) SS_CUDA(cudaEventRecord(h->ev_a, st));
-      if ((s = write_levels(h, m, W, (int)(it + 1), !done, st)) != SS_OK) return s;
+      if ((s = write_levels(h, &m, W, (int)(it + 1), !done, st)) != SS_OK) return s;
       if (prof) {  // the epoch's distance writes are work of its last level
         SS_CUDA(cudaEventRecord(h->ev_b, st));
         SS_CUDA(cudaEventSynchronize(h->ev_b));
