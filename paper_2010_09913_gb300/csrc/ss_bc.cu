@@ -143,12 +143,14 @@ struct BcVal<BC_FP64> {
   using T = double;
   T v = 0.0;
   static __device__ __forceinline__ T zero() { return 0.0; }
+  // (a skipped fp64 add frees the pipe, which an fp64 comparison would hold as long: eight of them
+  // to a group of gathers made lattices' levels 1.08 times slower)
   __device__ __forceinline__ void add(T x) {
-    if (x != 0.0) v += x;  // (a skipped fp64 add frees the pipe)
+    if (__double_as_longlong(x) != 0) v += x;
   }
   __device__ __forceinline__ void store(T* p) const { *p = v; }
   __device__ __forceinline__ unsigned long long merge(T* p) const {
-    if (v != 0.0) atomicAdd(p, v);
+    if (__double_as_longlong(v) != 0) atomicAdd(p, v);
     return 0ull;
   }
   __device__ __forceinline__ unsigned long long bits() const { return 0ull; }
