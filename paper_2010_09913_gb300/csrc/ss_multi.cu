@@ -173,12 +173,14 @@ __global__ void k_multi_root_levels(MultiDev m) {
 // Resident blocks asked of the compiler (0: its choice) so that MULTI_BATCH columns stay in
 // flight: left alone, it gave the plane form of some shapes fewer registers than the loads
 // take and a spill (64 sources in chunks of 64: 32 registers; Kronecker 20 in items of 1024
-// columns 2407 us, 1247 with 40; 128 sources there 1869 us, 1504 with 64; in chunks of 32
-// on G(1 M, 8n) 1071 us, 1031).  Writing distances at once they were 40 to 48 from the start.
+// columns 2407 us, 1247 with 40; 128 sources there 1869 us, 1504 with 64).  Two words in chunks
+// of 32 are worth 48: with 40 and a spill 100 sources on Kronecker 20 take 1029 us against
+// 1084, but 128 on a 512^2 lattice 39.3 ms against 36.1.
 template <int C, int W, int KEEP>
 __host__ __device__ constexpr int multi_blocks() {
   if (KEEP == KEEP_NOT) return 0;
   if (C == 64 && W == 2) return 8;
+  if (C == 32 && W == 2) return 20;
   return C * W == 64 ? 24 : 0;
 }
 
