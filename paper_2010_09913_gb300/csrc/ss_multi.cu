@@ -803,7 +803,9 @@ static ss_status launch_multi_one(const slimsell_graph* h, const MultiDev& m, bo
     for (Kernel kern : kernels)
       SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SMEM_LIMIT_BYTES));
   const size_t smem = (size_t)(m.d.smem_words + SMEM_GUARD) * 4;
-  kernels[(slimwork ? 1 : 0) + (m.long_epoch ? 2 : 0)]<<<pull_grid(h), MULTI_ONE_THREADS, smem, st>>>(m, il);
+  // every SM a block, as multi_one counts on (in pull_grid, a block per 128 items of 32 warps, G(400 K, 8n)
+  // gave 62 % of the SMs blocks: 529 us, 508 so)
+  kernels[(slimwork ? 1 : 0) + (m.long_epoch ? 2 : 0)]<<<h->num_sms, MULTI_ONE_THREADS, smem, st>>>(m, il);
   SS_CUDA(cudaGetLastError());
   return SS_OK;
 }
