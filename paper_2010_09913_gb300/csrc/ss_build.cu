@@ -444,12 +444,61 @@ static void launch_pack(const slimsell_graph* h, const int4* items, int n_items,
 // (hub chunks unsplit) are packed from a table of their own.
 constexpr int PACK_WIDTH = 1024;
 
+// The layout's tables, but for the work items and columns.
+static void add_tables(slimsell_graph* h, Slab& p) {
+  const size_t np = (size_t)h->n_pad;
+  p.add(&h->perm, np);
+  p.add(&h->invperm, (size_t)h->n);
+  p.add(&h->rdeg, np);
+  p.add(&h->cl, (size_t)h->n_c);
+  p.add(&h->cs, (size_t)h->n_c + 1);
+}
+
+// The BFS state whose size follows from n and nnz.
+static void add_state(slimsell_graph* h, Slab& p) {
+  const size_t np = (size_t)h->n_pad;
+  // bitmap words rounded up to whole int4 groups, plus one spare group
+  h->fb_words = (long long)((((np + 31) / 32) + 3) / 4 * 4 + 4);
+  h->units_cap = (long long)np + h->nnz / 256 + 1024;  // any frontier fits
+  h->iter_cap = 1 << 16;
+  p.add(&h->claim, np);
+  p.add(&h->vis, (size_t)h->fb_words);
+  p.add(&h->act, (size_t)h->n_c);
+  for (int b = 0; b < 2; ++b) p.add(&h->fb[b], (size_t)h->fb_words);
+  p.add(&h->fr, np);
+  p.add(&h->units, (size_t)h->units_cap);
+  p.add(&h->psum, np);
+  p.add(&h->touched, (size_t)h->fb_words);
+  p.add(&h->qcount, 1);
+  p.add(&h->ctl, 1);
+  p.add(&h->feats, SS_SELECTOR_FEATURES * (size_t)h->iter_cap);
+  p.add(&h->iters, (size_t)h->iter_cap);
+  p.add(&h->lstat, SS_LSTAT * (size_t)h->iter_cap);
+}
+
+static ss_status clear_state(slimsell_graph* h, cudaStream_t st) {
+  SS_CUDA(cudaMemsetAsync(h->psum, 0, sizeof(float) * (size_t)h->n_pad, st));
+  SS_CUDA(cudaMemsetAsync(h->touched, 0, sizeof(unsigned) * (size_t)h->fb_words, st));
+  SS_CUDA(cudaMemsetAsync(h->ctl, 0, sizeof(Ctl), st));
+  return SS_OK;
+}
+
+// The state of a handle whose build had no room for it beside the temporaries.
+static ss_status place_late_state(slimsell_graph* h, cudaStream_t st) {
+  Slab p;
+  add_state(h, p);
+  ss_status s = p.place(h, &h->slab[2]);
+  if (s == SS_OK) s = clear_state(h, st);
+  if (s != SS_OK) return s;
+  SS_CUDA(cudaStreamSynchronize(st));
+  return SS_OK;
+}
+
 static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const int* csr_col, void** temps,
                             cudaStream_t st) {
   const int n = h->n, C = h->C;
   const int n_c = h->n_c, n_pad = h->n_pad;
   const int grid = 8 * h->num_sms;
-  const size_t np = (size_t)n_pad;
   ss_status s;
 
   // temporaries (temps: allocations that the caller frees)
@@ -475,36 +524,25 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
     if ((s = t.place(nullptr, &temps[0])) != SS_OK) return s;
   }
 
-  // permanent arrays whose size follows from n and nnz: the layout's tables and the BFS state
-  // bitmap words rounded up to whole int4 groups, plus one spare group
-  h->fb_words = (long long)((((np + 31) / 32) + 3) / 4 * 4 + 4);
-  h->units_cap = (long long)np + h->nnz / 256 + 1024;  // any frontier fits
-  h->iter_cap = 1 << 16;
+  // permanent arrays whose size follows from n and nnz: the layout's tables and the BFS state,
+  // which waits for the temporaries to be gone where the device does not hold both
   {
     Slab p;
-    p.add(&h->perm, np);
-    p.add(&h->invperm, (size_t)n);
-    p.add(&h->rdeg, np);
-    p.add(&h->cl, (size_t)n_c);
-    p.add(&h->cs, (size_t)n_c + 1);
-    p.add(&h->claim, np);
-    p.add(&h->vis, (size_t)h->fb_words);
-    p.add(&h->act, (size_t)n_c);
-    for (int b = 0; b < 2; ++b) p.add(&h->fb[b], (size_t)h->fb_words);
-    p.add(&h->fr, np);
-    p.add(&h->units, (size_t)h->units_cap);
-    p.add(&h->psum, np);
-    p.add(&h->touched, (size_t)h->fb_words);
-    p.add(&h->qcount, 1);
-    p.add(&h->ctl, 1);
-    p.add(&h->feats, SS_SELECTOR_FEATURES * (size_t)h->iter_cap);
-    p.add(&h->iters, (size_t)h->iter_cap);
-    p.add(&h->lstat, SS_LSTAT * (size_t)h->iter_cap);
-    if ((s = p.place(h, &h->slab[0])) != SS_OK) return s;
+    add_tables(h, p);
+    add_state(h, p);
+    s = p.place(h, &h->slab[0]);
+    if (s == SS_OK) {
+      if ((s = clear_state(h, st)) != SS_OK) return s;
+    } else if (s == SS_ERR_OOM) {
+      cudaGetLastError();
+      set_error("");
+      h->claim = nullptr;
+      Slab q;
+      add_tables(h, q);
+      s = q.place(h, &h->slab[0]);
+    }
+    if (s != SS_OK) return s;
   }
-  SS_CUDA(cudaMemsetAsync(h->psum, 0, sizeof(float) * np, st));
-  SS_CUDA(cudaMemsetAsync(h->touched, 0, sizeof(unsigned) * (size_t)h->fb_words, st));
-  SS_CUDA(cudaMemsetAsync(h->ctl, 0, sizeof(Ctl), st));
 
   // 1. degrees and sort keys
   SS_CUDA(cudaMemsetAsync(flags, 0, 3 * sizeof(int), st));
@@ -642,7 +680,7 @@ void free_handle(slimsell_graph* h) {
   if (!h) return;
   ab_release(h);
   bc_release(h);
-  void* ptrs[] = {h->slab[0], h->slab[1], h->mlp, h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots, h->mplanes[0], h->mplanes[1]};
+  void* ptrs[] = {h->slab[0], h->slab[1], h->slab[2], h->mlp, h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots, h->mplanes[0], h->mplanes[1]};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->h_ctl) cudaFreeHost(h->h_ctl);
@@ -735,6 +773,7 @@ ss_status slimsell_build(const int64_t* d_row_ptr, const int32_t* d_col, int32_t
   if (s != SS_OK) cudaStreamSynchronize(st);  // queued work may still use the temporaries
   for (void* t : temps)
     if (t) cudaFree(t);
+  if (s == SS_OK && !h->claim) s = ss::place_late_state(h, st);
   if (s != SS_OK) {
     ss::free_handle(h);
     return s;

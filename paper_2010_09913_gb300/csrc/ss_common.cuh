@@ -148,7 +148,7 @@ struct slimsell_graph {
   int n_live = 0, n_busy = 0;
   int num_sms = 0;
   // device allocations of the layout and the BFS state: the arrays below lie in them
-  void* slab[2] = {nullptr, nullptr};
+  void* slab[3] = {nullptr, nullptr, nullptr};
   // layout
   int* perm = nullptr;
   int* invperm = nullptr;

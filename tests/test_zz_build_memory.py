@@ -1,0 +1,66 @@
+"""GPU: a build on a device whose free memory holds the layout with the build's temporaries, and
+the layout with the BFS state, but not all three: the state waits for the temporaries to be
+freed."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2010_09913_gb300 as ss
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _build():
+    ss.build()
+
+
+class Device:
+    """A graph of 2^25 vertices, a build and run of it, and the device filled beside them."""
+
+    def __init__(self):
+        n = self.n = 1 << 25  # about 28 bytes a vertex of temporaries, 24 of state, 12 of tables
+        row_ptr = np.zeros(n + 1, np.int64)
+        row_ptr[1:5] = [1, 3, 5, 6]
+        row_ptr[5:] = 6
+        self.rp = torch.from_numpy(row_ptr).cuda()
+        self.col = torch.tensor([1, 0, 2, 1, 3, 2], dtype=torch.int32, device="cuda")
+        self.out = torch.empty((2, n), dtype=torch.int32, device="cuda")
+        self.keep = []
+
+    def build(self):
+        return ss.SlimSellGraph(self.rp, self.col, C=32, sigma=None, split_w=256)
+
+    def run(self):
+        G, out = self.build(), self.out
+        G.bfs(0, "tropical", "slimwork", out[0], out[1])
+        torch.cuda.synchronize()
+        assert out[:, :5].cpu().tolist() == [[0, 1, 2, 3, -1], [0, 0, 1, 2, -1]] and int((out[0] >= 0).sum()) == 4
+        held = G.info().device_bytes
+        G.close()
+        torch.cuda.empty_cache()
+        return held
+
+    def leave(self, size):
+        """Fill the device up to `size` free bytes; what is free then."""
+        while True:
+            free = torch.cuda.mem_get_info()[0]
+            if free < size + (64 << 20):
+                return free
+            self.keep.append(torch.empty(min(free - size, 64 << 30) - (32 << 20), dtype=torch.uint8, device="cuda"))
+
+
+@pytest.fixture
+def device():
+    d = Device()
+    yield d
+    d.keep.clear()
+    torch.cuda.empty_cache()
+
+
+def test_state_waits_for_the_temporaries(device):
+    held = device.run()
+    free = device.leave(held + device.n * 12)  # the handle, and less than half of the temporaries
+    assert free < held + device.n * 24, (free, held)
+    assert device.run() == held
+    assert torch.cuda.mem_get_info()[0] >= free - (8 << 20)
