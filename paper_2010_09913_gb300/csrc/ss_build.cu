@@ -37,6 +37,7 @@ ss_status dmalloc(slimsell_graph* h, void** p, size_t bytes) {
   if (bytes == 0) bytes = 16;
   cudaError_t e = cudaMalloc(p, bytes);
   if (e != cudaSuccess) {
+    cudaGetLastError();  // the error is reported here, not by the next launch's check as well
     *p = nullptr;
     return cuda_fail(e, "cudaMalloc");
   }
@@ -534,7 +535,6 @@ static ss_status build_impl(slimsell_graph* h, const long long* row_ptr, const i
     if (s == SS_OK) {
       if ((s = clear_state(h, st)) != SS_OK) return s;
     } else if (s == SS_ERR_OOM) {
-      cudaGetLastError();
       set_error("");
       h->claim = nullptr;
       Slab q;

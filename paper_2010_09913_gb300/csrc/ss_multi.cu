@@ -909,9 +909,8 @@ static ss_status next_planes(slimsell_graph* h, MultiDev* m, bool long_epoch, cu
   unsigned long long*& p = h->mplanes[long_epoch ? 1 : 0];
   if (!p) {
     const ss_status s = dmalloc(h, (void**)&p, sizeof(unsigned long long) * planes * (size_t)h->n_pad * (size_t)h->multi_w);
-    if (s != SS_OK) {  // neither the launches' checks nor the user are to see it
-      cudaGetLastError();
-      set_error("");
+    if (s != SS_OK) {
+      set_error("");  // (the call goes on)
       return s;
     }
   }

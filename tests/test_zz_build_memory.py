@@ -64,3 +64,15 @@ def test_state_waits_for_the_temporaries(device):
     assert free < held + device.n * 24, (free, held)
     assert device.run() == held
     assert torch.cuda.mem_get_info()[0] >= free - (8 << 20)
+
+
+def test_out_of_memory_is_reported_once(device):
+    """A build that does not fit leaves nothing behind: no memory, and no error for the next."""
+    held = device.run()
+    free = device.leave(held // 2)
+    with pytest.raises(ss.SlimSellError):
+        device.build()
+    assert torch.cuda.mem_get_info()[0] >= free - (8 << 20)
+    device.keep.clear()
+    torch.cuda.empty_cache()
+    assert device.run() == held
