@@ -36,6 +36,10 @@ ss_status cuda_fail(cudaError_t e, const char* what) {
 ss_status dmalloc(slimsell_graph* h, void** p, size_t bytes) {
   if (bytes == 0) bytes = 16;
   cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && h && drop_planes(h)) {  // what a handle can do without goes first
+    cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();  // the error is reported here, not by the next launch's check as well
     *p = nullptr;

@@ -219,4 +219,5 @@ struct slimsell_graph {
 
 namespace ss {
 ss_status dmalloc(slimsell_graph* h, void** p, size_t bytes);
+bool drop_planes(slimsell_graph* h);  // give the multi-source level planes back; false: there were none
 }  // namespace ss

@@ -883,12 +883,12 @@ static bool multi_dense(const slimsell_graph* h) {
 // Multi-source scratch, grown on demand and kept with the handle.
 static ss_status ensure_multi_scratch(slimsell_graph* h, int W) {
   if (h->multi_w >= W) return SS_OK;
-  void* ptrs[] = {h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots, h->mplanes[0], h->mplanes[1]};
+  drop_planes(h);
+  void* ptrs[] = {h->mF[0], h->mF[1], h->mV, h->mxacc, h->mroots};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   h->mF[0] = h->mF[1] = h->mV = h->mxacc = nullptr;
   h->mroots = nullptr;
-  h->mplanes[0] = h->mplanes[1] = nullptr;
   h->multi_w = 0;
   const size_t words = (size_t)h->n_pad * W;
   ss_status s;
@@ -902,21 +902,41 @@ static ss_status ensure_multi_scratch(slimsell_graph* h, int W) {
   return SS_OK;
 }
 
+static size_t plane_bytes(const slimsell_graph* h, bool long_epoch) {
+  return sizeof(unsigned long long) * (long_epoch ? MULTI_LONG_PLANES : MULTI_SHORT_PLANES) * (size_t)h->n_pad *
+         (size_t)h->multi_w;
+}
+
+// The planes stay with the handle from call to call, but no other allocation of it fails for
+// them (dmalloc).
+bool drop_planes(slimsell_graph* h) {
+  bool any = false;
+  for (int i = 0; i < 2; ++i)
+    if (h->mplanes[i]) {
+      cudaFree(h->mplanes[i]);
+      h->mplanes[i] = nullptr;
+      h->device_bytes -= (long long)plane_bytes(h, i == 1);
+      any = true;
+    }
+  return any;
+}
+
 // Planes of the next epoch, cleared; allocated by the first call that wants them.
 // SS_ERR_OOM: the caller does with shorter epochs, or without.
 static ss_status next_planes(slimsell_graph* h, MultiDev* m, bool long_epoch, cudaStream_t st) {
-  const size_t planes = long_epoch ? MULTI_LONG_PLANES : MULTI_SHORT_PLANES;
   unsigned long long*& p = h->mplanes[long_epoch ? 1 : 0];
   if (!p) {
-    const ss_status s = dmalloc(h, (void**)&p, sizeof(unsigned long long) * planes * (size_t)h->n_pad * (size_t)h->multi_w);
+    const ss_status s = dmalloc(nullptr, (void**)&p, plane_bytes(h, long_epoch));
     if (s != SS_OK) {
       set_error("");  // (the call goes on)
       return s;
     }
+    h->device_bytes += (long long)plane_bytes(h, long_epoch);
   }
   m->planes = p;
   m->long_epoch = long_epoch ? 1 : 0;
-  SS_CUDA(cudaMemsetAsync(p, 0, sizeof(unsigned long long) * planes * (size_t)m->plane_words, st));
+  SS_CUDA(cudaMemsetAsync(p, 0, sizeof(unsigned long long) * (long_epoch ? MULTI_LONG_PLANES : MULTI_SHORT_PLANES) *
+                                    (size_t)m->plane_words, st));
   return SS_OK;
 }
 

@@ -1,10 +1,12 @@
-"""GPU: a build on a device whose free memory holds the layout with the build's temporaries, and
-the layout with the BFS state, but not all three: the state waits for the temporaries to be
-freed."""
+"""GPU: calls on a device that is nearly full: a build for which the device holds the layout with
+the build's temporaries, and the layout with the BFS state, but not all three; a build that
+does not fit; and a handle whose multi-source scratch must make room for other scratch."""
 import numpy as np
 import pytest
 import torch
 
+import graphgen as gg
+import oracle
 import paper_2010_09913_gb300 as ss
 
 pytestmark = pytest.mark.gpu
@@ -76,3 +78,32 @@ def test_out_of_memory_is_reported_once(device):
     device.keep.clear()
     torch.cuda.empty_cache()
     assert device.run() == held
+
+
+def test_level_planes_make_room_for_centrality(device):
+    """A multi-source run leaves its level planes with the handle; a centrality call whose scratch
+    does not fit beside them gets their memory, and the next multi-source run does without."""
+    g = gg.erdos_renyi(1 << 18, 12.0, seed=3)
+    G = ss.SlimSellGraph.from_host(g.row_ptr, g.col, C=32, sigma=g.n, split_w=256)
+    roots = torch.from_numpy(gg.roots(g, 1000, seed=4).astype(np.int32)).cuda()
+    src = gg.roots(g, 3, seed=5).astype(np.int32)
+    d_src = torch.from_numpy(src).cuda()
+    dist = torch.empty((g.n, 1000), dtype=torch.int32, device="cuda")
+    G.bfs_multi(roots, "slimwork", dist)
+    want = dist.clone()
+    planes = 32 * 16 * g.n  # 134 MB; the centrality scratch takes 1,536 bytes a row, 403 MB
+    torch.cuda.empty_cache()
+    held = G.info().device_bytes
+    free = device.leave(1536 * g.n - planes // 2)
+    assert free < 1536 * g.n
+    got = G.bc(d_src).cpu().numpy()
+    np.testing.assert_allclose(got, oracle.bc(g.row_ptr, g.col, src), rtol=1e-9, atol=1e-9 * got.max())
+    assert G.info().device_bytes < held + 1536 * g.n
+    dist.fill_(7)
+    G.bfs_multi(roots, "slimwork", dist)
+    device.keep.clear()
+    torch.cuda.empty_cache()
+    assert torch.equal(dist, want)
+    d = oracle.bfs_queue(g.row_ptr, g.col, int(roots[0]))
+    np.testing.assert_array_equal(dist[:, 0].cpu().numpy(), d)
+    G.close()
