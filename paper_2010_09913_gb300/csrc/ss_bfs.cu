@@ -1176,13 +1176,15 @@ static ss_status launch_filtered(const slimsell_graph* h, const Dev& d, const It
 // Graphs whose whole run goes into one launch (k_small): the fixed full and SlimWork
 // policies over SlimSell with the whole bitmap staged.  Where a run has the GPU to itself
 // that is a graph of up to SMALL_ROWS live rows (8 a thread of one CTA) and SMALL_DENSE_SLOTS
-// slots (what 16 CTAs stream in a few microseconds), whatever its layout, but for
-// layouts that are mostly padding, whose few long items leave most warps idle; and any
-// graph of up to SMALL_SLOTS slots.  One launch / grid-wide, SlimWork tropical, us a call that
-// is waited for:
+// slots (what 16 CTAs stream in a few microseconds) without items of more than SMALL_ITEM
+// slots, one of which would keep a warp busy for longer than the levels' launches take; and any
+// graph of up to SMALL_SLOTS slots.  One launch / grid-wide, SlimWork tropical, us a call
+// that is waited for:
 //   Kronecker 10 in chunks of 32 69 / 118, of 64 93 / 131, of 32 sorted in windows of 256 69 / 118;
 //   Kronecker 13 129 / 195, in chunks of 8 91 / 161; G(8 K, 8n) 82 / 165, G(8 K, 60n) 105 / 250;
-//   lattice 64^2 422 / 1202; Kronecker 11 unsorted in unsplit chunks of 64 (13 slots an edge) 465 / 413.
+//   lattice 64^2 422 / 1202; Kronecker 13 in chunks of 64 with items of 16 K slots 193 / 244, of
+//   64 K 402 / 388, of 150 K 742 / 616; Kronecker 10 there with one of 30 K 132 / 162, but sel-max
+//   over full passes 270 / 256, real 425 / 383, with items of 16 K 170 / 190 and 266 / 278.
 // It goes on to gain past SMALL_ROWS (lattice 128^2 823 / 1678, Kronecker 14 154 / 229), but the
 // adaptive policies do not run here, and from there on they, who scale, would lose to
 // plain SlimWork on small long-diameter graphs.
@@ -1205,6 +1207,7 @@ static ss_status launch_filtered(const slimsell_graph* h, const Dev& d, const It
 constexpr long long SMALL_SLOTS = SS_SMALL_SLOTS;                  // one run alone on the GPU
 constexpr int SMALL_ROWS = 8 << 10;
 constexpr long long SMALL_DENSE_SLOTS = 512 << 10;
+constexpr long long SMALL_ITEM = 16 << 10;
 constexpr long long SMALL_SLOTS_PER_CTA = SS_SMALL_SLOTS_PER_CTA;
 constexpr long long SMALL_BATCH_SLOTS = SS_SMALL_BATCH_SLOTS;      // many side by side
 constexpr long long SMALL_BATCH_MIN = SS_SMALL_BATCH_MIN;
@@ -1217,8 +1220,8 @@ static bool whole_run(const slimsell_graph* h, const Dev& d, int policy, long lo
          (long long)d.smem_words * 4 <= SS_SMEM_LIMIT_BYTES - 16 - (long long)sizeof(ItemCache) * PULL_THREADS;
 }
 static bool run_small(const slimsell_graph* h, const Dev& d, int policy) {
-  const bool rows = h->n_live <= SMALL_ROWS && h->slots <= 4 * h->nnz;
-  return whole_run(h, d, policy, rows ? SMALL_DENSE_SLOTS : SMALL_SLOTS);
+  const long long item = (long long)h->C * (h->split_w > 0 ? std::min(h->split_w, h->max_degree) : h->max_degree);
+  return whole_run(h, d, policy, h->n_live <= SMALL_ROWS && item <= SMALL_ITEM ? SMALL_DENSE_SLOTS : SMALL_SLOTS);
 }
 static size_t small_smem(const Dev& d) {
   return (size_t)(d.smem_words + SMEM_GUARD) * 4 + sizeof(ItemCache) * PULL_THREADS;

@@ -1,5 +1,5 @@
 """GPU: runs in one launch by the number of rows, on both sides of the limits (8,192 rows with
-a neighbour, 512 K slots, four slots an edge, 32 K slots), against the oracle and the
+a neighbour, 512 K slots, items of 16 K, 32 K slots), against the oracle and the
 grid-wide path (which the staged-prefix option forces)."""
 import numpy as np
 import pytest
@@ -30,7 +30,7 @@ GRAPHS = [gg.kronecker(10, seed=1), gg.kronecker(13, seed=2), gg.erdos_renyi(819
           with_isolated(gg.kronecker(11, seed=8), 3001)]
 
 
-@pytest.mark.parametrize("C,sigma,w", [(8, None, 64), (32, None, 256), (32, 256, 256), (64, 1, 4096)])
+@pytest.mark.parametrize("C,sigma,w", [(8, None, 64), (32, None, 256), (32, 256, 256), (64, 1, 4096), (64, None, 256)])
 @pytest.mark.parametrize("sr,policy", [("tropical", "slimwork"), ("real", "slimwork"), ("selmax", "full")])
 def test_runs_by_rows_match_oracle_and_grid(C, sigma, w, sr, policy):
     for g in GRAPHS:
