@@ -1219,9 +1219,12 @@ static bool whole_run(const slimsell_graph* h, const Dev& d, int policy, long lo
          h->slots <= max_slots && (long long)d.smem_words * 32 >= h->n_pad &&
          (long long)d.smem_words * 4 <= SS_SMEM_LIMIT_BYTES - 16 - (long long)sizeof(ItemCache) * PULL_THREADS;
 }
+static long long longest_item(const slimsell_graph* h) {  // slots
+  return (long long)h->C * (h->split_w > 0 ? std::min(h->split_w, h->max_degree) : h->max_degree);
+}
 static bool run_small(const slimsell_graph* h, const Dev& d, int policy) {
-  const long long item = (long long)h->C * (h->split_w > 0 ? std::min(h->split_w, h->max_degree) : h->max_degree);
-  return whole_run(h, d, policy, h->n_live <= SMALL_ROWS && item <= SMALL_ITEM ? SMALL_DENSE_SLOTS : SMALL_SLOTS);
+  const bool rows = h->n_live <= SMALL_ROWS && longest_item(h) <= SMALL_ITEM;
+  return whole_run(h, d, policy, rows ? SMALL_DENSE_SLOTS : SMALL_SLOTS);
 }
 static size_t small_smem(const Dev& d) {
   return (size_t)(d.smem_words + SMEM_GUARD) * 4 + sizeof(ItemCache) * PULL_THREADS;
@@ -1247,19 +1250,29 @@ int batch_ctas(const slimsell_graph* h, const Dev& d, int policy, long long batc
 // passes have the whole GPU, eight CTAs a twentieth of it; but a loop pays its launches, which
 // those of other loops queue behind (about 4 us a level and loop), and its grids wait for SMs
 // that clusters hold.  So the larger graphs run as clusters only where the batch's clusters,
-// those of graphs that earn a CTA or more (ctas), fill the GPU, or, for sparse graphs, whose
-// runs are many short levels, two fifths of it.  SlimWork, clusters / loops:
+// those of graphs that earn a CTA or more (ctas), fill the GPU, or two fifths of it where loops
+// are slow themselves: for sparse graphs, whose runs are many short levels, and for items past
+// SMALL_ITEM, whose one warp the rest of the GPU waits for (four fifths past eight times that,
+// which clusters are slow at too).  SlimWork, clusters / loops:
 //   Kronecker 16 (2.1 M slots) alone 202 us / 229, 17 (4.1 M) 261 / 192, 16 of 17 536 / 467, 64 1091 / 1648;
 //   G(60 K, 8n) (1 M) 175 / 181, G(120 K) (1.9 M) 271 / 188, 16 of it 535 / 476, 64 1056 / 1733;
 //   G(200 K) (3.2 M) 434 / 189, 16 of it 868 / 637, 64 1763 / 2363;
 //   lattice 300^2 (0.3 M) 2.3 ms / 3.6, 500^2 (0.9 M) 8.7 / 7.8, 16 of it 17.7 / 32.9,
 //   900^2 (3.1 M) 56 / 20, 4 of it 62 / 46, 16 of it 113 / 177;
-//   64 graphs of Kronecker 10 .. 17 (192 CTAs), all clusters 432 us, those of 17 in loops 503.
+//   64 graphs of Kronecker 10 .. 17 (192 CTAs), all clusters 432 us, those of 17 in loops 503;
+//   in chunks of 64 with items of 64 K slots, Kronecker 12 alone 287 / 281, 16 of it 422 / 731,
+//   of 260 K, 8 of Kronecker 15 1521 / 1280;
+//   finely split (items of 1 K slots) Kronecker 16 alone 200 / 168: past 1 M slots only graphs of
+//   longer items are clusters in any company.
 bool batch_small(const slimsell_graph* h, const Dev& d, int policy, long long ctas) {
   if (!whole_run(h, d, policy, SMALL_BATCH_SLOTS)) return false;
-  if (h->slots <= SMALL_BATCH_ALONE || h->n_live <= SMALL_BATCH_ROWS) return true;
-  const bool sparse = h->nnz < 8LL * h->n_live;
-  return ctas >= (sparse ? 2LL * h->num_sms / 5 : (long long)h->num_sms);
+  if (h->slots <= SMALL_BATCH_MIN) return true;
+  const long long item = longest_item(h);
+  if (item <= SMALL_ITEM && (h->slots <= SMALL_BATCH_ALONE ||
+                             (h->n_live <= SMALL_BATCH_ROWS && (h->slots <= 2 * SMALL_BATCH_ALONE || item >= SMALL_ITEM / 4))))
+    return true;
+  const int fifths = item > 8 * SMALL_ITEM ? 4 : item > SMALL_ITEM || h->nnz < 8LL * h->n_live ? 2 : 5;
+  return ctas >= (long long)fifths * h->num_sms / 5;
 }
 
 using SmallKernel = void (*)(Dev, SmallIo, int);

@@ -17,13 +17,16 @@ def _build():
     ss.build()
 
 
-@pytest.mark.parametrize("large,C", [("uniform", 32), ("lattice", 16)])
+@pytest.mark.parametrize("large,C", [("uniform", 32), ("lattice", 16), ("items", 64)])
 @pytest.mark.parametrize("copies,small", [(1, 0), (1, 30), (9, 3), (24, 2)])
 def test_routes_match_oracle(large, C, copies, small):
     # past the sizes that are a cluster in any company: 1.3 M slots, 80,000 rows; 0.6 M, 160,000
-    big = gg.erdos_renyi(80000, 16.0, seed=2) if large == "uniform" else gg.lattice(400, 0.05, seed=3)
+    # and items of more than 16 K slots
+    big = {"uniform": lambda: gg.erdos_renyi(80000, 16.0, seed=2), "lattice": lambda: gg.lattice(400, 0.05, seed=3),
+           "items": lambda: gg.kronecker(13, seed=4)}[large]()
+    w = 4096 if large == "items" else 256
     graphs = [big] * copies + [gg.kronecker(9, seed=40 + i) for i in range(small)]
-    Gs = [ss.SlimSellGraph.from_host(g.row_ptr, g.col, C=C, sigma=g.n, split_w=256) for g in graphs]
+    Gs = [ss.SlimSellGraph.from_host(g.row_ptr, g.col, C=C, sigma=g.n, split_w=w) for g in graphs]
     for sr in ("tropical", "selmax"):
         b = ss.slimsell_batch_create([G.h for G in Gs], ss.SEMIRINGS[sr], ss.V_SLIMWORK)
         roots = [int(gg.roots(g, copies + 1, seed=7)[i % copies]) for i, g in enumerate(graphs)]
