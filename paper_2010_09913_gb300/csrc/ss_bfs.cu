@@ -914,7 +914,7 @@ __device__ __forceinline__ void init_rows(const Dev& d, long long t0, long long 
 // bitmap, visited and value writes before the next level reads them (past L1), and
 // the counters travel through distributed shared memory, double-buffered by level
 // parity, so every thread takes the same exit.  Rank 0 keeps the control block in
-// shared memory and writes it back at the end.  Kronecker 10: 42 us; 64 graphs of scale
+// shared memory and writes it back at the end.  Kronecker 10: 39 us; 64 graphs of scale
 // 10 .. 17 in one batch 0.35 ms, 1.65 with a conditional loop of launches each.
 template <int SR, int C>
 __global__ void __launch_bounds__(PULL_THREADS, 1) k_small(Dev d, SmallIo io, int policy) {
